@@ -33,6 +33,7 @@
 #include <mutex>
 #include <tuple>
 
+#include "proj_finish.cuh"
 #include "tc_project.h"
 
 namespace tdb {
@@ -626,358 +627,6 @@ __global__ void k_selftest_mbar(unsigned* flags, long long limit) {
   __syncthreads();
 }
 
-// Finish, first launch.  The fused kernel leaves partial first contractions over the
-// tiles q of the contracted mode: Z1p at e + n1 (s + S q), e = i2 + N2 a, n1 = r1 N2
-// (mode 1 contracted), and Z2p at f + n2 (s + S q), f = i1 + N1 b, n2 = N1 r2 (mode 2
-// contracted), s the slice (i3 + N3 i4).  This launch sums them over q and contracts the
-// slices with B (S x J):
-//   Y_2[a + r1 (i2 + N2 j)] = sum_s Z1[e, s] B[s, j],    Y_1[f + n2 j] = sum_s Z2[f, s] B[s, j],
-// with B = A_3 (three modes), B[i3 + N3 i4, c + r3 d] = A_3[i3, c] A_4[i4, d] (four modes,
-// the Kronecker product that contracts modes 3 and 4 at once) or the 1 x 1 identity (two
-// modes).  It also writes Z1 = sum_q Z1p when there is more than one tile along mode 1
-// (the next launch forms Y_3 from it) and, in its first CTA, ||dV||_W^2 from the fused
-// kernel's per-CTA partials.  A CTA owns 256 elements of one side (a thread per element,
-// its slice values in registers) and one of `nsplit` slice ranges; the slices' rows of B
-// are staged in shared memory and read as float4 broadcasts, 32 outputs j at a time.
-// With nsplit > 1 each CTA writes its partial and k_tc_finish_red adds the partials of
-// every output in split order (so results do not vary from run to run).
-constexpr int FS_TE = 256, FS_SC = 16, FS_JB = 32, FS_JMAX = 128, FS_SPLIT_MAX = 32;
-constexpr int FS_CTAS = 2 * 152;   // split target: about two CTAs per SM
-constexpr int FS_NQ_MAX = 8;   // tiles along mode 1 or 2 loaded at once; more are added in order after them
-struct FinArgs {
-  const float* Z1p;
-  const float* Z2p;
-  int N1, N2, S, nq1, nq2, r1, r2;
-  const float* A3;       // N3 x r3 (null: two modes, B = [1])
-  const float* A4;       // N4 x r4 (null: three modes)
-  int N3, r3, N4, r4, J;
-  float* Z1;             // N2 x r1 x S, i2 fastest (written when nq1 > 1 and W is not fused)
-  // W = Z1 x_2 A_2^T (r1 x r2 x S: Y_3 for three modes) formed here when a first-side CTA
-  // holds whole i2 columns (te1 = N2 floor(256 / N2) elements, N2 <= 256)
-  float* W;
-  const float* A2;
-  int fuse_w, te1;
-  float* Y2;
-  float* Y1;
-  float* part;           // [tile][split][J][256]
-  int nsplit, nt1, nt2;
-  const double* npart;
-  int nnp;
-  unsigned long long* span;     // profiling words of the main kernel (see Params), or null
-  double* dv2;
-};
-
-// Row stride of A_2 in the fused finish's shared memory: = 4 (mod 32), so that the lanes
-// of a warp (eight columns b x four i2 phases) read 32 different banks.
-__host__ __device__ constexpr int a2_stride(int N2) { return N2 + ((36 - N2 % 32) % 32); }
-
-template <int NQ>   // tiles along the contracted mode, rounded up to a power of two (<= FS_NQ_MAX)
-__global__ void __launch_bounds__(FS_TE, 2) k_tc_finish_sk(FinArgs f) {
-  constexpr int SC = NQ <= 2 ? FS_SC : (NQ == 4 ? FS_SC / 2 : FS_SC / 4);   // slices per chunk
-  constexpr int BPT = FS_SC * FS_JMAX / FS_TE;      // B values a thread stages per chunk
-  extern __shared__ __align__(16) float fs_sm[];    // B rows of a slice chunk: [FS_SC][Jp]
-  __shared__ double dsh[32];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) grid_dep_launch();
-  const int tile = blockIdx.x / f.nsplit, sp = blockIdx.x % f.nsplit;
-  const bool first = tile < f.nt1;
-  const bool fw = first && f.fuse_w;
-  const int Jp0 = (f.J + 3) & ~3;
-  float* zs = fs_sm + FS_SC * Jp0;                     // fw: the chunk's z values [FS_SC][FS_TE]
-  float* a2s = zs + FS_SC * FS_TE;                     // fw: A_2 (N2 x r2, ld a2_stride(N2))
-  const int a2st = a2_stride(f.N2);
-  if (fw) {
-    // A_2 is an input of the step (not written by the main kernel): staged before the wait
-    for (int i0 = tid; i0 < f.N2 * f.r2; i0 += 4 * FS_TE) {
-      float v[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = i0 + k * FS_TE < f.N2 * f.r2 ? __ldg(&f.A2[i0 + k * FS_TE]) : 0.f;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int idx = i0 + k * FS_TE;
-        if (idx < f.N2 * f.r2) a2s[idx % f.N2 + a2st * (idx / f.N2)] = v[k];
-      }
-    }
-  }
-  // programmatic launch: the main kernel's results (partials, norms, span words) are
-  // complete and visible after this
-  grid_dep_wait();
-  if (blockIdx.x == gridDim.x - 1) {
-    // ||dV||_W^2: the main kernel's partials, eight loads in flight per thread (in the last
-    // CTA, a second-side one whenever there is one: those form no W)
-    double t = 0.0;
-    for (int i0 = tid; i0 < f.nnp; i0 += 8 * FS_TE) {
-      double v[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = i0 + k * FS_TE < f.nnp ? __ldcg(&f.npart[i0 + k * FS_TE]) : 0.0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) t += v[k];
-    }
-    t = block_sum(t, dsh);
-    if (tid == 0) *f.dv2 = t;
-    if (tid == 0 && f.span) {
-      // the main kernel has completed: its span into the sums, the words reset for the next
-      const unsigned long long a = f.span[0], b = f.span[1];
-      if (b > a) {
-        f.span[2] += b - a;
-        f.span[3] += 1;
-      }
-      f.span[0] = ~0ull;
-      f.span[1] = 0ull;
-    }
-  }
-  const int64_t ne = first ? (int64_t)f.r1 * f.N2 : (int64_t)f.N1 * f.r2;
-  const int te = first ? f.te1 : FS_TE;                // elements per CTA on this side
-  const int64_t e = (int64_t)(first ? tile : tile - f.nt1) * te + tid;
-  const bool in = tid < te && e < ne;
-  const int na = fw ? te / f.N2 : 0;                   // a1 values this CTA holds whole
-  const int a1_lo = fw ? tile * na : 0;
-  const int nq = first ? f.nq1 : f.nq2;
-  const float* Pp = (first ? f.Z1p : f.Z2p) + (in ? e : 0);
-  const bool write_z = first && f.nq1 > 1 && !f.fuse_w;
-  const int J = f.J, Jp = (J + 3) & ~3;
-  const int s_lo = (int)((int64_t)f.S * sp / f.nsplit), s_hi = (int)((int64_t)f.S * (sp + 1) / f.nsplit);
-  const int64_t qstride = ne * (int64_t)f.S;
-  float* mine = f.part + ((int64_t)tile * f.nsplit + sp) * (int64_t)J * FS_TE;
-  auto store = [&](int64_t ee, int j, float v) {
-    if (first) {
-      const int64_t a = ee / f.N2, i2 = ee - a * f.N2;
-      f.Y2[a + (int64_t)f.r1 * i2 + ne * (int64_t)j] = v;
-    } else {
-      f.Y1[ee + ne * (int64_t)j] = v;
-    }
-  };
-  for (int j0 = 0; j0 < J; j0 += FS_JB) {
-    const int jn = min(FS_JB, J - j0);
-    float acc[FS_JB];
-#pragma unroll
-    for (int t = 0; t < FS_JB; ++t) acc[t] = 0.f;
-    for (int s0 = s_lo; s0 < s_hi; s0 += SC) {
-      const int sc = min(SC, s_hi - s0);
-      // this element's slice values summed over q: every load of the chunk is issued
-      // into registers before the first addition
-      float raw[SC * NQ];
-#pragma unroll
-      for (int u = 0; u < SC; ++u) {
-        const float* pe = Pp + ne * (int64_t)(s0 + u);
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) raw[u * NQ + q] = (in && u < sc && q < nq) ? __ldcg(pe + qstride * q) : 0.f;
-      }
-      // this chunk's B rows, loaded beside the partials (staged in shared memory below)
-      float bpre[BPT];
-#pragma unroll
-      for (int k = 0; k < BPT; ++k) {
-        const int idx = tid + k * FS_TE;
-        float bv = 0.f;
-        if (idx < SC * Jp) {
-          const int sl = idx % SC, j = idx / SC;       // consecutive threads: consecutive slices
-          if (sl < sc && j < J) {
-            const int s = s0 + sl;
-            if (!f.A3) {
-              bv = 1.f;
-            } else if (!f.A4) {
-              bv = __ldg(&f.A3[s + (int64_t)f.N3 * j]);
-            } else {
-              const int i3 = s % f.N3, i4 = s / f.N3, c = j % f.r3, dd = j / f.r3;
-              bv = __ldg(&f.A3[i3 + (int64_t)f.N3 * c]) * __ldg(&f.A4[i4 + (int64_t)f.N4 * dd]);
-            }
-          }
-        }
-        bpre[k] = bv;
-      }
-      float z[SC];
-#pragma unroll
-      for (int u = 0; u < SC; ++u) {
-        float v = raw[u * NQ];
-#pragma unroll
-        for (int q = 1; q < NQ; ++q) v += raw[u * NQ + q];
-        if (NQ == FS_NQ_MAX && nq > NQ && in && u < sc) {
-          // a long mode (more than FS_NQ_MAX tiles): the rest in tile order
-          const float* pe = Pp + ne * (int64_t)(s0 + u);
-          for (int q = NQ; q < nq; ++q) v += __ldcg(pe + qstride * q);
-        }
-        z[u] = v;
-      }
-      if (write_z && j0 == 0 && in) {
-#pragma unroll
-        for (int u = 0; u < SC; ++u)
-          if (u < sc) f.Z1[e + ne * (int64_t)(s0 + u)] = z[u];
-      }
-      __syncthreads();                                   // the previous chunk is done with zs, fs_sm
-      if (fw && j0 == 0) {
-#pragma unroll
-        for (int u = 0; u < SC; ++u) zs[u * FS_TE + tid] = (in && u < sc) ? z[u] : 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < BPT; ++k) {
-        const int idx = tid + k * FS_TE;
-        if (idx < SC * Jp) fs_sm[(idx % SC) * Jp + idx / SC] = bpre[k];
-      }
-      __syncthreads();
-      if (fw && j0 == 0) {
-        // W[a1, a2, s] = sum_i2 Z1[i2, a1, s] A2[i2, a2] for this CTA's whole columns a1: a
-        // warp per (a1, eight a2, four slices); lane (b, phase) sums i2 = phase (mod 4) for
-        // the four slices side by side, then the four phases are added by shuffles
-        if ((f.N2 & 3) == 0) {
-          // whole float4 runs of i2: a thread per output (a1, slice, a2), a2 fastest, two
-          // chains (even and odd runs) added at the end
-          const int nout = na * sc * f.r2;
-          for (int o = tid; o < nout; o += FS_TE) {
-            const int b = o % f.r2, rest = o / f.r2, u = rest % sc, al = rest / sc;
-            const float4* zc = reinterpret_cast<const float4*>(zs + u * FS_TE + al * f.N2);
-            const float4* ac = reinterpret_cast<const float4*>(a2s + a2st * b);
-            float w0 = 0.f, w1 = 0.f;
-            const int nq4 = f.N2 >> 2;
-            int q = 0;
-#pragma unroll 2
-            for (; q + 1 < nq4; q += 2) {
-              const float4 z0 = zc[q], a0 = ac[q], z1 = zc[q + 1], a1v = ac[q + 1];
-              w0 = fmaf(z0.x, a0.x, w0); w0 = fmaf(z0.y, a0.y, w0); w0 = fmaf(z0.z, a0.z, w0); w0 = fmaf(z0.w, a0.w, w0);
-              w1 = fmaf(z1.x, a1v.x, w1); w1 = fmaf(z1.y, a1v.y, w1); w1 = fmaf(z1.z, a1v.z, w1); w1 = fmaf(z1.w, a1v.w, w1);
-            }
-            if (q < nq4) {
-              const float4 z0 = zc[q], a0 = ac[q];
-              w0 = fmaf(z0.x, a0.x, w0); w0 = fmaf(z0.y, a0.y, w0); w0 = fmaf(z0.z, a0.z, w0); w0 = fmaf(z0.w, a0.w, w0);
-            }
-            const int a1 = a1_lo + al;
-            if (a1 < f.r1) f.W[a1 + (int64_t)f.r1 * (b + (int64_t)f.r2 * (s0 + u))] = w0 + w1;
-          }
-        } else {
-          const int nbg = (f.r2 + 7) >> 3, nug = (sc + 3) >> 2;
-          const int nitem = na * nbg * nug;
-          const int bl = lane & 7, ph = lane >> 3;
-          for (int item = warp; item < nitem; item += FS_TE / 32) {
-            const int bg = item % nbg, rest = item / nbg, al = rest % na, u0 = 4 * (rest / na);
-            const int b = bg * 8 + bl;
-            const float* zc = zs + u0 * FS_TE + al * f.N2;
-            const float* ac = a2s + a2st * (b < f.r2 ? b : f.r2 - 1);
-            float w[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-            for (int i2 = ph; i2 < f.N2; i2 += 4) {
-              const float av = ac[i2];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) w[u] = fmaf(zc[u * FS_TE + i2], av, w[u]);
-            }
-            const int a1 = a1_lo + al;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              float x = w[u];
-              x += __shfl_xor_sync(0xffffffffu, x, 8);
-              x += __shfl_xor_sync(0xffffffffu, x, 16);
-              if (ph == 0 && b < f.r2 && a1 < f.r1 && u0 + u < sc)
-                f.W[a1 + (int64_t)f.r1 * (b + (int64_t)f.r2 * (s0 + u0 + u))] = x;
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < SC; ++u) {
-        const float* brow = fs_sm + u * Jp + j0;
-#pragma unroll
-        for (int t4 = 0; t4 < FS_JB / 4; ++t4) {
-          if (4 * t4 < jn) {
-            const float4 bb = *reinterpret_cast<const float4*>(brow + 4 * t4);
-            acc[4 * t4] = fmaf(bb.x, z[u], acc[4 * t4]);
-            acc[4 * t4 + 1] = fmaf(bb.y, z[u], acc[4 * t4 + 1]);
-            acc[4 * t4 + 2] = fmaf(bb.z, z[u], acc[4 * t4 + 2]);
-            acc[4 * t4 + 3] = fmaf(bb.w, z[u], acc[4 * t4 + 3]);
-          }
-        }
-      }
-    }
-    if (f.nsplit == 1) {
-      if (in) {
-#pragma unroll
-        for (int t = 0; t < FS_JB; ++t)
-          if (t < jn) store(e, j0 + t, acc[t]);
-      }
-    } else {
-#pragma unroll
-      for (int t = 0; t < FS_JB; ++t)
-        if (t < jn) mine[(int64_t)(j0 + t) * FS_TE + tid] = acc[t];
-    }
-  }
-}
-
-// Finish, split partials: output (e, j) of a tile is the sum of its nsplit partials in
-// split order (one thread per output, every load issued before the additions).
-__global__ void __launch_bounds__(256) k_tc_finish_red(FinArgs f) {
-  grid_dep_wait();                  // programmatic launch: the split partials are complete
-  const int J = f.J;
-  const int64_t per_tile = (int64_t)J * FS_TE;
-  const int64_t total = (int64_t)(f.nt1 + f.nt2) * per_tile;
-  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
-    const int tile = (int)(o / per_tile);
-    const int rem = (int)(o % per_tile);
-    const int j = rem / FS_TE, x = rem % FS_TE;
-    const bool first = tile < f.nt1;
-    const int64_t ne = first ? (int64_t)f.r1 * f.N2 : (int64_t)f.N1 * f.r2;
-    const int te = first ? f.te1 : FS_TE;
-    const int64_t e = (int64_t)(first ? tile : tile - f.nt1) * te + x;
-    if (x >= te || e >= ne) continue;
-    const float* base = f.part + (int64_t)tile * f.nsplit * per_tile + (int64_t)j * FS_TE + x;
-    float vals[FS_SPLIT_MAX];
-#pragma unroll
-    for (int q = 0; q < FS_SPLIT_MAX; ++q) vals[q] = q < f.nsplit ? __ldcg(&base[(int64_t)q * per_tile]) : 0.f;
-    float v = 0.f;
-#pragma unroll
-    for (int q = 0; q < FS_SPLIT_MAX; ++q) v += vals[q];
-    if (first) {
-      const int64_t a = e / f.N2, i2 = e - a * f.N2;
-      f.Y2[a + (int64_t)f.r1 * i2 + ne * (int64_t)j] = v;
-    } else {
-      f.Y1[e + ne * (int64_t)j] = v;
-    }
-  }
-}
-
-
-// Three-mode finish, second launch: Y_3 = Z1 x_2 A_2^T (r1 x r2 x S), a CTA per
-// slice, i2 in chunks of FB_CH staged in shared memory (thread per output (a1, a2)).
-// dS = Y_3 x_3 A_3^T follows in the update kernel.
-constexpr int FB_CH = 128;
-constexpr size_t kFinishBSmem = (size_t)(32 * FB_CH + 32 * (FB_CH + 1)) * sizeof(float);
-__global__ void __launch_bounds__(256) k_tc_finish_b(const float* __restrict__ Z1, int N2, int S, int r1, int r2,
-                                                     const float* __restrict__ A2, float* __restrict__ Y3) {
-  extern __shared__ float fb_sm[];
-  float* zs = fb_sm;                   // r1 x FB_CH (element a + r1 il), from Z1 at i2 + N2 a + r1 N2 s
-  float* as = zs + 32 * FB_CH;         // FB_CH x r2 (ld FB_CH + 1)
-  const int tid = threadIdx.x;
-  const int64_t n1 = (int64_t)r1 * N2;
-  for (int sl = blockIdx.x; sl < S; sl += gridDim.x) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int i0 = 0; i0 < N2; i0 += FB_CH) {
-      const int ch = min(FB_CH, N2 - i0);
-      const float* src = Z1 + i0 + n1 * sl;
-#pragma unroll 4
-      for (int e = tid; e < r1 * ch; e += 256) {
-        const int il = e % ch, a = e / ch;
-        zs[a + r1 * il] = __ldcg(&src[il + (int64_t)N2 * a]);
-      }
-#pragma unroll 4
-      for (int e = tid; e < ch * r2; e += 256) {
-        const int il = e % ch, b = e / ch;
-        as[il + (FB_CH + 1) * b] = __ldg(&A2[i0 + il + (int64_t)N2 * b]);
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int o = tid + 256 * j;
-        const int a1 = o % r1, a2 = o / r1;
-        if (a2 < r2)
-          for (int il = 0; il < ch; ++il) acc[j] = fmaf(as[il + (FB_CH + 1) * a2], zs[a1 + r1 * il], acc[j]);
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int o = tid + 256 * j;
-      const int a1 = o % r1, a2 = o / r1;
-      if (a2 < r2) Y3[a1 + (int64_t)r1 * (a2 + (int64_t)r2 * sl)] = acc[j];
-    }
-  }
-}
-
 // Copies of V_{k+1} and V_k with the rows of mode 1 padded to N1p (a multiple of 4, the
 // 16-byte row stride TMA needs) by zeros: a[i + N1p c] = (i < N1 ? V[i + N1 c] : 0).
 __global__ void k_pad_rows(const float* __restrict__ Vn, const float* __restrict__ Vp, int N1, int N1p, int64_t ncol,
@@ -996,16 +645,6 @@ __global__ void k_pad_rows(const float* __restrict__ Vn, const float* __restrict
 __global__ void k_weights_f(const double* w1, int N1, int L1, const double* w2, int N2, int L2, float* out) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < L1 + L2; i += gridDim.x * blockDim.x)
     out[i] = (i < L1) ? (i < N1 ? (float)w1[i] : 0.f) : (i - L1 < N2 ? (float)w2[i - L1] : 0.f);
-}
-
-__global__ void k_slice_weights(int p, const double* w3, int N3, const double* w4, int N4, double* out) {
-  int n = (p >= 3 ? N3 : 1) * (p >= 4 ? N4 : 1);
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    double v = 1.0;
-    if (p >= 3) v *= w3[s % N3];
-    if (p >= 4) v *= w4[s / N3];
-    out[s] = v;
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1172,11 +811,7 @@ void tc_carve(TcPlan& plan, Carver& cv, int p, const int64_t* N, const int* cap)
   }
   plan.w12f = cv.take<float>((size_t)(nq1 + nq2) * TILE);
   plan.npart = cv.take<double>((size_t)1024 * NUM_CONV_WARPS);
-  // finish: split partials ((FS_CTAS + tiles) x 256 x J floats bound nsplit x tiles x 256 x J
-  // for the split count the launch picks)
-  const int jmax = p == 2 ? 1 : (p == 3 ? cap[2] : cap[2] * cap[3]);
-  const int64_t ntmax = ((int64_t)cap[0] * N[1] + FS_TE - 1) / FS_TE + ((int64_t)N[0] * cap[1] + FS_TE - 1) / FS_TE;
-  plan.fpart_cap = (size_t)(FS_CTAS + ntmax) * FS_TE * jmax;
+  plan.fpart_cap = finish_part_elems(p, N, cap);
   plan.fpart = cv.take<float>(plan.fpart_cap);
 }
 
@@ -1279,98 +914,13 @@ tdb_status tc_project(TcPlan& plan, const float* Vn, const float* Vp, int p, con
     }
     count_launch();
   };
-  // finish: Y_1, Y_2 (and Z1) from the tile partials, the slices contracted with
-  // B = A_3 (x A_4); then Y_3 (three modes) or W = Z1 x_2 A_2^T (four modes) per slice
-  const int J = p == 2 ? 1 : (p == 3 ? r[2] : r[2] * r[3]);
-  // W = Z1 x_2 A_2^T inside the finish when its first-side CTAs can hold whole i2 columns
-  const bool fuse_w = p >= 3 && N2 <= FS_TE;
-  const int te1 = fuse_w ? N2 * (FS_TE / N2) : FS_TE;
-  const int nt1 = (int)(((int64_t)r[0] * N2 + te1 - 1) / te1);
-  const int nt2 = (int)(((int64_t)N1 * r[1] + FS_TE - 1) / FS_TE);
-  if (J > FS_JMAX) {
+  if (finish_outputs(p, r) > FS_JMAX) {
     err = "finish: r_3 r_4 above 128";
     return TDB_ERR_UNSUPPORTED;
   }
-  // splits per tile: the grid stays within the target (whole waves of resident CTAs: two
-  // per SM), at least one split
-  auto nsplit_for = [&](int target) {
-    int ns = (int)std::max<int64_t>(1, target / (nt1 + nt2));
-    ns = std::min({ns, std::max(1, nslice / FS_SC), FS_SPLIT_MAX});
-    while (ns > 1 && (size_t)ns * (nt1 + nt2) * FS_TE * J > plan.fpart_cap) --ns;
-    return ns;
-  };
-  FinArgs f;
-  f.Z1p = plan.z1p;
-  f.Z2p = plan.z2p;
-  f.N1 = N1;
-  f.N2 = N2;
-  f.S = nslice;
-  f.nq1 = nq1;
-  f.nq2 = nq2;
-  f.r1 = r[0];
-  f.r2 = r[1];
-  f.A3 = p >= 3 ? (const float*)A[2] : nullptr;
-  f.A4 = p >= 4 ? (const float*)A[3] : nullptr;
-  f.N3 = p >= 3 ? (int)N[2] : 1;
-  f.r3 = p >= 3 ? r[2] : 1;
-  f.N4 = p >= 4 ? (int)N[3] : 1;
-  f.r4 = p >= 4 ? r[3] : 1;
-  f.J = J;
-  f.Z1 = Z1;
-  f.W = p == 3 ? Y[2] : scratch;
-  f.A2 = (const float*)A[1];
-  f.fuse_w = fuse_w ? 1 : 0;
-  f.te1 = te1;
-  f.Y2 = Y[1];
-  f.Y1 = Y[0];
-  f.part = plan.fpart;
-  f.nt1 = nt1;
-  f.nt2 = nt2;
-  f.npart = plan.npart;
-  f.span = nullptr;
-  f.dv2 = dv2;
-  const size_t fsm = sizeof(float) * (FS_SC * ((J + 3) & ~3) +
-                                      (fuse_w ? FS_SC * FS_TE + (size_t)a2_stride(N2) * r[1] : 0));
-  if (fsm > 48 * 1024) {
-    static bool fs_attr = false;
-    if (!fs_attr) {
-      const int lim = 100 * 1024;
-      cudaFuncSetAttribute(k_tc_finish_sk<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      cudaFuncSetAttribute(k_tc_finish_sk<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      cudaFuncSetAttribute(k_tc_finish_sk<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      cudaFuncSetAttribute(k_tc_finish_sk<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      fs_attr = true;
-    }
-  }
-  const int nqm = std::max(nq1, nq2);
-  // both finishing kernels start by programmatic launch behind the kernel before them (their
-  // set-up overlaps its tail; they wait for it before reading its results)
-  auto launch_pdl = [&](auto kern, int grid, int block, size_t sm) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kern, f);
-    count_launch();
-  };
-  auto launch_finish = [&](int nsplit) {
-    f.nsplit = nsplit;
-    const int fgrid = (nt1 + nt2) * nsplit;
-    if (nqm <= 1) launch_pdl(k_tc_finish_sk<1>, fgrid, FS_TE, fsm);
-    else if (nqm <= 2) launch_pdl(k_tc_finish_sk<2>, fgrid, FS_TE, fsm);
-    else if (nqm <= 4) launch_pdl(k_tc_finish_sk<4>, fgrid, FS_TE, fsm);
-    else launch_pdl(k_tc_finish_sk<8>, fgrid, FS_TE, fsm);
-    if (nsplit > 1) {
-      const int64_t outs = (int64_t)(nt1 + nt2) * J * FS_TE;
-      launch_pdl(k_tc_finish_red, (int)std::min<int64_t>((outs + 255) / 256, 152 * 16), 256, 0);
-    }
-  };
+  Finish<float> fin;
+  fin.setup(p, N, r, A, Z1, plan.z1p, plan.z2p, nq1, nq2, scratch, Y, plan.fpart, plan.fpart_cap, plan.npart, dv2, s);
+  const int J = fin.J;
   // launch shape: tuned once per plan on its first call outside stream capture (cached
   // process-wide per shape); under capture before that, the full grid
   if (!plan.tuned) {
@@ -1387,8 +937,8 @@ tdb_status tc_project(TcPlan& plan, const float* Vn, const float* Vp, int p, con
         plan.from_cache = false;
       } else if (!tune_lookup(key, plan)) {
         tune_shape(plan, cmax, [&](int c) { launch_project(c, false); }, [&](int target) {
-          f.nnp = P.nq12 * plan.cstep * NUM_CONV_WARPS;
-          launch_finish(nsplit_for(target));
+          fin.f.nnp = P.nq12 * plan.cstep * NUM_CONV_WARPS;
+          fin.launch(fin.nsplit_for(target));
         }, s);
         tune_store(key, plan);
       }
@@ -1407,26 +957,10 @@ tdb_status tc_project(TcPlan& plan, const float* Vn, const float* Vp, int p, con
     err = std::string("k_tc_project launch: ") + cudaGetErrorString(e);
     return TDB_ERR_CUDA;
   }
-  f.nnp = grid * NUM_CONV_WARPS;
-  f.span = P.span;
-  launch_finish(nsplit_for(plan.tuned ? plan.fin_target : FS_CTAS));
-  if (p >= 3) {
-    if (!fuse_w) {
-      // Z1 summed over the mode-1 tiles: the partials themselves when there is one tile
-      const float* z1 = nq1 > 1 ? Z1 : plan.z1p;
-      float* out = p == 3 ? Y[2] : scratch;
-      k_tc_finish_b<<<std::min(nslice, 152 * 8), 256, kFinishBSmem, s>>>(z1, N2, nslice, r[0], r[1],
-                                                                         (const float*)A[1], out);
-      count_launch();
-    }
-    if (p == 4) {
-      // Y_3 = W x_4 A_4^T and Y_4 = W x_3 A_3^T from W = Z1 x_2 A_2^T (r1 x r2 x N3 x N4)
-      const int64_t L12 = (int64_t)r[0] * r[1];
-      launch_modeprod<float, float, float>(scratch, Y[2], (const float*)A[3], L12 * N[2], (int)N[3], r[3], 1, N[3], 1,
-                                           s);
-      launch_modeprod<float, float, float>(scratch, Y[3], (const float*)A[2], L12, (int)N[2], r[2], N[3], N[2], 1, s);
-    }
-  }
+  fin.f.nnp = grid * NUM_CONV_WARPS;
+  fin.f.span = P.span;
+  fin.launch(fin.nsplit_for(plan.tuned ? plan.fin_target : FS_CTAS));
+  fin.launch_rest(N, r, A, Y);
   if (!defer_ds) {
     // dS = Y_2 x_2 A_2^T (otherwise the update kernel forms it)
     int64_t Q = 1;

@@ -17,6 +17,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "mlp.h"
+#include "simt_project.h"
 #include "tc_project.h"
 
 namespace tdb {
@@ -143,6 +144,8 @@ struct tdb_ctx {
   // BF16 tensor-core projection
   TcPlan tc;
   bool use_tc = false;
+  // float and double projection (the contexts without the tensor cores)
+  SpPlan sp;
   // learned error estimator
   EstState est;
   float* mlpP = nullptr;
@@ -439,6 +442,8 @@ void carve(tdb_ctx* c, Carver& cv) {
   c->trX = cv.take<float>((size_t)c->tr_cap * MLP_F);
   c->trT = cv.take<float>(c->tr_cap);
   if (c->prec == TDB_BF16_TTM) tc_carve(c->tc, cv, c->p, c->N, c->cap);
+  else if (c->f64) sp_carve<double>(c->sp, cv, c->p, c->N, c->cap);
+  else sp_carve<float>(c->sp, cv, c->p, c->N, c->cap);
 }
 
 tdb_status validate(const tdb_config* cfg, std::string& err) {
@@ -511,6 +516,17 @@ WeightView weight_view(const tdb_ctx* c) {
     wv.w[n] = n < c->p ? c->w[n] : nullptr;
   }
   return wv;
+}
+
+// Whether a context without the tensor cores projects in one fused pass (simt_project.cu).
+// Measured per projection, fused against mode products: float 256 x 128 x 512 at ranks
+// (11, 8, 16) 60 against 430 us, double 126^3 at (5, 5, 5) 100 against 410 us.  Small double
+// tensors keep the mode products: at 64^3 the pass is latency-bound on both routes (12 us
+// apart), and an error 1e-8 of ||V||_W there rests on the last bits of the double state,
+// which the mode products' order of summation has always given.
+constexpr int64_t kSpDoubleMin = (int64_t)1 << 19;
+bool sp_route(const tdb_ctx* c) {
+  return !c->use_tc && sp_supported(c->p, c->r) && (!c->f64 || c->S >= kSpDoubleMin);
 }
 
 // ---------------------------------------------------------------------------
@@ -1072,7 +1088,8 @@ tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine
     ntiles += (ctx->N[n] + 31) / 32;
   }
   a.dS = ctx->dS;
-  a.ds_y2 = ctx->use_tc ? ctx->Y[1] : nullptr;       // the projection leaves dS to phase 1
+  // the fused projections leave dS to phase 1
+  a.ds_y2 = ctx->use_tc || sp_route(ctx) ? ctx->Y[1] : nullptr;
   a.dS_out = ctx->dS;
   a.T = ctx->T;
   a.T2 = ctx->T2;
@@ -1147,6 +1164,10 @@ tdb_status enqueue_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vp, bool all_paths
                      (const void* const*)ctx->A, (const double* const*)ctx->w, (float*)ctx->ping, (float*)ctx->pong,
                      (float*)ctx->dV, (float*)ctx->dS, (float* const*)ctx->Y, &ctx->rb_dev->dv2, ctx->flags, s, evm,
                      ctx->err, true, (float)scale, after_begin));
+    } else if (sp_route(ctx)) {
+      TRY(sp_project<Tc>(ctx->sp, Vn, Vfrom, p, ctx->N, ctx->r, (const void* const*)ctx->A,
+                         (const double* const*)ctx->w, (Tc*)ctx->ping, (Tc* const*)ctx->Y, &ctx->rb_dev->dv2,
+                         ctx->flags, s, evm, ctx->err, (Tc)scale));
     } else {
       launch_diff<Tc>(Vn, Vfrom, (Tc*)ctx->dV, ctx->S, s, (Tc)scale);
       launch_wnorm2<Tc>((const Tc*)ctx->dV, nullptr, weight_view(ctx), ctx->npart, ctx->nblk, &ctx->rb_dev->dv2,
@@ -1604,6 +1625,7 @@ tdb_status common_init(tdb_ctx** out, const tdb_config* cfg, void* ws, size_t ws
     launch_weights_T<double>(weight_view(ctx), (double*)ctx->w1T, (double*)ctx->wcolT, ctx->stream);
   else
     launch_weights_T<float>(weight_view(ctx), (float*)ctx->w1T, (float*)ctx->wcolT, ctx->stream);
+  if (!ctx->use_tc) sp_prepare(ctx->sp, ctx->p, ctx->N, (const double* const*)ctx->w, ctx->stream);
   memset(&ctx->est, 0, sizeof(ctx->est));
   ctx->est.last_log_eps = -30.0;
   ctx->est.max_skip = std::max(1, ctx->cfg.error_every);
