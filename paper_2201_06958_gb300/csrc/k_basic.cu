@@ -146,199 +146,66 @@ template void launch_wnorm2<double>(const double*, const double*, const WeightVi
 
 // Exact error of Eq. 2.20 without materialising V^TDB: with H = T x_2 U_2 ... x_p U_p
 // (r_1 x N_2 x ... x N_p), every mode-1 column of the reconstruction is U_1 H[:, c].
-// One warp per column, U_1 and w_1 staged in shared memory when they fit, the
-// column's H values broadcast by shuffles; w_1 and the column weights
-// w_c = prod_{m>1} w_m(i_m) in the compute type; per-column sums in the compute type,
-// double across columns.  Float with N_1 % 4 == 0: lanes own float4 row groups and a
-// warp works on two columns at once with all their loads issued before the
-// arithmetic (the pass is bound by how many bytes of V are in flight).  The last CTA
-// to finish adds the per-CTA partials in a fixed order and writes *out (no second
-// launch); `counter` is zero before and after.
-template <typename T>
-__global__ void __launch_bounds__(256) k_recon_err(const T* __restrict__ V, const T* __restrict__ U1,
-                                                   const T* __restrict__ H, int r1, int N1, unsigned ncol,
-                                                   const T* __restrict__ w1, const T* __restrict__ wcol,
-                                                   int stage_u1, double* __restrict__ partial,
-                                                   unsigned* __restrict__ counter, double* __restrict__ out,
-                                                   unsigned* flags, const int* __restrict__ gate) {
-  if (gate && *gate == 0) return;          // the estimator ruled this evaluation out
-  extern __shared__ __align__(16) unsigned char sm_re[];
-  T* U1s = (T*)sm_re;
-  T* w1s = U1s + (size_t)N1 * r1;
-  __shared__ double sh[32];
-  __shared__ bool last;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const T* Usrc = U1;
-  const T* wsrc = w1;
-  if (stage_u1) {
-    // every load of the staging issued before the first store (eight per thread in flight)
-    bool vec = false;
-    if constexpr (sizeof(T) == 4) vec = (N1 & 3) == 0;
-    if (vec) {
-      const float4* su = reinterpret_cast<const float4*>(U1);
-      float4* du = reinterpret_cast<float4*>(U1s);
-      const int nu4 = N1 * r1 / 4, nw4 = N1 / 4;
-#pragma unroll 8
-      for (int e = tid; e < nu4; e += blockDim.x) du[e] = __ldg(&su[e]);
-#pragma unroll 4
-      for (int e = tid; e < nw4; e += blockDim.x)
-        reinterpret_cast<float4*>(w1s)[e] = __ldg(&reinterpret_cast<const float4*>(w1)[e]);
-    } else {
-#pragma unroll 8
-      for (int e = tid; e < N1 * r1; e += blockDim.x) U1s[e] = U1[e];
-#pragma unroll 4
-      for (int e = tid; e < N1; e += blockDim.x) w1s[e] = w1[e];
-    }
-    __syncthreads();
-    Usrc = U1s;
-    wsrc = w1s;
-  }
-  double acc = 0.0;
-  bool bad = false;
-  const unsigned gw = blockIdx.x * nw + warp, tw = gridDim.x * nw;
-  bool done = false;
-  if constexpr (sizeof(T) == 4) {
-    if (stage_u1 && (N1 & 3) == 0) {
-      const int n4 = N1 >> 2;
-      const float4* U4 = reinterpret_cast<const float4*>(Usrc);
-      const float4* w4 = reinterpret_cast<const float4*>(wsrc);
-      const float4* V4 = reinterpret_cast<const float4*>(V);
-      const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (unsigned c0 = gw; c0 < ncol; c0 += 2 * tw) {
-        const unsigned c1 = c0 + tw;
-        const bool has1 = c1 < ncol;
-        const float hl0 = lane < r1 ? H[lane + (size_t)r1 * c0] : 0.f;
-        const float hl1 = (has1 && lane < r1) ? H[lane + (size_t)r1 * c1] : 0.f;
-        float s0 = 0.f, s1 = 0.f;
-        for (int g0 = 0; g0 < n4; g0 += 128) {
-          float4 v0[4], v1[4], q0[4], q1[4];
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int g = g0 + lane + 32 * t;
-            v0[t] = g < n4 ? V4[(size_t)n4 * c0 + g] : z4;
-            v1[t] = (has1 && g < n4) ? V4[(size_t)n4 * c1 + g] : z4;
-            q0[t] = z4;
-            q1[t] = z4;
-          }
-          for (int a = 0; a < r1; ++a) {
-            const float h0 = __shfl_sync(0xffffffffu, hl0, a), h1 = __shfl_sync(0xffffffffu, hl1, a);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              const int g = g0 + lane + 32 * t;
-              if (g < n4) {
-                const float4 u = U4[(size_t)n4 * a + g];
-                q0[t].x = fmaf(u.x, h0, q0[t].x); q0[t].y = fmaf(u.y, h0, q0[t].y);
-                q0[t].z = fmaf(u.z, h0, q0[t].z); q0[t].w = fmaf(u.w, h0, q0[t].w);
-                q1[t].x = fmaf(u.x, h1, q1[t].x); q1[t].y = fmaf(u.y, h1, q1[t].y);
-                q1[t].z = fmaf(u.z, h1, q1[t].z); q1[t].w = fmaf(u.w, h1, q1[t].w);
-              }
-            }
-          }
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int g = g0 + lane + 32 * t;
-            if (g < n4) {
-              const float4 w = w4[g];
-              const float d0[4] = {v0[t].x - q0[t].x, v0[t].y - q0[t].y, v0[t].z - q0[t].z, v0[t].w - q0[t].w};
-              const float d1[4] = {v1[t].x - q1[t].x, v1[t].y - q1[t].y, v1[t].z - q1[t].z, v1[t].w - q1[t].w};
-              const float wv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                bad |= !isfinite(d0[u]) || !isfinite(d1[u]);
-                s0 += wv[u] * d0[u] * d0[u];
-                s1 += wv[u] * d1[u] * d1[u];
-              }
-            }
-          }
-        }
-        acc += (double)(wcol[c0] * s0);
-        if (has1) acc += (double)(wcol[c1] * s1);
-      }
-      done = true;
-    }
-  }
-  if (!done) {
-    for (unsigned c = gw; c < ncol; c += tw) {
-      const T hl = lane < r1 ? H[lane + (size_t)r1 * c] : T(0);
-      T h[32];
-#pragma unroll
-      for (int a = 0; a < 32; ++a) h[a] = __shfl_sync(0xffffffffu, hl, a);
-      const T* vc = V + (size_t)N1 * c;
-      T s = T(0);
-      for (int i = lane; i < N1; i += 32) {
-        T rec = T(0);
-#pragma unroll
-        for (int a = 0; a < 32; ++a)
-          if (a < r1) rec += Usrc[i + N1 * a] * h[a];
-        const T d = vc[i] - rec;
-        bad |= !isfinite(d);
-        s += wsrc[i] * d * d;
-      }
-      acc += (double)(wcol[c] * s);
-    }
-  }
-  acc = block_sum(acc, sh);
-  if (bad && flags) atomicOr(flags, kFlagNonFinite);
-  if (tid == 0) {
-    partial[blockIdx.x] = acc;
-    __threadfence();
-    last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double t = 0.0;
-  for (int k = tid; k < (int)gridDim.x; k += blockDim.x) t += __ldcg(&partial[k]);
-  t = block_sum(t, sh);
-  if (tid == 0) {
-    *out = t;
-    atomicExch(counter, 0u);
-  }
-}
-
-// Float exact error, row-major variant: lane l of a warp owns rows i0 + R l .. i0 + R l + R - 1
-// of a block of 32 R rows, with U_1 of those rows (R x r_1) and w_1 in registers, and walks a
-// contiguous range of columns c.  Each column's R rows per lane, H[:, c] (lanes < r_1) and
-// w_c (lane 0) arrive by cp.async into a ring of D column slots per warp (D columns in
-// flight per warp, no registers held); H[:, c] is broadcast by shuffles.  Per column the
-// lane forms U_1 H[:, c] for its rows, the weighted squared difference, and adds w_c times
-// it to a float sum that goes into the double accumulator every D columns.
+// Lane l of a warp owns rows i0 + R l .. i0 + R l + R - 1 of a block of 32 R rows, with U_1 of
+// those rows (R x r_1) and w_1 in registers, and walks a contiguous range of columns c.  Each
+// column's R rows per lane, H[:, c] (lanes < r_1) and w_c (lane 0) arrive by cp.async into a
+// ring of D column slots per warp (D columns in flight per warp, no registers held); H[:, c]
+// is a broadcast read.  Per column the lane forms U_1 H[:, c] for its rows and the weighted
+// squared difference; w_c times it goes into a sum of the compute type that is added to the
+// double accumulator every D columns.  The last CTA to finish adds the per-CTA partials in a
+// fixed order and writes *out (no second launch); `counter` is zero before and after.
+// Double runs at 64 cycles per instruction and sub-partition, so there only the r_1 products
+// that exist are formed (float takes all RM, zeros past r_1).
+// Measured: 126^3 double at r_1 = 5, 54 us (8 double operations a point: 30 us at the issue
+// rate), where a warp per column with U_1 in shared memory and H[:, c] by shuffles took 156 us.
 constexpr int RE_D = 8;           // columns in flight per warp
-template <int R>
-__device__ __forceinline__ void cp_async_rows(float* dst, const float* src, bool valid) {
+template <int BYTES>
+__device__ __forceinline__ void cp_async_n(void* dst, const void* src, bool valid) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  const int n = valid ? 4 * R : 0;
-  if (R == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
-  else if (R == 2)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_async4(float* dst, const float* src, bool valid) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(d), "l"(src), "r"(valid ? BYTES : 0), "n"(BYTES)
+               : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <int R, int RM>
-__global__ void __launch_bounds__(256, 2) k_recon_err_rows(const float* __restrict__ V, const float* __restrict__ U1,
-                                                         const float* __restrict__ H, int r1, int N1, unsigned ncol,
-                                                         const float* __restrict__ w1, const float* __restrict__ wcol,
+// N consecutive values from 16-byte aligned (N sizeof(T) >= 16) shared memory
+template <typename T, int N>
+__device__ __forceinline__ void lds_run(const T* p, T* v) {
+  if constexpr (N * sizeof(T) % 16 == 0) {
+    constexpr int per = 16 / sizeof(T);
+#pragma unroll
+    for (int i = 0; i < N / per; ++i) {
+      if constexpr (sizeof(T) == 4) {
+        const float4 t = reinterpret_cast<const float4*>(p)[i];
+        v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w;
+      } else {
+        const double2 t = reinterpret_cast<const double2*>(p)[i];
+        v[2 * i] = t.x; v[2 * i + 1] = t.y;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = p[i];
+  }
+}
+
+template <typename T, int R, int RM>
+__global__ void __launch_bounds__(256, 2) k_recon_err_rows(const T* __restrict__ V, const T* __restrict__ U1,
+                                                         const T* __restrict__ H, int r1, int N1, unsigned ncol,
+                                                         const T* __restrict__ w1, const T* __restrict__ wcol,
                                                          int vec, double* __restrict__ partial,
                                                          unsigned* __restrict__ counter, double* __restrict__ out,
                                                          unsigned* flags, const int* __restrict__ gate) {
   if (gate && *gate == 0) return;          // the estimator ruled this evaluation out
-  constexpr int SLOT = 32 * R + RM + 4;    // floats per column slot: rows, H[:, c] (zero past r_1), w_c
-  __shared__ __align__(16) float ring[8][RE_D][SLOT];
+  constexpr int SLOT = 32 * R + RM + 4;    // values per column slot: rows, H[:, c] (zero past r_1), w_c
+  extern __shared__ __align__(16) unsigned char ring_raw[];
   __shared__ double sh[32];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  float (*slot)[SLOT] = ring[wib];
+  T (*slot)[SLOT] = (T(*)[SLOT])((T*)ring_raw + (size_t)wib * RE_D * SLOT);
   // H entries past r_1 are never copied: zero them once (they meet zero rows of U_1)
-  for (int e = lane; e < RE_D * RM; e += 32) slot[e / RM][32 * R + e % RM] = 0.f;
+  for (int e = lane; e < RE_D * RM; e += 32) slot[e / RM][32 * R + e % RM] = T(0);
   __syncwarp();
   const int nrb = (N1 + 32 * R - 1) / (32 * R);
   const unsigned gw = blockIdx.x * (blockDim.x >> 5) + wib, tw = gridDim.x * (blockDim.x >> 5);
@@ -347,34 +214,36 @@ __global__ void __launch_bounds__(256, 2) k_recon_err_rows(const float* __restri
   bool bad = false;
   const unsigned kk = gw % wpr;
   const unsigned c_lo = (unsigned)((uint64_t)ncol * kk / wpr), c_hi = (unsigned)((uint64_t)ncol * (kk + 1) / wpr);
-  if (gw < wpr * (unsigned)nrb && c_lo < c_hi) {
-    const int rb = (int)(gw / wpr);
+  // (a row block per group of wpr warps; the outer loop only where there are fewer warps than blocks)
+  for (unsigned rbw = gw / wpr; rbw < (unsigned)nrb && c_lo < c_hi; rbw += (tw >= (unsigned)nrb ? (unsigned)nrb : tw)) {
+    const int rb = (int)rbw;
     const int i0 = rb * 32 * R + R * lane;
-    float u[R][RM], wr[R];
+    T u[R][RM], wr[R];
 #pragma unroll
     for (int q = 0; q < R; ++q) {
       const int i = i0 + q;
-      wr[q] = i < N1 ? w1[i] : 0.f;
+      wr[q] = i < N1 ? w1[i] : T(0);
 #pragma unroll
-      for (int a = 0; a < RM; ++a) u[q][a] = (i < N1 && a < r1) ? U1[i + (size_t)N1 * a] : 0.f;
+      for (int a = 0; a < RM; ++a) u[q][a] = (i < N1 && a < r1) ? U1[i + (size_t)N1 * a] : T(0);
     }
     // source pointers of the next column to issue, advanced by one column per issue; past
     // c_hi the copies read nothing (zero bytes) from the last valid column
     const bool rows_in = i0 < N1;
-    const float* vsrc = V + (size_t)N1 * c_lo + (rows_in ? i0 : 0);
-    const float* hsrc = H + (size_t)r1 * c_lo + (lane < r1 ? lane : 0);
-    const float* wsrc = wcol + c_lo;
+    const T* vsrc = V + (size_t)N1 * c_lo + (rows_in ? i0 : 0);
+    const T* hsrc = H + (size_t)r1 * c_lo + (lane < r1 ? lane : 0);
+    const T* wsrc = wcol + c_lo;
     unsigned cnext = c_lo;
     auto issue = [&](int sl) {
       const bool in = cnext < c_hi;
       if (vec) {
-        cp_async_rows<R>(&slot[sl][R * lane], vsrc, in && rows_in);
+        cp_async_n<R * sizeof(T)>(&slot[sl][R * lane], vsrc, in && rows_in);
       } else {
 #pragma unroll
-        for (int q = 0; q < R; ++q) cp_async4(&slot[sl][R * lane + q], vsrc + (i0 + q < N1 ? q : 0), in && i0 + q < N1);
+        for (int q = 0; q < R; ++q)
+          cp_async_n<sizeof(T)>(&slot[sl][R * lane + q], vsrc + (i0 + q < N1 ? q : 0), in && i0 + q < N1);
       }
-      if (lane < r1) cp_async4(&slot[sl][32 * R + lane], hsrc, in);
-      if (lane == 0) cp_async4(&slot[sl][32 * R + RM], wsrc, in);
+      if (lane < r1) cp_async_n<sizeof(T)>(&slot[sl][32 * R + lane], hsrc, in);
+      if (lane == 0) cp_async_n<sizeof(T)>(&slot[sl][32 * R + RM], wsrc, in);
       cp_async_commit();
       if (in && cnext + 1 < c_hi) {
         vsrc += N1;
@@ -385,51 +254,41 @@ __global__ void __launch_bounds__(256, 2) k_recon_err_rows(const float* __restri
     };
 #pragma unroll
     for (int t = 0; t < RE_D; ++t) issue(t);
-    float csum = 0.f;
+    T csum = T(0);
     int sl = 0;
     for (unsigned c = c_lo; c < c_hi; ++c) {
       cp_async_wait<RE_D - 1>();           // this column's copies (the oldest group) have landed
       __syncwarp();
-      float v[R], h[RM];
-      if (R == 4) {
-        const float4 t4 = *reinterpret_cast<const float4*>(&slot[sl][4 * lane]);
-        v[0] = t4.x; v[1 % R] = t4.y; v[2 % R] = t4.z; v[3 % R] = t4.w;
-      } else if (R == 2) {
-        const float2 t2 = *reinterpret_cast<const float2*>(&slot[sl][2 * lane]);
-        v[0] = t2.x; v[1 % R] = t2.y;
-      } else {
-        v[0] = slot[sl][lane];
-      }
-#pragma unroll
-      for (int j = 0; j < RM / 4; ++j) {
-        const float4 t4 = *reinterpret_cast<const float4*>(&slot[sl][32 * R + 4 * j]);
-        h[4 * j] = t4.x; h[4 * j + 1] = t4.y; h[4 * j + 2] = t4.z; h[4 * j + 3] = t4.w;
-      }
-      const float wc = slot[sl][32 * R + RM];
+      T v[R], h[RM];
+      lds_run<T, R>(&slot[sl][R * lane], v);
+      lds_run<T, RM>(&slot[sl][32 * R], h);
+      const T wc = slot[sl][32 * R + RM];
       __syncwarp();
       issue(sl);                           // the slot refills with the column D ahead
-      float rec[R];
+      T rec[R];
 #pragma unroll
-      for (int q = 0; q < R; ++q) rec[q] = 0.f;
+      for (int q = 0; q < R; ++q) rec[q] = T(0);
 #pragma unroll
       for (int a = 0; a < RM; ++a)
+        if (sizeof(T) == 4 || a < r1)
 #pragma unroll
-        for (int q = 0; q < R; ++q) rec[q] = fmaf(u[q][a], h[a], rec[q]);
-      float s = 0.f;
+          for (int q = 0; q < R; ++q) rec[q] = fma(u[q][a], h[a], rec[q]);
+      T s = T(0);
 #pragma unroll
       for (int q = 0; q < R; ++q) {
-        const float d = v[q] - rec[q];
-        s = fmaf(wr[q] * d, d, s);
+        const T d = v[q] - rec[q];
+        s = fma(wr[q] * d, d, s);
       }
-      csum = fmaf(wc, s, csum);
+      csum = fma(wc, s, csum);
       if (++sl == RE_D) {
         sl = 0;
         bad |= !isfinite(csum);
         acc += (double)csum;
-        csum = 0.f;
+        csum = T(0);
       }
     }
     cp_async_wait<0>();
+    __syncwarp();
     bad |= !isfinite(csum);
     acc += (double)csum;
   }
@@ -456,36 +315,25 @@ template <typename T>
 void launch_recon_err(const T* V, const T* U1, const T* H, int r1, int N1, int64_t ncol, const T* w1, const T* wcol,
                       double* partial, unsigned* counter, int nblocks, double* out, unsigned* flags, cudaStream_t s,
                       const int* gate) {
-  if constexpr (sizeof(T) == 4) {
-    // the row-major variant: U_1 in registers, cp.async column ring
-    const uintptr_t va = (uintptr_t)V;
-    const int vec4 = (N1 % 4) == 0 && va % 16 == 0, vec2 = (N1 % 2) == 0 && va % 8 == 0;
-    const int blocks = std::max(1, std::min(nblocks, 2 * 152));
-    if (r1 <= 8)
-      k_recon_err_rows<4, 8><<<blocks, 256, 0, s>>>(V, U1, H, r1, N1, (unsigned)ncol, w1, wcol, vec4, partial,
-                                                    counter, out, flags, gate);
-    else if (r1 <= 16)
-      k_recon_err_rows<4, 16><<<blocks, 256, 0, s>>>(V, U1, H, r1, N1, (unsigned)ncol, w1, wcol, vec4, partial,
-                                                     counter, out, flags, gate);
-    else
-      k_recon_err_rows<2, 32><<<blocks, 256, 0, s>>>(V, U1, H, r1, N1, (unsigned)ncol, w1, wcol, vec2, partial,
-                                                     counter, out, flags, gate);
+  // rows per lane: 16 bytes of V (float ranks above 16: 8 bytes), so that U_1 stays in registers
+  const uintptr_t va = (uintptr_t)V;
+  const int blocks = std::max(1, std::min(nblocks, 2 * 152));
+  auto go = [&](auto kern, int R, int RM) {
+    const size_t sm = sizeof(T) * 8 * RE_D * (32 * R + RM + 4);
+    if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const int vec = N1 % R == 0 && va % (R * sizeof(T)) == 0;
+    kern<<<blocks, 256, sm, s>>>(V, U1, H, r1, N1, (unsigned)ncol, w1, wcol, vec, partial, counter, out, flags, gate);
     count_launch();
-    return;
+  };
+  if constexpr (sizeof(T) == 4) {
+    if (r1 <= 8) go(k_recon_err_rows<float, 4, 8>, 4, 8);
+    else if (r1 <= 16) go(k_recon_err_rows<float, 4, 16>, 4, 16);
+    else go(k_recon_err_rows<float, 2, 32>, 2, 32);
+  } else {
+    if (r1 <= 8) go(k_recon_err_rows<double, 2, 8>, 2, 8);
+    else if (r1 <= 16) go(k_recon_err_rows<double, 2, 16>, 2, 16);
+    else go(k_recon_err_rows<double, 1, 32>, 1, 32);
   }
-  const size_t st_bytes = (size_t)N1 * (r1 + 1) * sizeof(T);
-  const int stage = st_bytes <= 96 * 1024 ? 1 : 0;
-  static bool attr[2] = {false, false};
-  if (stage && !attr[sizeof(T) == 8]) {
-    cudaFuncSetAttribute(k_recon_err<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    attr[sizeof(T) == 8] = true;
-  }
-  // float4 path: two columns per warp and iteration
-  const int per_block = (sizeof(T) == 4 && stage && N1 % 4 == 0) ? 16 : 8;
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(nblocks, (ncol + per_block - 1) / per_block));
-  k_recon_err<T><<<blocks, 256, stage ? st_bytes : 0, s>>>(V, U1, H, r1, N1, (unsigned)ncol, w1, wcol, stage,
-                                                           partial, counter, out, flags, gate);
-  count_launch();
 }
 template void launch_recon_err<float>(const float*, const float*, const float*, int, int, int64_t, const float*,
                                       const float*, double*, unsigned*, int, double*, unsigned*, cudaStream_t,
