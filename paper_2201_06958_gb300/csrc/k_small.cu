@@ -1,8 +1,7 @@
 // k_small.cu - rank-sized algebra outside the per-step update (FP64): the weighted
 // Cholesky-QR of freshly computed bases at (re)initialisation,
 //   C_n = U^T W U = R^T R,  U <- U R^{-1},  A = W U
-// (the paper does not say how it keeps Eq. 2.6; this is the reading used), and a
-// single-CTA Jacobi eigensolver for small symmetric matrices.
+// (the paper does not say how it keeps Eq. 2.6; this is the reading used).
 //
 // Small r x r matrices are stored column-major with leading dimension 32
 // (TDB_MAX_RANK): A[a + 32 b].  N x r matrices are column-major with leading
@@ -122,67 +121,5 @@ void launch_orthonormalize(RowArgs& a, double* R, double* Rinv, unsigned* flags,
 }
 template void launch_orthonormalize<float>(RowArgs&, double*, double*, unsigned*, cudaStream_t);
 template void launch_orthonormalize<double>(RowArgs&, double*, double*, unsigned*, cudaStream_t);
-
-// ---------------------------------------------------------------------------
-// Standalone Jacobi on an n x n symmetric matrix (n <= 96), one CTA; eigenvalues
-// descending into ev, eigenvectors (columns, ld n) into Vout with the largest-
-// magnitude entry of each column made positive.
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void k_jacobi_eig(const T* __restrict__ Ain, int n, double* __restrict__ ev, T* __restrict__ Vout,
-                             int max_sweeps, T tol, unsigned* flags) {
-  extern __shared__ unsigned char smraw[];
-  const int lda = 97;
-  T* A = (T*)smraw;
-  T* V = A + lda * 96;
-  T* cs = V + lda * 96;
-  T* red = cs + 128;
-  int* pq = (int*)(red + 32);
-  __shared__ int order[96];
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    int i = e % n, j = e / n;
-    A[i + lda * j] = Ain[i + (int64_t)n * j];
-  }
-  __syncthreads();
-  int sw = jacobi_smem<T>(A, V, lda, n, max_sweeps, tol, cs, pq, red);
-  if (sw >= max_sweeps && threadIdx.x == 0 && flags) atomicOr(flags, kFlagEigNoConv);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int j = 0; j < n; ++j) order[j] = j;
-    for (int i = 0; i < n; ++i) {
-      int best = i;
-      for (int j = i + 1; j < n; ++j)
-        if (A[order[j] + lda * order[j]] > A[order[best] + lda * order[best]]) best = j;
-      int t = order[i]; order[i] = order[best]; order[best] = t;
-    }
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    int o = order[j];
-    ev[j] = (double)A[o + lda * o];
-    int im = 0;
-    T best = 0;
-    for (int i = 0; i < n; ++i) {
-      T v = fabs(V[i + lda * o]);
-      if (v > best) { best = v; im = i; }
-    }
-    T sgn = V[im + lda * o] < T(0) ? T(-1) : T(1);
-    for (int i = 0; i < n; ++i) Vout[i + (int64_t)n * j] = sgn * V[i + lda * o];
-  }
-}
-
-template <typename T>
-void launch_jacobi_eig(const T* A, int n, double* ev, T* V, unsigned* flags, cudaStream_t s) {
-  size_t sm = (2 * 97 * 96 + 128 + 32) * sizeof(T) + 128 * sizeof(int);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_jacobi_eig<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
-  T tol = sizeof(T) == 8 ? T(1e-15) : T(1e-6);
-  k_jacobi_eig<T><<<1, 512, sm, s>>>(A, n, ev, V, 40, tol, flags); count_launch();
-}
-template void launch_jacobi_eig<float>(const float*, int, double*, float*, unsigned*, cudaStream_t);
-template void launch_jacobi_eig<double>(const double*, int, double*, double*, unsigned*, cudaStream_t);
 
 }  // namespace tdb

@@ -159,37 +159,49 @@ void launch_sqrt_weights(const double* w, int n, float* ws, cudaStream_t s);
 void launch_weight_data(const float* V, int p, const int64_t* N, const float* const* ws, int64_t S, float* Vw,
                         cudaStream_t s);
 void launch_gram_weighted(const float* Vw, int64_t L, int64_t Nn, int64_t Q, double* part, size_t part_cap,
-                          double* C64, float* Cc, cudaStream_t s);
-size_t eig_si_scratch_floats(int n);
-// Leading k eigenpairs of the float Gram Cc (n x n) by block subspace iteration from
-// hash columns (the result depends on Cc only).
-tdb_status eig_si_float(const float* Cc, const double* C64, int n, int k, int iters, float* scratch, unsigned* bar,
-                        unsigned* flags, double* ev, double* Q, double* trace, cudaStream_t s);
+                          double* C64, cudaStream_t s);
+
+// k_eig_modes.cu: leading eigenpairs of several symmetric positive semi-definite matrices
+constexpr int kEigBlock = 50;              // most columns of a block: 16 more than the wanted pairs (<= 34)
+constexpr int kEigSweeps = 16;             // Jacobi sweeps at most
+constexpr int kEigPart = 3840;             // a CTA's partial sums: block^2 and its upper triangle, and 64
+struct EigProblem {
+  const double* C;                         // n x n, symmetric
+  int n, k;                                // k wanted pairs, k <= min(n, 34)
+  double* scratch;                         // eig_modes_scratch(n, k) doubles
+  double* ev;                              // k eigenvalues, descending
+  double* Q;                               // n x k eigenvectors, entry of largest magnitude positive
+  double* trace;
+};
+struct EigMode {
+  const double* C;
+  int n, m, k, mp;                         // m columns of the block, mp: padded to eight
+  int cta0, nct;                           // the CTAs of the group
+  double* Q;                               // n x m block, row-major (ld mp)
+  double* part;                            // per-CTA partial sums (stride pstride), and column statistics
+  int pstride;
+  double* sums;                            // the group's sums
+  double* rot;                             // Jacobi rotations, by sweep, round and pair
+  unsigned* bar;                           // group barrier
+  unsigned* done;                          // Jacobi sweeps done
+  double* ev;
+  double* out;
+  double* trace;
+  double tau, tol;
+};
+struct EigModes {
+  int p;
+  EigMode mode[kMaxModes];
+  unsigned* flags;
+};
+size_t eig_modes_scratch(int n, int k);
+// All p problems in one cooperative launch.  tau: relative accuracy of the matrices' entries
+// (what the iteration converges to); tol: off-diagonal mass left by the Jacobi.
+tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsigned* flags, cudaStream_t s);
 
 // k_hosvd.cu
 template <typename Tv>
-void launch_wgram(const Tv* V, const GramView& g, double* part, size_t part_cap, double* C64, void* Cc, int cc_float,
-                  cudaStream_t s);
-template <typename T>
-tdb_status eig_leading_small(const T* Cc, const double* C64, int n, int k, T* A_ws, T* V_ws, unsigned* flags,
-                             double* ev, double* Q, double* trace, double* scratch, cudaStream_t s);
-template <typename T>
-struct SubspaceWs {
-  T* Q;        // n x 64
-  T* Z;        // n x 64
-  T* X;        // n x 64
-  double* G;   // 64 x 64
-  double* R;   // 64 x 64
-  T* H;        // 64 x 64
-  T* JA;       // 64 x 64
-  T* JV;       // 64 x 64
-};
-template <typename T>
-// Q0 (nullable, n x k doubles, may be Q itself): warm start from a previous solve instead
-// of hash columns.
-tdb_status eig_subspace(const T* Cc, const double* C64, int n, int k, int iters, const SubspaceWs<T>& ws,
-                        unsigned* flags, double* ev, double* Q, double* trace, double* scratch, cudaStream_t s,
-                        const double* Q0 = nullptr);
+void launch_wgram(const Tv* V, const GramView& g, double* part, size_t part_cap, double* C64, cudaStream_t s);
 void launch_scale_basis(const double* Q, const double* w, int64_t n, int r, double* U, cudaStream_t s);
 void launch_merge_weights(const WeightView& wv, int skip, int64_t M, double* wq, cudaStream_t s);
 template <typename Tv>

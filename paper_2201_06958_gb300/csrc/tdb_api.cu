@@ -119,26 +119,14 @@ struct tdb_ctx {
   Readback* rb_dev;
   unsigned* flags;
   // HOSVD scratch
-  double* C64;
-  void* Cc;
-  void* jA;
-  void* jV;
-  void* siQ;
-  void* siZ;
-  void* siX;
-  double* siG;
-  double* siR;
-  void* siH;
-  void* siJA;
-  void* siJV;
+  double* C64[kMaxModes];         // the Gram of each mode (or of its short side)
+  double* eigws[kMaxModes];       // eigensolver scratch
   double* wpart;
-  float* eigf;                    // float eigensolver scratch (float compute types)
   float* wsf[kMaxModes];          // sqrt of the weights in float
   size_t wpart_cap = 0;
   double* ev[kMaxModes];
   double* Qeig[kMaxModes];
   double* trace;
-  double* eigscratch;
   double* Zs;                     // eigenvectors of the short-side Gram of a long mode (M x kcap)
   double* wq;                     // merged weights of the other modes and their square roots (2 M)
   // BF16 tensor-core projection
@@ -400,35 +388,21 @@ void carve(tdb_ctx* c, Carver& cv) {
   c->est_dev = cv.take<EstState>(1);
   c->flags = &c->rb_dev->flags;
   // HOSVD scratch (sized by the Gram dimension: N_n, or the short side of a long mode)
-  int64_t nn = (Ng + 1) & ~1;
-  c->C64 = cv.take<double>(Ng * Ng);
-  c->Cc = cv.take<char>(Ng * Ng * tsz);
-  // eigensolver blocks: double in every compute type (float contexts refine in double)
-  int64_t nsmall = std::min<int64_t>(nn, 96);
-  c->jA = cv.take<double>(nsmall * nsmall);
-  c->jV = cv.take<double>(nsmall * nsmall);
-  c->siQ = cv.take<double>(Ng * 64);
-  c->siZ = cv.take<double>(Ng * 64);
-  c->siX = cv.take<double>(Ng * 64);
-  c->siG = cv.take<double>(64 * 64);
-  c->siR = cv.take<double>(64 * 64);
-  c->siH = cv.take<double>(64 * 64);
-  c->siJA = cv.take<double>(64 * 64);
-  c->siJV = cv.take<double>(64 * 64);
   int ntile = (int)((Ng + 31) / 32);
   c->wpart_cap = std::max<size_t>((size_t)(ntile * (ntile + 1) / 2) * 8 * 1024, (size_t)152 * 64 * 64);
   c->wpart = cv.take<double>(c->wpart_cap);
-  c->eigf = c->f64 ? nullptr : cv.take<float>(eig_si_scratch_floats((int)Ng));
   for (int n = 0; n < p; ++n) c->wsf[n] = c->f64 ? nullptr : cv.take<float>(c->N[n]);
   for (int n = 0; n < p; ++n) {
     c->kcap[n] = (int)std::min<int64_t>(gram_dim(c, n), c->cap[n] + 2);
     c->ev[n] = cv.take<double>(c->kcap[n]);
     c->Qeig[n] = cv.take<double>(c->N[n] * c->kcap[n]);
+    const int64_t gd = gram_dim(c, n);
+    c->C64[n] = cv.take<double>(gd * gd);
+    c->eigws[n] = cv.take<double>(eig_modes_scratch((int)gd, c->kcap[n]));
   }
   c->trace = cv.take<double>(p);
   int kmax = 0;
   for (int n = 0; n < p; ++n) kmax = std::max(kmax, c->kcap[n]);
-  c->eigscratch = cv.take<double>(64 + Ng * (kmax + 2));
   c->Zs = cv.take<double>(Ng * kmax);
   c->wq = cv.take<double>(2 * Ng);
   c->mlpP = cv.take<float>(MLP_NPARAM);
@@ -687,65 +661,55 @@ tdb_status readback(tdb_ctx* ctx) {
 // ---------------------------------------------------------------------------
 // HOSVD: per-mode spectrum (leading eigenpairs and trace), then the truncated state
 // ---------------------------------------------------------------------------
-// Spectrum and leading eigenvectors of C_n for a long first or last mode n from the short
+// The weighted Gram of mode n into C64[n]; for a long first or last mode that of its short
 // side: K, the weighted Gram of the other modes' merged index (M x M, M = S / N_n), has the
 // nonzero eigenvalues of C_n, and its unit eigenvector z maps to C_n's as B z / sqrt(lambda)
-// (B the weighted unfolding; the thin SVD of B).  Float compute types read the weighted
-// data in ctx->rec and solve in double as for the direct route.
+// (B the weighted unfolding; the thin SVD of B).  Float compute types read the weighted data
+// in ctx->rec.
 template <typename Tc>
-tdb_status hosvd_short(tdb_ctx* ctx, const Tc* V, int n) {
+tdb_status mode_gram(tdb_ctx* ctx, const Tc* V, int n) {
   cudaStream_t s = ctx->stream;
   const int64_t Nn = ctx->N[n], M = ctx->S / Nn;
+  const bool shrt = short_side(ctx, n);
   const int first = (n == 0) ? 1 : 0;
-  const int k = ctx->kcap[n], Mi = (int)M;
-  tdb_status st;
   if (!ctx->f64) {
-    launch_gram_weighted((const float*)ctx->rec, first ? Nn : 1, M, first ? 1 : Nn, ctx->wpart, ctx->wpart_cap,
-                         ctx->C64, (float*)ctx->Cc, s);
-    CHECK_LAUNCH();
-    if (Mi <= 48) {
-      st = eig_leading_small<double>(ctx->C64, ctx->C64, Mi, k, (double*)ctx->jA, (double*)ctx->jV, ctx->flags,
-                                     ctx->ev[n], ctx->Zs, ctx->trace + n, ctx->eigscratch, s);
-    } else {
-      st = eig_si_float((const float*)ctx->Cc, ctx->C64, Mi, k, 24, ctx->eigf, ctx->bar, ctx->flags, ctx->ev[n],
-                        ctx->Zs, ctx->trace + n, s);
-      if (st == TDB_OK) {
-        SubspaceWs<double> ws{(double*)ctx->siQ, (double*)ctx->siZ, (double*)ctx->siX, ctx->siG, ctx->siR,
-                              (double*)ctx->siH, (double*)ctx->siJA, (double*)ctx->siJV};
-        st = eig_subspace<double>(ctx->C64, ctx->C64, Mi, k, 3, ws, ctx->flags, ctx->ev[n], ctx->Zs, ctx->trace + n,
-                                  ctx->eigscratch, s, ctx->Zs);
-      }
-    }
-    if (st != TDB_OK) { ctx->err = "eigensolver launch failed"; return st; }
-    launch_short_map<float>((const float*)ctx->rec, first, Nn, M, nullptr, nullptr, ctx->Zs, ctx->ev[n], k,
-                            ctx->Qeig[n], s);
+    int64_t L = 1, Q = 1;
+    for (int m = 0; m < n; ++m) L *= ctx->N[m];
+    for (int m = n + 1; m < ctx->p; ++m) Q *= ctx->N[m];
+    if (shrt)
+      launch_gram_weighted((const float*)ctx->rec, first ? Nn : 1, M, first ? 1 : Nn, ctx->wpart, ctx->wpart_cap,
+                           ctx->C64[n], s);
+    else
+      launch_gram_weighted((const float*)ctx->rec, L, Nn, Q, ctx->wpart, ctx->wpart_cap, ctx->C64[n], s);
   } else {
-    launch_merge_weights(weight_view(ctx), n, M, ctx->wq, s);
-    // K as the mode Gram of a two-mode view: (N_n, M) for the first mode, (M, N_n) for the last
     GramView g;
-    g.p = 2;
-    g.n = first;
     for (int m = 0; m < kMaxModes; ++m) { g.N[m] = 1; g.w[m] = nullptr; }
-    g.N[first ? 0 : 1] = Nn;
-    g.w[first ? 0 : 1] = ctx->w[n];
-    g.N[first ? 1 : 0] = M;
-    g.w[first ? 1 : 0] = ctx->wq;
-    g.Nn = M;
-    g.L = first ? Nn : 1;
-    g.Q = first ? 1 : Nn;
-    launch_wgram<Tc>(V, g, ctx->wpart, ctx->wpart_cap, ctx->C64, ctx->Cc, 0, s);
-    CHECK_LAUNCH();
-    if (Mi <= 96) {
-      st = eig_leading_small<Tc>((const Tc*)ctx->Cc, ctx->C64, Mi, k, (Tc*)ctx->jA, (Tc*)ctx->jV, ctx->flags,
-                                 ctx->ev[n], ctx->Zs, ctx->trace + n, ctx->eigscratch, s);
+    if (shrt) {
+      launch_merge_weights(weight_view(ctx), n, M, ctx->wq, s);
+      // K as the mode Gram of a two-mode view: (N_n, M) for the first mode, (M, N_n) for the last
+      g.p = 2;
+      g.n = first;
+      g.N[first ? 0 : 1] = Nn;
+      g.w[first ? 0 : 1] = ctx->w[n];
+      g.N[first ? 1 : 0] = M;
+      g.w[first ? 1 : 0] = ctx->wq;
+      g.Nn = M;
+      g.L = first ? Nn : 1;
+      g.Q = first ? 1 : Nn;
     } else {
-      SubspaceWs<Tc> ws{(Tc*)ctx->siQ, (Tc*)ctx->siZ, (Tc*)ctx->siX, ctx->siG, ctx->siR,
-                        (Tc*)ctx->siH, (Tc*)ctx->siJA, (Tc*)ctx->siJV};
-      st = eig_subspace<Tc>((const Tc*)ctx->Cc, ctx->C64, Mi, k, 24, ws, ctx->flags, ctx->ev[n], ctx->Zs,
-                            ctx->trace + n, ctx->eigscratch, s);
+      g.p = ctx->p;
+      g.n = n;
+      for (int m = 0; m < ctx->p; ++m) {
+        g.N[m] = ctx->N[m];
+        g.w[m] = ctx->w[m];
+      }
+      g.Nn = Nn;
+      g.L = 1;
+      for (int m = 0; m < n; ++m) g.L *= ctx->N[m];
+      g.Q = 1;
+      for (int m = n + 1; m < ctx->p; ++m) g.Q *= ctx->N[m];
     }
-    if (st != TDB_OK) { ctx->err = "eigensolver launch failed"; return st; }
-    launch_short_map<Tc>(V, first, Nn, M, ctx->w[n], ctx->wq + M, ctx->Zs, ctx->ev[n], k, ctx->Qeig[n], s);
+    launch_wgram<double>((const double*)V, g, ctx->wpart, ctx->wpart_cap, ctx->C64[n], s);
   }
   CHECK_LAUNCH();
   return TDB_OK;
@@ -755,80 +719,41 @@ template <typename Tc>
 tdb_status hosvd_spectrum(tdb_ctx* ctx, const Tc* V) {
   cudaStream_t s = ctx->stream;
   if (!ctx->f64) {
-    // float compute types: weight the data once, 64 x 64 Gram tiles, cooperative eigensolver
+    // float compute types: weight the data once, 64 x 64 Gram tiles
     for (int n = 0; n < ctx->p; ++n) launch_sqrt_weights(ctx->w[n], (int)ctx->N[n], ctx->wsf[n], s);
     launch_weight_data((const float*)V, ctx->p, ctx->N, ctx->wsf, ctx->S, (float*)ctx->rec, s);
     CHECK_LAUNCH();
-    for (int n = 0; n < ctx->p; ++n) {
-      if (short_side(ctx, n)) {
-        TRY(hosvd_short<Tc>(ctx, V, n));
-        continue;
-      }
-      int64_t L = 1, Q = 1;
-      for (int m = 0; m < n; ++m) L *= ctx->N[m];
-      for (int m = n + 1; m < ctx->p; ++m) Q *= ctx->N[m];
-      launch_gram_weighted((const float*)ctx->rec, L, ctx->N[n], Q, ctx->wpart, ctx->wpart_cap, ctx->C64,
-                           (float*)ctx->Cc, s);
-      CHECK_LAUNCH();
-      const int Nn = (int)ctx->N[n];
-      tdb_status st;
-      // The Gram is accurate to about 1e-9 of its largest entries (float products,
-      // float-float sums), but a float eigensolver resolves eigenvectors only where the
-      // eigenvalue gaps exceed about 1e-6 of the largest eigenvalue; the eigenvectors the
-      // rank rule keeps at gamma_th = 99.999 % sit below that.  So the solve is double: the
-      // single-CTA Jacobi on the double Gram for short modes, and for long ones the float
-      // subspace iteration as a warm start refined by three double iterations with
-      // Rayleigh-Ritz.
-      if (Nn <= 48) {
-        st = eig_leading_small<double>(ctx->C64, ctx->C64, Nn, ctx->kcap[n], (double*)ctx->jA, (double*)ctx->jV,
-                                       ctx->flags, ctx->ev[n], ctx->Qeig[n], ctx->trace + n, ctx->eigscratch, s);
-      } else {
-        st = eig_si_float((const float*)ctx->Cc, ctx->C64, Nn, ctx->kcap[n], 24, ctx->eigf, ctx->bar, ctx->flags,
-                          ctx->ev[n], ctx->Qeig[n], ctx->trace + n, s);
-        if (st == TDB_OK) {
-          SubspaceWs<double> ws{(double*)ctx->siQ, (double*)ctx->siZ, (double*)ctx->siX, ctx->siG, ctx->siR,
-                                (double*)ctx->siH, (double*)ctx->siJA, (double*)ctx->siJV};
-          st = eig_subspace<double>(ctx->C64, ctx->C64, Nn, ctx->kcap[n], 3, ws, ctx->flags, ctx->ev[n],
-                                    ctx->Qeig[n], ctx->trace + n, ctx->eigscratch, s, ctx->Qeig[n]);
-        }
-      }
-      if (st != TDB_OK) { ctx->err = "eigensolver launch failed"; return st; }
-      CHECK_LAUNCH();
-    }
-  } else
-  for (int n = 0; n < ctx->p; ++n) {
-    if (short_side(ctx, n)) {
-      TRY(hosvd_short<Tc>(ctx, V, n));
-      continue;
-    }
-    GramView g;
-    g.p = ctx->p;
-    g.n = n;
-    for (int m = 0; m < kMaxModes; ++m) {
-      g.N[m] = m < ctx->p ? ctx->N[m] : 1;
-      g.w[m] = m < ctx->p ? ctx->w[m] : nullptr;
-    }
-    g.Nn = ctx->N[n];
-    g.L = 1;
-    for (int m = 0; m < n; ++m) g.L *= ctx->N[m];
-    g.Q = 1;
-    for (int m = n + 1; m < ctx->p; ++m) g.Q *= ctx->N[m];
-    launch_wgram<Tc>(V, g, ctx->wpart, ctx->wpart_cap, ctx->C64, ctx->Cc, ctx->f64 ? 0 : 1, s);
-    CHECK_LAUNCH();
-    int Nn = (int)ctx->N[n];
-    tdb_status st;
-    if (Nn <= 96)
-      st = eig_leading_small<Tc>((const Tc*)ctx->Cc, ctx->C64, Nn, ctx->kcap[n], (Tc*)ctx->jA, (Tc*)ctx->jV,
-                                 ctx->flags, ctx->ev[n], ctx->Qeig[n], ctx->trace + n, ctx->eigscratch, s);
-    else {
-      SubspaceWs<Tc> ws{(Tc*)ctx->siQ, (Tc*)ctx->siZ, (Tc*)ctx->siX, ctx->siG, ctx->siR,
-                        (Tc*)ctx->siH, (Tc*)ctx->siJA, (Tc*)ctx->siJV};
-      st = eig_subspace<Tc>((const Tc*)ctx->Cc, ctx->C64, Nn, ctx->kcap[n], 24, ws, ctx->flags, ctx->ev[n],
-                            ctx->Qeig[n], ctx->trace + n, ctx->eigscratch, s);
-    }
-    if (st != TDB_OK) { ctx->err = "eigensolver launch failed"; return st; }
-    CHECK_LAUNCH();
   }
+  EigProblem pr[kMaxModes];
+  for (int n = 0; n < ctx->p; ++n) {
+    TRY(mode_gram<Tc>(ctx, V, n));
+    pr[n].C = ctx->C64[n];
+    pr[n].n = (int)gram_dim(ctx, n);
+    pr[n].k = ctx->kcap[n];
+    pr[n].scratch = ctx->eigws[n];
+    pr[n].ev = ctx->ev[n];
+    pr[n].Q = short_side(ctx, n) ? ctx->Zs : ctx->Qeig[n];
+    pr[n].trace = ctx->trace + n;
+  }
+  // Every mode's eigenpairs in double.  The float types' Gram is accurate to about 1e-9 of its
+  // largest entries (float products, float-float sums): the iteration goes a tenth below
+  // that.  (A float eigensolver resolves eigenvectors only where the eigenvalue gaps exceed
+  // about 1e-6 of the largest eigenvalue; those the rank rule keeps at gamma_th = 99.999 %
+  // sit below that.)
+  const tdb_status st = launch_eig_modes(pr, ctx->p, ctx->f64 ? 2e-16 : 1e-10, ctx->f64 ? 1e-15 : 1e-14, ctx->flags, s);
+  if (st != TDB_OK) { ctx->err = "eigensolver launch failed"; return st; }
+  for (int n = 0; n < ctx->p; ++n) {
+    if (!short_side(ctx, n)) continue;
+    const int first = (n == 0) ? 1 : 0;
+    const int64_t Nn = ctx->N[n], M = ctx->S / Nn;
+    if (ctx->f64)
+      launch_short_map<double>((const double*)V, first, Nn, M, ctx->w[n], ctx->wq + M, ctx->Zs, ctx->ev[n],
+                               ctx->kcap[n], ctx->Qeig[n], s);
+    else
+      launch_short_map<float>((const float*)ctx->rec, first, Nn, M, nullptr, nullptr, ctx->Zs, ctx->ev[n],
+                              ctx->kcap[n], ctx->Qeig[n], s);
+  }
+  CHECK_LAUNCH();
   // spectrum to host (needed by the rank rule)
   for (int n = 0; n < ctx->p; ++n) {
     ctx->h_ev[n].resize(ctx->kcap[n]);
