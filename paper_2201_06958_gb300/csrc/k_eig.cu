@@ -13,7 +13,8 @@ namespace tdb {
 
 namespace {
 
-constexpr int SY_T = 64;          // Gram output tile
+constexpr int SY_T = 64;          // Gram output tile of modes of up to 64 points
+constexpr int SY_B = 128;         // of longer ones
 constexpr int SY_K = 32;          // columns per chunk
 
 __device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
@@ -35,16 +36,35 @@ struct SqrtWeights {
   const float* ws[kMaxModes];
 };
 
-__global__ void k_weight_data(const float* __restrict__ V, SqrtWeights sw, int S, float* __restrict__ Vw) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < S; e += gridDim.x * blockDim.x) {
-    int rem = e;
-    float f = 1.f;
-    for (int n = 0; n < sw.p; ++n) {
-      const int i = rem % sw.N[n];
-      rem /= sw.N[n];
-      f *= sw.ws[n][i];
+// A warp per mode-1 column: the other modes' factors once per column, 16-byte accesses where
+// the columns allow them.  Bound: HBM, one read and one write of S floats (256 x 128 x 512:
+// 20 us; forming every element's index from its offset took 96 us).
+__global__ void __launch_bounds__(256) k_weight_data(const float* __restrict__ V, SqrtWeights sw, unsigned ncol, int vec,
+                                                     float* __restrict__ Vw) {
+  const int lane = threadIdx.x & 31;
+  const unsigned N1 = (unsigned)sw.N[0], nw = gridDim.x * (blockDim.x >> 5);
+  for (unsigned c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < ncol; c += nw) {
+    float f[kMaxModes - 1];
+    unsigned rem = c;
+#pragma unroll
+    for (int n = 1; n < kMaxModes; ++n) {
+      f[n - 1] = 1.f;
+      if (n < sw.p) {
+        f[n - 1] = sw.ws[n][rem % (unsigned)sw.N[n]];
+        rem /= (unsigned)sw.N[n];
+      }
     }
-    Vw[e] = V[e] * f;
+    const float* v = V + (size_t)N1 * c;
+    float* o = Vw + (size_t)N1 * c;
+    auto fac = [&](float w) { return ((w * f[0]) * f[1]) * f[2]; };
+    if (vec) {
+      for (unsigned i = 4 * lane; i < N1; i += 128) {
+        const float4 x = __ldcs((const float4*)(v + i)), w = __ldg((const float4*)(sw.ws[0] + i));
+        *(float4*)(o + i) = make_float4(x.x * fac(w.x), x.y * fac(w.y), x.z * fac(w.z), x.w * fac(w.w));
+      }
+    } else {
+      for (unsigned i = lane; i < N1; i += 32) o[i] = __ldcs(v + i) * fac(__ldg(sw.ws[0] + i));
+    }
   }
 }
 
@@ -53,7 +73,7 @@ __global__ void k_sqrt_weights(const double* __restrict__ w, int n, float* __res
 }
 
 // ---------------------------------------------------------------------------
-// Gram tiles: blockIdx.x = upper tile pair (ti <= tj) of 64 x 64, blockIdx.y =
+// Gram tiles of modes of up to 64 points: blockIdx.x = upper tile pair (ti <= tj) of 64 x 64, blockIdx.y =
 // column slice.  256 threads, 4 x 4 outputs each.  Column c of Vw_(n) is (l, q):
 // Vw[l + L (i + N q)].
 // ---------------------------------------------------------------------------
@@ -143,20 +163,150 @@ __global__ void __launch_bounds__(256) k_syrk_partial(const float* __restrict__ 
       out[(tr * 4 + x) + SY_T * (tc * 4 + y)] = (double)hi[x * 4 + y] + (double)lo[x * 4 + y];
 }
 
+// The same with 128 x 128 tiles and 8 x 8 outputs a thread (rows 4 tr .. and 64 + 4 tr ..,
+// columns 4 tc .. and 64 + 4 tc ..): a quarter of the shared-memory reads per product.  The
+// next chunk of 32 columns arrives by cp.async in a second buffer (no registers held: acc, hi
+// and lo take 192).  Rows of a column live in 16-byte granules, granule g of column k at
+// g ^ (k & 7), so that either loading writes without bank conflicts.  On a diagonal tile the
+// lower left quarter is left out (the finish reads the upper triangle).  Bound: FP32 issue at
+// eight warps per SM.  256 x 128 x 512: the three modes 0.75 ms, with 64 x 64 tiles 1.52 ms.
+__device__ __forceinline__ void sy_cp4(float* dst, const float* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void sy_cp16(float* dst, const float* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(in ? 16 : 0) : "memory");
+}
+constexpr size_t kSyrkBigSmem = 2 * 2 * sizeof(float) * SY_K * SY_B;
+__global__ void __launch_bounds__(256, 1) k_syrk_big(const float* __restrict__ Vw, int64_t L, int64_t Nn, int64_t Q,
+                                                     int ntile, int ksplit, double* __restrict__ part) {
+  int t = blockIdx.x, ti = 0;
+  while (t >= ntile - ti) { t -= ntile - ti; ++ti; }
+  const int tj = ti + t;
+  const bool diag = (ti == tj);
+  const int64_t ncol = L * Q;
+  const int64_t c0 = ncol * blockIdx.y / ksplit, c1 = ncol * (blockIdx.y + 1) / ksplit;
+  extern __shared__ __align__(16) float sy_sm[];            // [buffer][A, B][SY_K][SY_B]
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int tr = tid & 15, tc = tid >> 4;
+  const bool rows_fast = (L == 1);
+  const bool vec = rows_fast && (Nn & 3) == 0;
+  // columns fast: lanes take 8 columns x 4 rows (32-byte runs); this thread's column of group
+  // kg (of 8) is cb + 8 kg + (lane & 7), its element offset at row 0 kept with its l
+  int lc[4];
+  int64_t oc[4];
+#pragma unroll
+  for (int kg = 0; kg < 4; ++kg) {
+    const int64_t c = c0 + 8 * kg + (lane & 7);
+    lc[kg] = rows_fast ? 0 : (int)(c % L);
+    oc[kg] = rows_fast ? 0 : c % L + L * Nn * (c / L);
+  }
+  const int64_t wrap = L * (Nn - 1);                        // from the end of one l run to the next q's
+  auto issue = [&](int64_t cb, int buf) {
+    float* A = sy_sm + buf * 2 * SY_K * SY_B;
+    float* Bm = A + SY_K * SY_B;
+    if (rows_fast) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int k = w + 8 * u, at = k * SY_B + 4 * (lane ^ (k & 7));   // a column per warp and u
+        const int64_t c = cb + k;
+        const int ia = ti * SY_B + 4 * lane, ib = tj * SY_B + 4 * lane;
+        const float* src = Vw + Nn * (c < c1 ? c : c0);
+        if (vec) {
+          sy_cp16(A + at, src + (ia < Nn ? ia : 0), c < c1 && ia < Nn);
+          if (!diag) sy_cp16(Bm + at, src + (ib < Nn ? ib : 0), c < c1 && ib < Nn);
+        } else {
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            sy_cp4(A + at + x, src + (ia + x < Nn ? ia + x : 0), c < c1 && ia + x < Nn);
+            if (!diag) sy_cp4(Bm + at + x, src + (ib + x < Nn ? ib + x : 0), c < c1 && ib + x < Nn);
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int kg = 0; kg < 4; ++kg) {
+        const int kk = 8 * kg + (lane & 7);
+        const bool in = cb + kk < c1;
+        const float* src = Vw + (in ? oc[kg] : 0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int g = w + 8 * u, row = 4 * g + (lane >> 3), at = kk * SY_B + 4 * (g ^ (kk & 7)) + (lane >> 3);
+          const int ia = ti * SY_B + row, ib = tj * SY_B + row;
+          sy_cp4(A + at, src + (ia < Nn ? L * ia : 0), in && ia < Nn);
+          if (!diag) sy_cp4(Bm + at, src + (ib < Nn ? L * ib : 0), in && ib < Nn);
+        }
+        lc[kg] += SY_K;
+        oc[kg] += SY_K;
+        while (lc[kg] >= L) { lc[kg] -= (int)L; oc[kg] += wrap; }
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float hi[64], lo[64];
+#pragma unroll
+  for (int x = 0; x < 64; ++x) { hi[x] = 0.f; lo[x] = 0.f; }
+  issue(c0, 0);
+  int buf = 0;
+  for (int64_t cb = c0; cb < c1; cb += SY_K, buf ^= 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                        // this chunk is in; the other buffer is free
+    if (cb + SY_K < c1) issue(cb + SY_K, buf ^ 1);
+    const float* A = sy_sm + buf * 2 * SY_K * SY_B;
+    const float* Bm = diag ? A : A + SY_K * SY_B;
+    float acc[64];
+#pragma unroll
+    for (int x = 0; x < 64; ++x) acc[x] = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < SY_K; ++k) {
+      const int sw = k & 7;
+      const float4 a0 = *(const float4*)(A + k * SY_B + 4 * (tr ^ sw)), a1 = *(const float4*)(A + k * SY_B + 4 * ((16 + tr) ^ sw));
+      const float4 b0 = *(const float4*)(Bm + k * SY_B + 4 * (tc ^ sw)), b1 = *(const float4*)(Bm + k * SY_B + 4 * ((16 + tc) ^ sw));
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) acc[8 * x + y] = fmaf(av[x], bv[y], acc[8 * x + y]);
+      if (!diag)
+#pragma unroll
+        for (int x = 4; x < 8; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) acc[8 * x + y] = fmaf(av[x], bv[y], acc[8 * x + y]);
+#pragma unroll
+      for (int x = 4; x < 8; ++x)
+#pragma unroll
+        for (int y = 4; y < 8; ++y) acc[8 * x + y] = fmaf(av[x], bv[y], acc[8 * x + y]);
+    }
+#pragma unroll
+    for (int x = 0; x < 64; ++x) two_sum(hi[x], lo[x], acc[x]);
+  }
+  double* out = part + ((int64_t)blockIdx.x * ksplit + blockIdx.y) * SY_B * SY_B;
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 8; ++y) {
+      const int i = (x < 4 ? 4 * tr + x : 60 + 4 * tr + x), j = (y < 4 ? 4 * tc + y : 60 + 4 * tc + y);
+      out[i + SY_B * j] = (double)hi[8 * x + y] + (double)lo[8 * x + y];
+    }
+}
+
 // Sum the slices: C64, full n x n.
+template <int T>                  // the tile size
 __global__ void k_syrk_finish(int64_t Nn, int ntile, int ksplit, const double* __restrict__ part,
                               double* __restrict__ C64) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < Nn * Nn; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e % Nn, j = e / Nn;
     const int64_t a = i <= j ? i : j, b = i <= j ? j : i;
-    const int ti = (int)(a / SY_T), tj = (int)(b / SY_T);
+    const int ti = (int)(a / T), tj = (int)(b / T);
     const int pair = ti * ntile - ti * (ti - 1) / 2 + (tj - ti);
-    int x = (int)(a % SY_T), y = (int)(b % SY_T);
+    int x = (int)(a % T), y = (int)(b % T);
     if (ti == tj && x > y) { const int t = x; x = y; y = t; }
     double s = 0.0;
-    const double* src = part + (int64_t)pair * ksplit * SY_T * SY_T + x + SY_T * y;
+    const double* src = part + (int64_t)pair * ksplit * T * T + x + T * y;
 #pragma unroll 8
-    for (int k = 0; k < ksplit; ++k) s += src[(int64_t)k * SY_T * SY_T];
+    for (int k = 0; k < ksplit; ++k) s += src[(int64_t)k * T * T];
     C64[e] = s;
   }
 }
@@ -177,22 +327,51 @@ void launch_weight_data(const float* V, int p, const int64_t* N, const float* co
     sw.N[n] = n < p ? (int)N[n] : 1;
     sw.ws[n] = n < p ? ws[n] : nullptr;
   }
-  const int blocks = (int)std::min<int64_t>((S + 255) / 256, 152 * 8);
-  k_weight_data<<<blocks, 256, 0, s>>>(V, sw, (int)S, Vw);
+  const int64_t ncol = S / N[0];
+  const int blocks = (int)std::min<int64_t>((ncol + 7) / 8, 152 * 8);
+  const int vec = N[0] % 4 == 0 && ((uintptr_t)V & 15) == 0;      // (Vw and the weights are 256-byte aligned)
+  k_weight_data<<<blocks, 256, 0, s>>>(V, sw, (unsigned)ncol, vec, Vw);
   count_launch();
 }
 
-void launch_gram_weighted(const float* Vw, int64_t L, int64_t Nn, int64_t Q, double* part, size_t part_cap, double* C64,
+// Tiles and column slices of a Gram: about one CTA per SM, a slice not below 128 columns.
+struct GramSplit {
+  int tile, ntile, npair, ksplit;
+};
+static GramSplit gram_shape(int64_t Nn, int64_t ncol) {
+  GramSplit g;
+  g.tile = Nn <= SY_T ? SY_T : SY_B;
+  g.ntile = (int)((Nn + g.tile - 1) / g.tile);
+  g.npair = g.ntile * (g.ntile + 1) / 2;
+  // (slices rounded down where tiles of 128 fill the SMs once: a second, partial wave costs more)
+  const int want = g.tile == SY_T ? (152 + g.npair - 1) / g.npair : std::max(1, 152 / g.npair);
+  g.ksplit = (int)std::max<int64_t>(1, std::min<int64_t>(want, (ncol + 127) / 128));
+  return g;
+}
+
+size_t gram_part_elems(int64_t Nn, int64_t ncol) {
+  const GramSplit g = gram_shape(Nn, ncol);
+  return (size_t)g.npair * g.ksplit * g.tile * g.tile;
+}
+
+void launch_gram_weighted(const float* Vw, int64_t L, int64_t Nn, int64_t Q, double* part, double* C64,
                           cudaStream_t s) {
-  const int ntile = (int)((Nn + SY_T - 1) / SY_T);
-  const int npair = ntile * (ntile + 1) / 2;
-  const int64_t ncol = L * Q;
-  int ksplit = (int)std::max<int64_t>(1, std::min<int64_t>((152 + npair - 1) / npair, (ncol + 127) / 128));
-  while ((size_t)npair * ksplit * SY_T * SY_T > part_cap && ksplit > 1) --ksplit;
-  k_syrk_partial<<<dim3(npair, ksplit), 256, 0, s>>>(Vw, L, Nn, Q, ntile, ksplit, part);
-  count_launch();
+  const GramSplit g = gram_shape(Nn, L * Q);
   const int blocks = (int)std::min<int64_t>((Nn * Nn + 255) / 256, 1024);
-  k_syrk_finish<<<blocks, 256, 0, s>>>(Nn, ntile, ksplit, part, C64);
+  if (g.tile == SY_T) {
+    k_syrk_partial<<<dim3(g.npair, g.ksplit), 256, 0, s>>>(Vw, L, Nn, Q, g.ntile, g.ksplit, part);
+    count_launch();
+    k_syrk_finish<SY_T><<<blocks, 256, 0, s>>>(Nn, g.ntile, g.ksplit, part, C64);
+  } else {
+    static bool attr = false;
+    if (!attr) {
+      cudaFuncSetAttribute(k_syrk_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSyrkBigSmem);
+      attr = true;
+    }
+    k_syrk_big<<<dim3(g.npair, g.ksplit), 256, kSyrkBigSmem, s>>>(Vw, L, Nn, Q, g.ntile, g.ksplit, part);
+    count_launch();
+    k_syrk_finish<SY_B><<<blocks, 256, 0, s>>>(Nn, g.ntile, g.ksplit, part, C64);
+  }
   count_launch();
 }
 

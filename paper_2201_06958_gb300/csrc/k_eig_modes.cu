@@ -639,7 +639,7 @@ int em_cols(int n, int k) { return std::min(n, k + 16); }
 
 size_t eig_modes_scratch(int n, int k) {
   const size_t m = em_cols(n, k), mp = (m + 7) & ~(size_t)7;
-  return (size_t)n * mp + (size_t)152 * kEigPart + kEigPart +
+  return (size_t)n * mp + (size_t)std::min(152, n + 1) * kEigPart + kEigPart +
          (size_t)kEigSweeps * (EM_M - 1) * (EM_M / 2) * 2 + 8;
 }
 
@@ -684,7 +684,7 @@ tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsig
     w += (size_t)M.n * M.mp;
     M.part = w;
     M.pstride = kEigPart;
-    w += (size_t)152 * kEigPart;
+    w += (size_t)std::min(152, M.n + 1) * kEigPart;
     M.sums = w;
     w += kEigPart;
     M.rot = w;

@@ -158,8 +158,11 @@ tdb_status launch_update(UpdArgs& a, int grid_hint, cudaStream_t s);
 void launch_sqrt_weights(const double* w, int n, float* ws, cudaStream_t s);
 void launch_weight_data(const float* V, int p, const int64_t* N, const float* const* ws, int64_t S, float* Vw,
                         cudaStream_t s);
-void launch_gram_weighted(const float* Vw, int64_t L, int64_t Nn, int64_t Q, double* part, size_t part_cap,
-                          double* C64, cudaStream_t s);
+// Vw Vw^T of a mode of Nn points (L, Q: the sizes before and after it) into C64; part:
+// gram_part_elems(Nn, L Q) doubles.
+size_t gram_part_elems(int64_t Nn, int64_t ncol);
+void launch_gram_weighted(const float* Vw, int64_t L, int64_t Nn, int64_t Q, double* part, double* C64,
+                          cudaStream_t s);
 
 // k_eig_modes.cu: leading eigenpairs of several symmetric positive semi-definite matrices
 constexpr int kEigBlock = 50;              // most columns of a block: 16 more than the wanted pairs (<= 34)

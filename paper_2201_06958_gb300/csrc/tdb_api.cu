@@ -388,8 +388,14 @@ void carve(tdb_ctx* c, Carver& cv) {
   c->est_dev = cv.take<EstState>(1);
   c->flags = &c->rb_dev->flags;
   // HOSVD scratch (sized by the Gram dimension: N_n, or the short side of a long mode)
-  int ntile = (int)((Ng + 31) / 32);
-  c->wpart_cap = std::max<size_t>((size_t)(ntile * (ntile + 1) / 2) * 8 * 1024, (size_t)152 * 64 * 64);
+  if (c->f64) {
+    const int ntile = (int)((Ng + 31) / 32);
+    c->wpart_cap = std::max<size_t>((size_t)(ntile * (ntile + 1) / 2) * 8 * 1024, (size_t)152 * 64 * 64);
+  } else {
+    c->wpart_cap = 0;
+    for (int n = 0; n < p; ++n)
+      c->wpart_cap = std::max(c->wpart_cap, gram_part_elems(gram_dim(c, n), c->S / gram_dim(c, n)));
+  }
   c->wpart = cv.take<double>(c->wpart_cap);
   for (int n = 0; n < p; ++n) c->wsf[n] = c->f64 ? nullptr : cv.take<float>(c->N[n]);
   for (int n = 0; n < p; ++n) {
@@ -677,10 +683,9 @@ tdb_status mode_gram(tdb_ctx* ctx, const Tc* V, int n) {
     for (int m = 0; m < n; ++m) L *= ctx->N[m];
     for (int m = n + 1; m < ctx->p; ++m) Q *= ctx->N[m];
     if (shrt)
-      launch_gram_weighted((const float*)ctx->rec, first ? Nn : 1, M, first ? 1 : Nn, ctx->wpart, ctx->wpart_cap,
-                           ctx->C64[n], s);
+      launch_gram_weighted((const float*)ctx->rec, first ? Nn : 1, M, first ? 1 : Nn, ctx->wpart, ctx->C64[n], s);
     else
-      launch_gram_weighted((const float*)ctx->rec, L, Nn, Q, ctx->wpart, ctx->wpart_cap, ctx->C64[n], s);
+      launch_gram_weighted((const float*)ctx->rec, L, Nn, Q, ctx->wpart, ctx->C64[n], s);
   } else {
     GramView g;
     for (int m = 0; m < kMaxModes; ++m) { g.N[m] = 1; g.w[m] = nullptr; }
