@@ -10,6 +10,7 @@
 #include "kernels.h"
 
 #include <atomic>
+#include <type_traits>
 
 namespace tdb {
 
@@ -20,21 +21,6 @@ long long launches_so_far() { return g_launches.load(std::memory_order_relaxed);
 // ---------------------------------------------------------------------------
 // Elementwise
 // ---------------------------------------------------------------------------
-
-// out = scale (a - b): the snapshot difference (scale 1), or a scaled central difference
-template <typename T>
-__global__ void k_diff(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out, int64_t n, T scale) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (a[i] - b[i]) * scale;
-}
-
-template <typename T>
-void launch_diff(const T* a, const T* b, T* out, int64_t n, cudaStream_t s, T scale) {
-  int blocks = (int)std::min<int64_t>((n + 255) / 256, 152 * 16);
-  k_diff<T><<<blocks, 256, 0, s>>>(a, b, out, n, scale); count_launch();
-}
-template void launch_diff<float>(const float*, const float*, float*, int64_t, cudaStream_t, float);
-template void launch_diff<double>(const double*, const double*, double*, int64_t, cudaStream_t, double);
 
 // A = W U in the compute type: A[i + N a] = w[i] U[i + N a]  (Eq. 2.17).
 template <typename T>
@@ -69,80 +55,69 @@ template void launch_cast<double, float>(const double*, float*, int64_t, cudaStr
 template void launch_cast<float, double>(const float*, double*, int64_t, cudaStream_t);
 template void launch_cast<double, double>(const double*, double*, int64_t, cudaStream_t);
 
-// out = a + (double) b   (core Euler update T + dS, Sec. 2.3)
-template <typename Tb>
-__global__ void k_add(const double* __restrict__ a, const Tb* __restrict__ b, double* __restrict__ out, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = a[i] + (double)b[i];
-}
-template <typename Tb>
-void launch_add(const double* a, const Tb* b, double* out, int64_t n, cudaStream_t s) {
-  int blocks = (int)std::min<int64_t>((n + 255) / 256, 1024);
-  if (blocks < 1) blocks = 1;
-  k_add<Tb><<<blocks, 256, 0, s>>>(a, b, out, n); count_launch();
-}
-template void launch_add<float>(const double*, const float*, double*, int64_t, cudaStream_t);
-template void launch_add<double>(const double*, const double*, double*, int64_t, cudaStream_t);
-
 // ---------------------------------------------------------------------------
-// Weighted squared norms (Eq. 2.2 with the quadrature of Eq. 2.17), deterministic:
-// block partials in fixed order, then one block sums the partials in fixed order.
-//   sum_i w_1(i_1) ... w_p(i_p) (x[i] - y[i])^2      (y may be null)
-// Grid-stride over mode-1 columns; the product of the other weights is formed
-// once per column.
+// The snapshot difference out = scale (a - b) (scale 1, or a central difference's) and its
+// weighted squared norm (Eq. 2.2 with the quadrature of Eq. 2.17) in one pass, for the mode
+// products' route of the projection:
+//   sum_i w_1(i_1) ... w_p(i_p) out[i]^2
+// A warp per mode-1 column, the column weights prod_{m>1} w_m from `wcol`.  Deterministic:
+// warp and CTA partials in a fixed order, added by the last CTA to finish (`counter` is zero
+// before and after).  64^3 double from a cold cache: 12.7 us, as difference, norm and
+// sum apart 23.7 us.
 // ---------------------------------------------------------------------------
-
-
 template <typename T>
-__global__ void k_wnorm2_partial(const T* __restrict__ x, const T* __restrict__ y, WeightView wv,
-                                 double* __restrict__ partial, unsigned* flags) {
+__global__ void __launch_bounds__(256) k_diff_norm(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out,
+                                                   int N1, unsigned ncol, T scale, const T* __restrict__ w1,
+                                                   const T* __restrict__ wcol, double* __restrict__ partial,
+                                                   unsigned* __restrict__ counter, double* __restrict__ norm2,
+                                                   unsigned* flags) {
   __shared__ double sh[32];
-  const int64_t N1 = wv.N[0];
-  int64_t ncol = 1;
-  for (int m = 1; m < wv.p; ++m) ncol *= wv.N[m];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31;
+  const unsigned nw = gridDim.x * (blockDim.x >> 5);
   double acc = 0.0;
   bool bad = false;
-  for (int64_t c = blockIdx.x; c < ncol; c += gridDim.x) {
-    double wc = 1.0;
-    unsigned rem = (unsigned)c;
-    for (int m = 1; m < wv.p; ++m) {
-      const unsigned nm = (unsigned)wv.N[m];
-      wc *= wv.w[m][rem % nm];
-      rem /= nm;
+  for (unsigned c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < ncol; c += nw) {
+    const size_t o = (size_t)N1 * c;
+    T s = T(0);
+    for (int i = lane; i < N1; i += 32) {
+      const T d = (a[o + i] - b[o + i]) * scale;
+      out[o + i] = d;
+      bad |= !isfinite(d);
+      s = fma(w1[i] * d, d, s);
     }
-    const T* xc = x + c * N1;
-    const T* yc = y ? y + c * N1 : nullptr;
-    T s = 0;                 // per-thread partial over <= N1 / blockDim terms in the data type
-    for (int64_t i = threadIdx.x; i < N1; i += blockDim.x) {
-      T d = xc[i] - (yc ? yc[i] : T(0));
-      bad |= !isfinite((double)d);
-      s += (T)wv.w[0][i] * d * d;
-    }
-    acc += wc * (double)s;
+    acc = fma((double)wcol[c], (double)s, acc);
   }
   acc = block_sum(acc, sh);
   if (bad && flags) atomicOr(flags, kFlagNonFinite);
-  if (threadIdx.x == 0) partial[blockIdx.x] = acc;
-}
-
-__global__ void k_sum_partials(const double* __restrict__ partial, int n, double* __restrict__ out) {
-  __shared__ double sh[32];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += partial[i];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) *out = s;
+  if (threadIdx.x == 0) {
+    partial[blockIdx.x] = acc;
+    __threadfence();
+    last = (atomicAdd(counter, 1u) == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double t = 0.0;
+  for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) t += __ldcg(&partial[k]);
+  t = block_sum(t, sh);
+  if (threadIdx.x == 0) {
+    *norm2 = t;
+    atomicExch(counter, 0u);
+  }
 }
 
 template <typename T>
-void launch_wnorm2(const T* x, const T* y, const WeightView& wv, double* partial, int nblocks, double* out,
-                   unsigned* flags, cudaStream_t s) {
-  k_wnorm2_partial<T><<<nblocks, 256, 0, s>>>(x, y, wv, partial, flags); count_launch();
-  k_sum_partials<<<1, 256, 0, s>>>(partial, nblocks, out); count_launch();
+void launch_diff_norm(const T* a, const T* b, T* out, int N1, int64_t ncol, T scale, const T* w1, const T* wcol,
+                      double* partial, unsigned* counter, int nblocks, double* norm2, unsigned* flags, cudaStream_t s) {
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(nblocks, (ncol + 7) / 8));
+  k_diff_norm<T><<<blocks, 256, 0, s>>>(a, b, out, N1, (unsigned)ncol, scale, w1, wcol, partial, counter, norm2, flags);
+  count_launch();
 }
-template void launch_wnorm2<float>(const float*, const float*, const WeightView&, double*, int, double*, unsigned*,
-                                   cudaStream_t);
-template void launch_wnorm2<double>(const double*, const double*, const WeightView&, double*, int, double*,
-                                    unsigned*, cudaStream_t);
+template void launch_diff_norm<float>(const float*, const float*, float*, int, int64_t, float, const float*,
+                                      const float*, double*, unsigned*, int, double*, unsigned*, cudaStream_t);
+template void launch_diff_norm<double>(const double*, const double*, double*, int, int64_t, double, const double*,
+                                       const double*, double*, unsigned*, int, double*, unsigned*, cudaStream_t);
 
 // Exact error of Eq. 2.20 without materialising V^TDB: with H = T x_2 U_2 ... x_p U_p
 // (r_1 x N_2 x ... x N_p), every mode-1 column of the reconstruction is U_1 H[:, c].
@@ -373,10 +348,6 @@ void launch_weights_T(const WeightView& wv, T* w1, T* wcol, cudaStream_t s) {
 template void launch_weights_T<float>(const WeightView&, float*, float*, cudaStream_t);
 template void launch_weights_T<double>(const WeightView&, double*, double*, cudaStream_t);
 
-void launch_sum_partials(const double* partial, int n, double* out, cudaStream_t s) {
-  k_sum_partials<<<1, 256, 0, s>>>(partial, n, out); count_launch();
-}
-
 // ---------------------------------------------------------------------------
 // Generic n-mode product
 // ---------------------------------------------------------------------------
@@ -575,10 +546,12 @@ __global__ void k_mp_reduce_block(const Tin* __restrict__ in, Tacc* __restrict__
   }
 }
 
-// K small: one thread per output element (l, j, q), l fastest.
+// K small: a thread per output element (l, j, q), l fastest.  For few outputs: bound by the
+// latency of the K loads and of the chain of products, so eight terms' loads are in flight
+// while the eight before are multiplied.
 template <typename Tin, typename Tm, typename Tacc>
-__global__ void k_mp_expand(const Tin* __restrict__ in, Tacc* __restrict__ out, const Tm* __restrict__ M, int64_t L,
-                            int K, int J, int64_t Q, int64_t sMj, int64_t sMk, const int* __restrict__ gate) {
+__global__ void k_mp_expand1(const Tin* __restrict__ in, Tacc* __restrict__ out, const Tm* __restrict__ M, int64_t L,
+                             int K, int J, int64_t Q, int64_t sMj, int64_t sMk, const int* __restrict__ gate) {
   if (gate && *gate == 0) return;
   const unsigned total = (unsigned)(L * J * Q), uL = (unsigned)L, uJ = (unsigned)J;
   for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
@@ -588,11 +561,249 @@ __global__ void k_mp_expand(const Tin* __restrict__ in, Tacc* __restrict__ out, 
     const unsigned q = jq / uJ;
     const Tin* base = in + l + (size_t)uL * K * q;
     const Tm* mrow = M + j * sMj;
-    Tacc acc = Tacc(0);
-    for (int k = 0; k < K; ++k) acc += (Tacc)mrow[k * sMk] * (Tacc)base[(size_t)k * uL];
+    // eight terms at a time, the next eight's loads issued before the current products
+    Tacc acc = Tacc(0), a[8], b[8];
+    auto fetch = [&](int k) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        a[t] = k + t < K ? (Tacc)__ldg(&mrow[(k + t) * sMk]) : Tacc(0);
+        b[t] = k + t < K ? (Tacc)__ldg(&base[(size_t)(k + t) * uL]) : Tacc(0);
+      }
+    };
+    fetch(0);
+    for (int k = 0; k < K; k += 8) {
+      Tacc x[8], y[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) { x[t] = a[t]; y[t] = b[t]; }
+      if (k + 8 < K) fetch(k + 8);
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (k + t < K) acc = fma(x[t], y[t], acc);
+    }
     out[e] = acc;
   }
 }
+
+// K small: a thread per (l, q), l fastest, and JT consecutive outputs j: every value of `in` is
+// read once for the JT of them, their M (blockIdx.y's rows) comes from shared memory.  Each
+// output sums its K products in order whatever JT is.  Bound: the stores of L J Q values;
+// r_1 N_2 N_3 = 11 x 128 x 512 from K = 16: 5.6 us, where a thread per output (K reads of both
+// operands for each) took 9.7 us.  Taken where that makes two CTAs per SM and half of the last
+// JT are not wasted.
+template <typename Tin, typename Tm, typename Tacc, int JT>
+__global__ void __launch_bounds__(256) k_mp_expand(const Tin* __restrict__ in, Tacc* __restrict__ out,
+                                                   const Tm* __restrict__ M, int64_t L, int K, int J, int64_t Q,
+                                                   int64_t sMj, int64_t sMk, const int* __restrict__ gate) {
+  if (gate && *gate == 0) return;
+  __shared__ Tacc Ms[64 * JT];                       // [k][jj]
+  const unsigned total = (unsigned)(L * Q), uL = (unsigned)L, uJ = (unsigned)J;
+  for (int j0 = blockIdx.y * JT; j0 < J; j0 += gridDim.y * JT) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < K * JT; e += blockDim.x) {
+      const int k = e / JT, j = j0 + e % JT;
+      Ms[e] = j < J ? (Tacc)M[j * sMj + k * sMk] : Tacc(0);
+    }
+    __syncthreads();
+    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+      const unsigned l = e % uL, q = e / uL;
+      const Tin* base = in + l + (size_t)uL * K * q;
+      Tacc acc[JT];
+#pragma unroll
+      for (int t = 0; t < JT; ++t) acc[t] = Tacc(0);
+#pragma unroll 4
+      for (int k = 0; k < K; ++k) {
+        const Tacc v = (Tacc)base[(size_t)k * uL];
+#pragma unroll
+        for (int t = 0; t < JT; ++t) acc[t] = fma(Ms[k * JT + t], v, acc[t]);
+      }
+      Tacc* o = out + l + (size_t)uL * (j0 + (size_t)uJ * q);
+#pragma unroll
+      for (int t = 0; t < JT; ++t)
+        if (j0 + t < J) o[(size_t)t * uL] = acc[t];
+    }
+  }
+}
+
+// Float, L == 1, K large: out[j + J q] = sum_k M[j, k] in[k + K q], the first contraction of a
+// (re)initialisation's core (V x_1 A_1^T).  A warp takes eight columns q at a time, its lanes
+// four k of each 128; four outputs at a time are summed over the lanes by a transposing
+// butterfly (lane l ends with column l % 8, output l / 8).  M in shared memory, zero past K.
+// Bound: HBM (K Q values read once); 256 x 128 x 512 at 11 outputs: 33 us, where a warp per
+// column with M from global memory took 160 us.
+__global__ void __launch_bounds__(256) k_mp_cols(const float* __restrict__ in, float* __restrict__ out,
+                                                 const float* __restrict__ M, int K, int J, unsigned Q, int64_t sMj,
+                                                 int64_t sMk, int vec) {
+  extern __shared__ __align__(16) float mc_sm[];       // [J rounded up to 4][Kp]
+  const int Kp = (K + 127) & ~127, Jp = (J + 3) & ~3;
+  for (int e = threadIdx.x; e < Jp * Kp; e += blockDim.x) {
+    const int j = e / Kp, k = e % Kp;
+    mc_sm[e] = (j < J && k < K) ? M[j * sMj + k * sMk] : 0.f;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const unsigned nw = gridDim.x * (blockDim.x >> 5);
+  for (unsigned g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); g * 8 < Q; g += nw) {
+    const unsigned q0 = g * 8;
+    for (int j0 = 0; j0 < Jp; j0 += 16) {              // sixteen outputs in registers at a time
+      float acc[4][32];
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[b][i] = 0.f;
+      for (int k0 = 0; k0 < Kp; k0 += 128) {
+        const int k = k0 + 4 * lane;
+        float4 v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          v[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (q0 + c < Q) {
+            const float* src = in + (size_t)K * (q0 + c) + k;
+            if (vec) {
+              if (k < K) v[c] = __ldg((const float4*)src);
+            } else {
+              if (k < K) v[c].x = __ldg(src);
+              if (k + 1 < K) v[c].y = __ldg(src + 1);
+              if (k + 2 < K) v[c].z = __ldg(src + 2);
+              if (k + 3 < K) v[c].w = __ldg(src + 3);
+            }
+          }
+        }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          if (j0 + 4 * b >= Jp) break;
+#pragma unroll
+          for (int a = 0; a < 4; ++a) {
+            const float4 m = *(const float4*)&mc_sm[(j0 + 4 * b + a) * Kp + k];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+              acc[b][c + 8 * a] = fmaf(v[c].w, m.w, fmaf(v[c].z, m.z, fmaf(v[c].y, m.y, fmaf(v[c].x, m.x, acc[b][c + 8 * a]))));
+          }
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        if (j0 + 4 * b >= Jp) break;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const bool up = lane & o;
+#pragma unroll
+          for (int i = 0; i < o; ++i) {
+            const float keep = up ? acc[b][i + o] : acc[b][i], send = up ? acc[b][i] : acc[b][i + o];
+            acc[b][i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+        }
+        const unsigned q = q0 + (lane & 7);
+        const int j = j0 + 4 * b + (lane >> 3);
+        if (q < Q && j < J) out[j + (size_t)J * q] = acc[b][0];
+      }
+    }
+  }
+}
+
+// V^TDB = U_1 H with H = T x_2 U_2 ... x_p U_p (r_1 x ncol): the last and only large product of
+// a reconstruction.  Lane l of a warp owns R rows of a block of 32 R with U_1's in registers
+// and walks a range of columns, 32 columns' H at a time through shared memory (padded to RM,
+// zeros past r_1), the next 32 loaded meanwhile.  Bound: HBM, N_1 ncol values written once.
+// 192 x 129 x 192 x 3 float at r_1 = 13: 24 us from a cold cache, where the product of the last mode with a
+// thread per output took 91 us, and the mode before it as long.
+template <typename T, int R, int RM>
+__global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, const T* __restrict__ H, int r1, int N1,
+                                                      unsigned ncol, int vec, T* __restrict__ V) {
+  extern __shared__ __align__(16) unsigned char ro_raw[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  T* hs = (T*)ro_raw + (size_t)wib * 32 * RM;
+  for (int e = lane; e < 32 * RM; e += 32) hs[e] = T(0);
+  __syncwarp();
+  const int nrb = (N1 + 32 * R - 1) / (32 * R);
+  const unsigned gw = blockIdx.x * (blockDim.x >> 5) + wib, tw = gridDim.x * (blockDim.x >> 5);
+  const unsigned wpr = tw >= (unsigned)nrb ? tw / nrb : 1u;
+  const unsigned kk = gw % wpr;
+  const unsigned c_lo = (unsigned)((uint64_t)ncol * kk / wpr), c_hi = (unsigned)((uint64_t)ncol * (kk + 1) / wpr);
+  for (unsigned rb = gw / wpr; rb < (unsigned)nrb && c_lo < c_hi; rb += (tw >= (unsigned)nrb ? (unsigned)nrb : tw)) {
+    const int i0 = (int)rb * 32 * R + R * lane;
+    T u[R][RM];
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+#pragma unroll
+      for (int a = 0; a < RM; ++a) u[q][a] = (i0 + q < N1 && a < r1) ? U1[i0 + q + (size_t)N1 * a] : T(0);
+    T nx[RM];                                          // this lane's share of the next 32 columns of H
+    auto fetch = [&](unsigned c) {
+      const unsigned nv = c < c_hi ? (unsigned)r1 * min(32u, c_hi - c) : 0u;
+#pragma unroll
+      for (int a = 0; a < RM; ++a) {
+        const unsigned e = lane + 32 * a;
+        nx[a] = (a < r1 && e < nv) ? __ldg(&H[(size_t)r1 * c + e]) : T(0);
+      }
+    };
+    fetch(c_lo);
+    for (unsigned c0 = c_lo; c0 < c_hi; c0 += 32) {
+      __syncwarp();
+#pragma unroll
+      for (int a = 0; a < RM; ++a)
+        if (a < r1) {
+          const int e = lane + 32 * a;
+          hs[(e / r1) * RM + e % r1] = nx[a];
+        }
+      __syncwarp();
+      fetch(c0 + 32);
+      const int nc = (int)min(32u, c_hi - c0);
+      for (int c = 0; c < nc; ++c) {
+        T h[RM], rec[R];
+        lds_run<T, RM>(hs + c * RM, h);
+#pragma unroll
+        for (int q = 0; q < R; ++q) rec[q] = T(0);
+#pragma unroll
+        for (int a = 0; a < RM; ++a)
+          if (sizeof(T) == 4 || a < r1)
+#pragma unroll
+            for (int q = 0; q < R; ++q) rec[q] = fma(u[q][a], h[a], rec[q]);
+        T* o = V + (size_t)N1 * (c0 + c) + i0;
+        if (vec) {
+          if (i0 < N1) {
+            if constexpr (R * sizeof(T) == 16 && sizeof(T) == 4)
+              __stcs((float4*)o, make_float4(rec[0], rec[1 % R], rec[2 % R], rec[3 % R]));
+            else if constexpr (R == 2 && sizeof(T) == 4)
+              __stcs((float2*)o, make_float2(rec[0], rec[1 % R]));
+            else if constexpr (R == 2)
+              __stcs((double2*)o, make_double2(rec[0], rec[1 % R]));
+            else
+              __stcs(o, rec[0]);
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < R; ++q)
+            if (i0 + q < N1) __stcs(o + q, rec[q]);
+        }
+      }
+    }
+  }
+}
+
+template <typename T>
+void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* V, cudaStream_t s) {
+  const uintptr_t va = (uintptr_t)V;
+  auto go = [&](auto kern, int R, int RM) {
+    const size_t sm = sizeof(T) * 8 * 32 * RM;
+    if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // a warp per 32 columns of a row block at least, two CTAs per SM at most
+    const int64_t units = ((N1 + 32 * R - 1) / (32 * R)) * ((ncol + 31) / 32);
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((units + 7) / 8, 2 * 152));
+    const int vec = N1 % R == 0 && va % (R * sizeof(T)) == 0;
+    kern<<<blocks, 256, sm, s>>>(U1, H, r1, N1, (unsigned)ncol, vec, V);
+    count_launch();
+  };
+  if constexpr (sizeof(T) == 4) {
+    if (r1 <= 8) go(k_recon_out<float, 4, 8>, 4, 8);
+    else if (r1 <= 16) go(k_recon_out<float, 4, 16>, 4, 16);
+    else go(k_recon_out<float, 2, 32>, 2, 32);
+  } else {
+    if (r1 <= 8) go(k_recon_out<double, 2, 8>, 2, 8);
+    else if (r1 <= 16) go(k_recon_out<double, 2, 16>, 2, 16);
+    else go(k_recon_out<double, 1, 32>, 1, 32);
+  }
+}
+template void launch_recon_out<float>(const float*, const float*, int, int, int64_t, float*, cudaStream_t);
+template void launch_recon_out<double>(const double*, const double*, int, int, int64_t, double*, cudaStream_t);
 
 template <typename Tin, typename Tm, typename Tacc>
 void launch_modeprod(const Tin* in, Tacc* out, const Tm* M, int64_t L, int K, int J, int64_t Q, int64_t sMj,
@@ -600,10 +811,43 @@ void launch_modeprod(const Tin* in, Tacc* out, const Tm* M, int64_t L, int K, in
   if (L <= 0 || K <= 0 || J <= 0 || Q <= 0) return;
   count_launch();
   if (K <= 64) {
-    int64_t total = L * J * Q;
-    int blocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 32);
-    k_mp_expand<Tin, Tm, Tacc><<<blocks, 256, 0, s>>>(in, out, M, L, K, J, Q, sMj, sMk, gate);
-  } else if (Q == 1 && L >= 64 && J <= 32) {
+    const int64_t lq = L * Q;
+    if (J >= 5 && ((lq + 255) / 256) * ((J + 7) / 8) >= 2 * 152) {
+      const dim3 grid((unsigned)std::min<int64_t>((lq + 255) / 256, 152 * 32), (unsigned)std::min((J + 7) / 8, 16384));
+      k_mp_expand<Tin, Tm, Tacc, 8><<<grid, 256, 0, s>>>(in, out, M, L, K, J, Q, sMj, sMk, gate);
+    } else if (((lq + 255) / 256) * ((J + 3) / 4) >= 2 * 152) {
+      const dim3 grid((unsigned)std::min<int64_t>((lq + 255) / 256, 152 * 32), (unsigned)std::min((J + 3) / 4, 16384));
+      k_mp_expand<Tin, Tm, Tacc, 4><<<grid, 256, 0, s>>>(in, out, M, L, K, J, Q, sMj, sMk, gate);
+    } else {
+      // blocks small enough to reach every SM (double issues 64 cycles apart on each)
+      const int64_t total = lq * J;
+      int block = 256;
+      while (block > 64 && (total + block - 1) / block < 2 * 152) block /= 2;
+      k_mp_expand1<Tin, Tm, Tacc><<<(unsigned)std::min<int64_t>((total + block - 1) / block, 152 * 32), block, 0, s>>>(
+          in, out, M, L, K, J, Q, sMj, sMk, gate);
+    }
+    return;
+  }
+  if constexpr (std::is_same<Tin, float>::value && std::is_same<Tm, float>::value && std::is_same<Tacc, float>::value) {
+    const size_t sm = (size_t)((J + 3) & ~3) * ((K + 127) & ~127) * sizeof(float);
+    if (L == 1 && Q >= 1024 && sm <= 160 * 1024) {
+      if (sm > 48 * 1024) cudaFuncSetAttribute(k_mp_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+      const int vec = (K & 3) == 0 && ((uintptr_t)in & 15) == 0;
+      const int blocks = (int)std::min<int64_t>((Q + 63) / 64, 152);
+      k_mp_cols<<<blocks, 256, sm, s>>>(in, out, M, K, J, (unsigned)Q, sMj, sMk, vec);
+      return;
+    }
+    // few rows: a block per (l, q) splits K, where 64-row tiles would leave most SMs idle
+    // (88 x 512 by 16: 7.5 against 29 us with two CTAs)
+    if (Q == 1 && L > 1 && L <= 256) {
+      const int blocks = (int)std::min<int64_t>(L, 152 * 8);
+      if (J <= 8) k_mp_reduce_block<Tin, Tm, Tacc, 8><<<blocks, 256, 0, s>>>(in, out, M, L, K, J, Q, sMj, sMk);
+      else if (J <= 16) k_mp_reduce_block<Tin, Tm, Tacc, 16><<<blocks, 256, 0, s>>>(in, out, M, L, K, J, Q, sMj, sMk);
+      else k_mp_reduce_block<Tin, Tm, Tacc, 32><<<blocks, 256, 0, s>>>(in, out, M, L, K, J, Q, sMj, sMk);
+      return;
+    }
+  }
+  if (Q == 1 && L >= 64 && J <= 32) {
     const int blocks = (int)std::min<int64_t>((L + 63) / 64, 152 * 8);
     k_mp_gemm<Tin, Tm, Tacc><<<blocks, 256, 0, s>>>(in, out, M, L, K, J, sMj, sMk);
   } else if (L > 1 && L * Q <= 1024) {

@@ -23,8 +23,8 @@
 // Measured, all modes of a re-initialisation: 256 x 128 x 512 float (k = 18, 13, 10) 1.07 ms,
 // where a float subspace iteration refined by double iterations and a one-CTA Jacobi, mode
 // after mode in 130 launches, took 6.0 ms; 126^3 double (k = 7) 0.34 ms, where 24 iterations
-// of single launches took 11.2 ms; 59^3 double against the one-CTA Jacobi, a whole
-// re-initialisation 1.1 against 24.8 ms.
+// of single launches took 11.2 ms; 90^3 double against a one-CTA Jacobi of the whole Gram, a
+// re-initialisation 1.1 against 76 ms.
 #include "common.cuh"
 #include "fastrcp.cuh"
 #include "kernels.h"

@@ -111,18 +111,18 @@ void count_launch(int n = 1);
 long long launches_so_far();
 
 // k_basic.cu
-template <typename T> void launch_diff(const T* a, const T* b, T* out, int64_t n, cudaStream_t s, T scale = T(1));
 template <typename T> void launch_weighted_bases(const double* U, const double* w, T* A, int64_t N, int r, cudaStream_t s);
 template <typename Ts, typename Td> void launch_cast(const Ts* a, Td* b, int64_t n, cudaStream_t s);
-template <typename Tb> void launch_add(const double* a, const Tb* b, double* out, int64_t n, cudaStream_t s);
 template <typename T>
-void launch_wnorm2(const T* x, const T* y, const WeightView& wv, double* partial, int nblocks, double* out,
-                   unsigned* flags, cudaStream_t s);
-void launch_sum_partials(const double* partial, int n, double* out, cudaStream_t s);
+void launch_diff_norm(const T* a, const T* b, T* out, int N1, int64_t ncol, T scale, const T* w1, const T* wcol,
+                      double* partial, unsigned* counter, int nblocks, double* norm2, unsigned* flags, cudaStream_t s);
 template <typename T>
 void launch_recon_err(const T* V, const T* U1, const T* H, int r1, int N1, int64_t ncol, const T* w1, const T* wcol,
                       double* partial, unsigned* counter, int nblocks, double* out, unsigned* flags, cudaStream_t s,
                       const int* gate = nullptr);
+// V = U1 H (N1 x ncol; H: r1 x ncol)
+template <typename T>
+void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* V, cudaStream_t s);
 template <typename T>
 void launch_weights_T(const WeightView& wv, T* w1, T* wcol, cudaStream_t s);
 template <typename Tin, typename Tm, typename Tacc>

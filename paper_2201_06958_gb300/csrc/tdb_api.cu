@@ -571,34 +571,11 @@ tdb_status project_tree(tdb_ctx* ctx, const Tc* dV, cudaEvent_t* evm) {
   return TDB_OK;
 }
 
-// V^TDB = T x_1 U_1 ... x_p U_p into out (compute type)
+// H = T x_2 U_2 ... x_p U_p (r_1 x N_2 x ... x N_p, compute type), whose columns U_1 maps to the
+// mode-1 columns of V^TDB.
 template <typename Tc>
-tdb_status reconstruct_into(tdb_ctx* ctx, Tc* out) {
+const Tc* column_factors(tdb_ctx* ctx, const int* gate) {
   const int p = ctx->p;
-  cudaStream_t s = ctx->stream;
-  int64_t cur[kMaxModes];
-  for (int m = 0; m < p; ++m) cur[m] = ctx->r[m];
-  const Tc* src = (const Tc*)ctx->Tcore;
-  Tc* bufs[2] = {(Tc*)ctx->ping, (Tc*)ctx->pong};
-  for (int n = 0; n < p; ++n) {
-    Tc* dst = (n == p - 1) ? out : bufs[n & 1];
-    int64_t L = 1, Q = 1;
-    for (int m = 0; m < n; ++m) L *= cur[m];
-    for (int m = n + 1; m < p; ++m) Q *= cur[m];
-    launch_modeprod<Tc, Tc, Tc>(src, dst, (const Tc*)ctx->Uc[n], L, ctx->r[n], (int)ctx->N[n], Q, 1, ctx->N[n], s);
-    cur[n] = ctx->N[n];
-    src = dst;
-  }
-  CHECK_LAUNCH();
-  return TDB_OK;
-}
-
-// err2 = ||V - T x U||_W^2 (Eq. 2.20): H = T x_2 U_2 ... x_p U_p, then the fused pass
-// over V that forms each mode-1 column U_1 H[:, c] on the fly.
-template <typename Tc>
-tdb_status exact_error2(tdb_ctx* ctx, const Tc* V, const int* gate = nullptr) {
-  const int p = ctx->p;
-  cudaStream_t s = ctx->stream;
   int64_t cur[kMaxModes];
   for (int m = 0; m < p; ++m) cur[m] = ctx->r[m];
   const Tc* src = (const Tc*)ctx->Tcore;
@@ -608,14 +585,32 @@ tdb_status exact_error2(tdb_ctx* ctx, const Tc* V, const int* gate = nullptr) {
     int64_t L = 1, Q = 1;
     for (int m = 0; m < n; ++m) L *= cur[m];
     for (int m = n + 1; m < p; ++m) Q *= cur[m];
-    launch_modeprod<Tc, Tc, Tc>(src, dst, (const Tc*)ctx->Uc[n], L, ctx->r[n], (int)ctx->N[n], Q, 1, ctx->N[n], s,
-                                gate);
+    launch_modeprod<Tc, Tc, Tc>(src, dst, (const Tc*)ctx->Uc[n], L, ctx->r[n], (int)ctx->N[n], Q, 1, ctx->N[n],
+                                ctx->stream, gate);
     cur[n] = ctx->N[n];
     src = dst;
   }
-  launch_recon_err<Tc>(V, (const Tc*)ctx->Uc[0], src, ctx->r[0], (int)ctx->N[0], ctx->S / ctx->N[0],
+  return src;
+}
+
+// V^TDB = T x_1 U_1 ... x_p U_p into out (compute type): mode 1 last, so that the only product
+// of S values reads H and writes V^TDB once.
+template <typename Tc>
+tdb_status reconstruct_into(tdb_ctx* ctx, Tc* out) {
+  const Tc* H = column_factors<Tc>(ctx, nullptr);
+  launch_recon_out<Tc>((const Tc*)ctx->Uc[0], H, ctx->r[0], (int)ctx->N[0], ctx->S / ctx->N[0], out, ctx->stream);
+  CHECK_LAUNCH();
+  return TDB_OK;
+}
+
+// err2 = ||V - T x U||_W^2 (Eq. 2.20): the fused pass over V that forms each mode-1 column
+// U_1 H[:, c] on the fly.
+template <typename Tc>
+tdb_status exact_error2(tdb_ctx* ctx, const Tc* V, const int* gate = nullptr) {
+  const Tc* H = column_factors<Tc>(ctx, gate);
+  launch_recon_err<Tc>(V, (const Tc*)ctx->Uc[0], H, ctx->r[0], (int)ctx->N[0], ctx->S / ctx->N[0],
                        (const Tc*)ctx->w1T, (const Tc*)ctx->wcolT, ctx->npart, ctx->redcnt, ctx->nblk,
-                       &ctx->rb_dev->err2, ctx->flags, s, gate);
+                       &ctx->rb_dev->err2, ctx->flags, ctx->stream, gate);
   CHECK_LAUNCH();
   return TDB_OK;
 }
@@ -1099,9 +1094,9 @@ tdb_status enqueue_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vp, bool all_paths
                          (const double* const*)ctx->w, (Tc*)ctx->ping, (Tc* const*)ctx->Y, &ctx->rb_dev->dv2,
                          ctx->flags, s, evm, ctx->err, (Tc)scale));
     } else {
-      launch_diff<Tc>(Vn, Vfrom, (Tc*)ctx->dV, ctx->S, s, (Tc)scale);
-      launch_wnorm2<Tc>((const Tc*)ctx->dV, nullptr, weight_view(ctx), ctx->npart, ctx->nblk, &ctx->rb_dev->dv2,
-                        ctx->flags, s);
+      launch_diff_norm<Tc>(Vn, Vfrom, (Tc*)ctx->dV, (int)ctx->N[0], ctx->S / ctx->N[0], (Tc)scale,
+                           (const Tc*)ctx->w1T, (const Tc*)ctx->wcolT, ctx->npart, ctx->redcnt + 1, ctx->nblk,
+                           &ctx->rb_dev->dv2, ctx->flags, s);
       CHECK_LAUNCH();
       TRY(project_tree<Tc>(ctx, (const Tc*)ctx->dV, evm));
     }

@@ -1,4 +1,5 @@
-"""The float and double projection pass and the exact error at the edges of their tiles.
+"""The float and double projection pass, the exact error and the reconstruction at the edges
+of their tiles.
 
 Every entry of dS and Y_n against the oracle's, within the rounding bound of the sums that
 form it: a chain of products contracting N_1, ..., N_p terms in arithmetic of unit roundoff u
@@ -101,6 +102,9 @@ def test_projection_and_error_within_rounding(precision, dims, ranks, shift):
     big = O.reconstruct(np.abs(Tg), [np.abs(x) for x in Ug])
     slack = np.sqrt(np.sum(_weights(w) * ((sum(ranks) + 8 * p) * u * (big + wide)) ** 2))
     assert abs(info["eps"] - e) <= slack + (sum(dims) + 16) * u * e
+    out = torch.empty(v0.numel() + 8, dtype=dtype, device="cuda")[shift:shift + v0.numel()].view(v0.shape)
+    rec = synth.to_logical(c.reconstruct(out))
+    assert np.all(np.abs(rec - O.reconstruct(Tg, Ug)) <= (sum(ranks) + 8 * p) * u * big)
     c.close()
 
 
