@@ -122,23 +122,28 @@ template void launch_diff_norm<double>(const double*, const double*, double*, in
 // Exact error of Eq. 2.20 without materialising V^TDB: with H = T x_2 U_2 ... x_p U_p
 // (r_1 x N_2 x ... x N_p), every mode-1 column of the reconstruction is U_1 H[:, c].
 // Lane l of a warp owns rows i0 + R l .. i0 + R l + R - 1 of a block of 32 R rows, with U_1 of
-// those rows (R x r_1) and w_1 in registers, and walks a contiguous range of columns c.  Each
-// column's R rows per lane, H[:, c] (lanes < r_1) and w_c (lane 0) arrive by cp.async into a
-// ring of D column slots per warp (D columns in flight per warp, no registers held); H[:, c]
-// is a broadcast read.  Per column the lane forms U_1 H[:, c] for its rows and the weighted
-// squared difference; w_c times it goes into a sum of the compute type that is added to the
-// double accumulator every D columns.  The last CTA to finish adds the per-CTA partials in a
-// fixed order and writes *out (no second launch); `counter` is zero before and after.
-// Double runs at 64 cycles per instruction and sub-partition, so there only the r_1 products
-// that exist are formed (float takes all RM, zeros past r_1).
-// Measured: 126^3 double at r_1 = 5, 54 us (8 double operations a point: 30 us at the issue
-// rate), where a warp per column with U_1 in shared memory and H[:, c] by shuffles took 156 us.
+// those rows (R x r_1) and w_1 in registers, and walks a contiguous range of columns c.  Its R
+// rows of each column arrive by cp.async in a ring of D slots (D columns in flight per warp,
+// read back by the lane that copied them: no barrier); H and w_c come 32 columns at a time, H
+// through shared memory (rows padded to RM, zeros past r_1), w_c a column per lane.  Per column
+// the lane forms U_1 H[:, c] for its rows and the weighted squared difference; w_c times it
+// goes into a sum of the compute type that is added to the double accumulator every D columns.
+// The last CTA to finish adds the per-CTA partials in a fixed order and writes *out (no second
+// launch); `counter` is zero before and after.  Double runs at 64 cycles per instruction and
+// sub-partition, so there only the r_1 products that exist are formed (float takes all RM).
+// Measured from a cold cache: 256 x 128 x 512 float at r_1 = 11, 26 us (32 us with a column's H
+// and w_c copied by cp.async beside its rows and two warp barriers a column); 126^3 double at
+// r_1 = 5, 54 us (8 double operations a point: 30 us at the issue rate), where a warp per column
+// with U_1 in shared memory and H[:, c] by shuffles took 156 us.
 constexpr int RE_D = 8;           // columns in flight per warp
 template <int BYTES>
 __device__ __forceinline__ void cp_async_n(void* dst, const void* src, bool valid) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(d), "l"(src), "r"(valid ? BYTES : 0), "n"(BYTES)
-               : "memory");
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(d), "l"(src), "r"(valid ? BYTES : 0), "n"(BYTES)
+                 : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -165,6 +170,29 @@ __device__ __forceinline__ void lds_run(const T* p, T* v) {
   }
 }
 
+// 32 columns of an r1 x ncol matrix (contiguous), r1 values a lane in registers, and into the
+// warp's shared rows of RM
+template <typename T, int RM>
+struct ColChunk {
+  T nx[RM];
+  __device__ __forceinline__ void fetch(const T* __restrict__ H, int r1, unsigned c, unsigned c_hi, int lane) {
+    const unsigned nv = c < c_hi ? (unsigned)r1 * min(32u, c_hi - c) : 0u;
+#pragma unroll
+    for (int a = 0; a < RM; ++a) {
+      const unsigned e = lane + 32 * a;
+      nx[a] = (a < r1 && e < nv) ? __ldg(&H[(size_t)r1 * c + e]) : T(0);
+    }
+  }
+  __device__ __forceinline__ void put(T* hs, int r1, int lane) const {
+#pragma unroll
+    for (int a = 0; a < RM; ++a)
+      if (a < r1) {
+        const int e = lane + 32 * a;
+        hs[(e / r1) * RM + e % r1] = nx[a];
+      }
+  }
+};
+
 template <typename T, int R, int RM>
 __global__ void __launch_bounds__(256, 2) k_recon_err_rows(const T* __restrict__ V, const T* __restrict__ U1,
                                                          const T* __restrict__ H, int r1, int N1, unsigned ncol,
@@ -173,15 +201,13 @@ __global__ void __launch_bounds__(256, 2) k_recon_err_rows(const T* __restrict__
                                                          unsigned* __restrict__ counter, double* __restrict__ out,
                                                          unsigned* flags, const int* __restrict__ gate) {
   if (gate && *gate == 0) return;          // the estimator ruled this evaluation out
-  constexpr int SLOT = 32 * R + RM + 4;    // values per column slot: rows, H[:, c] (zero past r_1), w_c
   extern __shared__ __align__(16) unsigned char ring_raw[];
   __shared__ double sh[32];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  T (*slot)[SLOT] = (T(*)[SLOT])((T*)ring_raw + (size_t)wib * RE_D * SLOT);
-  // H entries past r_1 are never copied: zero them once (they meet zero rows of U_1)
-  for (int e = lane; e < RE_D * RM; e += 32) slot[e / RM][32 * R + e % RM] = T(0);
-  __syncwarp();
+  T* ring = (T*)ring_raw + (size_t)wib * (RE_D * 32 * R + 32 * RM) + R * lane;     // this lane's rows of slot 0
+  T* hs = (T*)ring_raw + (size_t)wib * (RE_D * 32 * R + 32 * RM) + RE_D * 32 * R;
+  for (int e = lane; e < 32 * RM; e += 32) hs[e] = T(0);
   const int nrb = (N1 + 32 * R - 1) / (32 * R);
   const unsigned gw = blockIdx.x * (blockDim.x >> 5) + wib, tw = gridDim.x * (blockDim.x >> 5);
   const unsigned wpr = tw >= (unsigned)nrb ? tw / nrb : 1u;   // warps per row block
@@ -190,9 +216,30 @@ __global__ void __launch_bounds__(256, 2) k_recon_err_rows(const T* __restrict__
   const unsigned kk = gw % wpr;
   const unsigned c_lo = (unsigned)((uint64_t)ncol * kk / wpr), c_hi = (unsigned)((uint64_t)ncol * (kk + 1) / wpr);
   // (a row block per group of wpr warps; the outer loop only where there are fewer warps than blocks)
-  for (unsigned rbw = gw / wpr; rbw < (unsigned)nrb && c_lo < c_hi; rbw += (tw >= (unsigned)nrb ? (unsigned)nrb : tw)) {
-    const int rb = (int)rbw;
-    const int i0 = rb * 32 * R + R * lane;
+  for (unsigned rb = gw / wpr; rb < (unsigned)nrb && c_lo < c_hi; rb += (tw >= (unsigned)nrb ? (unsigned)nrb : tw)) {
+    const int i0 = (int)rb * 32 * R + R * lane;
+    const bool rows_in = i0 < N1;
+    const T* vsrc = V + (size_t)N1 * c_lo + (rows_in ? i0 : 0);   // the next column to issue
+    unsigned cnext = c_lo;
+    auto issue = [&](int sl) {
+      const bool in = cnext < c_hi;
+      T* dst = ring + sl * 32 * R;
+      if (vec) {
+        cp_async_n<R * sizeof(T)>(dst, vsrc, in && rows_in);
+      } else {
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+          cp_async_n<sizeof(T)>(dst + q, vsrc + (i0 + q < N1 ? q : 0), in && i0 + q < N1);
+      }
+      cp_async_commit();
+      ++cnext;
+      if (cnext < c_hi) vsrc += N1;          // (past the end: zero bytes from the last column)
+    };
+#pragma unroll
+    for (int t = 0; t < RE_D; ++t) issue(t);
+    ColChunk<T, RM> hc;
+    hc.fetch(H, r1, c_lo, c_hi, lane);
+    T wn = c_lo + lane < c_hi ? __ldg(&wcol[c_lo + lane]) : T(0);
     T u[R][RM], wr[R];
 #pragma unroll
     for (int q = 0; q < R; ++q) {
@@ -201,71 +248,46 @@ __global__ void __launch_bounds__(256, 2) k_recon_err_rows(const T* __restrict__
 #pragma unroll
       for (int a = 0; a < RM; ++a) u[q][a] = (i < N1 && a < r1) ? U1[i + (size_t)N1 * a] : T(0);
     }
-    // source pointers of the next column to issue, advanced by one column per issue; past
-    // c_hi the copies read nothing (zero bytes) from the last valid column
-    const bool rows_in = i0 < N1;
-    const T* vsrc = V + (size_t)N1 * c_lo + (rows_in ? i0 : 0);
-    const T* hsrc = H + (size_t)r1 * c_lo + (lane < r1 ? lane : 0);
-    const T* wsrc = wcol + c_lo;
-    unsigned cnext = c_lo;
-    auto issue = [&](int sl) {
-      const bool in = cnext < c_hi;
-      if (vec) {
-        cp_async_n<R * sizeof(T)>(&slot[sl][R * lane], vsrc, in && rows_in);
-      } else {
-#pragma unroll
-        for (int q = 0; q < R; ++q)
-          cp_async_n<sizeof(T)>(&slot[sl][R * lane + q], vsrc + (i0 + q < N1 ? q : 0), in && i0 + q < N1);
-      }
-      if (lane < r1) cp_async_n<sizeof(T)>(&slot[sl][32 * R + lane], hsrc, in);
-      if (lane == 0) cp_async_n<sizeof(T)>(&slot[sl][32 * R + RM], wsrc, in);
-      cp_async_commit();
-      if (in && cnext + 1 < c_hi) {
-        vsrc += N1;
-        hsrc += r1;
-        wsrc += 1;
-      }
-      ++cnext;
-    };
-#pragma unroll
-    for (int t = 0; t < RE_D; ++t) issue(t);
     T csum = T(0);
-    int sl = 0;
-    for (unsigned c = c_lo; c < c_hi; ++c) {
-      cp_async_wait<RE_D - 1>();           // this column's copies (the oldest group) have landed
+    for (unsigned c0 = c_lo; c0 < c_hi; c0 += 32) {
       __syncwarp();
-      T v[R], h[RM];
-      lds_run<T, R>(&slot[sl][R * lane], v);
-      lds_run<T, RM>(&slot[sl][32 * R], h);
-      const T wc = slot[sl][32 * R + RM];
+      hc.put(hs, r1, lane);
+      const T wl = wn;
       __syncwarp();
-      issue(sl);                           // the slot refills with the column D ahead
-      T rec[R];
+      hc.fetch(H, r1, c0 + 32, c_hi, lane);
+      wn = c0 + 32 + lane < c_hi ? __ldg(&wcol[c0 + 32 + lane]) : T(0);
+      const int nc = (int)min(32u, c_hi - c0);
+      for (int cb = 0; cb < nc; cb += RE_D) {
 #pragma unroll
-      for (int q = 0; q < R; ++q) rec[q] = T(0);
+        for (int t = 0; t < RE_D; ++t) {
+          if (cb + t >= nc) break;
+          cp_async_wait<RE_D - 1>();         // this column's copies (the oldest group) have landed
+          T v[R], h[RM];
+          lds_run<T, R>(ring + t * 32 * R, v);
+          lds_run<T, RM>(hs + (cb + t) * RM, h);
+          issue(t);                          // the slot refills with the column D ahead
+          T rec[R];
 #pragma unroll
-      for (int a = 0; a < RM; ++a)
-        if (sizeof(T) == 4 || a < r1)
+          for (int q = 0; q < R; ++q) rec[q] = T(0);
 #pragma unroll
-          for (int q = 0; q < R; ++q) rec[q] = fma(u[q][a], h[a], rec[q]);
-      T s = T(0);
+          for (int a = 0; a < RM; ++a)
+            if (sizeof(T) == 4 || a < r1)
 #pragma unroll
-      for (int q = 0; q < R; ++q) {
-        const T d = v[q] - rec[q];
-        s = fma(wr[q] * d, d, s);
-      }
-      csum = fma(wc, s, csum);
-      if (++sl == RE_D) {
-        sl = 0;
+              for (int q = 0; q < R; ++q) rec[q] = fma(u[q][a], h[a], rec[q]);
+          T s = T(0);
+#pragma unroll
+          for (int q = 0; q < R; ++q) {
+            const T d = v[q] - rec[q];
+            s = fma(wr[q] * d, d, s);
+          }
+          csum = fma(__shfl_sync(0xffffffffu, wl, cb + t), s, csum);
+        }
         bad |= !isfinite(csum);
         acc += (double)csum;
         csum = T(0);
       }
     }
     cp_async_wait<0>();
-    __syncwarp();
-    bad |= !isfinite(csum);
-    acc += (double)csum;
   }
   acc = block_sum(acc, sh);
   if (bad && flags) atomicOr(flags, kFlagNonFinite);
@@ -294,14 +316,15 @@ void launch_recon_err(const T* V, const T* U1, const T* H, int r1, int N1, int64
   const uintptr_t va = (uintptr_t)V;
   const int blocks = std::max(1, std::min(nblocks, 2 * 152));
   auto go = [&](auto kern, int R, int RM) {
-    const size_t sm = sizeof(T) * 8 * RE_D * (32 * R + RM + 4);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = sizeof(T) * 8 * (RE_D * 32 * R + 32 * RM);
+    if (sm > 47 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     const int vec = N1 % R == 0 && va % (R * sizeof(T)) == 0;
     kern<<<blocks, 256, sm, s>>>(V, U1, H, r1, N1, (unsigned)ncol, w1, wcol, vec, partial, counter, out, flags, gate);
     count_launch();
   };
   if constexpr (sizeof(T) == 4) {
     if (r1 <= 8) go(k_recon_err_rows<float, 4, 8>, 4, 8);
+    else if (r1 <= 12) go(k_recon_err_rows<float, 4, 12>, 4, 12);
     else if (r1 <= 16) go(k_recon_err_rows<float, 4, 16>, 4, 16);
     else go(k_recon_err_rows<float, 2, 32>, 2, 32);
   } else {
@@ -726,26 +749,13 @@ __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, 
     for (int q = 0; q < R; ++q)
 #pragma unroll
       for (int a = 0; a < RM; ++a) u[q][a] = (i0 + q < N1 && a < r1) ? U1[i0 + q + (size_t)N1 * a] : T(0);
-    T nx[RM];                                          // this lane's share of the next 32 columns of H
-    auto fetch = [&](unsigned c) {
-      const unsigned nv = c < c_hi ? (unsigned)r1 * min(32u, c_hi - c) : 0u;
-#pragma unroll
-      for (int a = 0; a < RM; ++a) {
-        const unsigned e = lane + 32 * a;
-        nx[a] = (a < r1 && e < nv) ? __ldg(&H[(size_t)r1 * c + e]) : T(0);
-      }
-    };
-    fetch(c_lo);
+    ColChunk<T, RM> hc;
+    hc.fetch(H, r1, c_lo, c_hi, lane);
     for (unsigned c0 = c_lo; c0 < c_hi; c0 += 32) {
       __syncwarp();
-#pragma unroll
-      for (int a = 0; a < RM; ++a)
-        if (a < r1) {
-          const int e = lane + 32 * a;
-          hs[(e / r1) * RM + e % r1] = nx[a];
-        }
+      hc.put(hs, r1, lane);
       __syncwarp();
-      fetch(c0 + 32);
+      hc.fetch(H, r1, c0 + 32, c_hi, lane);
       const int nc = (int)min(32u, c_hi - c0);
       for (int c = 0; c < nc; ++c) {
         T h[RM], rec[R];
@@ -794,6 +804,7 @@ void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* 
   };
   if constexpr (sizeof(T) == 4) {
     if (r1 <= 8) go(k_recon_out<float, 4, 8>, 4, 8);
+    else if (r1 <= 12) go(k_recon_out<float, 4, 12>, 4, 12);
     else if (r1 <= 16) go(k_recon_out<float, 4, 16>, 4, 16);
     else go(k_recon_out<float, 2, 32>, 2, 32);
   } else {
