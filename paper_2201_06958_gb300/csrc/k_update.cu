@@ -4,14 +4,17 @@
 // one CTA per mode, and bounded grid barriers separate the phases.  Tc is the
 // compute type (float or double); the state (U, T, R, R^{-1}, G^{-1}) is double.
 //   1 rows : M = Y_(n) T_(n)^T, X = M G_n^{-1}, partial P = A^T X with A = W U   (Tc)
-//            (pseudo-inverse and complement projector, Sec. 2.2; Eq. 2.16 times dt)
+//            (pseudo-inverse and complement projector, Sec. 2.2; Eq. 2.16 times dt);
+//            dS = Y_2 x_2 A_2^T on the CTAs without rows (all of them where every one has some)
 //   2 rows : P_n = sum of the partials, E = X - U P_n (Tc), U' = U + E (double;
 //            Euler step, Sec. 2.3), partial C = U'^T W U' (Tc)
-//   3 mode : C_n = R^T R and R^{-1} (weighted Cholesky-QR, the reading used to keep
-//            Eq. 2.6 through the step)
-//   4 rows : U'' = U' R^{-1} (double), A = W U'' and U'' in Tc;
-//            core (T + dS) x_1 R_1 (double)
-//   5      : core x_n R_n for n = 2..p (T x U is left unchanged)
+//   3 rows : C_n = R^T R and R^{-1} (weighted Cholesky-QR, the reading used to keep Eq. 2.6
+//            through the step), by every CTA for the mode of its rows (the same instructions
+//            on the same sums; cheaper than one CTA's result through L2 and a barrier);
+//            U'' = U' R^{-1} (double), A = W U'' and U'' in Tc
+//   4 slabs: (T + dS) x_1 R_1 x_2 R_2, the r_1 x r_2 slabs of the core (double; T x U is left
+//            unchanged)
+//   5      : x_3 R_3 (x_4 R_4), the r_3 x r_4 fibers; the core and its copy in Tc
 //   6 tasks: partial G_n = T_(n) T_(n)^T over column slices (double)
 //   7 mode : G_n, G_n^{-1} by Gauss-Jordan (double); sigma^2 (Eq. 2.18) by a float
 //            Jacobi warm-started from the previous eigenvectors, then Rayleigh
@@ -35,7 +38,7 @@ namespace {
 
 constexpr int LD = kMaxRank;
 constexpr int UPD_THREADS = 1024;
-constexpr size_t kUpdSmem = 48 * 1024;   // largest phase: the Gram finish, 45.6 KB
+constexpr size_t kUpdSmem = 54 * 1024;   // largest phase: the rows of phase 1 in double, 49.3 KB
 constexpr int GJ_THREADS = 256;          // threads 0..255 invert G_n by Gauss-Jordan
 // Modes with more row tiles than this (more than 1024 points) have their per-tile partial
 // sums of P_n and C_n reduced once by the whole grid (reduce_long) instead of by every
@@ -110,48 +113,54 @@ __device__ void trinv_d(const double* L, double* Li, int r, double* dinv) {
 }
 
 // ---------------------------------------------------------------------------
-// Float Cholesky and triangular inverse by one warp (lane i owns row i; the
-// float compute type's Cholesky-QR).  S is r x r, ld LD, in shared memory.
+// Float Cholesky S = L L^T and Li = L^{-1} by one warp (the float compute type's Cholesky-QR),
+// r <= RM, ld LD, in shared memory.  Lane i keeps row i of S, then lane j column j of Li, in
+// registers: a step is one shuffle, one reciprocal and independent multiply-adds (working in
+// shared memory it waited for a load and a store per entry: 3.2 us at r = 6).
 // ---------------------------------------------------------------------------
-__device__ bool chol_warp_f(float* S, int r) {
+template <int RM>
+__device__ bool chol_inv_warp_f(float* S, float* Li, int r) {
   const int lane = threadIdx.x & 31;
   bool ok = true;
-  for (int k = 0; k < r; ++k) {
-    float d = S[k + LD * k];
+  float a[RM];
+#pragma unroll
+  for (int j = 0; j < RM; ++j) a[j] = (lane < r && j < r) ? S[lane + LD * j] : 0.f;
+#pragma unroll
+  for (int k = 0; k < RM; ++k) {
+    if (k >= r) break;
+    float d = __shfl_sync(0xffffffffu, a[k], k);
     if (!(d > 0.f)) { ok = false; d = 1.f; }
     const float inv = rsqrt_approx(d);
-    __syncwarp();
-    float lik = 0.f;
-    if (lane > k && lane < r) {
-      lik = S[lane + LD * k] * inv;
-      S[lane + LD * k] = lik;
+    const float lik = lane > k ? a[k] * inv : 0.f;
+#pragma unroll
+    for (int j = k + 1; j < RM; ++j) {
+      const float ljk = __shfl_sync(0xffffffffu, lik, j);
+      if (lane >= j) a[j] = fmaf(-lik, ljk, a[j]);
     }
-    if (lane == k) S[k + LD * k] = d * inv;
-    __syncwarp();
-    if (lane > k && lane < r)
-      for (int j = k + 1; j <= lane; ++j) S[lane + LD * j] = fmaf(-lik, S[j + LD * k], S[lane + LD * j]);
-    __syncwarp();
+    a[k] = lane > k ? lik : (lane == k ? d * inv : 0.f);
   }
-  for (int j = 1; j < r; ++j)
-    if (lane < j) S[lane + LD * j] = 0.f;
+#pragma unroll
+  for (int j = 0; j < RM; ++j)
+    if (lane < r && j < r) S[lane + LD * j] = a[j];
+  __syncwarp();
+  float x[RM];
+#pragma unroll
+  for (int i = 0; i < RM; ++i) x[i] = i == lane ? 1.f : 0.f;
+#pragma unroll
+  for (int k = 0; k < RM; ++k) {
+    if (k >= r) break;
+    if (lane <= k) {
+      x[k] = x[k] / S[k + LD * k];
+#pragma unroll
+      for (int i = k + 1; i < RM; ++i)
+        if (i < r) x[i] = fmaf(-S[i + LD * k], x[k], x[i]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+    if (lane < r && i < r) Li[i + LD * lane] = x[i];
   __syncwarp();
   return ok;
-}
-
-// Li = L^{-1} (lower) by column sweeps: lane j owns column j.
-__device__ void trinv_warp_f(const float* L, float* Li, int r) {
-  const int lane = threadIdx.x & 31;
-  for (int i = 0; i < r; ++i)
-    if (lane < r) Li[i + LD * lane] = (i == lane) ? 1.f : 0.f;
-  __syncwarp();
-  for (int k = 0; k < r; ++k) {
-    if (lane <= k && lane < r) {
-      const float x = Li[k + LD * lane] / L[k + LD * k];
-      Li[k + LD * lane] = x;
-      for (int i = k + 1; i < r; ++i) Li[i + LD * lane] = fmaf(-L[i + LD * k], x, Li[i + LD * lane]);
-    }
-  }
-  __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
@@ -302,7 +311,7 @@ __device__ double* gj_inverse(double* A0, double* A1, int r, int nthr, int bar, 
 }
 
 // Bounded grid barrier; every CTA is resident (cooperative launch, <= 1 CTA per SM).
-// The counter (zeroed before the launch) only grows: the k-th barrier (k from 1)
+// The counter (zeroed at the start of the step) only grows: the k-th barrier (k from 1)
 // waits for k * nblocks arrivals.  Release on arrival and acquire on the spin order
 // the CTA's writes before and its reads after the barrier.
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
@@ -357,7 +366,9 @@ __device__ __forceinline__ void stamp_flush(const unsigned long long* sh, unsign
 // ---------------------------------------------------------------------------
 
 // Partial G_n = T_(n) T_(n)^T over column slice `sp` of mode n: the slice is staged
-// in shared memory 32 columns at a time; one thread per upper-triangle entry.
+// in shared memory 32 columns at a time; one thread per upper-triangle entry, its sum in
+// CH interleaved chains (4 in the float types: a chain of 32 dependent double products is 2 us).
+template <int CH>
 __device__ void gram_partial(const ModeDesc& d, const double* T, double* gpart, int gsplit, int n, int sp,
                              double (*S)[33]) {
   const int r = d.r[n];
@@ -368,7 +379,9 @@ __device__ void gram_partial(const ModeDesc& d, const double* T, double* gpart, 
   int ta = 0, tb = 0;
   if ((int)threadIdx.x < ntri) tri_index(threadIdx.x, &ta, &tb);
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  double s = 0.0;
+  double sum[CH];
+#pragma unroll
+  for (int u = 0; u < CH; ++u) sum[u] = 0.0;
   for (int64_t cb = c0; cb < c1; cb += 32) {
     const int64_t c = cb + tx;
     double v = 0.0;
@@ -379,11 +392,14 @@ __device__ void gram_partial(const ModeDesc& d, const double* T, double* gpart, 
     S[ty][tx] = v;
     __syncthreads();
     if ((int)threadIdx.x < ntri) {
-#pragma unroll 8
-      for (int x = 0; x < 32; ++x) s = fma(S[ta][x], S[tb][x], s);
+#pragma unroll
+      for (int x = 0; x < 32; ++x) sum[x % CH] = fma(S[ta][x], S[tb][x], sum[x % CH]);
     }
     __syncthreads();
   }
+  double s = sum[0];
+#pragma unroll
+  for (int u = 1; u < CH; ++u) s += sum[u];
   if ((int)threadIdx.x < ntri) gpart[((int64_t)n * gsplit + sp) * LD * LD + ta + LD * tb] = s;
 }
 
@@ -546,19 +562,40 @@ __device__ __noinline__ void gram_finish(const ModeDesc& d, int n, const double*
 // Row-tile phases
 // ---------------------------------------------------------------------------
 
-// Phase 1 on one tile of mode n: M = Y_(n) T_(n)^T, X = M G^{-1}, partial P = A^T X.
+// N consecutive values (16-byte aligned) from shared memory
+template <typename Tc, int N>
+__device__ __forceinline__ void lds_vec(const Tc* p, Tc* v) {
+  constexpr int per = 16 / sizeof(Tc);
+#pragma unroll
+  for (int i = 0; i < N / per; ++i) {
+    if constexpr (sizeof(Tc) == 4) {
+      const float4 t = reinterpret_cast<const float4*>(p)[i];
+      v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w;
+    } else {
+      const double2 t = reinterpret_cast<const double2*>(p)[i];
+      v[2 * i] = t.x; v[2 * i + 1] = t.y;
+    }
+  }
+}
+
+// Phase 1 on one tile of mode n: M = Y_(n) T_(n)^T, X = M G^{-1}, partial P = A^T X.  The
+// columns come in chunks of CW, all of a chunk's loads in flight at once and the next chunk's
+// behind the products (32 columns at a time paid the L2 latency up to 19 times), read back as
+// 16-byte vectors.
 template <typename Tc>
 __device__ void rows_mxp(const UpdArgs& a, int n, int64_t i0, int tile, unsigned char* sm) {
+  constexpr int CW = sizeof(Tc) == 4 ? 128 : 64, CPT = CW / 32, LDC = CW + 16 / (int)sizeof(Tc);
+  constexpr int VN = 16 / sizeof(Tc);
   const ModeDesc& d = a.d;
   const int r = d.r[n];
   const int64_t N = d.N[n];
   const int li = threadIdx.x & 31, ca = threadIdx.x >> 5;
   const int64_t i = i0 + li;
-  Tc (*Ysh)[33] = (Tc(*)[33])sm;
-  Tc (*Tsh)[33] = Ysh + 32;
-  Tc (*Msh)[33] = Tsh + 32;
+  Tc (*Ysh)[LDC] = (Tc(*)[LDC])sm;
+  Tc (*Tsh)[LDC] = Ysh + 32;
+  Tc (*Msh)[33] = (Tc(*)[33])(Tsh + 32);
   Tc* Gi = (Tc*)(Msh + 32);
-  const int64_t L = prod_r_below(d, n), Q = prod_r_above(d, n);
+  const unsigned L = (unsigned)prod_r_below(d, n), ncol = L * (unsigned)prod_r_above(d, n);
   const Tc* Y = (const Tc*)a.Y[n];
   const Tc* Tm = (const Tc*)a.Tcore;
   if (sizeof(Tc) == 8) {
@@ -566,41 +603,52 @@ __device__ void rows_mxp(const UpdArgs& a, int n, int64_t i0, int tile, unsigned
   } else {
     for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) Gi[e] = (Tc)a.Ginvf[(int64_t)n * LD * LD + e];
   }
-  const int64_t ncol = L * Q;
   Tc s = Tc(0);
   // staging: for L == 1 the rows of Y_(n) (and the ranks of T_(n)) are contiguous, so
-  // lanes run along rows; otherwise along columns.  The next chunk is loaded into
-  // registers while the current one is multiplied.
+  // lanes run along rows; otherwise along columns
   const bool rows_fast = (L == 1);
   const int u = threadIdx.x & 31, v = threadIdx.x >> 5;
   const int srow = rows_fast ? u : v, scol = rows_fast ? v : u;
-  auto fetch = [&](int64_t c0, Tc* vy, Tc* vt) {
-    const int64_t c = c0 + scol;
-    const int64_t ii = i0 + srow;
-    *vy = Tc(0);
-    *vt = Tc(0);
-    if (c < ncol) {
-      const int64_t l = c % L, q = c / L;
-      if (ii < N) *vy = Y[l + L * (ii + N * q)];
-      if (srow < r) *vt = Tm[l + L * (srow + (int64_t)r * q)];
+  const bool yin = i0 + srow < N, tin = srow < r;
+  Tc vy[CPT], vt[CPT];
+  auto fetch = [&](unsigned c0) {
+#pragma unroll
+    for (int k = 0; k < CPT; ++k) {
+      const unsigned c = c0 + scol + 32 * k;
+      vy[k] = Tc(0);
+      vt[k] = Tc(0);
+      if (c < ncol) {
+        const unsigned q = c / L, l = c - q * L;
+        if (yin) vy[k] = Y[l + (size_t)L * (i0 + srow + (size_t)N * q)];
+        if (tin) vt[k] = Tm[l + (size_t)L * (srow + (size_t)r * q)];
+      }
     }
   };
-  Tc vy, vt;
-  fetch(0, &vy, &vt);
-  for (int64_t c0 = 0; c0 < ncol; c0 += 32) {
-    Ysh[srow][scol] = vy;
-    Tsh[srow][scol] = vt;
+  fetch(0);
+  for (unsigned c0 = 0; c0 < ncol; c0 += CW) {
+#pragma unroll
+    for (int k = 0; k < CPT; ++k) {
+      Ysh[srow][scol + 32 * k] = vy[k];
+      Tsh[srow][scol + 32 * k] = vt[k];
+    }
     __syncthreads();
-    if (c0 + 32 < ncol) fetch(c0 + 32, &vy, &vt);
+    if (c0 + CW < ncol) fetch(c0 + CW);
     if (ca < r) {
-#pragma unroll 8
-      for (int x = 0; x < 32; ++x) s += Ysh[li][x] * Tsh[ca][x];
+      const int nx = (int)min((unsigned)CW, (ncol - c0 + 31) & ~31u);     // (zeros past ncol)
+#pragma unroll 4
+      for (int x = 0; x < nx; x += VN) {
+        Tc y[VN], t[VN];
+        lds_vec<Tc, VN>(&Ysh[li][x], y);
+        lds_vec<Tc, VN>(&Tsh[ca][x], t);
+#pragma unroll
+        for (int w = 0; w < VN; ++w) s += y[w] * t[w];
+      }
     }
     __syncthreads();
   }
   if (ca < r) Msh[li][ca] = s;
-  Tc (*Ash)[33] = Ysh;
-  Tc (*Xsh)[33] = Tsh;
+  Tc (*Ash)[33] = (Tc(*)[33])sm;
+  Tc (*Xsh)[33] = Ash + 32;
   Ash[li][ca] = (ca < r && i < N) ? ((const Tc*)a.A[n])[i + N * ca] : Tc(0);
   __syncthreads();
   Tc x = Tc(0);
@@ -632,7 +680,8 @@ __device__ void rows_u1(const UpdArgs& a, int n, int64_t i0, int tile, unsigned 
   const int64_t i = i0 + li;
   Tc* Psh = (Tc*)sm;                         // LD*LD
   Tc (*Ush)[33] = (Tc(*)[33])(Psh + LD * LD);
-  Tc* wsh = (Tc*)(Ush + 32);                 // 32
+  Tc (*Wsh)[33] = Ush + 32;                  // U' W
+  const Tc wi = i < N ? (Tc)a.w[n][i] : Tc(0);
   const Tc* part = (const Tc*)a.part;
   const int nt = (int)((N + 31) / 32);
   {
@@ -650,7 +699,6 @@ __device__ void rows_u1(const UpdArgs& a, int n, int64_t i0, int tile, unsigned 
     Psh[e] = s;
   }
   Ush[li][ca] = (ca < r && i < N) ? ((const Tc*)a.Uc[n])[i + N * ca] : Tc(0);
-  if (threadIdx.x < 32) wsh[li] = (i < N) ? (Tc)a.w[n][i] : Tc(0);
   __syncthreads();
   Tc upc = Tc(0);
   if (ca < r && i < N) {
@@ -665,12 +713,13 @@ __device__ void rows_u1(const UpdArgs& a, int n, int64_t i0, int tile, unsigned 
   }
   __syncthreads();
   Ush[li][ca] = upc;
+  Wsh[li][ca] = upc * wi;
   __syncthreads();
   if ((int)threadIdx.x < r * r) {
     const int ra = threadIdx.x % r, rb = threadIdx.x / r;
     Tc acc = Tc(0);
 #pragma unroll 8
-    for (int t = 0; t < 32; ++t) acc += Ush[t][ra] * wsh[t] * Ush[t][rb];
+    for (int t = 0; t < 32; ++t) acc += Wsh[t][ra] * Ush[t][rb];
     ((Tc*)a.part)[(int64_t)a.d.p * a.ntile * LD * LD + ((int64_t)n * a.ntile + tile) * LD * LD + ra + LD * rb] = acc;
   }
   __syncthreads();
@@ -703,188 +752,144 @@ __device__ void reduce_long(const UpdArgs& a, int which) {
   }
 }
 
-// Phase 3 for mode n (one CTA): C_n from the partials, R (upper, C = R^T R) and R^{-1}.
+// Phase 3 for mode n: C_n from the partials, R (upper, C = R^T R) and R^{-1} into the first
+// two LD x LD doubles of sm (R, then R^{-1}); 24 KB of scratch after them.  Every CTA with
+// rows of the mode forms the same factors; `flag` only on one of them.
 template <typename Tc>
-__device__ void mode_cholqr(const UpdArgs& a, int n, unsigned char* sm) {
+__device__ void mode_cholqr(const UpdArgs& a, int n, unsigned char* sm, bool flag) {
   const ModeDesc& d = a.d;
   const int r = d.r[n];
   const int nt = (int)((d.N[n] + 31) / 32);
   const Tc* part = (const Tc*)a.part + (int64_t)d.p * a.ntile * LD * LD + (int64_t)n * a.ntile * LD * LD;
-  double* Rg = a.R + (int64_t)n * LD * LD;
-  double* Rig = a.Rinv + (int64_t)n * LD * LD;
+  double* Rs = (double*)sm;
+  double* Ris = Rs + LD * LD;
+  unsigned char* scr = (unsigned char*)(Ris + LD * LD);
   __shared__ bool ok_sh;
   __shared__ double dinv_sh;
+  const int e = threadIdx.x, ra = e % LD, rb = e / LD;      // (UPD_THREADS == LD * LD)
   if (!a.reorth) {
-    for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) Rg[e] = Rig[e] = (e % LD == e / LD) ? 1.0 : 0.0;
+    Rs[e] = Ris[e] = ra == rb ? 1.0 : 0.0;
+    __syncthreads();
     return;
   }
-  if (sizeof(Tc) == 8) {
-    double* C = (double*)sm;
+  Tc c = Tc(0);
+  if (ra < r && rb < r) {
+    if (nt > kTreeTiles)
+      c = __ldcg(&((const Tc*)a.red)[(int64_t)(kMaxModes + n) * LD * LD + e]);
+    else
+#pragma unroll 8
+      for (int t = 0; t < nt; ++t) c += __ldcg(&part[(int64_t)t * LD * LD + e]);
+  }
+  if constexpr (sizeof(Tc) == 8) {
+    double* C = (double*)scr;
     double* Li = C + LD * LD;
     double* dinv = Li + LD * LD;
-    for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-      const int ra = e % LD, rb = e / LD;
-      double s = 0.0;
-      if (ra < r && rb < r) {
-        if (nt > kTreeTiles)
-          s = (double)__ldcg(&((const Tc*)a.red)[(int64_t)(kMaxModes + n) * LD * LD + e]);
-        else
-#pragma unroll 8
-          for (int t = 0; t < nt; ++t) s += (double)__ldcg(&part[(int64_t)t * LD * LD + e]);
-      }
-      C[e] = s;
-    }
+    C[e] = c;
     __syncthreads();
-    if (!chol_d(C, r, &ok_sh, &dinv_sh) && threadIdx.x == 0) atomicOr(a.flags, kFlagCholQR);
+    if (!chol_d(C, r, &ok_sh, &dinv_sh) && threadIdx.x == 0 && flag) atomicOr(a.flags, kFlagCholQR);
     trinv_d(C, Li, r, dinv);
-    for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-      const int ra = e % LD, rb = e / LD;
-      Rg[e] = (ra < r && rb < r) ? C[rb + LD * ra] : 0.0;     // R = L^T
-      Rig[e] = (ra < r && rb < r) ? Li[rb + LD * ra] : 0.0;   // R^{-1} = L^{-T}
-    }
+    Rs[e] = (ra < r && rb < r) ? C[rb + LD * ra] : 0.0;     // R = L^T
+    Ris[e] = (ra < r && rb < r) ? Li[rb + LD * ra] : 0.0;   // R^{-1} = L^{-T}
   } else {
-    float* Cf = (float*)sm;                 // LD*LD
-    float* Lif = Cf + LD * LD;              // LD*LD
-    double* R0 = (double*)(Lif + LD * LD);  // LD*LD
-    double* Z0 = R0 + LD * LD;              // LD*LD
-    double* E = Z0 + LD * LD;               // LD*LD
-    __shared__ float fmax_sh;
-    for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-      const int ra = e % LD, rb = e / LD;
-      float s = 0.f;
-      if (ra < r && rb < r) {
-        if (nt > kTreeTiles)
-          s = (float)__ldcg(&((const Tc*)a.red)[(int64_t)(kMaxModes + n) * LD * LD + e]);
-        else
-#pragma unroll 8
-          for (int t = 0; t < nt; ++t) s += (float)__ldcg(&part[(int64_t)t * LD * LD + e]);
-      }
-      Cf[e] = s;
-    }
-    __syncthreads();
+    float* Cf = (float*)scr;                // LD*LD
+    float* F1 = Cf + LD * LD;               // LD*LD
+    __shared__ int fmax_sh;
+    if (threadIdx.x == 0) fmax_sh = 0;
     // C = I + D with D small after a step: R = I + F, F = Phi(D - F1^T F1), F1 = Phi(D),
     // Phi = upper triangle with the diagonal halved (R^T R = C up to O(|D|^3)), and
     // R^{-1} = I - F + F^2 - F^3 + F^4 (R R^{-1} = I + F^5).  Taken when max |F1| <= 2^-14,
     // so that |F^5| < 4e-14 for r <= 32.
-    float* F1 = Lif;
-    for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-      const int ra = e % LD, rb = e / LD;
-      float f = 0.f;
-      if (ra < r && rb < r && ra <= rb) f = (ra == rb) ? 0.5f * (Cf[e] - 1.f) : Cf[e];
-      F1[e] = f;
-    }
-    if (threadIdx.x == 0) fmax_sh = 0.f;
+    const bool up = ra <= rb && rb < r;
+    const float f1 = up ? (ra == rb ? 0.5f * (c - 1.f) : c) : 0.f;
+    Cf[e] = c;
+    F1[e] = f1;
+    // this thread's entry of the packed upper triangle (the products below are triangular and
+    // end in double, which a warp without an entry must not issue)
+    const int ntri = r * (r + 1) / 2;
+    int ia = 0, jb = 0;
+    if (e < ntri) tri_index(e, &ia, &jb);
     __syncthreads();
     {
-      float m = 0.f;
-      for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-        const float v = fabsf(F1[e]);
-        m = (v == v) ? fmaxf(m, v) : 3.0e38f;      // a NaN takes the Cholesky path, which flags it
-      }
+      float m = fabsf(f1);
+      m = (m == m) ? m : 3.0e38f;              // a NaN takes the Cholesky path, which flags it
       for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax((int*)&fmax_sh, __float_as_int(m));
+      if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(&fmax_sh, __float_as_int(m));
     }
     __syncthreads();
-    if (fmax_sh <= 6.103515625e-05f) {
-      float* Fs = (float*)R0;                // LD*LD float: F
-      float* F2 = Fs + LD * LD;              // F^2
-      float* F3 = F2 + LD * LD;              // F^3
-      float* F4 = F3 + LD * LD;              // F^4
-      for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {   // F = Phi(D - F1^T F1)
-        const int ra = e % LD, rb = e / LD;
-        float f = 0.f;
-        if (ra < r && rb < r && ra <= rb) {
-          float q = 0.f;
-          for (int k = 0; k <= ra; ++k) q = fmaf(F1[k + LD * ra], F1[k + LD * rb], q);
-          f = (ra == rb) ? F1[e] - 0.5f * q : Cf[e] - q;
+    if (__int_as_float(fmax_sh) <= 6.103515625e-05f) {
+      float* Fs = F1 + LD * LD;                // LD*LD: F
+      float* F2 = Fs + LD * LD;                // LD*LD: F^2
+      Rs[e] = Ris[e] = 0.0;
+      float f = 0.f, f2 = 0.f;
+      if (e < ntri) {                          // F = Phi(D - F1^T F1)
+        float q = 0.f;
+        for (int k = 0; k <= ia; ++k) q = fmaf(F1[k + LD * ia], F1[k + LD * jb], q);
+        f = (ia == jb) ? F1[ia + LD * jb] - 0.5f * q : Cf[ia + LD * jb] - q;
+        Fs[ia + LD * jb] = f;
+      }
+      __syncthreads();
+      if (e < ntri) {
+        for (int k = ia; k <= jb; ++k) f2 = fmaf(Fs[ia + LD * k], Fs[k + LD * jb], f2);
+        F2[ia + LD * jb] = f2;
+      }
+      __syncthreads();
+      if (e < ntri) {
+        float f3 = 0.f, f4 = 0.f;
+        for (int k = ia; k <= jb; ++k) {
+          f3 = fmaf(F2[ia + LD * k], Fs[k + LD * jb], f3);
+          f4 = fmaf(F2[ia + LD * k], F2[k + LD * jb], f4);
         }
-        Fs[e] = f;
+        const double id = ia == jb ? 1.0 : 0.0, fd = (double)f;
+        Rs[ia + LD * jb] = id + fd;
+        Ris[ia + LD * jb] = (((id - fd) + (double)f2) - (double)f3) + (double)f4;
+      }
+    } else {
+      float* Lif = F1;                         // LD*LD
+      double* Z0 = (double*)(F1 + LD * LD);    // LD*LD
+      double* E = Z0 + LD * LD;                // LD*LD
+      if (threadIdx.x < 32) {
+        const bool good = r <= 8 ? chol_inv_warp_f<8>(Cf, Lif, r)
+                                 : (r <= 16 ? chol_inv_warp_f<16>(Cf, Lif, r) : chol_inv_warp_f<32>(Cf, Lif, r));
+        if (!good && threadIdx.x == 0 && flag) atomicOr(a.flags, kFlagCholQR);
+      }
+      Rs[e] = Ris[e] = Z0[e] = 0.0;
+      __syncthreads();
+      if (e < ntri) {
+        Rs[ia + LD * jb] = (double)Cf[jb + LD * ia];            // R0 = L^T (upper)
+        Z0[ia + LD * jb] = (double)Lif[jb + LD * ia];           // Z0 = L^{-T}, float accurate
       }
       __syncthreads();
-      for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-        const int ra = e % LD, rb = e / LD;
-        float q = 0.f;
-        if (ra < r && rb < r && ra <= rb)
-          for (int k = ra; k <= rb; ++k) q = fmaf(Fs[ra + LD * k], Fs[k + LD * rb], q);
-        F2[e] = q;
+      // one Newton step in double: Z1 = Z0 + Z0 (I - R0 Z0); all three are upper triangular
+      if (e < ntri) {
+        double x = (ia == jb) ? 1.0 : 0.0;
+        for (int k = ia; k <= jb; ++k) x = fma(-Rs[ia + LD * k], Z0[k + LD * jb], x);
+        E[ia + LD * jb] = x;
       }
       __syncthreads();
-      for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-        const int ra = e % LD, rb = e / LD;
-        float q = 0.f;
-        if (ra < r && rb < r && ra <= rb)
-          for (int k = ra; k <= rb; ++k) q = fmaf(F2[ra + LD * k], Fs[k + LD * rb], q);
-        F3[e] = q;
-      }
-      __syncthreads();
-      for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-        const int ra = e % LD, rb = e / LD;
-        float q = 0.f;
-        if (ra < r && rb < r && ra <= rb)
-          for (int k = ra; k <= rb; ++k) q = fmaf(F2[ra + LD * k], F2[k + LD * rb], q);
-        F4[e] = q;
-      }
-      __syncthreads();
-      for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-        const int ra = e % LD, rb = e / LD;
-        const double id = (ra == rb && ra < r) ? 1.0 : 0.0;
-        Rg[e] = id + (double)Fs[e];
-        Rig[e] = (((id - (double)Fs[e]) + (double)F2[e]) - (double)F3[e]) + (double)F4[e];
-      }
-      return;
-    }
-    if (threadIdx.x < 32) {
-      const bool good = chol_warp_f(Cf, r);
-      if (!good && threadIdx.x == 0) atomicOr(a.flags, kFlagCholQR);
-      trinv_warp_f(Cf, Lif, r);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-      const int ra = e % LD, rb = e / LD;
-      const bool in = ra < r && rb < r;
-      R0[e] = in ? (double)Cf[rb + LD * ra] : 0.0;            // R0 = L^T (upper)
-      Z0[e] = in ? (double)Lif[rb + LD * ra] : 0.0;           // Z0 = L^{-T}, float accurate
-    }
-    __syncthreads();
-    // one Newton step in double: Z1 = Z0 + Z0 (I - R0 Z0); all three are upper triangular
-    const int ntri = r * (r + 1) / 2;
-    for (int e = threadIdx.x; e < ntri; e += blockDim.x) {
-      int ia, jb;
-      tri_index(e, &ia, &jb);
-      double s = (ia == jb) ? 1.0 : 0.0;
-      for (int k = ia; k <= jb; ++k) s = fma(-R0[ia + LD * k], Z0[k + LD * jb], s);
-      E[ia + LD * jb] = s;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) {
-      const int ia = e % LD, jb = e / LD;
-      double z = 0.0;
-      if (ia < r && jb < r && ia <= jb) {
-        z = Z0[e];
+      if (e < ntri) {
+        double z = Z0[ia + LD * jb];
         for (int k = ia; k <= jb; ++k) z = fma(Z0[ia + LD * k], E[k + LD * jb], z);
+        Ris[ia + LD * jb] = z;
       }
-      Rg[e] = R0[e];
-      Rig[e] = z;
     }
   }
+  __syncthreads();
 }
 
-// Phase 4 on one tile of mode n: U'' = U' R^{-1}, A = W U'' and U'' in the compute type.
+// Phase 3 on one tile of mode n: U'' = U' R^{-1}, A = W U'' and U'' in the compute type.
 template <typename Tc>
-__device__ void rows_u2(const UpdArgs& a, int n, int64_t i0, unsigned char* sm) {
+__device__ void rows_u2(const UpdArgs& a, int n, int64_t i0, const double* Ris, unsigned char* scr) {
   const ModeDesc& d = a.d;
   const int r = d.r[n];
   const int64_t N = d.N[n];
   const int li = threadIdx.x & 31, ca = threadIdx.x >> 5;
   const int64_t i = i0 + li;
-  double (*Ush)[LD + 1] = (double(*)[LD + 1])sm;
-  double* Rsh = (double*)(Ush + 32);
-  for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) Rsh[e] = __ldcg(&a.Rinv[(int64_t)n * LD * LD + e]);
+  double (*Ush)[LD + 1] = (double(*)[LD + 1])scr;
   if (ca < r) Ush[li][ca] = (i < N) ? __ldcg(&a.Up[n][i + N * ca]) : 0.0;
   __syncthreads();
   if (ca < r && i < N) {
     double s = 0.0;
-    for (int b = 0; b <= ca; ++b) s = fma(Ush[li][b], Rsh[b + LD * ca], s);
+    for (int b = 0; b <= ca; ++b) s = fma(Ush[li][b], Ris[b + LD * ca], s);
     a.U[n][i + N * ca] = s;
     ((Tc*)a.A[n])[i + N * ca] = (Tc)(a.w[n][i] * s);
     ((Tc*)a.Uc[n])[i + N * ca] = (Tc)s;
@@ -892,46 +897,90 @@ __device__ void rows_u2(const UpdArgs& a, int n, int64_t i0, unsigned char* sm) 
   __syncthreads();
 }
 
-// Core mode product dst = src x_n R_n (R_n upper triangular); the first mode adds dS
-// to T (Heun's second stage: forms (T0 + T + dS) / 2; the midpoint scheme's: T0 + dS).  Work is split by mode-n fibers (the r_n entries at fixed other indices):
-// each pass stages F fibers per CTA in shared memory (one coalesced load per
-// thread), F chosen so that every CTA of the grid has some.
+// Phase 4: dst = (T + dS) x_1 R_1 x_2 R_2 (Heun's second stage: ((T0 + T + dS) / 2), the
+// midpoint scheme's: (T0 + dS)), slab by slab: r_1 x r_2 entries at fixed other indices, F
+// slabs at a time staged in shared memory, F chosen so that every CTA of the grid has some.
+// With two modes the one slab is the core: it is read whole before it is written.
 template <typename Tc>
-__device__ void core_mode(const UpdArgs& a, int n, const double* src, double* dst, unsigned char* sm) {
+__device__ void core_12(const UpdArgs& a, unsigned char* sm) {
   const ModeDesc& d = a.d;
-  const int r = d.r[n];
-  const int64_t L = prod_r_below(d, n);
-  const int64_t nfib = prod_r(d) / r;
-  const int64_t per_cta = (nfib + gridDim.x - 1) / gridDim.x;
-  const int F = (int)(per_cta < UPD_THREADS / r ? per_cta : UPD_THREADS / r);
-  double* Rsh = (double*)sm;            // LD*LD
-  double* Xs = Rsh + LD * LD;           // r x F <= UPD_THREADS
-  for (int e = threadIdx.x; e < LD * LD; e += blockDim.x) Rsh[e] = __ldcg(&a.R[(int64_t)n * LD * LD + e]);
+  const int r1 = d.r[0], r2 = d.r[1], ns = r1 * r2;
+  const int64_t nslab = prod_r_above(d, 1);
+  const int64_t per_cta = (nslab + gridDim.x - 1) / gridDim.x;
+  const int F = (int)(per_cta < UPD_THREADS / ns ? per_cta : UPD_THREADS / ns);
+  if (blockIdx.x * (int64_t)F >= nslab) return;
+  double* R1 = (double*)sm;             // LD*LD each
+  double* R2 = R1 + LD * LD;
+  double* Xs = R2 + LD * LD;            // F slabs <= UPD_THREADS
+  double* Ys = Xs + UPD_THREADS;
+  R1[threadIdx.x] = __ldcg(&a.R[threadIdx.x]);
+  R2[threadIdx.x] = __ldcg(&a.R[LD * LD + threadIdx.x]);
   const Tc* dS = (const Tc*)a.dS;
-  const int t = threadIdx.x, fl = t % F, j = t / F;
-  for (int64_t f0 = blockIdx.x * (int64_t)F; f0 < nfib; f0 += (int64_t)gridDim.x * F) {
-    const int64_t f = f0 + fl;
-    const bool act = j < r && f < nfib;
-    int64_t idx = 0;
+  const int t = threadIdx.x, fl = t / ns, e = t - fl * ns, i = e % r1, j = e / r1;
+  for (int64_t f0 = blockIdx.x * (int64_t)F; f0 < nslab; f0 += (int64_t)gridDim.x * F) {
+    const bool act = fl < F && f0 + fl < nslab;
+    const int64_t idx = (f0 + fl) * ns + e;
     if (act) {
-      const int64_t l = f % L, q = f / L;
-      idx = l + L * (j + (int64_t)r * q);
-      if (n != 0)
-        Xs[j * F + fl] = __ldcg(&src[idx]);
-      else if (a.T0 && a.combine == 2)
-        Xs[j * F + fl] = a.T0[idx] + (double)dS[idx];
-      else if (a.T0)
-        Xs[j * F + fl] = 0.5 * ((src[idx] + a.T0[idx]) + (double)dS[idx]);
-      else
-        Xs[j * F + fl] = src[idx] + (double)dS[idx];
+      if (a.T0 && a.combine == 2) Xs[t] = a.T0[idx] + (double)dS[idx];
+      else if (a.T0) Xs[t] = 0.5 * ((a.T[idx] + a.T0[idx]) + (double)dS[idx]);
+      else Xs[t] = a.T[idx] + (double)dS[idx];
     }
     __syncthreads();
     if (act) {
       double s = 0.0;
-      for (int k = j; k < r; ++k) s = fma(Rsh[j + LD * k], Xs[k * F + fl], s);
-      dst[idx] = s;
+      for (int k = i; k < r1; ++k) s = fma(R1[i + LD * k], Xs[fl * ns + k + r1 * j], s);
+      Ys[t] = s;
     }
     __syncthreads();
+    if (act) {
+      double s = 0.0;
+      for (int k = j; k < r2; ++k) s = fma(R2[j + LD * k], Ys[fl * ns + i + r1 * k], s);
+      if (d.p == 2) {
+        a.T[idx] = s;
+        if (sizeof(Tc) == 4) ((float*)a.Tcore)[idx] = (float)s;
+      } else {
+        a.T2[idx] = s;
+      }
+    }
+  }
+}
+
+// Phase 5: T = T2 x_3 R_3 (x_4 R_4) and its copy in the compute type, by r_3 x r_4 fibers (the
+// entries at fixed first two indices), F at a time, neighbouring fibers on neighbouring threads.
+template <typename Tc>
+__device__ void core_34(const UpdArgs& a, unsigned char* sm) {
+  const ModeDesc& d = a.d;
+  const int r3 = d.r[2], r4 = d.p == 4 ? d.r[3] : 1, nf = r3 * r4;
+  const int64_t L = prod_r_below(d, 2);
+  const int64_t per_cta = (L + gridDim.x - 1) / gridDim.x;
+  const int F = (int)(per_cta < UPD_THREADS / nf ? per_cta : UPD_THREADS / nf);
+  if (blockIdx.x * (int64_t)F >= L) return;
+  double* R3 = (double*)sm;
+  double* R4 = R3 + LD * LD;
+  double* Xs = R4 + LD * LD;            // F fibers <= UPD_THREADS, element (c, d) of fiber f at f + F (c + r3 d)
+  double* Ys = Xs + UPD_THREADS;
+  R3[threadIdx.x] = __ldcg(&a.R[2 * LD * LD + threadIdx.x]);
+  if (d.p == 4) R4[threadIdx.x] = __ldcg(&a.R[3 * LD * LD + threadIdx.x]);
+  const int t = threadIdx.x, fl = t % F, e = t / F, c = e % r3, dd = e / r3;
+  for (int64_t f0 = blockIdx.x * (int64_t)F; f0 < L; f0 += (int64_t)gridDim.x * F) {
+    const bool act = e < nf && f0 + fl < L;
+    const int64_t idx = f0 + fl + L * e;
+    if (act) Xs[t] = __ldcg(&a.T2[idx]);
+    __syncthreads();
+    double s = 0.0;
+    if (act) {
+      for (int k = c; k < r3; ++k) s = fma(R3[c + LD * k], Xs[fl + F * (k + r3 * dd)], s);
+      if (d.p == 4) Ys[t] = s;
+    }
+    __syncthreads();
+    if (act) {
+      if (d.p == 4) {
+        s = 0.0;
+        for (int k = dd; k < r4; ++k) s = fma(R4[dd + LD * k], Ys[fl + F * (c + r3 * k)], s);
+      }
+      a.T[idx] = s;
+      if (sizeof(Tc) == 4) ((float*)a.Tcore)[idx] = (float)s;
+    }
   }
 }
 
@@ -965,15 +1014,16 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_update(UpdArgs a) {
   };
 
   // 1: M, X, partial P; dS = Y_2 x_2 A_2^T when the projection left it
+  // (on the CTAs without rows where those hold all of it at once, else on all)
+  const unsigned dsc0 = (int64_t)nb - ntiles_total >= update_ds_ctas(prod_r(d)) ? (unsigned)ntiles_total : 0u;
   for (int task = blockIdx.x; task < ntiles_total; task += nb) {
     int n, t;
     tile_of(task, &n, &t);
     rows_mxp<Tc>(a, n, (int64_t)t * 32, t, smraw);
   }
-  if (a.ds_y2) {
+  if (a.ds_y2 && blockIdx.x >= dsc0) {
     // dS = Y_2 x_2 A_2^T (Eqs. 2.15/2.16: dS = Y_n x_n A_n^T for every n), read from
-    // phase 4 on.  Eight consecutive threads share one element (every CTA takes a share
-    // of the elements): each sums every eighth i2 with all its loads in flight, then the
+    // phase 4 on.  Eight consecutive threads share one element: each sums every eighth i2 with all its loads in flight, then the
     // eight partial sums are added by shuffles in a fixed order.
     const Tc* Y2 = (const Tc*)a.ds_y2;
     const Tc* A2 = (const Tc*)a.A[1];
@@ -982,10 +1032,10 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_update(UpdArgs a) {
     const int64_t tot = prod_r(d);
     const int grp = threadIdx.x >> 3, part = threadIdx.x & 7;
     const int ngrp = blockDim.x >> 3;
-    const int64_t stride = (int64_t)nb * ngrp;
+    const int64_t stride = (int64_t)(nb - dsc0) * ngrp;
     const int64_t rounds = (tot + stride - 1) / stride;
     for (int64_t k = 0; k < rounds; ++k) {
-      const int64_t e = blockIdx.x + (int64_t)nb * grp + stride * k;
+      const int64_t e = (blockIdx.x - dsc0) + (int64_t)(nb - dsc0) * grp + stride * k;
       Tc acc = Tc(0);
       if (e < tot) {
         const int a1 = (int)(e % r1);
@@ -1023,55 +1073,63 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_update(UpdArgs a) {
     if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   }
 
-  // 3: Cholesky-QR factors, one CTA per mode
-  for (int n = blockIdx.x; n < p; n += nb) mode_cholqr<Tc>(a, n, smraw);
+  // 3: Cholesky-QR factors of the mode of this CTA's rows; U''
+  {
+    double* Rs = (double*)smraw;
+    int have = -1;
+    for (int task = blockIdx.x; task < ntiles_total; task += nb) {
+      int n, t;
+      tile_of(task, &n, &t);
+      if (n != have) mode_cholqr<Tc>(a, n, smraw, t == 0);
+      have = n;
+      rows_u2<Tc>(a, n, (int64_t)t * 32, Rs + LD * LD, (unsigned char*)(Rs + 2 * LD * LD));
+      if (t == 0) {
+        a.R[(int64_t)n * LD * LD + threadIdx.x] = Rs[threadIdx.x];
+        a.Rinv[(int64_t)n * LD * LD + threadIdx.x] = Rs[LD * LD + threadIdx.x];
+      }
+    }
+  }
   if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   stamp(st_sh, a.stamps, ++nst);
 
-  // 4: U'' and the core product of mode 1; 5: the other modes (T -> T2 -> T ...)
-  for (int task = blockIdx.x; task < ntiles_total; task += nb) {
-    int n, t;
-    tile_of(task, &n, &t);
-    rows_u2<Tc>(a, n, (int64_t)t * 32, smraw);
-  }
-  for (int n = 0; n < p; ++n) {
-    const double* src = (n & 1) ? a.T2 : a.T;
-    double* dst = (n & 1) ? a.T : a.T2;
-    core_mode<Tc>(a, n, src, dst, smraw);
+  // 4, 5: the core
+  core_12<Tc>(a, smraw);
+  if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
+  stamp(st_sh, a.stamps, ++nst);
+  if (p > 2) {
+    core_34<Tc>(a, smraw);
     if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
-    stamp(st_sh, a.stamps, ++nst);
   }
+  stamp(st_sh, a.stamps, ++nst);
 
-  // 6: final core in T, compute-type copy, Gram partials
-  {
-    const double* Tfin = (p & 1) ? a.T2 : a.T;
-    const int64_t Rprod = prod_r(d);
-    const int64_t gstr = (int64_t)nb * blockDim.x;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < Rprod; e += gstr) {
-      const double v = __ldcg(&Tfin[e]);
-      if (p & 1) a.T[e] = v;
-      if (sizeof(Tc) == 4) ((float*)a.Tcore)[e] = (float)v;
-    }
-    for (int task = blockIdx.x; task < p * a.gsplit; task += nb)
-      gram_partial(d, Tfin, a.gpart, a.gsplit, task / a.gsplit, task % a.gsplit, (double(*)[33])smraw);
+  // 6: Gram partials
+  for (int task = blockIdx.x; task < p * a.gsplit; task += nb)
+    gram_partial<sizeof(Tc) == 4 ? 4 : 1>(d, a.T, a.gpart, a.gsplit, task / a.gsplit, task % a.gsplit,
+                                          (double(*)[33])smraw);
+  if (a.skip_finish) {
+    // (the finish is another launch: the kernel's end orders it)
+    stamp(st_sh, a.stamps, ++nst);
+    stamp(st_sh, a.stamps, ++nst);
+    stamp_flush(st_sh, a.stamps, nst);
+    return;
   }
   if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   stamp(st_sh, a.stamps, ++nst);
 
   // 7: G, G^{-1}, sigma^2 (or a separate launch beside the exact error)
-  if (!a.skip_finish)
-    for (int n = blockIdx.x; n < p; n += nb)
-      gram_finish(d, n, a.gpart, a.gsplit, a.G, a.Ginv, a.Ginvf, a.sig2, a.Vprev, a.warm, a.flags, smraw);
+  for (int n = blockIdx.x; n < p; n += nb)
+    gram_finish(d, n, a.gpart, a.gsplit, a.G, a.Ginv, a.Ginvf, a.sig2, a.Vprev, a.warm, a.flags, smraw);
   stamp(st_sh, a.stamps, ++nst);
   stamp_flush(st_sh, a.stamps, nst);
 }
 
 // The Gram refresh of phases 6-7 as two ordinary launches (after (re)initialisation
-// and state loads), bit-identical to the fused path.
+// and state loads), bit-identical to the fused path of the same compute type.
+template <int CH>
 __global__ void __launch_bounds__(UPD_THREADS, 1) k_gram_partial(ModeDesc d, const double* T, double* gpart,
                                                                  int gsplit) {
   __shared__ double S[32][33];
-  gram_partial(d, T, gpart, gsplit, blockIdx.x / gsplit, blockIdx.x % gsplit, S);
+  gram_partial<CH>(d, T, gpart, gsplit, blockIdx.x / gsplit, blockIdx.x % gsplit, S);
 }
 
 __global__ void __launch_bounds__(UPD_THREADS, 1) k_gram_finish(ModeDesc d, const double* gpart, int gsplit, double* G,
@@ -1094,7 +1152,9 @@ void launch_gram_finish(const ModeDesc& d, const double* Gpart, int nsplit, doub
 
 void launch_gram(const ModeDesc& d, const double* T, double* Gpart, int nsplit, double* G, double* Ginv,
                  float* Ginvf, double* sig2, float* Vprev, int warm, unsigned* flags, cudaStream_t s) {
-  k_gram_partial<<<d.p * nsplit, UPD_THREADS, 0, s>>>(d, T, Gpart, nsplit); count_launch();
+  if (Ginvf) k_gram_partial<4><<<d.p * nsplit, UPD_THREADS, 0, s>>>(d, T, Gpart, nsplit);
+  else k_gram_partial<1><<<d.p * nsplit, UPD_THREADS, 0, s>>>(d, T, Gpart, nsplit);
+  count_launch();
   launch_gram_finish(d, Gpart, nsplit, G, Ginv, Ginvf, sig2, Vprev, warm, flags, s);
 }
 
@@ -1115,7 +1175,6 @@ tdb_status launch_update(UpdArgs& a, int grid_hint, cudaStream_t s) {
   }
   // every CTA is resident (one per SM at most), so the grid barriers cannot deadlock
   const int grid = std::max(a.d.p, std::min(nsm, grid_hint));
-  cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), s);
   // cooperative launch through the extensible API, which stream capture records as a
   // cooperative kernel node
   cudaLaunchConfig_t cfg = {};

@@ -85,7 +85,7 @@ struct UpdArgs {
   const double* T0;
   const double* U0[kMaxModes];
   int combine;                   // with T0: 1 = Heun's mean (T0 + T + dT) / 2, 2 = T0 + dT (midpoint)
-  unsigned* bar;                 // arrival counter of the grid barriers (zeroed per launch)
+  unsigned* bar;                 // arrival counter of the grid barriers (zero at the launch)
   unsigned long long* stamps;    // per-phase timer stamps (profiling), or null
   unsigned* flags;
 };
@@ -150,7 +150,10 @@ void launch_gram(const ModeDesc& d, const double* T, double* Gpart, int nsplit, 
 template <typename Tc>
 void launch_orthonormalize(RowArgs& a, double* R, double* Rinv, unsigned* flags, cudaStream_t s);
 
-// k_update.cu
+// CTAs that hold all of dS = Y_2 x_2 A_2^T at once (eight threads of 1024 per element)
+__host__ __device__ inline int64_t update_ds_ctas(int64_t rprod) { return (rprod + 127) / 128; }
+
+// k_update.cu: a.bar must hold zero
 template <typename Tc>
 tdb_status launch_update(UpdArgs& a, int grid_hint, cudaStream_t s);
 

@@ -44,7 +44,7 @@ struct Readback {
 // sigma^2 the step starts from (the estimator's features), and lets the projection that
 // follows start its set-up early (programmatic launch).  One CTA.
 __global__ void k_step_begin(Readback* rb, const int* need_h, const EstState* est_h, EstState* est_d,
-                             const double* sig2, double* sig2_lag, int nsig) {
+                             const double* sig2, double* sig2_lag, int nsig, unsigned* bar) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   unsigned* w = (unsigned*)rb;
   for (int i = threadIdx.x; i < (int)(sizeof(Readback) / 4); i += blockDim.x) w[i] = 0u;
@@ -54,6 +54,7 @@ __global__ void k_step_begin(Readback* rb, const int* need_h, const EstState* es
   for (int i = threadIdx.x; i < nsig; i += blockDim.x) sig2_lag[i] = sig2[i];
   __syncthreads();
   if (threadIdx.x == 0) rb->need = *(volatile const int*)need_h;
+  if (threadIdx.x < 2) bar[threadIdx.x] = 0u;          // the updates' grid barriers
 }
 
 // The step's last kernel: sigma^2 into the step record, and the record to pinned host memory
@@ -1019,7 +1020,7 @@ void prepare_step(tdb_ctx* ctx) {
 // (the mean of y_k and the predicted state plus the increment), 2 = the midpoint scheme's
 // second stage (y_k plus the increment taken at the midpoint state).
 template <typename Tc>
-tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine) {
+tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine, int stage) {
   const int p = ctx->p;
   UpdArgs a;
   memset(&a, 0, sizeof(a));
@@ -1061,10 +1062,13 @@ tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine
   a.warm = ctx->warm ? 1 : 0;
   a.reorth = reorth ? 1 : 0;
   a.skip_finish = skip_finish ? 1 : 0;
-  a.bar = ctx->bar;
+  a.bar = ctx->bar + stage;          // (both words zeroed when the step begins)
   a.stamps = ctx->prof ? ctx->stamps : nullptr;
   a.flags = ctx->flags;
-  const int64_t hint = std::max<int64_t>({ntiles, (int64_t)p * a.gsplit, Rprod / 2048});
+  // a few more CTAs take dS beside the rows (2 us of phase 1 at 1408 elements); more than 16
+  // would cost the barriers, and other members of a batch their SMs, more than that gives
+  const int64_t dsc = a.ds_y2 && update_ds_ctas(Rprod) <= 16 ? update_ds_ctas(Rprod) : 0;
+  const int64_t hint = std::max<int64_t>({ntiles + dsc, (int64_t)p * a.gsplit, Rprod / 2048});
   const tdb_status us = launch_update<Tc>(a, (int)std::min<int64_t>(hint, 1 << 20), ctx->stream);
   if (us != TDB_OK) {
     ctx->err = us == TDB_ERR_UNSUPPORTED ? "cooperative launch unsupported" : "fused update launch failed";
@@ -1097,13 +1101,14 @@ tdb_status enqueue_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vp, bool all_paths
   ctx->main_from_start = pdl;        // the projection's start event is the step's (ev[0])
   if (begin_kernel) {
     k_step_begin<<<1, 256, 0, s>>>(ctx->rb_dev, ctx->need_pin_d, ctx->est_pin_d, ctx->est_dev, ctx->sig2,
-                                   ctx->sig2_lag, p * kMaxRank);
+                                   ctx->sig2_lag, p * kMaxRank, ctx->bar);
     count_launch();
   } else {
     CK(cudaMemsetAsync(ctx->rb_dev, 0, sizeof(Readback), s));
     CK(cudaMemcpyAsync(&ctx->rb_dev->need, ctx->need_pin, sizeof(int), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(ctx->est_dev, ctx->est_pin, sizeof(EstState), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(ctx->sig2_lag, ctx->sig2, sizeof(double) * p * kMaxRank, cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemsetAsync(ctx->bar, 0, 2 * sizeof(unsigned), s));
   }
   int64_t Rprod = 1;
   for (int n = 0; n < p; ++n) Rprod *= ctx->r[n];
@@ -1139,14 +1144,14 @@ tdb_status enqueue_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vp, bool all_paths
     if (scheme == TDB_HEUN) TRY(project(nullptr, Vp, 1.0, false));
     else if (Vpp) TRY(project(nullptr, Vpp, 0.25, false));
     else TRY(project(nullptr, Vp, 0.5, false));
-    TRY(fused_update<Tc>(ctx, false, false, 0));
+    TRY(fused_update<Tc>(ctx, false, false, 0, 0));
   }
   TRY(project(ev ? ev + 4 : nullptr, Vp, 1.0, pdl));
   if (ev) CK(record_timing_event(ev[1], s));
   // a3..a6 and the refresh of G_n, G_n^{-1}, sigma^(n): one cooperative launch (second
   // stages: the increment at the intermediate state, combined with y_k)
   TRY(fused_update<Tc>(ctx, ctx->cfg.reorth != 0, split,
-                       scheme == TDB_HEUN ? 1 : (scheme == TDB_RK2_CENTRAL ? 2 : 0)));
+                       scheme == TDB_HEUN ? 1 : (scheme == TDB_RK2_CENTRAL ? 2 : 0), scheme == TDB_EULER ? 0 : 1));
   if (ev) CK(record_timing_event(ev[2], s));
   // the estimator's gate decides the error evaluation only in TDB_ERRMODE_MLP; otherwise
   // its decision goes to a scratch word and the host's schedule stands
