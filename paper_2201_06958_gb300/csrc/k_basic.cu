@@ -22,23 +22,49 @@ long long launches_so_far() { return g_launches.load(std::memory_order_relaxed);
 // Elementwise
 // ---------------------------------------------------------------------------
 
-// A = W U in the compute type: A[i + N a] = w[i] U[i + N a]  (Eq. 2.17).
+// Everything of a state (T, U_n) that other kernels read beside it, in one launch: the core and
+// the bases in the compute type (float types) and, if asked for, A_n = W_n U_n (Eq. 2.17); with
+// `src` the state is first taken from there (T, then U_1 .. U_p, as a saved state holds it).
+// One launch instead of two or three per mode: a state load is launches and copies.
 template <typename T>
-__global__ void k_weighted_bases(const double* __restrict__ U, const double* __restrict__ w, T* __restrict__ A,
-                                 int64_t N, int r) {
-  const unsigned n = (unsigned)N, tot = (unsigned)(N * r);
-  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += gridDim.x * blockDim.x)
-    A[e] = (T)(w[e % n] * U[e]);
+__global__ void __launch_bounds__(256) k_state_views(StateViews v) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < v.total; e += (int64_t)gridDim.x * blockDim.x) {
+    if (e < v.nT) {
+      const double x = v.src ? v.src[e] : v.T[e];
+      if (v.src) v.T[e] = x;
+      if (v.Tcore != v.T) ((T*)v.Tcore)[e] = (T)x;
+      continue;
+    }
+    int64_t k = e - v.nT;
+    int n = 0;
+    while (k >= v.N[n] * v.r[n]) { k -= v.N[n] * v.r[n]; ++n; }
+    const double x = v.src ? v.src[e] : v.U[n][k];
+    if (v.src) v.U[n][k] = x;
+    ((T*)v.Uc[n])[k] = (T)x;
+    if (v.bases) ((T*)v.A[n])[k] = (T)(v.w[n][k % v.N[n]] * x);
+  }
 }
-
+// The reverse: T, U_1 .. U_p one after another, for one copy to the host.
+__global__ void __launch_bounds__(256) k_state_pack(StateViews v, double* __restrict__ out) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < v.total; e += (int64_t)gridDim.x * blockDim.x) {
+    int64_t k = e - v.nT;
+    int n = 0;
+    if (k >= 0)
+      while (k >= v.N[n] * v.r[n]) { k -= v.N[n] * v.r[n]; ++n; }
+    out[e] = k < 0 ? v.T[e] : v.U[n][k];
+  }
+}
 template <typename T>
-void launch_weighted_bases(const double* U, const double* w, T* A, int64_t N, int r, cudaStream_t s) {
-  int64_t n = N * r;
-  int blocks = (int)std::min<int64_t>((n + 255) / 256, 1024);
-  k_weighted_bases<T><<<blocks, 256, 0, s>>>(U, w, A, N, r); count_launch();
+void launch_state_views(const StateViews& v, cudaStream_t s) {
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((v.total + 255) / 256, 152 * 8));
+  k_state_views<T><<<blocks, 256, 0, s>>>(v); count_launch();
 }
-template void launch_weighted_bases<float>(const double*, const double*, float*, int64_t, int, cudaStream_t);
-template void launch_weighted_bases<double>(const double*, const double*, double*, int64_t, int, cudaStream_t);
+template void launch_state_views<float>(const StateViews&, cudaStream_t);
+template void launch_state_views<double>(const StateViews&, cudaStream_t);
+void launch_state_pack(const StateViews& v, double* out, cudaStream_t s) {
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((v.total + 255) / 256, 152 * 8));
+  k_state_pack<<<blocks, 256, 0, s>>>(v, out); count_launch();
+}
 
 template <typename Ts, typename Td>
 __global__ void k_cast(const Ts* __restrict__ a, Td* __restrict__ b, int64_t n) {

@@ -111,7 +111,20 @@ void count_launch(int n = 1);
 long long launches_so_far();
 
 // k_basic.cu
-template <typename T> void launch_weighted_bases(const double* U, const double* w, T* A, int64_t N, int r, cudaStream_t s);
+struct StateViews {
+  const double* src;             // the state to take, or null: T and U hold it
+  double* T;
+  double* U[kMaxModes];
+  const double* w[kMaxModes];
+  void* Tcore;                   // compute-type core (T itself in FP64)
+  void* A[kMaxModes];
+  void* Uc[kMaxModes];
+  int64_t N[kMaxModes], nT, total;
+  int r[kMaxModes];
+  int bases;                     // form A_n too
+};
+template <typename T> void launch_state_views(const StateViews& v, cudaStream_t s);
+void launch_state_pack(const StateViews& v, double* out, cudaStream_t s);
 template <typename Ts, typename Td> void launch_cast(const Ts* a, Td* b, int64_t n, cudaStream_t s);
 template <typename T>
 void launch_diff_norm(const T* a, const T* b, T* out, int N1, int64_t ncol, T scale, const T* w1, const T* wcol,

@@ -101,6 +101,7 @@ struct tdb_ctx {
   void* Uc[kMaxModes];
   double* Ubak[kMaxModes];
   double* T;
+  double* packed;                 // T, U_1 .. U_p one after another: states on their way from or to the host
   double* T2;
   double* Tbak;
   void* Tcore;                    // compute-type core (alias of T in FP64 mode)
@@ -367,6 +368,11 @@ void carve(tdb_ctx* c, Carver& cv) {
     c->Y[n] = cv.take<char>(ysz * tsz);
   }
   c->T = cv.take<double>(Rprod);
+  {
+    int64_t tot = Rprod;
+    for (int n = 0; n < p; ++n) tot += c->N[n] * c->cap[n];
+    c->packed = cv.take<double>(tot);
+  }
   c->T2 = cv.take<double>(Rprod);
   c->Tbak = cv.take<double>(Rprod);
   c->Tcore = c->f64 ? (void*)c->T : (void*)cv.take<char>(Rprod * tsz);
@@ -635,21 +641,34 @@ tdb_status exact_error2(tdb_ctx* ctx, const Tc* V, const int* gate = nullptr) {
   return TDB_OK;
 }
 
-// Refresh everything derived from (T, U): compute-type copies, weighted bases,
-// G_n, its inverse and sigma^(n) (Eq. 2.18).
-template <typename Tc>
-tdb_status refresh_derived(tdb_ctx* ctx, bool bases_too) {
-  cudaStream_t s = ctx->stream;
-  int64_t Rprod = 1;
-  for (int n = 0; n < ctx->p; ++n) Rprod *= ctx->r[n];
-  if (!ctx->f64) launch_cast<double, float>(ctx->T, (float*)ctx->Tcore, Rprod, s);
+StateViews state_views(const tdb_ctx* ctx, bool bases, const double* src) {
+  StateViews v;
+  memset(&v, 0, sizeof(v));
+  v.src = src;
+  v.T = ctx->T;
+  v.Tcore = ctx->Tcore;
+  v.bases = bases ? 1 : 0;
+  v.nT = 1;
+  for (int n = 0; n < ctx->p; ++n) v.nT *= ctx->r[n];
+  v.total = v.nT;
   for (int n = 0; n < ctx->p; ++n) {
-    if (bases_too) launch_weighted_bases<Tc>(ctx->U[n], ctx->w[n], (Tc*)ctx->A[n], ctx->N[n], ctx->r[n], s);
-    if (ctx->f64)
-      cudaMemcpyAsync(ctx->Uc[n], ctx->U[n], sizeof(double) * ctx->N[n] * ctx->r[n], cudaMemcpyDeviceToDevice, s);
-    else
-      launch_cast<double, float>(ctx->U[n], (float*)ctx->Uc[n], ctx->N[n] * ctx->r[n], s);
+    v.U[n] = ctx->U[n];
+    v.w[n] = ctx->w[n];
+    v.A[n] = ctx->A[n];
+    v.Uc[n] = ctx->Uc[n];
+    v.N[n] = ctx->N[n];
+    v.r[n] = ctx->r[n];
+    v.total += ctx->N[n] * ctx->r[n];
   }
+  return v;
+}
+
+// Refresh everything derived from (T, U): compute-type copies, weighted bases,
+// G_n, its inverse and sigma^(n) (Eq. 2.18).  src: a packed state to take first.
+template <typename Tc>
+tdb_status refresh_derived(tdb_ctx* ctx, bool bases_too, const double* src = nullptr) {
+  cudaStream_t s = ctx->stream;
+  launch_state_views<Tc>(state_views(ctx, bases_too, src), s);
   ModeDesc d = mode_desc(ctx);
   const int nsplit = gram_split(ctx->r, ctx->p, ctx->gsplit);
   launch_gram(d, ctx->T, ctx->Gpart, nsplit, ctx->G, ctx->Ginv, ctx->Ginvf, ctx->sig2, ctx->Vprev, ctx->warm ? 1 : 0, ctx->flags, s);
@@ -1760,13 +1779,30 @@ tdb_status tdb_reinit(tdb_ctx* ctx, const void* V_now) {
 tdb_status tdb_get_factors(tdb_ctx* ctx, double* core, double* const* U, int* ranks) {
   if (!ctx) return TDB_ERR_INVALID_ARG;
   if (!ctx->ready) { ctx->err = "not initialised"; return TDB_ERR_STATE; }
-  int64_t Rprod = 1;
-  for (int n = 0; n < ctx->p; ++n) Rprod *= ctx->r[n];
-  if (core) CK(cudaMemcpyAsync(core, ctx->T, sizeof(double) * Rprod, cudaMemcpyDeviceToHost, ctx->stream));
-  if (U)
-    for (int n = 0; n < ctx->p; ++n)
-      if (U[n]) CK(cudaMemcpyAsync(U[n], ctx->U[n], sizeof(double) * ctx->N[n] * ctx->r[n], cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  if (core || U) {
+    // packed on the device, so that one copy leaves it
+    const StateViews v = state_views(ctx, false, nullptr);
+    launch_state_pack(v, ctx->packed, ctx->stream);
+    CHECK_LAUNCH();
+    std::vector<double> h;
+    try {
+      h.resize((size_t)v.total);
+    } catch (const std::bad_alloc&) {
+      ctx->err = "out of host memory";
+      return TDB_ERR_CUDA;
+    }
+    CK(cudaMemcpyAsync(h.data(), ctx->packed, sizeof(double) * v.total, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    const double* src = h.data();
+    if (core) memcpy(core, src, sizeof(double) * v.nT);
+    src += v.nT;
+    for (int n = 0; n < ctx->p; ++n) {
+      if (U && U[n]) memcpy(U[n], src, sizeof(double) * ctx->N[n] * ctx->r[n]);
+      src += ctx->N[n] * ctx->r[n];
+    }
+  } else {
+    CK(cudaStreamSynchronize(ctx->stream));
+  }
   if (ranks)
     for (int n = 0; n < ctx->p; ++n) ranks[n] = ctx->r[n];
   return TDB_OK;
@@ -1825,12 +1861,10 @@ tdb_status tdb_save_state(tdb_ctx* ctx, void* buf, size_t* bytes) {
   double* d = (double*)(h + 10);
   for (size_t i = 0; i < ctx->history.size(); ++i) d[i] = ctx->history[i];
   d += ctx->history.size();
-  CK(cudaMemcpyAsync(d, ctx->T, 8 * Rprod, cudaMemcpyDeviceToHost, ctx->stream));
-  d += Rprod;
-  for (int n = 0; n < ctx->p; ++n) {
-    CK(cudaMemcpyAsync(d, ctx->U[n], 8 * ctx->N[n] * ctx->r[n], cudaMemcpyDeviceToHost, ctx->stream));
-    d += ctx->N[n] * ctx->r[n];
-  }
+  const StateViews v = state_views(ctx, false, nullptr);
+  launch_state_pack(v, ctx->packed, ctx->stream);
+  CHECK_LAUNCH();
+  CK(cudaMemcpyAsync(d, ctx->packed, 8 * v.total, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   *bytes = need;
   return TDB_OK;
@@ -1856,14 +1890,11 @@ tdb_status tdb_load_state(tdb_ctx* ctx, const void* buf, size_t bytes, const voi
   const double* d = (const double*)(h + 10);
   ctx->history.assign(d, d + nh);
   d += nh;
-  CK(cudaMemcpyAsync(ctx->T, d, 8 * Rprod, cudaMemcpyHostToDevice, ctx->stream));
-  d += Rprod;
-  for (int n = 0; n < ctx->p; ++n) {
-    CK(cudaMemcpyAsync(ctx->U[n], d, 8 * ctx->N[n] * ctx->r[n], cudaMemcpyHostToDevice, ctx->stream));
-    d += ctx->N[n] * ctx->r[n];
-  }
+  int64_t total = Rprod;
+  for (int n = 0; n < ctx->p; ++n) total += ctx->N[n] * ctx->r[n];
+  CK(cudaMemcpyAsync(ctx->packed, d, 8 * total, cudaMemcpyHostToDevice, ctx->stream));
   ctx->warm = false;
-  tdb_status st = ctx->f64 ? refresh_derived<double>(ctx, true) : refresh_derived<float>(ctx, true);
+  tdb_status st = ctx->f64 ? refresh_derived<double>(ctx, true, ctx->packed) : refresh_derived<float>(ctx, true, ctx->packed);
   if (st != TDB_OK) return st;
   TRY(readback(ctx));
   ctx->V_prev = V_prev;
