@@ -165,32 +165,67 @@ __device__ bool chol_inv_warp_f(float* S, float* Li, int r) {
 
 // ---------------------------------------------------------------------------
 // Cyclic Jacobi on a symmetric float matrix (n <= 32, ld LD, shared) by a group of
-// `gs` threads (gt = index in the group, hardware barrier `bar`), Brent-Luk
-// round-robin ordering as jacobi_smem: eigenvalues end on the diagonal of A and the
-// vectors in V.  Stops when the off-diagonal mass is below tol^2 of the diagonal
+// JG = 256 threads (gt = index in the group, hardware barrier `bar`), Brent-Luk
+// round-robin ordering: eigenvalues end on the diagonal of the returned buffer (A or B) and
+// the vectors in V.  Stops when the off-diagonal mass is below tol^2 of the diagonal
 // mass, after max_sweeps, or when a sweep after the second no longer halves it
-// (the float rounding floor).  red holds >= 2 * gs / 32 floats.
+// (the float rounding floor).  red holds >= 16 floats.
+//
+// A round is one chain (the pair's entries, its rotation, the 2 x 2 block) between barriers;
+// every thread forms the two rotations its block needs itself, from the buffer the round
+// reads, and writes the block to the other one, so a round has one barrier.  (The rotations
+// formed by half the pairs' threads and passed through shared memory: two barriers and 0.5 us
+// a round.)  V's entries belong to one thread in a round and stay in place.
 // ---------------------------------------------------------------------------
-__device__ int jacobi_group(float* A, float* V, int n, int max_sweeps, float tol, float* cs, int* pq, float* red,
-                            int gt, int gs, int bar) {
+__device__ __forceinline__ void jacobi_pair(int nn, int rd, int k, int& p, int& q) {
+  if (k == 0) {
+    p = rd;
+    q = nn - 1;
+  } else {
+    p = rd + k;
+    if (p >= nn - 1) p -= nn - 1;
+    q = rd - k;
+    if (q < 0) q += nn - 1;
+  }
+}
+__device__ __forceinline__ void jacobi_rotation(float app, float aqq, float apq, float thr, float& c, float& s) {
+  c = 1.f;
+  s = 0.f;
+  if (apq != 0.f && apq * apq > thr * thr * fabsf(app * aqq)) {
+    // tan of the rotation angle, t = sign(theta) / (|theta| + sqrt(theta^2 + 1)),
+    // with approximate reciprocals: c^2 + s^2 = 1 holds whatever t's rounding
+    const float theta = (aqq - app) * rcp_approx(2.f * apq);
+    const float at = fabsf(theta);
+    const float x = fmaf(at, at, 1.f);
+    const float root = (at < 1e18f) ? x * rsqrt_approx(x) : at;
+    const float t = copysignf(rcp_approx(at + root), theta);
+    c = rsqrt_approx(fmaf(t, t, 1.f));
+    s = t * c;
+  }
+}
+constexpr int JG = 256;
+__device__ float* jacobi_group(float* A, float* B, float* V, int n, int max_sweeps, float tol, float* red, int gt,
+                               int bar) {
   const int nn = (n + 1) & ~1, half = nn / 2;
-  const int nw = gs >> 5, gl = gt & 31, gw = gt >> 5;
-  for (int e = gt; e < nn * nn; e += gs) {
+  constexpr int nw = JG >> 5;
+  const int gl = gt & 31, gw = gt >> 5;
+  for (int e = gt; e < nn * nn; e += JG) {
     const int i = e % nn, j = e / nn;
     if (i >= n || j >= n) A[i + LD * j] = 0.f;
     V[i + LD * j] = (i == j) ? 1.f : 0.f;
   }
-  // the block (I, J) and the V entries (i, J) owned by this thread, fixed for all rounds
+  // the block (I, J) and the V entries (i, J) of this thread, fixed for all rounds
   const int bI = gt % half, bJ = gt / half;
   const bool has_b = gt < half * half;
   const int nv = nn * half;
-  named_bar(bar, gs);
+  const int v0 = gt < nv ? gt : -1, v1 = gt + JG < nv ? gt + JG : -1;
+  const int vi0 = v0 % nn, vJ0 = v0 / nn, vi1 = v1 % nn, vJ1 = v1 / nn;
+  named_bar(bar, JG);
   const float thr = tol * 1e-3f;
   float off_prev = 0.f;
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     float off = 0.f, dia = 0.f;
-    for (int e = gt; e < nn * nn; e += gs) {
+    for (int e = gt; e < nn * nn; e += JG) {
       const int i = e % nn, j = e / nn;
       const float v = A[i + LD * j];
       if (i == j) dia += v * v; else off += v * v;
@@ -198,66 +233,51 @@ __device__ int jacobi_group(float* A, float* V, int n, int max_sweeps, float tol
     off = warp_sum(off);
     dia = warp_sum(dia);
     if (gl == 0) { red[gw] = off; red[nw + gw] = dia; }
-    named_bar(bar, gs);
+    named_bar(bar, JG);
     off = 0.f;
     dia = 0.f;
     for (int w = 0; w < nw; ++w) { off += red[w]; dia += red[nw + w]; }
-    named_bar(bar, gs);
+    named_bar(bar, JG);
     if (off <= tol * tol * dia || dia == 0.f) break;
     if (sweep >= 2 && off > 0.5f * off_prev) break;
     off_prev = off;
+    auto rotation = [&](int p, int q, float& c, float& s) {
+      jacobi_rotation(A[p + LD * p], A[q + LD * q], A[p + LD * q], thr, c, s);
+    };
+    auto turn = [&](int rd, int i, int J) {              // V's entry (i, pair J)
+      int p, q;
+      jacobi_pair(nn, rd, J, p, q);
+      float c, s;
+      rotation(p, q, c, s);
+      const float vp = V[i + LD * p], vq = V[i + LD * q];
+      V[i + LD * p] = c * vp - s * vq;
+      V[i + LD * q] = s * vp + c * vq;
+    };
     for (int rd = 0; rd < nn - 1; ++rd) {
-      if (gt < half) {
-        const int k = gt;
-        int p = rd, q = nn - 1;
-        if (k > 0) {
-          p = rd + k;
-          if (p >= nn - 1) p -= nn - 1;
-          q = rd - k;
-          if (q < 0) q += nn - 1;
-        }
-        const float app = A[p + LD * p], aqq = A[q + LD * q], apq = A[p + LD * q];
-        float c = 1.f, s = 0.f;
-        if (apq != 0.f && apq * apq > thr * thr * fabsf(app * aqq)) {
-          // tan of the rotation angle, t = sign(theta) / (|theta| + sqrt(theta^2 + 1)),
-          // with approximate reciprocals: c^2 + s^2 = 1 holds whatever t's rounding
-          const float theta = (aqq - app) * rcp_approx(2.f * apq);
-          const float at = fabsf(theta);
-          const float x = fmaf(at, at, 1.f);
-          const float root = (at < 1e18f) ? x * rsqrt_approx(x) : at;
-          const float t = copysignf(rcp_approx(at + root), theta);
-          c = rsqrt_approx(fmaf(t, t, 1.f));
-          s = t * c;
-        }
-        cs[2 * k] = c;
-        cs[2 * k + 1] = s;
-        pq[2 * k] = p;
-        pq[2 * k + 1] = q;
-      }
-      named_bar(bar, gs);
       if (has_b) {
-        const int pI = pq[2 * bI], qI = pq[2 * bI + 1], pJ = pq[2 * bJ], qJ = pq[2 * bJ + 1];
-        const float cI = cs[2 * bI], sI = cs[2 * bI + 1], cJ = cs[2 * bJ], sJ = cs[2 * bJ + 1];
+        int pI, qI, pJ, qJ;
+        jacobi_pair(nn, rd, bI, pI, qI);
+        jacobi_pair(nn, rd, bJ, pJ, qJ);
         const float b00 = A[pI + LD * pJ], b01 = A[pI + LD * qJ], b10 = A[qI + LD * pJ], b11 = A[qI + LD * qJ];
+        float cI, sI, cJ, sJ;
+        rotation(pI, qI, cI, sI);
+        rotation(pJ, qJ, cJ, sJ);
         const float c00 = cJ * b00 - sJ * b01, c01 = sJ * b00 + cJ * b01;
         const float c10 = cJ * b10 - sJ * b11, c11 = sJ * b10 + cJ * b11;
-        A[pI + LD * pJ] = cI * c00 - sI * c10;
-        A[pI + LD * qJ] = cI * c01 - sI * c11;
-        A[qI + LD * pJ] = sI * c00 + cI * c10;
-        A[qI + LD * qJ] = sI * c01 + cI * c11;
+        B[pI + LD * pJ] = cI * c00 - sI * c10;
+        B[pI + LD * qJ] = cI * c01 - sI * c11;
+        B[qI + LD * pJ] = sI * c00 + cI * c10;
+        B[qI + LD * qJ] = sI * c01 + cI * c11;
       }
-      for (int e = gt; e < nv; e += gs) {
-        const int i = e % nn, J = e / nn;
-        const int pJ = pq[2 * J], qJ = pq[2 * J + 1];
-        const float cJ = cs[2 * J], sJ = cs[2 * J + 1];
-        const float vp = V[i + LD * pJ], vq = V[i + LD * qJ];
-        V[i + LD * pJ] = cJ * vp - sJ * vq;
-        V[i + LD * qJ] = sJ * vp + cJ * vq;
-      }
-      named_bar(bar, gs);
+      if (v0 >= 0) turn(rd, vi0, vJ0);
+      if (v1 >= 0) turn(rd, vi1, vJ1);
+      named_bar(bar, JG);
+      float* t = A;
+      A = B;
+      B = t;
     }
   }
-  return sweep;
+  return A;
 }
 
 // Gauss-Jordan inversion of the SPD matrix in A0 (r x r, ld LD, shared) by the
@@ -407,7 +427,7 @@ __device__ void gram_partial(const ModeDesc& d, const double* T, double* gpart, 
 // while threads 256..511 run the float Jacobi on Vp^T (G / scale) Vp (Vp the previous
 // eigenvectors, identity when cold); then Rayleigh quotients v^T G v / v^T v in
 // double, sorted descending by an integer key; the sorted eigenvectors become the
-// next warm start.  One CTA of UPD_THREADS threads; smraw holds >= 46 KB.
+// next warm start.  One CTA of UPD_THREADS threads; smraw holds >= 50 KB.
 __device__ __noinline__ void gram_finish(const ModeDesc& d, int n, const double* gpart, int gsplit, double* Gout,
                                          double* Ginv, float* Ginvf, double* sig2, float* Vprev, int warm,
                                          unsigned* flags, unsigned char* smraw) {
@@ -421,17 +441,15 @@ __device__ __noinline__ void gram_finish(const ModeDesc& d, int n, const double*
   float* Af = Vps + LD * LD;           // LD*LD
   float* Vf = Af + LD * LD;            // LD*LD  (Af and Vf later hold W in double)
   float* Wf = Vf + LD * LD;            // LD*LD
-  float* cs = Wf + LD * LD;            // 64
-  float* red = cs + 64;                // 64
-  int* pq = (int*)(red + 64);          // 64
-  int* slot = pq + 64;                 // LD
+  float* Bf = Wf + LD * LD;            // LD*LD: the Jacobi's other buffer
+  float* red = Bf + LD * LD;           // 64
+  int* slot = (int*)(red + 64);        // LD
   double* GW = Ai;
   double* Wd = (double*)Af;
   __shared__ int bad_sh, gjbad_sh;
   __shared__ float scale_sh;
   __shared__ double ipk_sh[2];
   const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
-  constexpr int JG = 256;              // Jacobi group: threads [JG, 2 JG)
   float* Vp = Vprev + (int64_t)n * LD * LD;
   if (tid == 0) bad_sh = 0;
   for (int e = tid; e < LD * LD; e += blockDim.x) {
@@ -491,7 +509,7 @@ __device__ __noinline__ void gram_finish(const ModeDesc& d, int n, const double*
       }
     }
     named_bar(2, JG);
-    jacobi_group(Af, Vf, r, warm ? 2 : 30, 1e-6f, cs, pq, red, gt, JG, 2);
+    jacobi_group(Af, Bf, Vf, r, warm ? 2 : 30, 1e-6f, red, gt, 2);
     for (int e = gt; e < r * r; e += JG) {               // eigenvectors in the original basis
       const int a = e % r, b = e / r;
       float s = Vf[a + LD * b];

@@ -1102,10 +1102,9 @@ template <typename Tc>
 tdb_status enqueue_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vp, bool all_paths, const Tc* Vpp = nullptr) {
   cudaStream_t s = ctx->stream;
   const int p = ctx->p;
-  // exact error every step, or gated by the estimator: the G_n refresh (G_n, G_n^{-1},
-  // sigma^(n)) runs beside the error on the context's second stream
-  const bool split = (ctx->cfg.error_mode == TDB_ERRMODE_EXACT || ctx->cfg.error_mode == TDB_ERRMODE_MLP) &&
-                     ctx->aux && ctx->ev_fork && ctx->ev_join;
+  // the G_n refresh (G_n, G_n^{-1}, sigma^(n)) runs beside the features and the error on the
+  // context's second stream
+  const bool split = ctx->aux && ctx->ev_fork && ctx->ev_join;
   cudaEvent_t* ev = ctx->prof ? ctx->pev : nullptr;
   const int scheme = ctx->cfg.integrator;
   // the step opens with one small kernel (step record cleared, host words fetched, the
