@@ -340,8 +340,11 @@ void launch_recon_err(const T* V, const T* U1, const T* H, int r1, int N1, int64
                       const int* gate) {
   // rows per lane: 16 bytes of V (float ranks above 16: 8 bytes), so that U_1 stays in registers
   const uintptr_t va = (uintptr_t)V;
-  const int blocks = std::max(1, std::min(nblocks, 2 * 152));
   auto go = [&](auto kern, int R, int RM) {
+    // two CTAs per SM at most, and at least a ring of columns for every warp (a small tensor's
+    // warps would spend their time on U_1, and a batch's members on each other's SMs)
+    const int64_t units = ((N1 + 32 * R - 1) / (32 * R)) * ncol;
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>({(units + 8 * RE_D - 1) / (8 * RE_D), nblocks, 2 * 152}));
     const size_t sm = sizeof(T) * 8 * (RE_D * 32 * R + 32 * RM);
     if (sm > 47 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     const int vec = N1 % R == 0 && va % (R * sizeof(T)) == 0;

@@ -227,12 +227,23 @@ namespace tdb {
 // re-initialisation + 1), log10 of the previous step's residual.  The network predicts
 // the change of log10 error over the step, so the estimate chains from the previous
 // error and the features do not depend on which steps were evaluated exactly.
-__global__ void __launch_bounds__(256) k_est_features(const EstState* __restrict__ stp, const float* __restrict__ dS, int nds,
-                                                      const double* __restrict__ dv2, const double* __restrict__ sig2,
-                                                      int4 ranks, int p, const float* __restrict__ P,
-                                                      const float* __restrict__ norm, float* __restrict__ feat,
-                                                      double* __restrict__ est, int* __restrict__ need,
-                                                      double* __restrict__ ds2_out) {
+constexpr int EF_BATCH = 32;
+struct EstBatch {
+  EstArgs a[EF_BATCH];
+};
+__global__ void __launch_bounds__(256) k_est_features(const __grid_constant__ EstBatch B) {
+  const EstArgs& A = B.a[blockIdx.x];
+  const EstState* __restrict__ stp = A.st;
+  const float* __restrict__ dS = A.dS;
+  const int nds = A.nds, p = A.p;
+  const double* __restrict__ dv2 = A.dv2;
+  const double* __restrict__ sig2 = A.sig2;
+  const float* __restrict__ P = A.P;
+  const float* __restrict__ norm = A.norm;
+  float* __restrict__ feat = A.feat;
+  double* __restrict__ est = A.est;
+  int* __restrict__ need = A.need;
+  double* __restrict__ ds2_out = A.ds2;
   // The features are float-valued and ||dS|| is only as accurate as the projection,
   // so everything is float except the difference ||dV||^2 - ||dS||^2 (double: it can
   // cancel).  One CTA; the launch is latency-bound, so every global load is issued up
@@ -261,7 +272,7 @@ __global__ void __launch_bounds__(256) k_est_features(const EstState* __restrict
   for (int k = 0; k < H / 4; ++k) w2r[k] = W2[j * H + q * (H / 4) + k];
   const float b2v = b2[j], w3v = w3[j];
   const float tiny = 1e-30f;
-  const int rr[4] = {ranks.x, ranks.y, ranks.z, ranks.w};
+  const int rr[4] = {A.ranks[0], A.ranks[1], A.ranks[2], A.ranks[3]};
   if (wid == 1) {                       // sum of the mode-1 sigma^2 (kept part)
     float v = lane < rr[0] ? fmaxf((float)sig2[lane], 0.f) : 0.f;
     v = warp_sum(v);
@@ -343,12 +354,14 @@ __global__ void __launch_bounds__(256) k_est_features(const EstState* __restrict
   }
 }
 
-void est_features(const EstState* st_dev, const float* dS, int nds, const double* dv2, const double* sig2,
-                  const int* ranks, int p, const float* P, const float* norm, float* feat, double* est, int* need,
-                  double* ds2, cudaStream_t s) {
-  int4 rk = make_int4(ranks[0], p > 1 ? ranks[1] : 1, p > 2 ? ranks[2] : 1, p > 3 ? ranks[3] : 1);
-  k_est_features<<<1, 256, 0, s>>>(st_dev, dS, nds, dv2, sig2, rk, p, P, norm, feat, est, need, ds2);
-  count_launch();
+void est_features(const EstArgs* args, int n, cudaStream_t s) {
+  for (int i0 = 0; i0 < n; i0 += EF_BATCH) {
+    EstBatch B;
+    const int m = std::min(EF_BATCH, n - i0);
+    for (int i = 0; i < m; ++i) B.a[i] = args[i0 + i];
+    k_est_features<<<m, 256, 0, s>>>(B);
+    count_launch();
+  }
 }
 
 // Standardise the trace in place: norm = [mean_f (F), sd_f (F), mean_t, sd_t].

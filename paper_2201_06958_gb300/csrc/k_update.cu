@@ -749,11 +749,11 @@ __device__ void rows_u1(const UpdArgs& a, int n, int64_t i0, int tile, unsigned 
 // every run).  Results go to red[which][n], read by every tile of phase 2 (P_n) or by
 // the Cholesky-QR of phase 3 (C_n).
 template <typename Tc>
-__device__ void reduce_long(const UpdArgs& a, int which) {
+__device__ void reduce_long(const UpdArgs& a, int which, unsigned bid, unsigned nb) {
   const ModeDesc& d = a.d;
   const int lane = threadIdx.x & 31;
-  const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int64_t gw = (int64_t)bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int64_t nw = (int64_t)nb * (blockDim.x >> 5);
   const Tc* part = (const Tc*)a.part + (int64_t)which * d.p * a.ntile * LD * LD;
   Tc* red = (Tc*)a.red + (int64_t)which * kMaxModes * LD * LD;
   for (int64_t task = gw; task < (int64_t)d.p * LD * LD; task += nw) {
@@ -920,13 +920,13 @@ __device__ void rows_u2(const UpdArgs& a, int n, int64_t i0, const double* Ris, 
 // slabs at a time staged in shared memory, F chosen so that every CTA of the grid has some.
 // With two modes the one slab is the core: it is read whole before it is written.
 template <typename Tc>
-__device__ void core_12(const UpdArgs& a, unsigned char* sm) {
+__device__ void core_12(const UpdArgs& a, unsigned char* sm, unsigned bid, unsigned nb) {
   const ModeDesc& d = a.d;
   const int r1 = d.r[0], r2 = d.r[1], ns = r1 * r2;
   const int64_t nslab = prod_r_above(d, 1);
-  const int64_t per_cta = (nslab + gridDim.x - 1) / gridDim.x;
+  const int64_t per_cta = (nslab + nb - 1) / nb;
   const int F = (int)(per_cta < UPD_THREADS / ns ? per_cta : UPD_THREADS / ns);
-  if (blockIdx.x * (int64_t)F >= nslab) return;
+  if (bid * (int64_t)F >= nslab) return;
   double* R1 = (double*)sm;             // LD*LD each
   double* R2 = R1 + LD * LD;
   double* Xs = R2 + LD * LD;            // F slabs <= UPD_THREADS
@@ -935,7 +935,7 @@ __device__ void core_12(const UpdArgs& a, unsigned char* sm) {
   R2[threadIdx.x] = __ldcg(&a.R[LD * LD + threadIdx.x]);
   const Tc* dS = (const Tc*)a.dS;
   const int t = threadIdx.x, fl = t / ns, e = t - fl * ns, i = e % r1, j = e / r1;
-  for (int64_t f0 = blockIdx.x * (int64_t)F; f0 < nslab; f0 += (int64_t)gridDim.x * F) {
+  for (int64_t f0 = bid * (int64_t)F; f0 < nslab; f0 += (int64_t)nb * F) {
     const bool act = fl < F && f0 + fl < nslab;
     const int64_t idx = (f0 + fl) * ns + e;
     if (act) {
@@ -966,13 +966,13 @@ __device__ void core_12(const UpdArgs& a, unsigned char* sm) {
 // Phase 5: T = T2 x_3 R_3 (x_4 R_4) and its copy in the compute type, by r_3 x r_4 fibers (the
 // entries at fixed first two indices), F at a time, neighbouring fibers on neighbouring threads.
 template <typename Tc>
-__device__ void core_34(const UpdArgs& a, unsigned char* sm) {
+__device__ void core_34(const UpdArgs& a, unsigned char* sm, unsigned bid, unsigned nb) {
   const ModeDesc& d = a.d;
   const int r3 = d.r[2], r4 = d.p == 4 ? d.r[3] : 1, nf = r3 * r4;
   const int64_t L = prod_r_below(d, 2);
-  const int64_t per_cta = (L + gridDim.x - 1) / gridDim.x;
+  const int64_t per_cta = (L + nb - 1) / nb;
   const int F = (int)(per_cta < UPD_THREADS / nf ? per_cta : UPD_THREADS / nf);
-  if (blockIdx.x * (int64_t)F >= L) return;
+  if (bid * (int64_t)F >= L) return;
   double* R3 = (double*)sm;
   double* R4 = R3 + LD * LD;
   double* Xs = R4 + LD * LD;            // F fibers <= UPD_THREADS, element (c, d) of fiber f at f + F (c + r3 d)
@@ -980,7 +980,7 @@ __device__ void core_34(const UpdArgs& a, unsigned char* sm) {
   R3[threadIdx.x] = __ldcg(&a.R[2 * LD * LD + threadIdx.x]);
   if (d.p == 4) R4[threadIdx.x] = __ldcg(&a.R[3 * LD * LD + threadIdx.x]);
   const int t = threadIdx.x, fl = t % F, e = t / F, c = e % r3, dd = e / r3;
-  for (int64_t f0 = blockIdx.x * (int64_t)F; f0 < L; f0 += (int64_t)gridDim.x * F) {
+  for (int64_t f0 = bid * (int64_t)F; f0 < L; f0 += (int64_t)nb * F) {
     const bool act = e < nf && f0 + fl < L;
     const int64_t idx = f0 + fl + L * e;
     if (act) Xs[t] = __ldcg(&a.T2[idx]);
@@ -1002,6 +1002,112 @@ __device__ void core_34(const UpdArgs& a, unsigned char* sm) {
   }
 }
 
+// The row tiles of all modes, numbered mode after mode.
+struct RowTiles {
+  int base[kMaxModes + 1];
+  bool tree;                               // a mode above kTreeTiles row tiles
+  __device__ explicit RowTiles(const ModeDesc& d) {
+    int tot = 0;
+    tree = false;
+    for (int n = 0; n < d.p; ++n) {
+      const int nt = (int)((d.N[n] + 31) / 32);
+      base[n] = tot;
+      tot += nt;
+      tree |= nt > kTreeTiles;
+    }
+    for (int n = d.p; n <= kMaxModes; ++n) base[n] = tot;
+  }
+  __device__ int total() const { return base[kMaxModes]; }
+  __device__ void find(int task, int* n_out, int* t_out) const {
+    int n = 0;
+    while (task >= base[n + 1]) ++n;
+    *n_out = n;
+    *t_out = task - base[n];
+  }
+};
+
+// Phase 1: M, X, partial P; dS = Y_2 x_2 A_2^T when the projection left it.  (Every phase takes
+// the CTA's index among the nb that share the state: the whole grid, or a member's part of a
+// batch's.  The values do not depend on nb.)
+template <typename Tc>
+__device__ void phase_rows1(const UpdArgs& a, const RowTiles& rt, unsigned char* smraw, unsigned bid, unsigned nb) {
+  const ModeDesc& d = a.d;
+  for (int task = bid; task < rt.total(); task += nb) {
+    int n, t;
+    rt.find(task, &n, &t);
+    rows_mxp<Tc>(a, n, (int64_t)t * 32, t, smraw);
+  }
+  // (dS on the CTAs without rows where those hold all of it at once, else on all)
+  const unsigned dsc0 = (int64_t)nb - rt.total() >= update_ds_ctas(prod_r(d)) ? (unsigned)rt.total() : 0u;
+  if (!a.ds_y2 || bid < dsc0) return;
+  // dS = Y_2 x_2 A_2^T (Eqs. 2.15/2.16: dS = Y_n x_n A_n^T for every n), read from phase 4 on.
+  // Eight consecutive threads share one element: each sums every eighth i2 with all its loads
+  // in flight, then the eight partial sums are added by shuffles in a fixed order.
+  const Tc* Y2 = (const Tc*)a.ds_y2;
+  const Tc* A2 = (const Tc*)a.A[1];
+  const int r1 = d.r[0], r2 = d.r[1];
+  const int N2 = (int)d.N[1];
+  const int64_t tot = prod_r(d);
+  const int grp = threadIdx.x >> 3, part = threadIdx.x & 7;
+  const int ngrp = blockDim.x >> 3;
+  const int64_t stride = (int64_t)(nb - dsc0) * ngrp;
+  const int64_t rounds = (tot + stride - 1) / stride;
+  for (int64_t k = 0; k < rounds; ++k) {
+    const int64_t e = (bid - dsc0) + (int64_t)(nb - dsc0) * grp + stride * k;
+    Tc acc = Tc(0);
+    if (e < tot) {
+      const int a1 = (int)(e % r1);
+      const int64_t rest = e / r1;
+      const int b = (int)(rest % r2);
+      const int64_t q = rest / r2;
+      const Tc* y = Y2 + a1 + (int64_t)r1 * N2 * q;      // Y_2[a1 + r1 (i2 + N2 q)]
+      const Tc* A = A2 + (int64_t)N2 * b;
+#pragma unroll 16
+      for (int i2 = part; i2 < N2; i2 += 8) acc += __ldcg(&y[(int64_t)r1 * i2]) * A[i2];
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (e < tot && part == 0) ((Tc*)a.dS_out)[e] = acc;
+  }
+}
+
+// Phase 2: P, U', partial C
+template <typename Tc>
+__device__ void phase_rows2(const UpdArgs& a, const RowTiles& rt, unsigned char* smraw, unsigned bid, unsigned nb) {
+  for (int task = bid; task < rt.total(); task += nb) {
+    int n, t;
+    rt.find(task, &n, &t);
+    rows_u1<Tc>(a, n, (int64_t)t * 32, t, smraw);
+  }
+}
+
+// Phase 3: Cholesky-QR factors of the mode of this CTA's rows; U''
+template <typename Tc>
+__device__ void phase_rows3(const UpdArgs& a, const RowTiles& rt, unsigned char* smraw, unsigned bid, unsigned nb) {
+  double* Rs = (double*)smraw;
+  int have = -1;
+  for (int task = bid; task < rt.total(); task += nb) {
+    int n, t;
+    rt.find(task, &n, &t);
+    if (n != have) mode_cholqr<Tc>(a, n, smraw, t == 0);
+    have = n;
+    rows_u2<Tc>(a, n, (int64_t)t * 32, Rs + LD * LD, (unsigned char*)(Rs + 2 * LD * LD));
+    if (t == 0) {
+      a.R[(int64_t)n * LD * LD + threadIdx.x] = Rs[threadIdx.x];
+      a.Rinv[(int64_t)n * LD * LD + threadIdx.x] = Rs[LD * LD + threadIdx.x];
+    }
+  }
+}
+
+// Phase 6: Gram partials
+template <typename Tc>
+__device__ void phase_grams(const UpdArgs& a, unsigned char* smraw, unsigned bid, unsigned nb) {
+  for (int task = bid; task < a.d.p * a.gsplit; task += nb)
+    gram_partial<sizeof(Tc) == 4 ? 4 : 1>(a.d, a.T, a.gpart, a.gsplit, task / a.gsplit, task % a.gsplit,
+                                          (double(*)[33])smraw);
+}
+
 template <typename Tc>
 __global__ void __launch_bounds__(UPD_THREADS, 1) k_update(UpdArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1012,118 +1118,35 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_update(UpdArgs a) {
   int nst = 0;
   unsigned nbar = 0;
   stamp(st_sh, a.stamps, 0);
-  const ModeDesc& d = a.d;
-  const int p = d.p;
-  const unsigned nb = gridDim.x;
-
-  int ntiles_total = 0, tile_base[kMaxModes + 1];
-  for (int n = 0; n < p; ++n) {
-    tile_base[n] = ntiles_total;
-    ntiles_total += (int)((d.N[n] + 31) / 32);
-  }
-  tile_base[p] = ntiles_total;
-  bool tree = false;
-  for (int n = 0; n < p; ++n) tree |= (d.N[n] + 31) / 32 > kTreeTiles;
-  auto tile_of = [&](int task, int* n_out, int* t_out) {
-    int n = 0;
-    while (task >= tile_base[n + 1]) ++n;
-    *n_out = n;
-    *t_out = task - tile_base[n];
-  };
-
-  // 1: M, X, partial P; dS = Y_2 x_2 A_2^T when the projection left it
-  // (on the CTAs without rows where those hold all of it at once, else on all)
-  const unsigned dsc0 = (int64_t)nb - ntiles_total >= update_ds_ctas(prod_r(d)) ? (unsigned)ntiles_total : 0u;
-  for (int task = blockIdx.x; task < ntiles_total; task += nb) {
-    int n, t;
-    tile_of(task, &n, &t);
-    rows_mxp<Tc>(a, n, (int64_t)t * 32, t, smraw);
-  }
-  if (a.ds_y2 && blockIdx.x >= dsc0) {
-    // dS = Y_2 x_2 A_2^T (Eqs. 2.15/2.16: dS = Y_n x_n A_n^T for every n), read from
-    // phase 4 on.  Eight consecutive threads share one element: each sums every eighth i2 with all its loads in flight, then the
-    // eight partial sums are added by shuffles in a fixed order.
-    const Tc* Y2 = (const Tc*)a.ds_y2;
-    const Tc* A2 = (const Tc*)a.A[1];
-    const int r1 = d.r[0], r2 = d.r[1];
-    const int N2 = (int)d.N[1];
-    const int64_t tot = prod_r(d);
-    const int grp = threadIdx.x >> 3, part = threadIdx.x & 7;
-    const int ngrp = blockDim.x >> 3;
-    const int64_t stride = (int64_t)(nb - dsc0) * ngrp;
-    const int64_t rounds = (tot + stride - 1) / stride;
-    for (int64_t k = 0; k < rounds; ++k) {
-      const int64_t e = (blockIdx.x - dsc0) + (int64_t)(nb - dsc0) * grp + stride * k;
-      Tc acc = Tc(0);
-      if (e < tot) {
-        const int a1 = (int)(e % r1);
-        const int64_t rest = e / r1;
-        const int b = (int)(rest % r2);
-        const int64_t q = rest / r2;
-        const Tc* y = Y2 + a1 + (int64_t)r1 * N2 * q;      // Y_2[a1 + r1 (i2 + N2 q)]
-        const Tc* A = A2 + (int64_t)N2 * b;
-#pragma unroll 16
-        for (int i2 = part; i2 < N2; i2 += 8) acc += __ldcg(&y[(int64_t)r1 * i2]) * A[i2];
-      }
-      acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-      if (e < tot && part == 0) ((Tc*)a.dS_out)[e] = acc;
-    }
-  }
+  const int p = a.d.p;
+  const unsigned bid = blockIdx.x, nb = gridDim.x;
+  const RowTiles rt(a.d);
+  phase_rows1<Tc>(a, rt, smraw, bid, nb);
   if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   stamp(st_sh, a.stamps, ++nst);
-  if (tree) {
-    reduce_long<Tc>(a, 0);
+  if (rt.tree) {
+    reduce_long<Tc>(a, 0, bid, nb);
     if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   }
-
-  // 2: P, U', partial C
-  for (int task = blockIdx.x; task < ntiles_total; task += nb) {
-    int n, t;
-    tile_of(task, &n, &t);
-    rows_u1<Tc>(a, n, (int64_t)t * 32, t, smraw);
-  }
+  phase_rows2<Tc>(a, rt, smraw, bid, nb);
   if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   stamp(st_sh, a.stamps, ++nst);
-  if (tree && a.reorth) {
-    reduce_long<Tc>(a, 1);
+  if (rt.tree && a.reorth) {
+    reduce_long<Tc>(a, 1, bid, nb);
     if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   }
-
-  // 3: Cholesky-QR factors of the mode of this CTA's rows; U''
-  {
-    double* Rs = (double*)smraw;
-    int have = -1;
-    for (int task = blockIdx.x; task < ntiles_total; task += nb) {
-      int n, t;
-      tile_of(task, &n, &t);
-      if (n != have) mode_cholqr<Tc>(a, n, smraw, t == 0);
-      have = n;
-      rows_u2<Tc>(a, n, (int64_t)t * 32, Rs + LD * LD, (unsigned char*)(Rs + 2 * LD * LD));
-      if (t == 0) {
-        a.R[(int64_t)n * LD * LD + threadIdx.x] = Rs[threadIdx.x];
-        a.Rinv[(int64_t)n * LD * LD + threadIdx.x] = Rs[LD * LD + threadIdx.x];
-      }
-    }
-  }
+  phase_rows3<Tc>(a, rt, smraw, bid, nb);
   if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   stamp(st_sh, a.stamps, ++nst);
-
-  // 4, 5: the core
-  core_12<Tc>(a, smraw);
+  core_12<Tc>(a, smraw, bid, nb);
   if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   stamp(st_sh, a.stamps, ++nst);
   if (p > 2) {
-    core_34<Tc>(a, smraw);
+    core_34<Tc>(a, smraw, bid, nb);
     if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   }
   stamp(st_sh, a.stamps, ++nst);
-
-  // 6: Gram partials
-  for (int task = blockIdx.x; task < p * a.gsplit; task += nb)
-    gram_partial<sizeof(Tc) == 4 ? 4 : 1>(d, a.T, a.gpart, a.gsplit, task / a.gsplit, task % a.gsplit,
-                                          (double(*)[33])smraw);
+  phase_grams<Tc>(a, smraw, bid, nb);
   if (a.skip_finish) {
     // (the finish is another launch: the kernel's end orders it)
     stamp(st_sh, a.stamps, ++nst);
@@ -1133,12 +1156,46 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_update(UpdArgs a) {
   }
   if (!grid_sync(a.bar, ++nbar, nb, a.flags, &abort_sh)) return;
   stamp(st_sh, a.stamps, ++nst);
-
   // 7: G, G^{-1}, sigma^2 (or a separate launch beside the exact error)
-  for (int n = blockIdx.x; n < p; n += nb)
-    gram_finish(d, n, a.gpart, a.gsplit, a.G, a.Ginv, a.Ginvf, a.sig2, a.Vprev, a.warm, a.flags, smraw);
+  for (int n = bid; n < p; n += nb)
+    gram_finish(a.d, n, a.gpart, a.gsplit, a.G, a.Ginv, a.Ginvf, a.sig2, a.Vprev, a.warm, a.flags, smraw);
   stamp(st_sh, a.stamps, ++nst);
   stamp_flush(st_sh, a.stamps, nst);
+}
+
+// One phase of the updates of up to kUpdBatch states (members of a batch) in an ordinary
+// launch: CTAs base[m] .. base[m + 1] - 1 are member m's.  The phases are the fused kernel's,
+// the end of a launch taking the place of the grid barrier, so that no member's CTAs hold an
+// SM while they wait and none needs to be resident with the others of its grid.
+struct UpdBatch {
+  int n;
+  int base[kUpdBatch + 1];
+  UpdArgs a[kUpdBatch];
+};
+enum { PH_ROWS1, PH_SUM_P, PH_ROWS2, PH_SUM_C, PH_ROWS3, PH_CORE12, PH_CORE34, PH_GRAMS, PH_FINISH };
+template <typename Tc, int PH>
+__global__ void __launch_bounds__(UPD_THREADS, 1) k_update_batch(const __grid_constant__ UpdBatch B) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  int m = 0;
+  while ((int)blockIdx.x >= B.base[m + 1]) ++m;
+  const UpdArgs& a = B.a[m];
+  const unsigned bid = blockIdx.x - B.base[m], nb = B.base[m + 1] - B.base[m];
+  if constexpr (PH == PH_CORE12) {
+    core_12<Tc>(a, smraw, bid, nb);
+  } else if constexpr (PH == PH_CORE34) {
+    core_34<Tc>(a, smraw, bid, nb);
+  } else if constexpr (PH == PH_GRAMS) {
+    phase_grams<Tc>(a, smraw, bid, nb);
+  } else if constexpr (PH == PH_FINISH) {
+    gram_finish(a.d, bid, a.gpart, a.gsplit, a.G, a.Ginv, a.Ginvf, a.sig2, a.Vprev, a.warm, a.flags, smraw);
+  } else if constexpr (PH == PH_SUM_P || PH == PH_SUM_C) {
+    reduce_long<Tc>(a, PH == PH_SUM_C, bid, nb);
+  } else {
+    const RowTiles rt(a.d);
+    if constexpr (PH == PH_ROWS1) phase_rows1<Tc>(a, rt, smraw, bid, nb);
+    else if constexpr (PH == PH_ROWS2) phase_rows2<Tc>(a, rt, smraw, bid, nb);
+    else phase_rows3<Tc>(a, rt, smraw, bid, nb);
+  }
 }
 
 // The Gram refresh of phases 6-7 as two ordinary launches (after (re)initialisation
@@ -1211,6 +1268,71 @@ tdb_status launch_update(UpdArgs& a, int grid_hint, cudaStream_t s) {
 }
 template tdb_status launch_update<float>(UpdArgs&, int, cudaStream_t);
 template tdb_status launch_update<double>(UpdArgs&, int, cudaStream_t);
+
+namespace {
+template <int PH>
+void launch_phase(UpdBatch& B, cudaStream_t s) {
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_update_batch<float, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpdSmem);
+    attr = true;
+  }
+  if (B.base[B.n] == 0) return;
+  k_update_batch<float, PH><<<B.base[B.n], UPD_THREADS, kUpdSmem, s>>>(B);
+  count_launch();
+}
+}  // namespace
+
+void launch_update_batch(const UpdArgs* args, int n, int part, cudaStream_t s) {
+  for (int i0 = 0; i0 < n; i0 += kUpdBatch) {
+    UpdBatch B;
+    B.n = std::min(kUpdBatch, n - i0);
+    bool tree = false, tree_c = false;
+    for (int m = 0; m < B.n; ++m) {
+      B.a[m] = args[i0 + m];
+      for (int k = 0; k < B.a[m].d.p; ++k)
+        if ((B.a[m].d.N[k] + 31) / 32 > kTreeTiles) {
+          tree = true;
+          tree_c |= B.a[m].reorth != 0;
+        }
+    }
+    // a phase's CTAs per member
+    auto count = [&](auto&& of) {
+      B.base[0] = 0;
+      for (int m = 0; m < B.n; ++m) B.base[m + 1] = B.base[m] + (int)std::min<int64_t>(of(B.a[m]), 1 << 16);
+    };
+    auto tiles = [](const UpdArgs& a) {
+      int64_t t = 0;
+      for (int k = 0; k < a.d.p; ++k) t += (a.d.N[k] + 31) / 32;
+      return t;
+    };
+    if (part == 1) {
+      count([](const UpdArgs& a) { return (int64_t)a.d.p; });
+      launch_phase<PH_FINISH>(B, s);
+      continue;
+    }
+    count([&](const UpdArgs& a) { return tiles(a) + (a.ds_y2 ? std::min<int64_t>(update_ds_ctas(prod_r(a.d)), 16) : 0); });
+    launch_phase<PH_ROWS1>(B, s);
+    if (tree) {
+      count([](const UpdArgs& a) { return (int64_t)a.d.p * 8; });
+      launch_phase<PH_SUM_P>(B, s);
+    }
+    count(tiles);
+    launch_phase<PH_ROWS2>(B, s);
+    if (tree_c) {
+      count([](const UpdArgs& a) { return a.reorth ? (int64_t)a.d.p * 8 : (int64_t)0; });
+      launch_phase<PH_SUM_C>(B, s);
+    }
+    count(tiles);
+    launch_phase<PH_ROWS3>(B, s);
+    count([](const UpdArgs& a) { return std::min<int64_t>(prod_r_above(a.d, 1), 16); });
+    launch_phase<PH_CORE12>(B, s);
+    count([](const UpdArgs& a) { return a.d.p > 2 ? std::min<int64_t>((prod_r(a.d) + 1023) / 1024, 16) : (int64_t)0; });
+    launch_phase<PH_CORE34>(B, s);
+    count([](const UpdArgs& a) { return (int64_t)a.d.p * a.gsplit; });
+    launch_phase<PH_GRAMS>(B, s);
+  }
+}
 
 // ---------------------------------------------------------------------------
 // Diagnostics (tdb_selftest_recip, tdb_selftest_timeout): the double reciprocal helpers

@@ -170,6 +170,11 @@ __host__ __device__ inline int64_t update_ds_ctas(int64_t rprod) { return (rprod
 template <typename Tc>
 tdb_status launch_update(UpdArgs& a, int grid_hint, cudaStream_t s);
 
+// The updates of n states of the float compute type, phase by phase over all of them:
+// part 0 = phases 1-6, part 1 = phase 7 (G_n, G_n^{-1}, sigma^(n)).
+constexpr int kUpdBatch = 16;
+void launch_update_batch(const UpdArgs* args, int n, int part, cudaStream_t s);
+
 // k_eig.cu (float compute types)
 void launch_sqrt_weights(const double* w, int n, float* ws, cudaStream_t s);
 void launch_weight_data(const float* V, int p, const int64_t* N, const float* const* ws, int64_t S, float* Vw,

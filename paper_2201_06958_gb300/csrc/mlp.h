@@ -26,11 +26,22 @@ struct EstState {
   double novelty_z;          // exact when a standardised feature leaves [-z, z]
 };
 
-// Features of the current step, the estimate and the gate (one CTA).
-// st_dev: device copy of the estimator state for this step.
-void est_features(const EstState* st_dev, const float* dS, int nds, const double* dv2, const double* sig2,
-                  const int* ranks, int p, const float* P, const float* norm, float* feat, double* est, int* need,
-                  double* ds2, cudaStream_t s);
+// Features of the current step, the estimate and the gate (one CTA a state).
+struct EstArgs {
+  const EstState* st;        // device copy of the estimator state for this step
+  const float* dS;
+  int nds;
+  const double* dv2;
+  const double* sig2;        // of the state the step started from
+  int ranks[4], p;
+  const float* P;
+  const float* norm;
+  float* feat;
+  double* est;
+  int* need;
+  double* ds2;
+};
+void est_features(const EstArgs* args, int n, cudaStream_t s);
 void est_normalize(float* X, float* t, int n, float* norm, cudaStream_t s);
 void est_init_params(float* P, unsigned long long seed, cudaStream_t s);
 

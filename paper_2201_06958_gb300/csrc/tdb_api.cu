@@ -42,32 +42,48 @@ struct Readback {
 // The step's first kernel: clears the step record, fetches the host's gate word and the
 // estimator state from pinned host memory (read through its device mapping), keeps the
 // sigma^2 the step starts from (the estimator's features), and lets the projection that
-// follows start its set-up early (programmatic launch).  One CTA.
-__global__ void k_step_begin(Readback* rb, const int* need_h, const EstState* est_h, EstState* est_d,
-                             const double* sig2, double* sig2_lag, int nsig, unsigned* bar) {
+// follows start its set-up early (programmatic launch).  One CTA a state.
+struct StepArgs {
+  Readback* rb;
+  Readback* rb_host;         // mapped pinned memory
+  const int* need_h;
+  const EstState* est_h;
+  EstState* est_d;
+  const double* sig2;
+  double* sig2_lag;
+  unsigned* bar;             // the updates' grid barriers
+  int nsig;
+};
+constexpr int kStepBatch = 32;
+struct StepBatch {
+  StepArgs a[kStepBatch];
+};
+__global__ void k_step_begin(const __grid_constant__ StepBatch B) {
+  const StepArgs& a = B.a[blockIdx.x];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  unsigned* w = (unsigned*)rb;
+  unsigned* w = (unsigned*)a.rb;
   for (int i = threadIdx.x; i < (int)(sizeof(Readback) / 4); i += blockDim.x) w[i] = 0u;
-  const unsigned* es = (const unsigned*)est_h;
-  unsigned* ed = (unsigned*)est_d;
+  const unsigned* es = (const unsigned*)a.est_h;
+  unsigned* ed = (unsigned*)a.est_d;
   for (int i = threadIdx.x; i < (int)(sizeof(EstState) / 4); i += blockDim.x) ed[i] = es[i];
-  for (int i = threadIdx.x; i < nsig; i += blockDim.x) sig2_lag[i] = sig2[i];
+  for (int i = threadIdx.x; i < a.nsig; i += blockDim.x) a.sig2_lag[i] = a.sig2[i];
   __syncthreads();
-  if (threadIdx.x == 0) rb->need = *(volatile const int*)need_h;
-  if (threadIdx.x < 2) bar[threadIdx.x] = 0u;          // the updates' grid barriers
+  if (threadIdx.x == 0) a.rb->need = *(volatile const int*)a.need_h;
+  if (threadIdx.x < 2) a.bar[threadIdx.x] = 0u;
 }
 
 // The step's last kernel: sigma^2 into the step record, and the record to pinned host memory
-// through its device mapping (one launch instead of two copies, ~5 us a step).  One CTA.
-__global__ void k_step_end(Readback* rb, const double* sig2, int nsig, Readback* host) {
-  const unsigned long long* src = (const unsigned long long*)rb;
-  unsigned long long* dst = (unsigned long long*)host;
+// through its device mapping (one launch instead of two copies, ~5 us a step).  One CTA a state.
+__global__ void k_step_end(const __grid_constant__ StepBatch B) {
+  const StepArgs& a = B.a[blockIdx.x];
+  const unsigned long long* src = (const unsigned long long*)a.rb;
+  unsigned long long* dst = (unsigned long long*)a.rb_host;
   const int first = (int)(offsetof(Readback, sig2) / 8);
   for (int i = threadIdx.x; i < (int)(sizeof(Readback) / 8); i += blockDim.x) {
     unsigned long long v = src[i];
-    if (i >= first && i - first < nsig) {
-      v = (unsigned long long)__double_as_longlong(sig2[i - first]);
-      ((unsigned long long*)rb)[i] = v;
+    if (i >= first && i - first < a.nsig) {
+      v = (unsigned long long)__double_as_longlong(a.sig2[i - first]);
+      ((unsigned long long*)a.rb)[i] = v;
     }
     dst[i] = v;
   }
@@ -244,6 +260,7 @@ struct tdb_batch {
   std::vector<tdb_ctx*> m;
   cudaStream_t main = nullptr;       // the caller's stream: graphs are launched here
   cudaStream_t cap = nullptr;        // private origin stream of the recording
+  std::vector<cudaStream_t> aux;     // G_n refreshes beside the errors, one a group
   std::vector<cudaStream_t> st;
   cudaEvent_t fork = nullptr;
   std::vector<cudaEvent_t> join;
@@ -261,6 +278,7 @@ struct tdb_batch {
     if (fork) cudaEventDestroy(fork);
     for (auto q : st) cudaStreamDestroy(q);
     if (cap) cudaStreamDestroy(cap);
+    for (auto q : aux) cudaStreamDestroy(q);
   }
 };
 
@@ -677,12 +695,36 @@ tdb_status refresh_derived(tdb_ctx* ctx, bool bases_too, const double* src = nul
   return TDB_OK;
 }
 
+StepArgs step_args(const tdb_ctx* ctx) {
+  StepArgs a;
+  a.rb = ctx->rb_dev;
+  a.rb_host = ctx->rb_pin_d;
+  a.need_h = ctx->need_pin_d;
+  a.est_h = ctx->est_pin_d;
+  a.est_d = ctx->est_dev;
+  a.sig2 = ctx->sig2;
+  a.sig2_lag = ctx->sig2_lag;
+  a.bar = ctx->bar;
+  a.nsig = ctx->p * kMaxRank;
+  return a;
+}
+// The opening (open) or closing kernel of the steps of n contexts.
+void launch_steps(tdb_ctx* const* c, int n, bool open, cudaStream_t s) {
+  for (int i0 = 0; i0 < n; i0 += kStepBatch) {
+    StepBatch B;
+    const int m = std::min(kStepBatch, n - i0);
+    for (int i = 0; i < m; ++i) B.a[i] = step_args(c[i0 + i]);
+    if (open) k_step_begin<<<m, 256, 0, s>>>(B);
+    else k_step_end<<<m, 160, 0, s>>>(B);
+    count_launch();
+  }
+}
+
 // The step record: sigma^2 into the record, then the record to pinned host memory.
 tdb_status readback_enqueue(tdb_ctx* ctx) {
   cudaStream_t s = ctx->stream;
   if (ctx->rb_pin_d) {
-    k_step_end<<<1, 160, 0, s>>>(ctx->rb_dev, ctx->sig2, ctx->p * kMaxRank, ctx->rb_pin_d);
-    count_launch();
+    launch_steps(&ctx, 1, false, s);
     CHECK_LAUNCH();
     return TDB_OK;
   }
@@ -1038,14 +1080,11 @@ void prepare_step(tdb_ctx* ctx) {
 // the current state; with the state of step k kept in Tbak / Ubak, 1 = Heun's second stage
 // (the mean of y_k and the predicted state plus the increment), 2 = the midpoint scheme's
 // second stage (y_k plus the increment taken at the midpoint state).
-template <typename Tc>
-tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine, int stage) {
+UpdArgs update_args(const tdb_ctx* ctx, bool reorth, bool skip_finish, int combine, int stage) {
   const int p = ctx->p;
   UpdArgs a;
   memset(&a, 0, sizeof(a));
   a.d = mode_desc(ctx);
-  int64_t Rprod = 1, ntiles = 0;
-  for (int n = 0; n < p; ++n) Rprod *= ctx->r[n];
   for (int n = 0; n < p; ++n) {
     a.Y[n] = ctx->Y[n];
     a.U[n] = ctx->U[n];
@@ -1055,7 +1094,6 @@ tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine
     a.A[n] = ctx->A[n];
     a.Uc[n] = ctx->Uc[n];
     a.U0[n] = combine ? ctx->Ubak[n] : nullptr;
-    ntiles += (ctx->N[n] + 31) / 32;
   }
   a.dS = ctx->dS;
   // the fused projections leave dS to phase 1
@@ -1084,6 +1122,18 @@ tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine
   a.bar = ctx->bar + stage;          // (both words zeroed when the step begins)
   a.stamps = ctx->prof ? ctx->stamps : nullptr;
   a.flags = ctx->flags;
+  return a;
+}
+
+template <typename Tc>
+tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine, int stage) {
+  UpdArgs a = update_args(ctx, reorth, skip_finish, combine, stage);
+  const int p = ctx->p;
+  int64_t Rprod = 1, ntiles = 0;
+  for (int n = 0; n < p; ++n) {
+    Rprod *= ctx->r[n];
+    ntiles += (ctx->N[n] + 31) / 32;
+  }
   // a few more CTAs take dS beside the rows (2 us of phase 1 at 1408 elements); more than 16
   // would cost the barriers, and other members of a batch their SMs, more than that gives
   const int64_t dsc = a.ds_y2 && update_ds_ctas(Rprod) <= 16 ? update_ds_ctas(Rprod) : 0;
@@ -1095,6 +1145,51 @@ tdb_status fused_update(tdb_ctx* ctx, bool reorth, bool skip_finish, int combine
   }
   CHECK_LAUNCH();
   return TDB_OK;
+}
+
+// a1 + a2: the difference scale (Vn - Vfrom) and its projection onto the current bases
+template <typename Tc>
+tdb_status project_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vfrom, double scale, cudaEvent_t* evm, bool after_begin) {
+  cudaStream_t s = ctx->stream;
+  const int p = ctx->p;
+  if (ctx->use_tc) {
+    TRY(tc_project(ctx->tc, (const float*)Vn, (const float*)Vfrom, ctx->p, ctx->N, ctx->r,
+                   (const void* const*)ctx->A, (const double* const*)ctx->w, (float*)ctx->ping, (float*)ctx->pong,
+                   (float*)ctx->dV, (float*)ctx->dS, (float* const*)ctx->Y, &ctx->rb_dev->dv2, ctx->flags, s, evm,
+                   ctx->err, true, (float)scale, after_begin));
+  } else if (sp_route(ctx)) {
+    TRY(sp_project<Tc>(ctx->sp, Vn, Vfrom, p, ctx->N, ctx->r, (const void* const*)ctx->A,
+                       (const double* const*)ctx->w, (Tc*)ctx->ping, (Tc* const*)ctx->Y, &ctx->rb_dev->dv2,
+                       ctx->flags, s, evm, ctx->err, (Tc)scale));
+  } else {
+    launch_diff_norm<Tc>(Vn, Vfrom, (Tc*)ctx->dV, (int)ctx->N[0], ctx->S / ctx->N[0], (Tc)scale,
+                         (const Tc*)ctx->w1T, (const Tc*)ctx->wcolT, ctx->npart, ctx->redcnt + 1, ctx->nblk,
+                         &ctx->rb_dev->dv2, ctx->flags, s);
+    CHECK_LAUNCH();
+    TRY(project_tree<Tc>(ctx, (const Tc*)ctx->dV, evm));
+  }
+  return TDB_OK;
+}
+
+// The estimator's features of a float context.  Its gate decides the error evaluation only in
+// TDB_ERRMODE_MLP; otherwise its decision goes to a scratch word and the host's schedule stands.
+EstArgs feature_args(const tdb_ctx* ctx) {
+  EstArgs a;
+  a.st = ctx->est_dev;
+  a.dS = (const float*)ctx->dS;
+  a.nds = 1;
+  for (int n = 0; n < ctx->p; ++n) a.nds *= ctx->r[n];
+  a.dv2 = &ctx->rb_dev->dv2;
+  a.sig2 = ctx->sig2_lag;
+  for (int n = 0; n < kMaxModes; ++n) a.ranks[n] = n < ctx->p ? ctx->r[n] : 1;
+  a.p = ctx->p;
+  a.P = ctx->mlpP;
+  a.norm = ctx->mlpNorm;
+  a.feat = ctx->rb_dev->feat;
+  a.est = &ctx->rb_dev->est;
+  a.need = ctx->cfg.error_mode == TDB_ERRMODE_MLP ? &ctx->rb_dev->need : ctx->need_scratch;
+  a.ds2 = &ctx->rb_dev->ds2;
+  return a;
 }
 
 // Vpp: the snapshot before Vp (central differences of TDB_RK2_CENTRAL), or null.
@@ -1118,9 +1213,7 @@ tdb_status enqueue_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vp, bool all_paths
   if (ev) CK(record_timing_event(ev[0], s));
   ctx->main_from_start = pdl;        // the projection's start event is the step's (ev[0])
   if (begin_kernel) {
-    k_step_begin<<<1, 256, 0, s>>>(ctx->rb_dev, ctx->need_pin_d, ctx->est_pin_d, ctx->est_dev, ctx->sig2,
-                                   ctx->sig2_lag, p * kMaxRank, ctx->bar);
-    count_launch();
+    launch_steps(&ctx, 1, true, s);
   } else {
     CK(cudaMemsetAsync(ctx->rb_dev, 0, sizeof(Readback), s));
     CK(cudaMemcpyAsync(&ctx->rb_dev->need, ctx->need_pin, sizeof(int), cudaMemcpyHostToDevice, s));
@@ -1130,25 +1223,8 @@ tdb_status enqueue_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vp, bool all_paths
   }
   int64_t Rprod = 1;
   for (int n = 0; n < p; ++n) Rprod *= ctx->r[n];
-  // a1 + a2: difference scale (Vn - Vfrom) and its projection onto the current bases
-  auto project = [&](cudaEvent_t* evm, const Tc* Vfrom, double scale, bool after_begin) -> tdb_status {
-    if (ctx->use_tc) {
-      TRY(tc_project(ctx->tc, (const float*)Vn, (const float*)Vfrom, ctx->p, ctx->N, ctx->r,
-                     (const void* const*)ctx->A, (const double* const*)ctx->w, (float*)ctx->ping, (float*)ctx->pong,
-                     (float*)ctx->dV, (float*)ctx->dS, (float* const*)ctx->Y, &ctx->rb_dev->dv2, ctx->flags, s, evm,
-                     ctx->err, true, (float)scale, after_begin));
-    } else if (sp_route(ctx)) {
-      TRY(sp_project<Tc>(ctx->sp, Vn, Vfrom, p, ctx->N, ctx->r, (const void* const*)ctx->A,
-                         (const double* const*)ctx->w, (Tc*)ctx->ping, (Tc* const*)ctx->Y, &ctx->rb_dev->dv2,
-                         ctx->flags, s, evm, ctx->err, (Tc)scale));
-    } else {
-      launch_diff_norm<Tc>(Vn, Vfrom, (Tc*)ctx->dV, (int)ctx->N[0], ctx->S / ctx->N[0], (Tc)scale,
-                           (const Tc*)ctx->w1T, (const Tc*)ctx->wcolT, ctx->npart, ctx->redcnt + 1, ctx->nblk,
-                           &ctx->rb_dev->dv2, ctx->flags, s);
-      CHECK_LAUNCH();
-      TRY(project_tree<Tc>(ctx, (const Tc*)ctx->dV, evm));
-    }
-    return TDB_OK;
+  auto project = [&](cudaEvent_t* evm, const Tc* Vfrom, double scale, bool after_begin) {
+    return project_step<Tc>(ctx, Vn, Vfrom, scale, evm, after_begin);
   };
   if (scheme == TDB_HEUN || scheme == TDB_RK2_CENTRAL) {
     // first stage: keep y_k = (T, U_n), then an Euler increment at y_k gives the
@@ -1171,16 +1247,11 @@ tdb_status enqueue_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vp, bool all_paths
   TRY(fused_update<Tc>(ctx, ctx->cfg.reorth != 0, split,
                        scheme == TDB_HEUN ? 1 : (scheme == TDB_RK2_CENTRAL ? 2 : 0), scheme == TDB_EULER ? 0 : 1));
   if (ev) CK(record_timing_event(ev[2], s));
-  // the estimator's gate decides the error evaluation only in TDB_ERRMODE_MLP; otherwise
-  // its decision goes to a scratch word and the host's schedule stands
   const bool mlp = ctx->cfg.error_mode == TDB_ERRMODE_MLP;
   auto features = [&](cudaStream_t q) {
     if (ctx->f64) return;
-    int64_t nds = 1;
-    for (int n = 0; n < p; ++n) nds *= ctx->r[n];
-    est_features(ctx->est_dev, (const float*)ctx->dS, (int)nds, &ctx->rb_dev->dv2, ctx->sig2_lag, ctx->r, p,
-                 ctx->mlpP, ctx->mlpNorm, ctx->rb_dev->feat, &ctx->rb_dev->est,
-                 mlp ? &ctx->rb_dev->need : ctx->need_scratch, &ctx->rb_dev->ds2, q);
+    const EstArgs ea = feature_args(ctx);
+    est_features(&ea, 1, q);
   };
   // a7: error, exact or estimated (the estimator's features and gate first).  Recorded
   // steps enqueue the error kernels on every step, gated by the device word.
@@ -2084,7 +2155,102 @@ tdb_status tdb_batch_create(tdb_batch** out, tdb_ctx* const* members, int n, int
     delete b;
     return TDB_ERR_CUDA;
   }
+  for (int k = 0; k < ns; ++k) {
+    cudaStream_t q = nullptr;
+    if (cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking) != cudaSuccess) {
+      delete b;
+      return TDB_ERR_CUDA;
+    }
+    b->aux.push_back(q);
+  }
   *out = b;
+  return TDB_OK;
+}
+
+// Whether a member's step can be recorded phase by phase with the others': one Euler stage of
+// the float compute type, not profiled.
+static bool phase_batchable(const tdb_ctx* c) {
+  return !c->f64 && c->cfg.integrator == TDB_EULER && !c->prof && c->rb_pin_d && c->need_pin_d && c->est_pin_d;
+}
+
+// Every member's step into the recording, phase by phase: the members' projections and exact
+// errors side by side on the streams (member i on stream i mod nstreams), and everything
+// between (the opening and closing kernels, the update's phases, the estimator's features, the
+// G_n refresh) in launches over all members of a group.  A member's own cooperative update
+// held up to 54 CTAs of 1024 threads for its 50 us of barriers, and eight streams of ~170 us a
+// member step overlapped less than twofold; the values are those of the member's own step.
+// A group is the members of a run of streams, about kUpdBatch of them, so that the groups'
+// phases fill the SMs beside one another.
+static tdb_status batch_phases(tdb_batch* b, int parity) {
+  const int n = (int)b->m.size(), ns = (int)b->st.size();
+  const int ngroup = std::max(1, std::min(ns, (n + kUpdBatch - 1) / kUpdBatch));
+  cudaEventRecord(b->fork, b->cap);
+  for (int g = 0; g < ngroup; ++g) {
+    const int k0 = ns * g / ngroup, k1 = ns * (g + 1) / ngroup;        // the group's streams
+    std::vector<tdb_ctx*> mem;
+    std::vector<int> at, who;                                          // stream and member index
+    for (int i = 0; i < n; ++i)
+      if (i % ns >= k0 && i % ns < k1) {
+        mem.push_back(b->m[i]);
+        at.push_back(i % ns);
+        who.push_back(i);
+      }
+    cudaStream_t lead = b->st[k0], aux = b->aux[g];
+    cudaStreamWaitEvent(lead, b->fork, 0);
+    auto each = [&](auto&& work) -> tdb_status {
+      cudaEventRecord(b->join[k0], lead);
+      for (int k = k0 + 1; k < k1; ++k) cudaStreamWaitEvent(b->st[k], b->join[k0], 0);
+      for (size_t i = 0; i < mem.size(); ++i) {
+        tdb_ctx* c = mem[i];
+        cudaStream_t own = c->stream;
+        c->stream = b->st[at[i]];
+        const tdb_status st = work(c);
+        c->stream = own;
+        if (st != TDB_OK) {
+          b->err = "member " + std::to_string(who[i]) + ": " + c->err;
+          return st;
+        }
+      }
+      for (int k = k0 + 1; k < k1; ++k) {
+        cudaEventRecord(b->join[k], b->st[k]);
+        cudaStreamWaitEvent(lead, b->join[k], 0);
+      }
+      return TDB_OK;
+    };
+    const int m = (int)mem.size();
+    launch_steps(mem.data(), m, true, lead);
+    tdb_status st = each([&](tdb_ctx* c) {
+      if (c->use_tc) c->tc.span = nullptr;
+      return project_step<float>(c, (const float*)c->slot[parity], (const float*)c->slot[1 - parity], 1.0, nullptr,
+                                 false);
+    });
+    if (st != TDB_OK) return st;
+    std::vector<UpdArgs> ua(m);
+    std::vector<EstArgs> ea(m);
+    for (int i = 0; i < m; ++i) {
+      ua[i] = update_args(mem[i], mem[i]->cfg.reorth != 0, true, 0, 0);
+      ea[i] = feature_args(mem[i]);
+    }
+    launch_update_batch(ua.data(), m, 0, lead);
+    cudaEventRecord(b->join[k0], lead);
+    cudaStreamWaitEvent(aux, b->join[k0], 0);
+    launch_update_batch(ua.data(), m, 1, aux);
+    est_features(ea.data(), m, lead);
+    st = each([&](tdb_ctx* c) {
+      return exact_error2<float>(c, (const float*)c->slot[parity],
+                                 c->cfg.error_mode == TDB_ERRMODE_EXACT ? nullptr : &c->rb_dev->need);
+    });
+    if (st != TDB_OK) return st;
+    cudaEventRecord(b->join[k0], aux);
+    cudaStreamWaitEvent(lead, b->join[k0], 0);
+    launch_steps(mem.data(), m, false, lead);
+    cudaEventRecord(b->join[k0], lead);
+    cudaStreamWaitEvent(b->cap, b->join[k0], 0);
+  }
+  if (cudaGetLastError() != cudaSuccess) {
+    b->err = "batch recording: a launch failed";
+    return TDB_ERR_CUDA;
+  }
   return TDB_OK;
 }
 
@@ -2098,19 +2264,25 @@ static tdb_status batch_capture(tdb_batch* b, int parity) {
   }
   tdb_status st = TDB_OK;
   const long long l0 = launches_so_far();
-  cudaEventRecord(b->fork, b->cap);
-  for (size_t k = 0; k < b->st.size(); ++k) cudaStreamWaitEvent(b->st[k], b->fork, 0);
-  for (size_t i = 0; i < b->m.size() && st == TDB_OK; ++i) {
-    tdb_ctx* c = b->m[i];
-    cudaStream_t own = c->stream;
-    c->stream = b->st[i % b->st.size()];
-    st = enqueue_any(c, parity);
-    c->stream = own;
-    if (st != TDB_OK) b->err = "member " + std::to_string(i) + ": " + c->err;
-  }
-  for (size_t k = 0; k < b->st.size(); ++k) {
-    cudaEventRecord(b->join[k], b->st[k]);
-    cudaStreamWaitEvent(b->cap, b->join[k], 0);
+  bool phases = b->m.size() > 1;
+  for (tdb_ctx* c : b->m) phases = phases && phase_batchable(c);
+  if (phases) {
+    st = batch_phases(b, parity);
+  } else {
+    cudaEventRecord(b->fork, b->cap);
+    for (size_t k = 0; k < b->st.size(); ++k) cudaStreamWaitEvent(b->st[k], b->fork, 0);
+    for (size_t i = 0; i < b->m.size() && st == TDB_OK; ++i) {
+      tdb_ctx* c = b->m[i];
+      cudaStream_t own = c->stream;
+      c->stream = b->st[i % b->st.size()];
+      st = enqueue_any(c, parity);
+      c->stream = own;
+      if (st != TDB_OK) b->err = "member " + std::to_string(i) + ": " + c->err;
+    }
+    for (size_t k = 0; k < b->st.size(); ++k) {
+      cudaEventRecord(b->join[k], b->st[k]);
+      cudaStreamWaitEvent(b->cap, b->join[k], 0);
+    }
   }
   b->gcount[parity] = launches_so_far() - l0;
   count_launch(-(int)b->gcount[parity]);
