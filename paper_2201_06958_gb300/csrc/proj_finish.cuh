@@ -64,19 +64,97 @@ struct __align__(16) Quad {
   T x, y, z, w;
 };
 
-// NQ: tiles along the contracted mode, rounded up to a power of two (<= FS_NQ_MAX).  Double
-// keeps a quarter of the outputs and half of the slices of float in registers at a time
-// (two CTAs per SM within 128 registers a thread).
-template <typename T, int NQ>
+// acc[0 .. 3] += b z; float as two pairs of multiply-adds (one issue slot each).
+__device__ __forceinline__ void fma4(double (&acc)[4], const Quad<double>& b, double z) {
+  acc[0] = fma(b.x, z, acc[0]);
+  acc[1] = fma(b.y, z, acc[1]);
+  acc[2] = fma(b.z, z, acc[2]);
+  acc[3] = fma(b.w, z, acc[3]);
+}
+__device__ __forceinline__ void fma4(float (&acc)[4], const Quad<float>& b, float z) {
+  const float2 zz = make_float2(z, z);
+  const float2 lo = __ffma2_rn(make_float2(b.x, b.y), zz, make_float2(acc[0], acc[1]));
+  const float2 hi = __ffma2_rn(make_float2(b.z, b.w), zz, make_float2(acc[2], acc[3]));
+  acc[0] = lo.x;
+  acc[1] = lo.y;
+  acc[2] = hi.x;
+  acc[3] = hi.y;
+}
+
+// W[a1, b, s] = sum_i2 Z1[i2, a1, s] A2[i2, b] of a finish CTA's whole columns a1 = a1_lo + al
+// (al < na) and sc staged slices: eight lanes share a tile of TU slices x 8 / TU columns b, each
+// taking every eighth run of VEC values of i2 (the lanes' runs are neighbours: no bank
+// conflicts), and a transposing butterfly leaves one sum to each lane.
+template <typename T, int VEC, int TU>
+__device__ __forceinline__ void finish_w(const FinArgs<T>& f, const T* zs, const T* a2s, int a2st, int na, int a1_lo,
+                                         int s0, int sc) {
+  constexpr int TB = 8 / TU;
+  const int kp = threadIdx.x & 7, nbg = (f.r2 + TB - 1) / TB, nug = (sc + TU - 1) / TU;
+  const int ntile = nbg * nug * na;
+  for (int t0 = 4 * (threadIdx.x >> 5); t0 < ntile; t0 += FS_TE / 8) {      // four tiles a warp
+    const int mine = t0 + ((threadIdx.x >> 3) & 3), tile = min(mine, ntile - 1);
+    const int bg = tile % nbg, rest = tile / nbg, ug = rest % nug, al = rest / nug;
+    const T* zc = zs + TU * ug * FS_TE + al * f.N2;
+    T w[8];                                                // [b][u]
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = T(0);
+    for (int i2 = VEC * kp; i2 < f.N2; i2 += 8 * VEC) {
+      if constexpr (VEC == 4) {
+        Quad<T> z[TU];
+#pragma unroll
+        for (int u = 0; u < TU; ++u) z[u] = *reinterpret_cast<const Quad<T>*>(zc + u * FS_TE + i2);
+#pragma unroll
+        for (int b = 0; b < TB; ++b) {
+          const Quad<T> x = *reinterpret_cast<const Quad<T>*>(a2s + a2st * min(TB * bg + b, f.r2 - 1) + i2);
+#pragma unroll
+          for (int u = 0; u < TU; ++u)
+            w[TU * b + u] = fma(z[u].x, x.x, fma(z[u].y, x.y, fma(z[u].z, x.z, fma(z[u].w, x.w, w[TU * b + u]))));
+        }
+      } else {
+        T z[TU];
+#pragma unroll
+        for (int u = 0; u < TU; ++u) z[u] = zc[u * FS_TE + i2];
+#pragma unroll
+        for (int b = 0; b < TB; ++b) {
+          const T x = a2s[a2st * min(TB * bg + b, f.r2 - 1) + i2];
+#pragma unroll
+          for (int u = 0; u < TU; ++u) w[TU * b + u] = fma(z[u], x, w[TU * b + u]);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const bool up = kp & o;
+#pragma unroll
+      for (int i = 0; i < o; ++i) {
+        const T keep = up ? w[i + o] : w[i], send = up ? w[i] : w[i + o];
+        w[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
+    const int u = TU * ug + kp % TU, b = TB * bg + kp / TU, a = a1_lo + al;
+    if (mine < ntile && u < sc && b < f.r2 && a < f.r1)
+      f.W[a + (int64_t)f.r1 * (b + (int64_t)f.r2 * (s0 + u))] = w[0];
+  }
+}
+
+// NQ: tiles along the contracted mode, rounded up to a power of two (<= FS_NQ_MAX); JB:
+// outputs j at a time (float 8, 16, 32 or 64, the least that holds all J, with fewer slices at
+// 64; double 8, and half of the slices: two CTAs per SM within 128 registers a thread).
+// Bound: latency of the partials, chunk after chunk.  256 x 128 x 512 at ranks (11, 8, 16) 13.6
+// us cold (19.9 with 32 outputs tested in groups of four, chunks of 16 and 7 slices and a
+// thread per W output), 256 x 128 x 24 x 20 at (13, 3, 15, 3), 45 outputs, 22 us (27: the partials read
+// once per 32 outputs), 126^3 double 31.8 us (33.2).
+template <typename T, int NQ, int JB>
 __global__ void __launch_bounds__(FS_TE, 2) k_finish_sk(FinArgs<T> f) {
   constexpr int WIDE = sizeof(T) / 4;                                       // 1 float, 2 double
-  constexpr int FS_JB = 32 / (WIDE * WIDE);                                 // outputs j at a time
-  constexpr int SC = (NQ <= 2 ? FS_SC : (NQ == 4 ? FS_SC / 2 : FS_SC / 4)) / WIDE;   // slices per chunk
-  constexpr int BPT = (SC * FS_JMAX + FS_TE - 1) / FS_TE;   // B values a thread stages per chunk
+  constexpr int SC0 = (NQ <= 2 ? FS_SC : (NQ == 4 ? FS_SC / 2 : FS_SC / 4)) / WIDE;
+  constexpr int SC = JB == 64 && SC0 > FS_SC / 2 ? FS_SC / 2 : SC0;         // slices per chunk
+  constexpr bool ONE = sizeof(T) == 4 && JB <= 32;          // J <= JB: one pass over j
+  constexpr int BPT = (SC * (ONE ? JB : FS_JMAX) + FS_TE - 1) / FS_TE;   // B values a thread stages per chunk
   extern __shared__ __align__(16) unsigned char fs_raw[];
   T* fs_sm = (T*)fs_raw;                            // B rows of a slice chunk: [FS_SC][Jp]
   __shared__ double dsh[32];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x;
   if (tid == 0) fin_dep_launch();
   const int tile = blockIdx.x / f.nsplit, sp = blockIdx.x % f.nsplit;
   const bool first = tile < f.nt1;
@@ -146,13 +224,16 @@ __global__ void __launch_bounds__(FS_TE, 2) k_finish_sk(FinArgs<T> f) {
       f.Y1[ee + ne * (int64_t)j] = v;
     }
   };
-  for (int j0 = 0; j0 < J; j0 += FS_JB) {
-    const int jn = min(FS_JB, J - j0);
-    T acc[FS_JB];
+  // chunks of equal length (at most SC slices)
+  const int nch = (s_hi - s_lo + SC - 1) / SC;
+  for (int j0 = 0; j0 < (ONE ? 1 : J); j0 += JB) {
+    const int jn = min(JB, J - j0);
+    T acc[JB / 4][4];
 #pragma unroll
-    for (int t = 0; t < FS_JB; ++t) acc[t] = T(0);
-    for (int s0 = s_lo; s0 < s_hi; s0 += SC) {
-      const int sc = min(SC, s_hi - s0);
+    for (int t = 0; t < JB; ++t) acc[t / 4][t % 4] = T(0);
+    for (int ch = 0; ch < nch; ++ch) {
+      const int s0 = s_lo + (s_hi - s_lo) * ch / nch;
+      const int sc = s_lo + (s_hi - s_lo) * (ch + 1) / nch - s0;
       // this element's slice values summed over q: every load of the chunk is issued
       // into registers before the first addition
       T raw[SC * NQ];
@@ -214,86 +295,29 @@ __global__ void __launch_bounds__(FS_TE, 2) k_finish_sk(FinArgs<T> f) {
       }
       __syncthreads();
       if (fw && j0 == 0) {
-        // W[a1, a2, s] = sum_i2 Z1[i2, a1, s] A2[i2, a2] for this CTA's whole columns a1: a
-        // warp per (a1, eight a2, four slices); lane (b, phase) sums i2 = phase (mod 4) for
-        // the four slices side by side, then the four phases are added by shuffles
-        if ((f.N2 & 3) == 0) {
-          // whole float4 runs of i2: a thread per output (a1, slice, a2), a2 fastest, two
-          // chains (even and odd runs) added at the end
-          const int nout = na * sc * f.r2;
-          for (int o = tid; o < nout; o += FS_TE) {
-            const int b = o % f.r2, rest = o / f.r2, u = rest % sc, al = rest / sc;
-            const Quad<T>* zc = reinterpret_cast<const Quad<T>*>(zs + u * FS_TE + al * f.N2);
-            const Quad<T>* ac = reinterpret_cast<const Quad<T>*>(a2s + a2st * b);
-            T w0 = T(0), w1 = T(0);
-            const int nq4 = f.N2 >> 2;
-            int q = 0;
-#pragma unroll 2
-            for (; q + 1 < nq4; q += 2) {
-              const Quad<T> z0 = zc[q], a0 = ac[q], z1 = zc[q + 1], a1v = ac[q + 1];
-              w0 = fma(z0.x, a0.x, w0); w0 = fma(z0.y, a0.y, w0); w0 = fma(z0.z, a0.z, w0); w0 = fma(z0.w, a0.w, w0);
-              w1 = fma(z1.x, a1v.x, w1); w1 = fma(z1.y, a1v.y, w1); w1 = fma(z1.z, a1v.z, w1); w1 = fma(z1.w, a1v.w, w1);
-            }
-            if (q < nq4) {
-              const Quad<T> z0 = zc[q], a0 = ac[q];
-              w0 = fma(z0.x, a0.x, w0); w0 = fma(z0.y, a0.y, w0); w0 = fma(z0.z, a0.z, w0); w0 = fma(z0.w, a0.w, w0);
-            }
-            const int a1 = a1_lo + al;
-            if (a1 < f.r1) f.W[a1 + (int64_t)f.r1 * (b + (int64_t)f.r2 * (s0 + u))] = w0 + w1;
-          }
-        } else {
-          const int nbg = (f.r2 + 7) >> 3, nug = (sc + 3) >> 2;
-          const int nitem = na * nbg * nug;
-          const int bl = lane & 7, ph = lane >> 3;
-          for (int item = warp; item < nitem; item += FS_TE / 32) {
-            const int bg = item % nbg, rest = item / nbg, al = rest % na, u0 = 4 * (rest / na);
-            const int b = bg * 8 + bl;
-            const T* zc = zs + u0 * FS_TE + al * f.N2;
-            const T* ac = a2s + a2st * (b < f.r2 ? b : f.r2 - 1);
-            T w[4] = {T(0), T(0), T(0), T(0)};
-#pragma unroll 4
-            for (int i2 = ph; i2 < f.N2; i2 += 4) {
-              const T av = ac[i2];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) w[u] = fma(zc[u * FS_TE + i2], av, w[u]);
-            }
-            const int a1 = a1_lo + al;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              T x = w[u];
-              x += __shfl_xor_sync(0xffffffffu, x, 8);
-              x += __shfl_xor_sync(0xffffffffu, x, 16);
-              if (ph == 0 && b < f.r2 && a1 < f.r1 && u0 + u < sc)
-                f.W[a1 + (int64_t)f.r1 * (b + (int64_t)f.r2 * (s0 + u0 + u))] = x;
-            }
-          }
-        }
+        constexpr int TU = SC < 4 ? SC : 4;
+        if ((f.N2 & 3) == 0) finish_w<T, 4, TU>(f, zs, a2s, a2st, na, a1_lo, s0, sc);
+        else finish_w<T, 1, TU>(f, zs, a2s, a2st, na, a1_lo, s0, sc);
       }
 #pragma unroll
       for (int u = 0; u < SC; ++u) {
+        if (u >= sc) break;
         const T* brow = fs_sm + u * Jp + j0;
 #pragma unroll
-        for (int t4 = 0; t4 < FS_JB / 4; ++t4) {
-          if (4 * t4 < jn) {
-            const Quad<T> bb = *reinterpret_cast<const Quad<T>*>(brow + 4 * t4);
-            acc[4 * t4] = fma(bb.x, z[u], acc[4 * t4]);
-            acc[4 * t4 + 1] = fma(bb.y, z[u], acc[4 * t4 + 1]);
-            acc[4 * t4 + 2] = fma(bb.z, z[u], acc[4 * t4 + 2]);
-            acc[4 * t4 + 3] = fma(bb.w, z[u], acc[4 * t4 + 3]);
-          }
-        }
+        for (int t4 = 0; t4 < JB / 4; ++t4)
+          if (4 * t4 < jn) fma4(acc[t4], *reinterpret_cast<const Quad<T>*>(brow + 4 * t4), z[u]);
       }
     }
     if (f.nsplit == 1) {
       if (in) {
 #pragma unroll
-        for (int t = 0; t < FS_JB; ++t)
-          if (t < jn) store(e, j0 + t, acc[t]);
+        for (int t = 0; t < JB; ++t)
+          if (t < jn) store(e, j0 + t, acc[t / 4][t % 4]);
       }
     } else {
 #pragma unroll
-      for (int t = 0; t < FS_JB; ++t)
-        if (t < jn) mine[(int64_t)(j0 + t) * FS_TE + tid] = acc[t];
+      for (int t = 0; t < JB; ++t)
+        if (t < jn) mine[(int64_t)(j0 + t) * FS_TE + tid] = acc[t / 4][t % 4];
     }
   }
 }
@@ -462,15 +486,6 @@ struct Finish {
     f.npart = npart;
     f.dv2 = dv2;
     smem = sizeof(T) * (FS_SC * ((J + 3) & ~3) + (fuse_w ? FS_SC * FS_TE + (size_t)a2_stride(N2) * r[1] : 0));
-    static bool attr = false;
-    if (smem > 48 * 1024 && !attr) {
-      const int lim = sizeof(T) * (FS_SC * FS_JMAX + FS_SC * FS_TE + a2_stride(FS_TE) * kMaxRank);
-      cudaFuncSetAttribute(k_finish_sk<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      cudaFuncSetAttribute(k_finish_sk<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      cudaFuncSetAttribute(k_finish_sk<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      cudaFuncSetAttribute(k_finish_sk<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      attr = true;
-    }
   }
 
   // A split takes at least 16 slices in float and 4 in double, whose arithmetic (64 cycles per
@@ -504,13 +519,29 @@ struct Finish {
     count_launch();
   }
 
+  template <int JB>
+  void launch_sk(int grid) {
+    auto go = [&](auto kern) {
+      if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      launch_pdl(kern, grid, smem);
+    };
+    if (nqm <= 1) go(k_finish_sk<T, 1, JB>);
+    else if (nqm <= 2) go(k_finish_sk<T, 2, JB>);
+    else if (nqm <= 4) go(k_finish_sk<T, 4, JB>);
+    else go(k_finish_sk<T, 8, JB>);
+  }
+
   void launch(int nsplit) {
     f.nsplit = nsplit;
     const int grid = (nt1 + nt2) * nsplit;
-    if (nqm <= 1) launch_pdl(k_finish_sk<T, 1>, grid, smem);
-    else if (nqm <= 2) launch_pdl(k_finish_sk<T, 2>, grid, smem);
-    else if (nqm <= 4) launch_pdl(k_finish_sk<T, 4>, grid, smem);
-    else launch_pdl(k_finish_sk<T, 8>, grid, smem);
+    if constexpr (sizeof(T) == 4) {
+      if (J <= 8) launch_sk<8>(grid);
+      else if (J <= 16) launch_sk<16>(grid);
+      else if (J <= 32) launch_sk<32>(grid);
+      else launch_sk<64>(grid);
+    } else {
+      launch_sk<8>(grid);
+    }
     if (nsplit > 1) {
       const int64_t outs = (int64_t)(nt1 + nt2) * J * FS_TE;
       launch_pdl(k_finish_red<T>, (int)std::min<int64_t>((outs + 255) / 256, 152 * 16), 0);
