@@ -142,7 +142,7 @@ __device__ __forceinline__ void finish_w(const FinArgs<T>& f, const T* zs, const
 // 64; double 8, and half of the slices: two CTAs per SM within 128 registers a thread).
 // Bound: latency of the partials, chunk after chunk.  256 x 128 x 512 at ranks (11, 8, 16) 13.6
 // us cold (19.9 with 32 outputs tested in groups of four, chunks of 16 and 7 slices and a
-// thread per W output), 256 x 128 x 24 x 20 at (13, 3, 15, 3), 45 outputs, 22 us (27: the partials read
+// thread per W output), 192 x 129 x 192 x 3 at (13, 3, 15, 3), 45 outputs, 22 us (27: the partials read
 // once per 32 outputs), 126^3 double 31.8 us (33.2).
 template <typename T, int NQ, int JB>
 __global__ void __launch_bounds__(FS_TE, 2) k_finish_sk(FinArgs<T> f) {

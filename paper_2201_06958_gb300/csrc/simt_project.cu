@@ -6,12 +6,13 @@
 //   Z1 = dV x_1 A_1^T (summed over the tile's i1) and Z2 = dV x_2 A_2^T (over its i2),
 // with ||dV||_W^2 and the finiteness check on the way; proj_finish.cuh contracts the rest.
 //
-// Bound: float by issue (about 80 of 160 issue slots per 128 points are the products at ranks
-// (11, 8); the rest forms the sums over the lanes, the difference and the norm), double by
-// its arithmetic (two lanes per clock and SM).  256 x 128 x 512 float at ranks (11, 8, 16):
-// 58 us, where difference, norm and the mode products that contract S points took 428 us;
-// 126^3 double at (5, 5, 5): 87 us against 251 us.  One CTA of eight warps per SM with the
-// next rows prefetched into registers measured the same as three of four without.
+// Bound: float by latency (12 warps an SM of one group after the other: loads, then products
+// through shared memory), double by its arithmetic (two lanes per clock and SM).  256 x 128 x
+// 512 float at ranks (11, 8, 16): 53 us (58 with the sums of Z1 over the lanes formed by a
+// butterfly of 31 shuffles and nothing fetched ahead), where difference, norm and the mode
+// products that contract S points took 428 us; 126^3 double at (5, 5, 5): 87 us against 251
+// us.  One CTA of eight warps per SM with the next rows prefetched into registers measured the
+// same as three of four without.
 #include "proj_finish.cuh"
 #include "simt_project.h"
 
@@ -55,9 +56,21 @@ struct SpCfg<float> { static constexpr int G = 8; };
 template <>
 struct SpCfg<double> { static constexpr int G = 4; };
 
+// Copies of an A_2 value in shared memory: float reads pairs (a, a) for its paired
+// multiply-adds.  A warp's shared values: the differences of a group (float, rows SP_DLD
+// apart), then its sums of Z2.
+template <typename T>
+constexpr int kSpDup = sizeof(T) == 4 ? 2 : 1;
+constexpr int SP_DLD = SP_T1 + 4;
+template <typename T>
+constexpr int sp_warp_elems(int rb) {
+  return sizeof(T) == 4 && rb * SP_T1 < SpCfg<float>::G * SP_DLD ? SpCfg<float>::G * SP_DLD : rb * SP_T1;
+}
+
 template <typename T, int RB>
 constexpr size_t sp_smem(int ti2) {
-  return sizeof(T) * ((size_t)RB * SP_T1 + (size_t)ti2 * RB + ti2 + (size_t)RB * ti2 + (size_t)SP_WARPS * RB * SP_T1);
+  return sizeof(T) * ((size_t)RB * SP_T1 + (size_t)ti2 * RB * kSpDup<T> + ti2 + (size_t)RB * ti2 +
+                      (size_t)SP_WARPS * sp_warp_elems<T>(RB));
 }
 
 __device__ __forceinline__ unsigned expo_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
@@ -70,9 +83,11 @@ constexpr unsigned kExpInf = sizeof(T) == 4 ? 0x7f800000u : 0x7ff00000u;
 // G rows at a time in registers:
 //   Z2: four i1 x RB accumulators per lane, A_2's row read as a broadcast; the eight warps'
 //       sums are added through shared memory at the end of the slice.
-//   Z1: per group of 32 / G ranks the lane's sums over its four i1 of G rows are added over
-//       the 32 lanes by a transposing butterfly (31 shuffles for 32 sums, lane l ends with
-//       row l % G, rank l / G), and leave through a shared tile.
+//   Z1: float: the group's differences are staged in shared memory and multiplied by A_1 as a
+//       small matrix product, four rows x every fourth rank a lane.  Double: per group of
+//       32 / G ranks the lane's sums over its four i1 of G rows are added over the 32 lanes by
+//       a transposing butterfly (31 shuffles for 32 sums, lane l ends with row l % G, rank
+//       l / G).  Either leaves through a shared tile.
 // Every sum has a fixed order.  Several CTAs of four warps per SM cover the loads of one
 // another (a warp's group is 8 KB).
 template <typename T, int RB>
@@ -81,10 +96,11 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
   extern __shared__ __align__(16) unsigned char sp_raw[];
   const int ti2 = P.ti2;
   T* A1s = (T*)sp_raw;                         // [RB][128]
-  T* A2s = A1s + RB * SP_T1;                   // [ti2][RB]
-  T* Z1s = A2s + ti2 * RB;                     // [RB][ti2]
+  T* A2s = A1s + RB * SP_T1;                   // [ti2][RB], each value kSpDup times
+  T* Z1s = A2s + ti2 * RB * kSpDup<T>;         // [RB][ti2]
   T* Z2s = Z1s + RB * ti2;                     // [4][RB][128]
-  T* w2s = Z2s + SP_WARPS * RB * SP_T1;        // [ti2]
+  constexpr int ZW = sp_warp_elems<T>(RB);     // a warp's part of it
+  T* w2s = Z2s + SP_WARPS * ZW;                // [ti2]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) fin_dep_launch();
   const int nq12 = P.nq1 * P.nq2;
@@ -102,7 +118,9 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
   }
   for (int e = tid; e < RB * ti2; e += SP_THREADS) {
     const int b = e / ti2, x = e % ti2, i = b2 + x;
-    A2s[x * RB + b] = (b < n2 && i < N2) ? P.A2[i + (int64_t)N2 * (r0 + b)] : T(0);
+    const T a = (b < n2 && i < N2) ? P.A2[i + (int64_t)N2 * (r0 + b)] : T(0);
+#pragma unroll
+    for (int u = 0; u < kSpDup<T>; ++u) A2s[(x * RB + b) * kSpDup<T> + u] = a;
   }
   for (int x = tid; x < ti2; x += SP_THREADS) w2s[x] = b2 + x < N2 ? (T)P.w2[b2 + x] : T(0);
   T w1r[4];
@@ -153,6 +171,20 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
       }
     }
   };
+  // The next group's rows into L2 while this one is computed (a group is 12 000 cycles of its
+  // warp): lane l takes 128 bytes of row l / 4 of both snapshots.
+  auto fetch_l2 = [&](int sl, int grp) {
+    constexpr int SEG = SP_T1 * (int)sizeof(T) / 128;        // 128-byte pieces of a row
+#pragma unroll
+    for (int u = lane; u < G * SEG; u += 32) {
+      const int g = u / SEG, i = b1 + (u % SEG) * (128 / (int)sizeof(T)), x = warp * wrows + grp * G + g;
+      if (grp * G + g < wrows && b2 + x < N2 && i < N1) {
+        const int64_t off = ((int64_t)sl * N2 + b2 + x) * N1 + i;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(P.Vn + off));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(P.Vp + off));
+      }
+    }
+  };
   double acc_norm = 0.0;
   bool bad = false;
   for (int sl = s_first; sl < P.nslice; sl += P.cstep) {
@@ -168,6 +200,8 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
       {
         T rn[G][4], rp[G][4];
         load(sl, grp, rn, rp);
+        if (grp + 1 < ngrp) fetch_l2(sl, grp + 1);
+        else if (sl + P.cstep < P.nslice) fetch_l2(sl + P.cstep, 0);
         bool odd = false;                                  // a row sum that is not finite
 #pragma unroll
         for (int g = 0; g < G; ++g) {
@@ -191,54 +225,124 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
 #pragma unroll
       for (int g = 0; g < G; ++g) {
         if (grp * G + g >= wrows) break;
-        const Quad<T>* a2 = reinterpret_cast<const Quad<T>*>(A2s + (x0 + g) * RB);
+        const Quad<T>* a2 = reinterpret_cast<const Quad<T>*>(A2s + (x0 + g) * RB * kSpDup<T>);
+        if constexpr (sizeof(T) == 4) {
+          const float2 d0 = make_float2(d[g][0], d[g][1]), d1 = make_float2(d[g][2], d[g][3]);
 #pragma unroll
-        for (int b4 = 0; b4 < RB / 4; ++b4) {
-          if (4 * b4 >= n2) break;
-          const Quad<T> a = a2[b4];
-          const T av[4] = {a.x, a.y, a.z, a.w};
+          for (int b2x = 0; b2x < RB / 2; ++b2x) {
+            if (b2x % 2 == 0 && 2 * b2x >= n2) break;
+            const Quad<T> a = a2[b2x];
 #pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (sizeof(T) == 4 || 4 * b4 + u < n2)
+            for (int u = 0; u < 2; ++u) {
+              T (&c)[4] = acc2[2 * b2x + u];
+              const float2 aa = u ? make_float2(a.z, a.w) : make_float2(a.x, a.y);
+              const float2 lo = __ffma2_rn(d0, aa, make_float2(c[0], c[1]));
+              const float2 hi = __ffma2_rn(d1, aa, make_float2(c[2], c[3]));
+              c[0] = lo.x; c[1] = lo.y; c[2] = hi.x; c[3] = hi.y;
+            }
+          }
+        } else {
 #pragma unroll
-              for (int j = 0; j < 4; ++j) acc2[4 * b4 + u][j] = fma(d[g][j], av[u], acc2[4 * b4 + u][j]);
+          for (int b4 = 0; b4 < RB / 4; ++b4) {
+            if (4 * b4 >= n2) break;
+            const Quad<T> a = a2[b4];
+            const T av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (4 * b4 + u < n2)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc2[4 * b4 + u][j] = fma(d[g][j], av[u], acc2[4 * b4 + u][j]);
+          }
         }
       }
-      // Z1: AG ranks of mode 1 at a time over the G rows
+      if constexpr (sizeof(T) == 4) {
+        // Z1: a small matrix product.  The group's G x 128 differences are staged for the warp;
+        // lane (kq, rg, ag) sums every fourth run of four i1 for four rows and the ranks ag,
+        // ag + 4, ..., and the four kq lanes' sums are added by a transposing exchange.
+        T* ds = Z2s + warp * ZW;
+        __syncwarp();
 #pragma unroll
-      for (int ag = 0; ag < RB / AG; ++ag) {
-        if (AG * ag >= n1) break;
-        T v[32];
+        for (int g = 0; g < G; ++g)
+          *reinterpret_cast<float4*>(ds + g * SP_DLD + 4 * lane) = make_float4(d[g][0], d[g][1], d[g][2], d[g][3]);
+        __syncwarp();
+        const int kq = lane & 3, rg = (lane >> 2) & 1, ag = lane >> 3;
+        float2 z[RB / 4][4];
 #pragma unroll
-        for (int aa = 0; aa < AG; ++aa) {
-          if (sizeof(T) == 8 && AG * ag + aa >= n1) {
+        for (int t = 0; t < RB / 4; ++t)
 #pragma unroll
-            for (int g = 0; g < G; ++g) v[g + G * aa] = T(0);
-            continue;
+          for (int r = 0; r < 4; ++r) z[t][r] = make_float2(0.f, 0.f);
+#pragma unroll 2
+        for (int q = kq; q < SP_T1 / 4; q += 4) {
+          float4 x[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) x[r] = *reinterpret_cast<const float4*>(ds + (4 * rg + r) * SP_DLD + 4 * q);
+#pragma unroll
+          for (int t = 0; t < RB / 4; ++t) {
+            if (4 * t >= n1) break;
+            const float4 a = *reinterpret_cast<const float4*>(A1s + (ag + 4 * t) * SP_T1 + 4 * q);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              z[t][r] = __ffma2_rn(make_float2(x[r].x, x[r].y), make_float2(a.x, a.y), z[t][r]);
+              z[t][r] = __ffma2_rn(make_float2(x[r].z, x[r].w), make_float2(a.z, a.w), z[t][r]);
+            }
           }
-          const Quad<T> a = *reinterpret_cast<const Quad<T>*>(A1s + (AG * ag + aa) * SP_T1 + 4 * lane);
-#pragma unroll
-          for (int g = 0; g < G; ++g)
-            v[g + G * aa] = fma(d[g][3], a.w, fma(d[g][2], a.z, fma(d[g][1], a.y, d[g][0] * a.x)));
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const bool up = lane & o;
+        for (int t = 0; t < RB / 4; ++t) {
+          if (4 * t >= n1) break;
+          T v[4];
 #pragma unroll
-          for (int i = 0; i < o; ++i) {
-            const T keep = up ? v[i + o] : v[i], send = up ? v[i] : v[i + o];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          for (int r = 0; r < 4; ++r) v[r] = z[t][r].x + z[t][r].y;
+#pragma unroll
+          for (int o = 2; o > 0; o >>= 1) {
+            const bool up = kq & o;
+#pragma unroll
+            for (int i = 0; i < o; ++i) {
+              const T keep = up ? v[i + o] : v[i], send = up ? v[i] : v[i + o];
+              v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
           }
+          const int g = 4 * rg + kq;
+          if (grp * G + g < wrows) Z1s[(ag + 4 * t) * ti2 + x0 + g] = v[0];
         }
-        const int g = lane % G, a = AG * ag + lane / G;
-        if (grp * G + g < wrows) Z1s[a * ti2 + x0 + g] = v[0];
+      } else {
+        // Z1: AG ranks of mode 1 at a time over the G rows
+#pragma unroll
+        for (int ag = 0; ag < RB / AG; ++ag) {
+          if (AG * ag >= n1) break;
+          T v[32];
+#pragma unroll
+          for (int aa = 0; aa < AG; ++aa) {
+            if (AG * ag + aa >= n1) {
+#pragma unroll
+              for (int g = 0; g < G; ++g) v[g + G * aa] = T(0);
+              continue;
+            }
+            const Quad<T> a = *reinterpret_cast<const Quad<T>*>(A1s + (AG * ag + aa) * SP_T1 + 4 * lane);
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+              v[g + G * aa] = fma(d[g][3], a.w, fma(d[g][2], a.z, fma(d[g][1], a.y, d[g][0] * a.x)));
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < o; ++i) {
+              const T keep = up ? v[i + o] : v[i], send = up ? v[i] : v[i + o];
+              v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+          }
+          const int g = lane % G, a = AG * ag + lane / G;
+          if (grp * G + g < wrows) Z1s[a * ti2 + x0 + g] = v[0];
+        }
       }
     }
     if (r0 == 0) acc_norm += P.wsl[sl] * (double)nrm;
     // the slice's partials leave: Z1 as it is, Z2 summed over the warps in order
+    __syncwarp();
 #pragma unroll
     for (int b = 0; b < RB; ++b)
-      *reinterpret_cast<Quad<T>*>(Z2s + ((warp * RB + b) * SP_T1) + 4 * lane) =
+      *reinterpret_cast<Quad<T>*>(Z2s + warp * ZW + b * SP_T1 + 4 * lane) =
           Quad<T>{acc2[b][0], acc2[b][1], acc2[b][2], acc2[b][3]};
     __syncthreads();
     for (int e = tid; e < n1 * ti2; e += SP_THREADS) {
@@ -250,7 +354,7 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
       const int at = vec ? x : 4 * (x & 31) + (x >> 5);
       T s = Z2s[b * SP_T1 + at];
 #pragma unroll
-      for (int w = 1; w < SP_WARPS; ++w) s += Z2s[(w * RB + b) * SP_T1 + at];
+      for (int w = 1; w < SP_WARPS; ++w) s += Z2s[w * ZW + b * SP_T1 + at];
       if (b1 + x < N1) P.Z2p[(((int64_t)q2 * P.nslice + sl) * P.r2 + r0 + b) * N1 + b1 + x] = s * P.dscale;
     }
     __syncthreads();
