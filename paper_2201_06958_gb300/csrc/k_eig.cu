@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(256) k_syrk_partial(const float* __restrict__ 
 // and lo take 192).  Rows of a column live in 16-byte granules, granule g of column k at
 // g ^ (k & 7), so that either loading writes without bank conflicts.  On a diagonal tile the
 // lower left quarter is left out (the finish reads the upper triangle).  Bound: FP32 issue at
-// eight warps per SM.  256 x 128 x 512: the three modes 0.75 ms, with 64 x 64 tiles 1.52 ms.
+// eight warps per SM (paired multiply-adds do not help: 0.82 ms).  256 x 128 x 512: the three
+// modes 0.75 ms, with 64 x 64 tiles 1.52 ms.
 __device__ __forceinline__ void sy_cp4(float* dst, const float* src, bool in) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
                "r"(in ? 4 : 0) : "memory");
@@ -292,22 +293,33 @@ __global__ void __launch_bounds__(256, 1) k_syrk_big(const float* __restrict__ V
     }
 }
 
-// Sum the slices: C64, full n x n.
+// Sum the slices: C64, full n x n, from the entries on and above the diagonal.  32 entries a
+// CTA, eight groups of slices side by side.
 template <int T>                  // the tile size
-__global__ void k_syrk_finish(int64_t Nn, int ntile, int ksplit, const double* __restrict__ part,
-                              double* __restrict__ C64) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < Nn * Nn; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e % Nn, j = e / Nn;
-    const int64_t a = i <= j ? i : j, b = i <= j ? j : i;
-    const int ti = (int)(a / T), tj = (int)(b / T);
-    const int pair = ti * ntile - ti * (ti - 1) / 2 + (tj - ti);
-    int x = (int)(a % T), y = (int)(b % T);
-    if (ti == tj && x > y) { const int t = x; x = y; y = t; }
+__global__ void __launch_bounds__(256) k_syrk_finish(int64_t Nn, int ntile, int ksplit, const double* __restrict__ part,
+                                                     double* __restrict__ C64) {
+  __shared__ double sh[8][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t e0 = blockIdx.x * (int64_t)32; e0 < Nn * Nn; e0 += gridDim.x * (int64_t)32) {
+    const int64_t i = (e0 + lane) % Nn, j = (e0 + lane) / Nn;
+    const bool in = j < Nn && i <= j;
     double s = 0.0;
-    const double* src = part + (int64_t)pair * ksplit * T * T + x + T * y;
+    if (in) {
+      const int ti = (int)(i / T), tj = (int)(j / T);
+      const int pair = ti * ntile - ti * (ti - 1) / 2 + (tj - ti);
+      const double* src = part + (int64_t)pair * ksplit * T * T + i % T + T * (j % T);
 #pragma unroll 8
-    for (int k = 0; k < ksplit; ++k) s += src[(int64_t)k * T * T];
-    C64[e] = s;
+      for (int k = w; k < ksplit; k += 8) s += src[(int64_t)k * T * T];
+    }
+    __syncthreads();
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && in) {
+#pragma unroll
+      for (int v = 1; v < 8; ++v) s += sh[v][lane];
+      C64[i + Nn * j] = s;
+      C64[j + Nn * i] = s;
+    }
   }
 }
 
@@ -357,7 +369,7 @@ size_t gram_part_elems(int64_t Nn, int64_t ncol) {
 void launch_gram_weighted(const float* Vw, int64_t L, int64_t Nn, int64_t Q, double* part, double* C64,
                           cudaStream_t s) {
   const GramSplit g = gram_shape(Nn, L * Q);
-  const int blocks = (int)std::min<int64_t>((Nn * Nn + 255) / 256, 1024);
+  const int blocks = (int)std::min<int64_t>((Nn * Nn + 31) / 32, 152 * 8);
   if (g.tile == SY_T) {
     k_syrk_partial<<<dim3(g.npair, g.ksplit), 256, 0, s>>>(Vw, L, Nn, Q, g.ntile, g.ksplit, part);
     count_launch();

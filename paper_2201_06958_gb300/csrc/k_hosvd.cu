@@ -21,12 +21,19 @@ __device__ __forceinline__ double column_weight(const GramView& g, int64_t c) {
   return wc;
 }
 
+// Bound: issue of the double multiply-adds (64 cycles a warp and sub-partition).  256 threads
+// of 2 x 2 entries, so that four CTAs per SM cover each other's loads and barriers (1024
+// threads of one entry left one CTA per SM: 126^3, one mode, 373 us, now 319); a diagonal tile forms the
+// 528 entries on and above its diagonal only.
+constexpr int WG_T = 256;
 template <typename Tv>
-__global__ void k_wgram_partial(const Tv* __restrict__ V, GramView g, int ntile, int ksplit, double* __restrict__ part) {
+__global__ void __launch_bounds__(WG_T, 4) k_wgram_partial(const Tv* __restrict__ V, const __grid_constant__ GramView g, int ntile, int ksplit,
+                                                           double* __restrict__ part) {
   // blockIdx.x: upper tile pair (ti <= tj), blockIdx.y: column slice
   int t = blockIdx.x, ti = 0;
   while (t >= ntile - ti) { t -= ntile - ti; ++ti; }
   const int tj = ti + t;
+  const bool diag = ti == tj;
   const int64_t i0 = (int64_t)ti * 32, j0 = (int64_t)tj * 32;
   const int64_t ncol = g.L * g.Q;
   const int64_t c0 = ncol * blockIdx.y / ksplit, c1 = ncol * (blockIdx.y + 1) / ksplit;
@@ -34,52 +41,117 @@ __global__ void k_wgram_partial(const Tv* __restrict__ V, GramView g, int ntile,
   __shared__ Tv Bs[32][33];
   __shared__ double wcol[32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  double acc = 0.0;
+  // entries (bx | bx + 16, by | by + 16); on a diagonal tile (bx, by + 16), and of thread
+  // t < 136 (ax, ay) and (ax + 16, ay + 16) with ax <= ay
+  const int bx = threadIdx.x & 15, by = threadIdx.x >> 4;
+  int ay = (int)((sqrtf(8.f * (float)threadIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((ay + 1) * (ay + 2) / 2 <= (int)threadIdx.x) ++ay;
+  while (ay * (ay + 1) / 2 > (int)threadIdx.x) --ay;
+  const int ax = (int)threadIdx.x - ay * (ay + 1) / 2;
+  double acc00 = 0.0, acc01 = 0.0, acc10 = 0.0, acc11 = 0.0;
   const bool ifast = (g.L == 1);
+  // columns fast: this thread's column is cb + tx, kept as (l, q)
+  int64_t l = ifast ? 0 : (c0 + tx) % g.L, q = ifast ? 0 : (c0 + tx) / g.L;
+  const int64_t dl = 32 % g.L, dq = 32 / g.L;
   for (int64_t cb = c0; cb < c1; cb += 32) {
+    Tv va[4], vb[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int ri = ifast ? tx : ty + 8 * u;
+      const int64_t c = cb + (ifast ? ty + 8 * u : tx);
+      const int64_t ia = i0 + ri, ib = j0 + ri;
+      const int64_t at = ifast ? g.Nn * c : l + g.L * g.Nn * q;
+      va[u] = (c < c1 && ia < g.Nn) ? V[at + g.L * ia] : Tv(0);
+      vb[u] = (c < c1 && ib < g.Nn) ? V[at + g.L * ib] : Tv(0);
+    }
+    l += dl;
+    q += dq;
+    if (l >= g.L) { l -= g.L; ++q; }
     if (threadIdx.x < 32) {
-      int64_t c = cb + threadIdx.x;
+      const int64_t c = cb + threadIdx.x;
       wcol[threadIdx.x] = (c < c1) ? column_weight(g, c) : 0.0;
     }
     __syncthreads();
-    // load tiles: element (i, c) with (row, col) = ifast ? (tx, ty) : (ty, tx)
-    {
-      int ri = ifast ? tx : ty, cc = ifast ? ty : tx;
-      int64_t c = cb + cc;
-      Tv va = 0, vb = 0;
-      if (c < c1) {
-        int64_t l = c % g.L, q = c / g.L;
-        int64_t ia = i0 + ri, ib = j0 + ri;
-        if (ia < g.Nn) va = V[l + g.L * (ia + g.Nn * q)];
-        if (ib < g.Nn) vb = V[l + g.L * (ib + g.Nn * q)];
-      }
-      As[ri][cc] = (Tv)((double)va * wcol[cc]);
-      Bs[ri][cc] = vb;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int ri = ifast ? tx : ty + 8 * u, cc = ifast ? ty + 8 * u : tx;
+      As[ri][cc] = (Tv)((double)va[u] * wcol[cc]);
+      Bs[ri][cc] = vb[u];
     }
     __syncthreads();
-    Tv s = 0;
+    if (!diag) {
+      Tv s00 = 0, s01 = 0, s10 = 0, s11 = 0;
 #pragma unroll 8
-    for (int k = 0; k < 32; ++k) s += As[tx][k] * Bs[ty][k];
-    acc += (double)s;
+      for (int k = 0; k < 32; ++k) {
+        const Tv a0 = As[bx][k], a1 = As[bx + 16][k], b0 = Bs[by][k], b1 = Bs[by + 16][k];
+        s00 += a0 * b0;
+        s01 += a0 * b1;
+        s10 += a1 * b0;
+        s11 += a1 * b1;
+      }
+      acc00 += (double)s00;
+      acc01 += (double)s01;
+      acc10 += (double)s10;
+      acc11 += (double)s11;
+    } else {
+      Tv s = 0;
+#pragma unroll 8
+      for (int k = 0; k < 32; ++k) s += As[bx][k] * Bs[by + 16][k];
+      acc01 += (double)s;
+      if (ay < 16) {
+        Tv s00 = 0, s11 = 0;
+#pragma unroll 8
+        for (int k = 0; k < 32; ++k) {
+          s00 += As[ax][k] * Bs[ay][k];
+          s11 += As[ax + 16][k] * Bs[ay + 16][k];
+        }
+        acc00 += (double)s00;
+        acc11 += (double)s11;
+      }
+    }
     __syncthreads();
   }
-  part[((int64_t)blockIdx.x * ksplit + blockIdx.y) * 1024 + tx + 32 * ty] = acc;
+  double* out = part + ((int64_t)blockIdx.x * ksplit + blockIdx.y) * 1024;
+  out[bx + 32 * (by + 16)] = acc01;
+  if (!diag) {
+    out[bx + 32 * by] = acc00;
+    out[bx + 16 + 32 * by] = acc10;
+    out[bx + 16 + 32 * (by + 16)] = acc11;
+  } else if (ay < 16) {
+    out[ax + 32 * ay] = acc00;
+    out[ax + 16 + 32 * (ay + 16)] = acc11;
+  }
 }
 
-__global__ void k_wgram_finish(GramView g, int ntile, int ksplit, const double* __restrict__ part,
-                               double* __restrict__ C64) {
+// The slices' sums, scaled, for the entries on and above the diagonal, and mirrored: 32 entries
+// a CTA, eight groups of slices side by side.
+__global__ void __launch_bounds__(256) k_wgram_finish(GramView g, int ntile, int ksplit, const double* __restrict__ part,
+                                                      double* __restrict__ C64) {
+  __shared__ double sh[8][33];
   const int64_t Nn = g.Nn;
   const double* wn = g.w[g.n];
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < Nn * Nn; e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t i = e % Nn, j = e / Nn;
-    int64_t a = i <= j ? i : j, b = i <= j ? j : i;
-    int ti = (int)(a / 32), tj = (int)(b / 32);
-    int pair = ti * ntile - ti * (ti - 1) / 2 + (tj - ti);
-    int tx = (int)(a % 32), ty = (int)(b % 32);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t e0 = blockIdx.x * (int64_t)32; e0 < Nn * Nn; e0 += gridDim.x * (int64_t)32) {
+    const int64_t i = (e0 + lane) % Nn, j = (e0 + lane) / Nn;
+    const bool in = j < Nn && i <= j;
     double s = 0.0;
-    for (int k = 0; k < ksplit; ++k) s += part[((int64_t)pair * ksplit + k) * 1024 + tx + 32 * ty];
-    s *= sqrt(wn[i] * wn[j]);
-    C64[e] = s;
+    if (in) {
+      const int ti = (int)(i / 32), tj = (int)(j / 32);
+      const int pair = ti * ntile - ti * (ti - 1) / 2 + (tj - ti);
+      const double* src = part + (int64_t)pair * ksplit * 1024 + i % 32 + 32 * (j % 32);
+#pragma unroll 8
+      for (int k = w; k < ksplit; k += 8) s += src[(int64_t)k * 1024];
+    }
+    __syncthreads();
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && in) {
+#pragma unroll
+      for (int v = 1; v < 8; ++v) s += sh[v][lane];
+      s *= sqrt(wn[i] * wn[j]);
+      C64[i + Nn * j] = s;
+      C64[j + Nn * i] = s;
+    }
   }
 }
 
@@ -90,8 +162,8 @@ void launch_wgram(const Tv* V, const GramView& g, double* part, size_t part_cap,
   int64_t ncol = g.L * g.Q;
   int ksplit = (int)std::max<int64_t>(1, std::min<int64_t>((152 * 4 + npair - 1) / npair, (ncol + 255) / 256));
   while ((size_t)npair * ksplit * 1024 > part_cap && ksplit > 1) --ksplit;
-  k_wgram_partial<Tv><<<dim3(npair, ksplit), 1024, 0, s>>>(V, g, ntile, ksplit, part); count_launch();
-  int blocks = (int)std::min<int64_t>((g.Nn * g.Nn + 255) / 256, 1024);
+  k_wgram_partial<Tv><<<dim3(npair, ksplit), WG_T, 0, s>>>(V, g, ntile, ksplit, part); count_launch();
+  const int blocks = (int)std::min<int64_t>((g.Nn * g.Nn + 31) / 32, 152 * 8);
   k_wgram_finish<<<blocks, 256, 0, s>>>(g, ntile, ksplit, part, C64); count_launch();
 }
 template void launch_wgram<double>(const double*, const GramView&, double*, size_t, double*, cudaStream_t);
