@@ -845,6 +845,120 @@ void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* 
 template void launch_recon_out<float>(const float*, const float*, int, int, int64_t, float*, cudaStream_t);
 template void launch_recon_out<double>(const double*, const double*, int, int, int64_t, double*, cudaStream_t);
 
+// H = T x_2 U_2 x_3 U_3 (x_4 U_4) in float, r_1 x N_2 x slices, in one launch: a CTA forms the
+// r_1 x r_2 slice G = sum_j T[:, :, j] c_j, c_j = U_3[i_3, c] U_4[i_4, d] over the J = r_3 r_4
+// pairs, then its block of columns G U_2[i_2, :]^T.  Bound: latency; 256 x 128 x 512 at (11, 8,
+// 16) CC_ONE us against 9.1 in two mode products with the gap between them.
+constexpr int CC_T = 256, CC_JMAX = 1024, CC_NB = 256, CC_PRE = 16;
+struct CoreCols {
+  const float* T;
+  const float* U2;
+  const float* U3;
+  const float* U4;               // null: three modes
+  float* H;
+  int r1, r2, r3, J, N2, N3, N4, nb;         // nb: columns i_2 of a CTA
+};
+__global__ void __launch_bounds__(CC_T) k_core_cols(CoreCols a, const int* __restrict__ gate) {
+  if (gate && *gate == 0) return;
+  extern __shared__ __align__(16) float cc_sm[];
+  const int r12 = a.r1 * a.r2, neg = (r12 + 31) >> 5;       // groups of 32 entries of G
+  float* cj = cc_sm;                                       // J
+  float* G = cj + a.J;                                     // r12
+  float* U2s = G + r12;                                    // r2 x nb
+  float* red = U2s + a.r2 * a.nb;                          // groups of j x 32 neg
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int s = blockIdx.x, i3 = s % a.N3, i4 = s / a.N3;
+  const int lo = blockIdx.y * a.nb, nc = min(a.nb, a.N2 - lo);
+  for (int j = t; j < a.J; j += CC_T) {
+    const float c = __ldg(&a.U3[i3 + a.N3 * (j % a.r3)]);
+    cj[j] = a.U4 ? c * __ldg(&a.U4[i4 + a.N4 * (j / a.r3)]) : c;
+  }
+  for (int b = w; b < a.r2; b += CC_T / 32)
+    for (int il = lane; il < a.nb; il += 32) U2s[il + a.nb * b] = il < nc ? __ldg(&a.U2[lo + il + a.N2 * b]) : 0.f;
+  // the eight warps over the groups of entries and, where these are few, over runs of j; the
+  // first CC_PRE values of T are on their way before the wait for c_j
+  const int js = max(1, (CC_T / 32) / neg), nq = neg * js;
+  float pre[CC_PRE];
+  {
+    const int e = 32 * (w % neg) + lane, jlo = a.J * (w / neg) / js, jhi = a.J * (w / neg + 1) / js;
+#pragma unroll
+    for (int u = 0; u < CC_PRE; ++u)
+      pre[u] = (w < nq && e < r12 && jlo + u < jhi) ? __ldg(&a.T[e + (size_t)r12 * (jlo + u)]) : 0.f;
+  }
+  __syncthreads();
+  for (int q = w; q < nq; q += CC_T / 32) {
+    const int eg = q % neg, jg = q / neg, e = 32 * eg + lane;
+    const int jlo = a.J * jg / js, jhi = a.J * (jg + 1) / js;
+    const float* src = a.T + (e < r12 ? e : 0);
+    float g = 0.f;
+    int j = jlo;
+    if (q == w) {
+#pragma unroll
+      for (int u = 0; u < CC_PRE; ++u)
+        if (jlo + u < jhi) g = fmaf(pre[u], cj[jlo + u], g);
+      j = min(jhi, jlo + CC_PRE);
+    }
+#pragma unroll 8
+    for (; j < jhi; ++j) g = fmaf(__ldg(&src[(size_t)r12 * j]), cj[j], g);
+    if (js > 1) red[jg * 32 * neg + e] = g;
+    else if (e < r12) G[e] = g;
+  }
+  __syncthreads();
+  if (js > 1) {
+    if (t < r12) {
+      float g = red[t];
+      for (int jg = 1; jg < js; ++jg) g += red[jg * 32 * neg + t];
+      G[t] = g;
+    }
+    __syncthreads();
+  }
+  // output a1 + r1 il, a1 and il carried from one to the next
+  float* out = a.H + (size_t)a.r1 * (lo + (size_t)a.N2 * s);
+  const int dil = CC_T / a.r1, da = CC_T - dil * a.r1;
+  int il = t / a.r1, a1 = t - il * a.r1;
+  for (int e = t; e < a.r1 * nc; e += CC_T) {
+    float h = 0.f;
+#pragma unroll 8
+    for (int b = 0; b < a.r2; ++b) h = fmaf(G[a1 + a.r1 * b], U2s[il + a.nb * b], h);
+    out[e] = h;
+    il += dil;
+    a1 += da;
+    if (a1 >= a.r1) { a1 -= a.r1; ++il; }
+  }
+}
+
+// Three and four modes, where forming G again for every slice and column block costs less than
+// the launch it saves (2^24 multiply-adds, 2 us); false: not taken.
+bool launch_core_cols(const float* T, const float* const* U, int p, const int64_t* N, const int* r, float* H,
+                      cudaStream_t s, const int* gate) {
+  if (p < 3 || p > 4) return false;
+  CoreCols a;
+  a.T = T;
+  a.U2 = U[1];
+  a.U3 = U[2];
+  a.U4 = p == 4 ? U[3] : nullptr;
+  a.H = H;
+  a.r1 = r[0];
+  a.r2 = r[1];
+  a.r3 = r[2];
+  a.J = r[2] * (p == 4 ? r[3] : 1);
+  a.N2 = (int)N[1];
+  a.N3 = (int)N[2];
+  a.N4 = p == 4 ? (int)N[3] : 1;
+  const int64_t ns = (int64_t)a.N3 * a.N4;
+  // columns of a CTA: two CTAs per SM where the slices alone are fewer, 16 columns at least
+  const int64_t sub = std::max<int64_t>((a.N2 + CC_NB - 1) / CC_NB, std::min<int64_t>((2 * 152 + ns - 1) / ns, (a.N2 + 15) / 16));
+  a.nb = (int)((a.N2 + sub - 1) / sub);
+  const int64_t ny = (a.N2 + a.nb - 1) / a.nb;
+  const int r12 = a.r1 * a.r2, neg = (r12 + 31) / 32;
+  if (a.J > CC_JMAX || ny > 65535 || (int64_t)r12 * a.J * ns * ny > (1 << 24)) return false;
+  const size_t sm = sizeof(float) * (a.J + r12 + (size_t)a.r2 * a.nb + 32 * std::max(8, neg));
+  if (sm > 48 * 1024) return false;
+  k_core_cols<<<dim3((unsigned)ns, (unsigned)ny), CC_T, sm, s>>>(a, gate);
+  count_launch();
+  return true;
+}
+
 template <typename Tin, typename Tm, typename Tacc>
 void launch_modeprod(const Tin* in, Tacc* out, const Tm* M, int64_t L, int K, int J, int64_t Q, int64_t sMj,
                      int64_t sMk, cudaStream_t s, const int* gate) {

@@ -136,6 +136,9 @@ void launch_recon_err(const T* V, const T* U1, const T* H, int r1, int N1, int64
 // V = U1 H (N1 x ncol; H: r1 x ncol)
 template <typename T>
 void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* V, cudaStream_t s);
+// H = T x_2 U_2 ... x_p U_p in one launch (three and four modes of few enough products), or false
+bool launch_core_cols(const float* T, const float* const* U, int p, const int64_t* N, const int* r, float* H,
+                      cudaStream_t s, const int* gate);
 template <typename T>
 void launch_weights_T(const WeightView& wv, T* w1, T* wcol, cudaStream_t s);
 template <typename Tin, typename Tm, typename Tacc>

@@ -624,6 +624,11 @@ const Tc* column_factors(tdb_ctx* ctx, const int* gate) {
   for (int m = 0; m < p; ++m) cur[m] = ctx->r[m];
   const Tc* src = (const Tc*)ctx->Tcore;
   Tc* bufs[2] = {(Tc*)ctx->ping, (Tc*)ctx->pong};
+  if constexpr (sizeof(Tc) == 4) {
+    const float* U[kMaxModes];
+    for (int n = 0; n < p; ++n) U[n] = (const float*)ctx->Uc[n];
+    if (launch_core_cols(src, U, p, ctx->N, ctx->r, bufs[(p - 1) & 1], ctx->stream, gate)) return bufs[(p - 1) & 1];
+  }
   for (int n = 1; n < p; ++n) {
     Tc* dst = bufs[n & 1];
     int64_t L = 1, Q = 1;
@@ -827,7 +832,7 @@ tdb_status hosvd_spectrum(tdb_ctx* ctx, const Tc* V) {
   // that.  (A float eigensolver resolves eigenvectors only where the eigenvalue gaps exceed
   // about 1e-6 of the largest eigenvalue; those the rank rule keeps at gamma_th = 99.999 %
   // sit below that.)
-  const tdb_status st = launch_eig_modes(pr, ctx->p, ctx->f64 ? 2e-16 : 1e-10, ctx->f64 ? 1e-15 : 1e-14, ctx->flags, s);
+  const tdb_status st = launch_eig_modes(pr, ctx->p, ctx->f64 ? 2e-16 : 1e-10, ctx->f64 ? 1e-15 : 1e-12, ctx->flags, s);
   if (st != TDB_OK) { ctx->err = "eigensolver launch failed"; return st; }
   for (int n = 0; n < ctx->p; ++n) {
     if (!short_side(ctx, n)) continue;
