@@ -570,6 +570,34 @@ tdb_status project_tree(tdb_ctx* ctx, const Tc* dV, cudaEvent_t* evm) {
   };
   Tc* ping = (Tc*)ctx->ping;
   Tc* pong = (Tc*)ctx->pong;
+  if (p == 3 && ctx->aux && ctx->ev_fork && ctx->ev_join) {
+    // Three modes: six launches, each too small to fill the GPU, in two chains on the context's
+    // streams: Z1 = dV x_1 A_1^T, Y_3, dS beside dV x_2 A_2^T, Y_1 and (once Z1 is there) Y_2.
+    // 64^3 double: 67 us, one after another 86 us.
+    for (int m = 0; m < p; ++m) dims[m] = ctx->N[m];
+    int64_t side[kMaxModes];
+    for (int m = 0; m < p; ++m) side[m] = ctx->N[m];
+    CK(cudaEventRecord(ctx->ev_fork, s));
+    CK(cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
+    if (evm) record_timing_event(evm[0], s);
+    mp(dV, ping, 0, dims);
+    if (evm) record_timing_event(evm[1], s);
+    CK(cudaEventRecord(ctx->ev_fork, s));
+    cudaStream_t lead = s;
+    s = ctx->aux;
+    mp(dV, pong, 1, side);
+    mp(pong, (Tc*)ctx->Y[0], 2, side);
+    CK(cudaStreamWaitEvent(s, ctx->ev_fork, 0));
+    for (int m = 0; m < p; ++m) side[m] = dims[m];
+    mp(ping, (Tc*)ctx->Y[1], 2, side);
+    CK(cudaEventRecord(ctx->ev_join, s));
+    s = lead;
+    mp(ping, (Tc*)ctx->Y[2], 1, dims);
+    mp((const Tc*)ctx->Y[2], (Tc*)ctx->dS, 2, dims);
+    CK(cudaStreamWaitEvent(s, ctx->ev_join, 0));
+    CHECK_LAUNCH();
+    return TDB_OK;
+  }
   // Z1 = dV x_1 A_1^T, then each Y_n (n >= 2) contracts the remaining modes but n
   for (int m = 0; m < p; ++m) dims[m] = ctx->N[m];
   if (evm) record_timing_event(evm[0], s);
