@@ -701,7 +701,8 @@ tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsig
     cudaMemsetAsync(M.bar, 0, 8 * sizeof(unsigned), s);
   }
   if (cta > nsm || smem > optin) return TDB_ERR_UNSUPPORTED;
-  cudaFuncSetAttribute(k_eig_modes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the limit, not this launch's need: another thread's launch may need more)
+  cudaFuncSetAttribute(k_eig_modes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)optin);
   void* args[] = {(void*)&a};
   const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_eig_modes, cta, EM_T, args, smem, s);
   count_launch();
