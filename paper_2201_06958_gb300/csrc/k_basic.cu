@@ -150,18 +150,22 @@ template void launch_diff_norm<double>(const double*, const double*, double*, in
 // Lane l of a warp owns rows i0 + R l .. i0 + R l + R - 1 of a block of 32 R rows, with U_1 of
 // those rows (R x r_1) and w_1 in registers, and walks a contiguous range of columns c.  Its R
 // rows of each column arrive by cp.async in a ring of D slots (D columns in flight per warp,
-// read back by the lane that copied them: no barrier); H and w_c come 32 columns at a time, H
-// through shared memory (rows padded to RM, zeros past r_1), w_c a column per lane.  Per column
+// read back by the lane that copied them: no barrier); H and w_c come 32 columns at a time, H by
+// cp.async into one of two halves of shared rows padded to RM (zeros past r_1), w_c a column per
+// lane.  Per column
 // the lane forms U_1 H[:, c] for its rows and the weighted squared difference; w_c times it
 // goes into a sum of the compute type that is added to the double accumulator every D columns.
 // The last CTA to finish adds the per-CTA partials in a fixed order and writes *out (no second
 // launch); `counter` is zero before and after.  Double runs at 64 cycles per instruction and
-// sub-partition, so there only the r_1 products that exist are formed (float takes all RM).
-// Measured from a cold cache: 256 x 128 x 512 float at r_1 = 11, 26 us (32 us with a column's H
-// and w_c copied by cp.async beside its rows and two warp barriers a column); 126^3 double at
+// sub-partition, so there only the r_1 products that exist are formed (float takes all RM, in
+// pairs).  Measured from a cold cache: 256 x 128 x 512 float at r_1 = 11, 25.4 us (26.7 with H
+// through registers, which spilled above rank 12, and single products; 32 with a column's H
+// and w_c copied beside its rows and two warp barriers a column); 126^3 double at
 // r_1 = 5, 54 us (8 double operations a point: 30 us at the issue rate), where a warp per column
 // with U_1 in shared memory and H[:, c] by shuffles took 156 us.
 constexpr int RE_D = 8;           // columns in flight per warp
+template <int N>
+using IntC = std::integral_constant<int, N>;
 template <int BYTES>
 __device__ __forceinline__ void cp_async_n(void* dst, const void* src, bool valid) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -196,26 +200,68 @@ __device__ __forceinline__ void lds_run(const T* p, T* v) {
   }
 }
 
-// 32 columns of an r1 x ncol matrix (contiguous), r1 values a lane in registers, and into the
-// warp's shared rows of RM
+// Columns of a chunk: 32, or 16 where two chunks of 32 would leave one CTA per SM.
 template <typename T, int RM>
-struct ColChunk {
-  T nx[RM];
-  __device__ __forceinline__ void fetch(const T* __restrict__ H, int r1, unsigned c, unsigned c_hi, int lane) {
-    const unsigned nv = c < c_hi ? (unsigned)r1 * min(32u, c_hi - c) : 0u;
-#pragma unroll
-    for (int a = 0; a < RM; ++a) {
-      const unsigned e = lane + 32 * a;
-      nx[a] = (a < r1 && e < nv) ? __ldg(&H[(size_t)r1 * c + e]) : T(0);
-    }
+constexpr int kChunk = sizeof(T) * RM <= 128 ? 32 : 16;
+
+// A chunk of columns of an r1 x ncol matrix (contiguous) on their way by cp.async into a warp's
+// shared rows of RM.  Value e goes to row e / r1, entry e % r1 (stepped, not divided).
+template <typename T, int RM>
+__device__ __forceinline__ void fetch_columns(T* dst, const T* __restrict__ H, int r1, unsigned c, unsigned c_hi,
+                                              int lane) {
+  const int nv = c < c_hi ? r1 * (int)min((unsigned)kChunk<T, RM>, c_hi - c) : 0;
+  const T* src = H + (size_t)r1 * (nv ? c : 0);
+  const int dq = 32 / r1, dr = 32 - dq * r1, q = lane / r1;
+  int rem = lane - q * r1, off = q * RM + rem;
+#pragma unroll 1
+  for (int e = lane; e < kChunk<T, RM> * r1; e += 32) {       // (unrolled, its offsets would stay in registers)
+    cp_async_n<sizeof(T)>(dst + off, e < nv ? src + e : src, e < nv);
+    off += dq * RM + dr;
+    rem += dr;
+    if (rem >= r1) { rem -= r1; off += RM - r1; }
   }
-  __device__ __forceinline__ void put(T* hs, int r1, int lane) const {
+}
+
+// U_1 of a lane's R rows in registers, and its product with one column of H.  Float: paired
+// multiply-adds over (a, a + 1), the even and the odd terms' sums added last; double: only the
+// r_1 products that exist.
+template <typename T, int R, int RM>
+struct RowBlock {
+  T u[R][RM];
+  __device__ __forceinline__ void load(const T* __restrict__ U1, int i0, int N1, int r1) {
 #pragma unroll
-    for (int a = 0; a < RM; ++a)
-      if (a < r1) {
-        const int e = lane + 32 * a;
-        hs[(e / r1) * RM + e % r1] = nx[a];
+    for (int q = 0; q < R; ++q)
+#pragma unroll
+      for (int a = 0; a < RM; ++a) u[q][a] = (i0 + q < N1 && a < r1) ? U1[i0 + q + (size_t)N1 * a] : T(0);
+  }
+  __device__ __forceinline__ void times(const T* h, int r1, T* rec) const {
+    if constexpr (sizeof(T) == 4) {
+      float2 acc[R];
+#pragma unroll
+      for (int q = 0; q < R; ++q) acc[q] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int a4 = 0; a4 < RM / 4; ++a4) {
+        const float4 x = reinterpret_cast<const float4*>(h)[a4];
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+          acc[q] = __ffma2_rn(make_float2(u[q][4 * a4], u[q][4 * a4 + 1]), make_float2(x.x, x.y), acc[q]);
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+          acc[q] = __ffma2_rn(make_float2(u[q][4 * a4 + 2], u[q][4 * a4 + 3]), make_float2(x.z, x.w), acc[q]);
       }
+#pragma unroll
+      for (int q = 0; q < R; ++q) rec[q] = acc[q].x + acc[q].y;
+    } else {
+      T x[RM];
+      lds_run<T, RM>(h, x);
+#pragma unroll
+      for (int q = 0; q < R; ++q) rec[q] = T(0);
+#pragma unroll
+      for (int a = 0; a < RM; ++a)
+        if (a < r1)
+#pragma unroll
+          for (int q = 0; q < R; ++q) rec[q] = fma(u[q][a], x[a], rec[q]);
+    }
   }
 };
 
@@ -227,13 +273,14 @@ __global__ void __launch_bounds__(256, 2) k_recon_err_rows(const T* __restrict__
                                                          unsigned* __restrict__ counter, double* __restrict__ out,
                                                          unsigned* flags, const int* __restrict__ gate) {
   if (gate && *gate == 0) return;          // the estimator ruled this evaluation out
+  constexpr int CC = kChunk<T, RM>;
   extern __shared__ __align__(16) unsigned char ring_raw[];
   __shared__ double sh[32];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  T* ring = (T*)ring_raw + (size_t)wib * (RE_D * 32 * R + 32 * RM) + R * lane;     // this lane's rows of slot 0
-  T* hs = (T*)ring_raw + (size_t)wib * (RE_D * 32 * R + 32 * RM) + RE_D * 32 * R;
-  for (int e = lane; e < 32 * RM; e += 32) hs[e] = T(0);
+  T* ring = (T*)ring_raw + (size_t)wib * (RE_D * 32 * R + 2 * CC * RM) + R * lane;     // this lane's rows of slot 0
+  T* hs = (T*)ring_raw + (size_t)wib * (RE_D * 32 * R + 2 * CC * RM) + RE_D * 32 * R;  // two chunks of H
+  for (int e = lane; e < 2 * CC * RM; e += 32) hs[e] = T(0);
   const int nrb = (N1 + 32 * R - 1) / (32 * R);
   const unsigned gw = blockIdx.x * (blockDim.x >> 5) + wib, tw = gridDim.x * (blockDim.x >> 5);
   const unsigned wpr = tw >= (unsigned)nrb ? tw / nrb : 1u;   // warps per row block
@@ -261,45 +308,37 @@ __global__ void __launch_bounds__(256, 2) k_recon_err_rows(const T* __restrict__
       ++cnext;
       if (cnext < c_hi) vsrc += N1;          // (past the end: zero bytes from the last column)
     };
+    __syncwarp();                            // hs cleared, and the row block before is done with it
+    fetch_columns<T, RM>(hs, H, r1, c_lo, c_hi, lane);
 #pragma unroll
     for (int t = 0; t < RE_D; ++t) issue(t);
-    ColChunk<T, RM> hc;
-    hc.fetch(H, r1, c_lo, c_hi, lane);
-    T wn = c_lo + lane < c_hi ? __ldg(&wcol[c_lo + lane]) : T(0);
-    T u[R][RM], wr[R];
+    T wn = lane < CC && c_lo + lane < c_hi ? __ldg(&wcol[c_lo + lane]) : T(0);
+    RowBlock<T, R, RM> ub;
+    ub.load(U1, i0, N1, r1);
+    T wr[R];
 #pragma unroll
-    for (int q = 0; q < R; ++q) {
-      const int i = i0 + q;
-      wr[q] = i < N1 ? w1[i] : T(0);
-#pragma unroll
-      for (int a = 0; a < RM; ++a) u[q][a] = (i < N1 && a < r1) ? U1[i + (size_t)N1 * a] : T(0);
-    }
+    for (int q = 0; q < R; ++q) wr[q] = i0 + q < N1 ? w1[i0 + q] : T(0);
     T csum = T(0);
-    for (unsigned c0 = c_lo; c0 < c_hi; c0 += 32) {
-      __syncwarp();
-      hc.put(hs, r1, lane);
+    int par = 0;                             // the half of hs that holds this chunk
+    for (unsigned c0 = c_lo; c0 < c_hi; c0 += CC, par ^= 1) {
+      // this chunk's H is in the group of the first column issued after it: older than the
+      // RE_D - 1 that may be open
+      cp_async_wait<RE_D - 1>();
       const T wl = wn;
       __syncwarp();
-      hc.fetch(H, r1, c0 + 32, c_hi, lane);
-      wn = c0 + 32 + lane < c_hi ? __ldg(&wcol[c0 + 32 + lane]) : T(0);
-      const int nc = (int)min(32u, c_hi - c0);
+      fetch_columns<T, RM>(hs + CC * RM * (par ^ 1), H, r1, c0 + CC, c_hi, lane);
+      const T* hc = hs + CC * RM * par;
+      wn = lane < CC && c0 + CC + lane < c_hi ? __ldg(&wcol[c0 + CC + lane]) : T(0);
+      const int nc = (int)min((unsigned)CC, c_hi - c0);
       for (int cb = 0; cb < nc; cb += RE_D) {
 #pragma unroll
         for (int t = 0; t < RE_D; ++t) {
           if (cb + t >= nc) break;
           cp_async_wait<RE_D - 1>();         // this column's copies (the oldest group) have landed
-          T v[R], h[RM];
+          T v[R], rec[R];
           lds_run<T, R>(ring + t * 32 * R, v);
-          lds_run<T, RM>(hs + (cb + t) * RM, h);
           issue(t);                          // the slot refills with the column D ahead
-          T rec[R];
-#pragma unroll
-          for (int q = 0; q < R; ++q) rec[q] = T(0);
-#pragma unroll
-          for (int a = 0; a < RM; ++a)
-            if (sizeof(T) == 4 || a < r1)
-#pragma unroll
-              for (int q = 0; q < R; ++q) rec[q] = fma(u[q][a], h[a], rec[q]);
+          ub.times(hc + (cb + t) * RM, r1, rec);
           T s = T(0);
 #pragma unroll
           for (int q = 0; q < R; ++q) {
@@ -340,26 +379,27 @@ void launch_recon_err(const T* V, const T* U1, const T* H, int r1, int N1, int64
                       const int* gate) {
   // rows per lane: 16 bytes of V (float ranks above 16: 8 bytes), so that U_1 stays in registers
   const uintptr_t va = (uintptr_t)V;
-  auto go = [&](auto kern, int R, int RM) {
+  auto go = [&](auto kern, auto rows, auto rmax) {
+    constexpr int R = decltype(rows)::value, RM = decltype(rmax)::value;
     // two CTAs per SM at most, and at least a ring of columns for every warp (a small tensor's
     // warps would spend their time on U_1, and a batch's members on each other's SMs)
     const int64_t units = ((N1 + 32 * R - 1) / (32 * R)) * ncol;
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>({(units + 8 * RE_D - 1) / (8 * RE_D), nblocks, 2 * 152}));
-    const size_t sm = sizeof(T) * 8 * (RE_D * 32 * R + 32 * RM);
+    const size_t sm = sizeof(T) * 8 * (RE_D * 32 * R + 2 * kChunk<T, RM> * RM);
     if (sm > 47 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     const int vec = N1 % R == 0 && va % (R * sizeof(T)) == 0;
     kern<<<blocks, 256, sm, s>>>(V, U1, H, r1, N1, (unsigned)ncol, w1, wcol, vec, partial, counter, out, flags, gate);
     count_launch();
   };
   if constexpr (sizeof(T) == 4) {
-    if (r1 <= 8) go(k_recon_err_rows<float, 4, 8>, 4, 8);
-    else if (r1 <= 12) go(k_recon_err_rows<float, 4, 12>, 4, 12);
-    else if (r1 <= 16) go(k_recon_err_rows<float, 4, 16>, 4, 16);
-    else go(k_recon_err_rows<float, 2, 32>, 2, 32);
+    if (r1 <= 8) go(k_recon_err_rows<float, 4, 8>, IntC<4>(), IntC<8>());
+    else if (r1 <= 12) go(k_recon_err_rows<float, 4, 12>, IntC<4>(), IntC<12>());
+    else if (r1 <= 16) go(k_recon_err_rows<float, 4, 16>, IntC<4>(), IntC<16>());
+    else go(k_recon_err_rows<float, 2, 32>, IntC<2>(), IntC<32>());
   } else {
-    if (r1 <= 8) go(k_recon_err_rows<double, 2, 8>, 2, 8);
-    else if (r1 <= 16) go(k_recon_err_rows<double, 2, 16>, 2, 16);
-    else go(k_recon_err_rows<double, 1, 32>, 1, 32);
+    if (r1 <= 8) go(k_recon_err_rows<double, 2, 8>, IntC<2>(), IntC<8>());
+    else if (r1 <= 16) go(k_recon_err_rows<double, 2, 16>, IntC<2>(), IntC<16>());
+    else go(k_recon_err_rows<double, 1, 32>, IntC<1>(), IntC<32>());
   }
 }
 template void launch_recon_err<float>(const float*, const float*, const float*, int, int, int64_t, const float*,
@@ -754,18 +794,19 @@ __global__ void __launch_bounds__(256) k_mp_cols(const float* __restrict__ in, f
 
 // V^TDB = U_1 H with H = T x_2 U_2 ... x_p U_p (r_1 x ncol): the last and only large product of
 // a reconstruction.  Lane l of a warp owns R rows of a block of 32 R with U_1's in registers
-// and walks a range of columns, 32 columns' H at a time through shared memory (padded to RM,
-// zeros past r_1), the next 32 loaded meanwhile.  Bound: HBM, N_1 ncol values written once.
-// 192 x 129 x 192 x 3 float at r_1 = 13: 24 us from a cold cache, where the product of the last mode with a
-// thread per output took 91 us, and the mode before it as long.
+// and walks a range of columns, 32 columns' H at a time in shared memory (padded to RM, zeros past
+// r_1), the next 32 on their way by cp.async.  Bound: HBM, N_1 ncol values written once.
+// 256 x 128 x 512 float at r_1 = 11, 17.7 us from a cold cache (18.3 with H through registers);
+// a whole reconstruction of 192 x 129 x 192 x 3 at r_1 = 13 31.7 us (33.0), where the product
+// of the last mode with a thread per output took 91 us, and the mode before it as long.
 template <typename T, int R, int RM>
 __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, const T* __restrict__ H, int r1, int N1,
                                                       unsigned ncol, int vec, T* __restrict__ V) {
+  constexpr int CC = kChunk<T, RM>;
   extern __shared__ __align__(16) unsigned char ro_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  T* hs = (T*)ro_raw + (size_t)wib * 32 * RM;
-  for (int e = lane; e < 32 * RM; e += 32) hs[e] = T(0);
-  __syncwarp();
+  T* hs = (T*)ro_raw + (size_t)wib * 2 * CC * RM;       // two chunks of H
+  for (int e = lane; e < 2 * CC * RM; e += 32) hs[e] = T(0);
   const int nrb = (N1 + 32 * R - 1) / (32 * R);
   const unsigned gw = blockIdx.x * (blockDim.x >> 5) + wib, tw = gridDim.x * (blockDim.x >> 5);
   const unsigned wpr = tw >= (unsigned)nrb ? tw / nrb : 1u;
@@ -773,29 +814,22 @@ __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, 
   const unsigned c_lo = (unsigned)((uint64_t)ncol * kk / wpr), c_hi = (unsigned)((uint64_t)ncol * (kk + 1) / wpr);
   for (unsigned rb = gw / wpr; rb < (unsigned)nrb && c_lo < c_hi; rb += (tw >= (unsigned)nrb ? (unsigned)nrb : tw)) {
     const int i0 = (int)rb * 32 * R + R * lane;
-    T u[R][RM];
-#pragma unroll
-    for (int q = 0; q < R; ++q)
-#pragma unroll
-      for (int a = 0; a < RM; ++a) u[q][a] = (i0 + q < N1 && a < r1) ? U1[i0 + q + (size_t)N1 * a] : T(0);
-    ColChunk<T, RM> hc;
-    hc.fetch(H, r1, c_lo, c_hi, lane);
-    for (unsigned c0 = c_lo; c0 < c_hi; c0 += 32) {
+    __syncwarp();                            // hs cleared, and the row block before is done with it
+    fetch_columns<T, RM>(hs, H, r1, c_lo, c_hi, lane);
+    cp_async_commit();
+    RowBlock<T, R, RM> ub;
+    ub.load(U1, i0, N1, r1);
+    int par = 0;                             // the half of hs that holds this chunk
+    for (unsigned c0 = c_lo; c0 < c_hi; c0 += CC, par ^= 1) {
+      cp_async_wait<0>();
       __syncwarp();
-      hc.put(hs, r1, lane);
-      __syncwarp();
-      hc.fetch(H, r1, c0 + 32, c_hi, lane);
-      const int nc = (int)min(32u, c_hi - c0);
+      fetch_columns<T, RM>(hs + CC * RM * (par ^ 1), H, r1, c0 + CC, c_hi, lane);
+      cp_async_commit();
+      const T* hc = hs + CC * RM * par;
+      const int nc = (int)min((unsigned)CC, c_hi - c0);
       for (int c = 0; c < nc; ++c) {
-        T h[RM], rec[R];
-        lds_run<T, RM>(hs + c * RM, h);
-#pragma unroll
-        for (int q = 0; q < R; ++q) rec[q] = T(0);
-#pragma unroll
-        for (int a = 0; a < RM; ++a)
-          if (sizeof(T) == 4 || a < r1)
-#pragma unroll
-            for (int q = 0; q < R; ++q) rec[q] = fma(u[q][a], h[a], rec[q]);
+        T rec[R];
+        ub.times(hc + c * RM, r1, rec);
         T* o = V + (size_t)N1 * (c0 + c) + i0;
         if (vec) {
           if (i0 < N1) {
@@ -815,14 +849,16 @@ __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, 
         }
       }
     }
+    cp_async_wait<0>();
   }
 }
 
 template <typename T>
 void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* V, cudaStream_t s) {
   const uintptr_t va = (uintptr_t)V;
-  auto go = [&](auto kern, int R, int RM) {
-    const size_t sm = sizeof(T) * 8 * 32 * RM;
+  auto go = [&](auto kern, auto rows, auto rmax) {
+    constexpr int R = decltype(rows)::value, RM = decltype(rmax)::value;
+    const size_t sm = sizeof(T) * 8 * 2 * kChunk<T, RM> * RM;
     if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     // a warp per 32 columns of a row block at least, two CTAs per SM at most
     const int64_t units = ((N1 + 32 * R - 1) / (32 * R)) * ((ncol + 31) / 32);
@@ -832,14 +868,14 @@ void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* 
     count_launch();
   };
   if constexpr (sizeof(T) == 4) {
-    if (r1 <= 8) go(k_recon_out<float, 4, 8>, 4, 8);
-    else if (r1 <= 12) go(k_recon_out<float, 4, 12>, 4, 12);
-    else if (r1 <= 16) go(k_recon_out<float, 4, 16>, 4, 16);
-    else go(k_recon_out<float, 2, 32>, 2, 32);
+    if (r1 <= 8) go(k_recon_out<float, 4, 8>, IntC<4>(), IntC<8>());
+    else if (r1 <= 12) go(k_recon_out<float, 4, 12>, IntC<4>(), IntC<12>());
+    else if (r1 <= 16) go(k_recon_out<float, 4, 16>, IntC<4>(), IntC<16>());
+    else go(k_recon_out<float, 2, 32>, IntC<2>(), IntC<32>());
   } else {
-    if (r1 <= 8) go(k_recon_out<double, 2, 8>, 2, 8);
-    else if (r1 <= 16) go(k_recon_out<double, 2, 16>, 2, 16);
-    else go(k_recon_out<double, 1, 32>, 1, 32);
+    if (r1 <= 8) go(k_recon_out<double, 2, 8>, IntC<2>(), IntC<8>());
+    else if (r1 <= 16) go(k_recon_out<double, 2, 16>, IntC<2>(), IntC<16>());
+    else go(k_recon_out<double, 1, 32>, IntC<1>(), IntC<32>());
   }
 }
 template void launch_recon_out<float>(const float*, const float*, int, int, int64_t, float*, cudaStream_t);
@@ -848,7 +884,7 @@ template void launch_recon_out<double>(const double*, const double*, int, int, i
 // H = T x_2 U_2 x_3 U_3 (x_4 U_4) in float, r_1 x N_2 x slices, in one launch: a CTA forms the
 // r_1 x r_2 slice G = sum_j T[:, :, j] c_j, c_j = U_3[i_3, c] U_4[i_4, d] over the J = r_3 r_4
 // pairs, then its block of columns G U_2[i_2, :]^T.  Bound: latency; 256 x 128 x 512 at (11, 8,
-// 16) CC_ONE us against 9.1 in two mode products with the gap between them.
+// 16) 8.2 us against 9.1 in two mode products with the gap between them.
 constexpr int CC_T = 256, CC_JMAX = 1024, CC_NB = 256, CC_PRE = 16;
 struct CoreCols {
   const float* T;
