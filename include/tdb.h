@@ -374,9 +374,16 @@ tdb_status tdb_project_noalloc(int ndim, const int64_t* dims, const int* ranks, 
  *   returns TDB_ERR_TIMEOUT (the expected result), TDB_OK if the wait ended otherwise,
  *   TDB_ERR_INVALID_ARG for bad arguments or TDB_ERR_CUDA.  The CUDA context stays
  *   usable afterwards.
+ * tdb_selftest_eig_split: how the HOSVD's eigensolver shares num_sms SMs of smem_bytes
+ *   shared memory per CTA out to nmodes mode Grams of n[i] points with k[i] wanted pairs:
+ *   ctas[i] (one for the Jacobi and the rest for the rows) and the shared memory of the
+ *   launch.  Host arithmetic only (no GPU needed).  TDB_ERR_UNSUPPORTED where they do not
+ *   suffice, TDB_ERR_INVALID_ARG for bad arguments.
  * ------------------------------------------------------------------------- */
 tdb_status tdb_selftest_recip(const double* x, double* rcp, double* rsqrt, int64_t n, void* stream);
 tdb_status tdb_selftest_timeout(int which, int64_t limit_cycles, unsigned* scratch, void* stream);
+tdb_status tdb_selftest_eig_split(int nmodes, const int* n, const int* k, int num_sms, int64_t smem_bytes, int* ctas,
+                                  int64_t* smem);
 
 /* The launch shape the tensor-core projection's tuner chose for this context (TDB_BF16_TTM
  * only; the paper has no counterpart).  The tile is fixed (128 x 128, eight strips); the

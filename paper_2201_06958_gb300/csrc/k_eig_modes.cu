@@ -649,6 +649,48 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
 
 int em_cols(int n, int k) { return std::min(n, k + 16); }
 
+// The CTAs of each mode (the Jacobi's and those that own rows), and the shared memory of the
+// launch.  A row CTA holds its rows of Q and Z in shared memory, so a mode takes at least the CTAs
+// that its rows need for that (110 rows and more of the widest block fill one); past that the SMs
+// are shared in proportion to n^2, the entries of C that a product reads, and a mode whose vectors
+// are all kept (no products) takes no more than leave eight rows, one per warp, to a CTA.  (By n^2
+// alone a mode of 119 points beside one of 1024 got one CTA, and the launch was refused.)
+// False: not on this many SMs.
+struct EmSplit {
+  int nct[kMaxModes];
+  size_t smem;
+};
+bool em_split(const int* n, const int* k, int p, int nsm, size_t limit, EmSplit& out) {
+  double tot = 0.0;
+  for (int i = 0; i < p; ++i) tot += (double)n[i] * n[i];
+  const int avail = nsm - 2 * p;
+  int need[kMaxModes], sum = 0;
+  for (int i = 0; i < p; ++i) {
+    const int m = em_cols(n[i], k[i]), mp = (m + 7) & ~7;
+    if (em_smem(1, mp) > limit) return false;
+    int rows = n[i];                         // the most rows of a CTA
+    if (em_smem(rows, mp) > limit) rows = (int)((limit - em_smem(0, mp)) / (em_smem(1, mp) - em_smem(0, mp)));
+    need[i] = (n[i] + rows - 1) / rows;
+    const int want = avail > 0 ? (int)((double)avail * ((double)n[i] * n[i] / tot)) : 0;
+    const int most = m == n[i] ? (n[i] + EM_W - 1) / EM_W : n[i];
+    out.nct[i] = 1 + std::max(need[i], std::min(std::max(want, 1), most));
+    sum += out.nct[i];
+  }
+  for (; sum > nsm; --sum) {                 // the mode with the most to spare gives one up
+    int best = 0;
+    for (int i = 1; i < p; ++i)
+      if (out.nct[i] - need[i] > out.nct[best] - need[best]) best = i;
+    if (out.nct[best] - 1 <= need[best]) return false;
+    --out.nct[best];
+  }
+  out.smem = 0;
+  for (int i = 0; i < p; ++i) {
+    const int nb = out.nct[i] - 1, mp = (em_cols(n[i], k[i]) + 7) & ~7;
+    out.smem = std::max(out.smem, em_smem((n[i] + nb - 1) / nb, mp));
+  }
+  return true;
+}
+
 }  // namespace
 
 size_t eig_modes_scratch(int n, int k) {
@@ -658,27 +700,34 @@ size_t eig_modes_scratch(int n, int k) {
 }
 
 tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsigned* flags, cudaStream_t s) {
-  static int nsm = 0;
-  static size_t optin = 0;
-  if (nsm == 0) {
-    int dev = 0, coop = 0, lim = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (!coop) return TDB_ERR_UNSUPPORTED;
-    optin = (size_t)lim - 2048;
-    nsm = std::min(sms, 152);
+  // (read once; what the device gives less than 2 KB for the kernel's static shared memory)
+  struct Device {
+    int nsm = 0, coop = 0;
+    size_t optin = 0;
+  };
+  static const Device dev = [] {
+    Device d;
+    int id = 0, lim = 0;
+    cudaGetDevice(&id);
+    cudaDeviceGetAttribute(&d.nsm, cudaDevAttrMultiProcessorCount, id);
+    cudaDeviceGetAttribute(&d.coop, cudaDevAttrCooperativeLaunch, id);
+    cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, id);
+    d.nsm = std::min(d.nsm, 152);
+    d.optin = (size_t)std::max(lim - 2048, 0);
+    return d;
+  }();
+  if (!dev.coop) return TDB_ERR_UNSUPPORTED;
+  int n[kMaxModes], k[kMaxModes];
+  for (int i = 0; i < p; ++i) {
+    n[i] = pr[i].n;
+    k[i] = pr[i].k;
+    if (k[i] > n[i] || em_cols(n[i], k[i]) > EM_M) return TDB_ERR_INVALID_ARG;
   }
+  EmSplit split;
+  if (!em_split(n, k, p, dev.nsm, dev.optin, split)) return TDB_ERR_UNSUPPORTED;
   EigModes a;
   a.p = p;
   a.flags = flags;
-  // CTAs per mode: in proportion to the n^2 m of its products, at least what keeps eight rows
-  // (one per warp) or fewer to a CTA where the SMs allow it; one CTA more for the Jacobi
-  double tot = 0.0;
-  for (int i = 0; i < p; ++i) tot += (double)pr[i].n * pr[i].n;
-  const int avail = nsm - 2 * p;
-  size_t smem = 0;
   int cta = 0;
   for (int i = 0; i < p; ++i) {
     EigMode& M = a.mode[i];
@@ -686,11 +735,8 @@ tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsig
     M.n = pr[i].n;
     M.k = pr[i].k;
     M.m = em_cols(M.n, M.k);
-    if (M.m > EM_M || M.k > M.m) return TDB_ERR_INVALID_ARG;
     M.mp = (M.m + 7) & ~7;
-    const int want = (int)((double)avail * ((double)M.n * M.n / tot));
-    const int most = M.m == M.n ? (M.n + EM_W - 1) / EM_W : M.n;
-    M.nct = 1 + std::max(1, std::min(want, most));
+    M.nct = split.nct[i];
     M.cta0 = cta;
     cta += M.nct;
     double* w = pr[i].scratch;
@@ -710,17 +756,28 @@ tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsig
     M.trace = pr[i].trace;
     M.tau = tau;
     M.tol = tol;
-    const int rows = (M.n + M.nct - 2) / (M.nct - 1);
-    smem = std::max(smem, em_smem(rows, M.mp));
     cudaMemsetAsync(M.bar, 0, 8 * sizeof(unsigned), s);
   }
-  if (cta > nsm || smem > optin) return TDB_ERR_UNSUPPORTED;
   // (the limit, not this launch's need: another thread's launch may need more)
-  cudaFuncSetAttribute(k_eig_modes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)optin);
+  cudaFuncSetAttribute(k_eig_modes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev.optin);
   void* args[] = {(void*)&a};
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_eig_modes, cta, EM_T, args, smem, s);
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_eig_modes, cta, EM_T, args, split.smem, s);
   count_launch();
   return e == cudaSuccess ? TDB_OK : TDB_ERR_CUDA;
 }
 
 }  // namespace tdb
+
+extern "C" tdb_status tdb_selftest_eig_split(int nmodes, const int* n, const int* k, int num_sms,
+                                             int64_t smem_bytes, int* ctas, int64_t* smem) {
+  using namespace tdb;
+  if (nmodes < 1 || nmodes > kMaxModes || !n || !k || !ctas || !smem || num_sms < 1 || smem_bytes < 1)
+    return TDB_ERR_INVALID_ARG;
+  for (int i = 0; i < nmodes; ++i)
+    if (n[i] < 1 || k[i] < 1 || k[i] > n[i] || em_cols(n[i], k[i]) > EM_M) return TDB_ERR_INVALID_ARG;
+  EmSplit split;
+  if (!em_split(n, k, nmodes, num_sms, (size_t)smem_bytes, split)) return TDB_ERR_UNSUPPORTED;
+  for (int i = 0; i < nmodes; ++i) ctas[i] = split.nct[i];
+  *smem = (int64_t)split.smem;
+  return TDB_OK;
+}

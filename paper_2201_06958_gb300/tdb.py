@@ -110,6 +110,7 @@ EXPORTS = [
     "tdb_estimator_params", "tdb_estimator_trace", "tdb_set_input_slots", "tdb_push_slot",
     "tdb_batch_create", "tdb_batch_push", "tdb_batch_last_error", "tdb_batch_destroy", "tdb_get_graph_counters",
     "tdb_selftest_recip", "tdb_selftest_timeout", "tdb_tc_tuning", "tdb_estimator_load_trace",
+    "tdb_selftest_eig_split",
 ]
 
 
@@ -188,6 +189,9 @@ def load(path: str = LIB_PATH):
     lib.tdb_selftest_recip.restype = st
     lib.tdb_selftest_timeout.argtypes = [C.c_int, C.c_int64, vp, vp]
     lib.tdb_selftest_timeout.restype = st
+    lib.tdb_selftest_eig_split.argtypes = [C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int), C.c_int, C.c_int64,
+                                           C.POINTER(C.c_int), C.POINTER(C.c_int64)]
+    lib.tdb_selftest_eig_split.restype = st
     lib.tdb_mlp_param_count.argtypes = []
     lib.tdb_mlp_param_count.restype = C.c_int
     lib.tdb_mlp_forward.argtypes = [vp, vp, C.c_int, vp, vp]
