@@ -13,7 +13,10 @@
 //            publishes its rotations sweep by sweep; the other CTAs apply them to their rows
 //            of Q meanwhile, so no vector matrix is formed.
 //   output   the k leading columns, unit length, entry of largest magnitude positive.
-// A mode of at most m points skips the iteration (Q = I, H = C).
+// A mode of at most m points skips the iteration (Q = I, H = C).  A mode of up to 96 points whose
+// iteration has not settled after 27 rounds is solved whole in the same way: a spectrum that
+// hardly decays (noise) would take hundreds, and its vectors were still off by up to 0.3 in angle.
+// (A longer mode keeps the block that it has by then.)
 //
 // Bound: chains of dependent double operations on one CTA (GB300 issues one double warp
 // instruction per 64 cycles per SM sub-partition), so the design cuts the number of chains
@@ -40,6 +43,7 @@ constexpr int EM_RC = 8;                    // rows of C Z formed at a time
 constexpr int EM_MP = (EM_M + 7) & ~7;      // columns padded to whole groups of eight (56)
 constexpr int EM_ITERS = 27;                // iterations at most
 constexpr int EM_SWEEPS = kEigSweeps;
+constexpr int EM_D = kEigWhole, EM_DLD = EM_D + 1;   // most points of a mode solved whole (96)
 
 __device__ __forceinline__ unsigned em_ld_acquire(const unsigned* p) {
   unsigned v;
@@ -247,18 +251,24 @@ __device__ __forceinline__ void em_pair(int nn, int rd, int k, int& p, int& q) {
   }
 }
 
+// (c, s) pairs of one sweep over m indices.
+__host__ __device__ inline int64_t em_sweep_pairs(int m) {
+  const int64_t nn = (m + 1) & ~1;
+  return (nn - 1) * (nn / 2);
+}
+
 // One sweep's rotations (rounds x pairs of (c, s)) applied to the rows A (nr x m, ld mp): a
-// warp per row, a lane per pair.
+// warp per row, a lane per pair (or two).
 __device__ void em_apply_sweep(double* A, int nr, int m, int mp, const double2* rot) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nn = (m + 1) & ~1, half = nn / 2;
   for (int r = w; r < nr; r += EM_W) {
     double* row = A + r * mp;
     for (int rd = 0; rd < nn - 1; ++rd) {
-      if (lane < half) {
+      for (int k = lane; k < half; k += 32) {
         int p, q;
-        em_pair(nn, rd, lane, p, q);
-        const double2 cs = __ldcg(&rot[rd * half + lane]);
+        em_pair(nn, rd, k, p, q);
+        const double2 cs = __ldcg(&rot[rd * half + k]);
         const double vp = row[p], vq = row[q];
         row[p] = fma(cs.x, vp, -(cs.y * vq));
         row[q] = fma(cs.y, vp, cs.x * vq);
@@ -268,23 +278,24 @@ __device__ void em_apply_sweep(double* A, int nr, int m, int mp, const double2* 
   }
 }
 
-// Cyclic Jacobi on the symmetric H (m x m, full, ld EM_LD; row and column nn - 1 zero for odd
-// m) by this CTA, the rotations of sweep s written to rot[s] and announced through *done
-// (s + 1; the last one with kEmLast set).  Every pair rotates: the block's columns are not
+// Cyclic Jacobi on the symmetric H (m x m, full, ld LDH; row and column nn - 1 zero for odd
+// m; NB blocks of 2 x 2 a thread at most) by this CTA, the rotations of sweep s written to rot[s]
+// and announced through *done (s + 1; the last one with kEmLast set).  Every pair rotates: the block's columns are not
 // sorted, so a wanted Ritz value can sit in its tail.  The angle's tangent is float (a rotation by it
 // leaves 1e-7 of the pair's off-diagonal, which the next sweep takes), its cosine and sine
 // double.  The 2 x 2 blocks above the diagonal are updated and mirrored.  Ends when the
 // off-diagonal mass is below tol^2 of the diagonal's, or at the rounding
 // floor (a sweep after the third that does not quarter it).
 constexpr unsigned kEmLast = 0x80000000u;
+template <int NB, int LDH>
 __device__ bool em_jacobi(double* H, int m, double tol, double2* rot, unsigned* done, double* cs, int* pq,
                           double* red) {
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int nn = (m + 1) & ~1, half = nn / 2, nblk = half * (half + 1) / 2;
   // this thread's blocks (I <= J), the same in every round
-  int blk[2];
+  int blk[NB];
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
+  for (int u = 0; u < NB; ++u) {
     const int e = t + EM_T * u;
     int J = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
     while ((J + 1) * (J + 2) / 2 <= e) ++J;
@@ -297,7 +308,7 @@ __device__ bool em_jacobi(double* H, int m, double tol, double2* rot, unsigned* 
     double off = 0.0, dia = 0.0;
     for (int e = t; e < m * m; e += EM_T) {
       const int i = e % m, j = e / m;
-      const double v = H[i + EM_LD * j];
+      const double v = H[i + LDH * j];
       if (i == j) dia = fma(v, v, dia);
       else if (i < j) off = fma(v, v, off);
     }
@@ -317,12 +328,12 @@ __device__ bool em_jacobi(double* H, int m, double tol, double2* rot, unsigned* 
       if (t == 0) em_st_release(done, (unsigned)sweep | kEmLast);
       return conv || sweep < EM_SWEEPS;
     }
-    double2* out = rot + (int64_t)sweep * (EM_M - 1) * (EM_M / 2);
+    double2* out = rot + sweep * em_sweep_pairs(m);
     for (int rd = 0; rd < nn - 1; ++rd) {
       if (t < half) {
         int p, q;
         em_pair(nn, rd, t, p, q);
-        const double app = H[p + EM_LD * p], aqq = H[q + EM_LD * q], apq = H[p + EM_LD * q];
+        const double app = H[p + LDH * p], aqq = H[q + LDH * q], apq = H[p + LDH * q];
         double c = 1.0, s = 0.0;
         const float fpq = (float)apq;
         if (fabsf(fpq) > 1e-30f && fpq * fpq > 1e-32f * fabsf((float)app * (float)aqq)) {
@@ -341,28 +352,28 @@ __device__ bool em_jacobi(double* H, int m, double tol, double2* rot, unsigned* 
       }
       __syncthreads();
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < NB; ++u) {
         if (blk[u] < 0) continue;
         const int I = blk[u] & 255, J = blk[u] >> 8;
         const int pI = pq[2 * I], qI = pq[2 * I + 1], pJ = pq[2 * J], qJ = pq[2 * J + 1];
         const double cI = cs[2 * I], sI = cs[2 * I + 1], cJ = cs[2 * J], sJ = cs[2 * J + 1];
-        const double b00 = H[pI + EM_LD * pJ], b01 = H[pI + EM_LD * qJ], b10 = H[qI + EM_LD * pJ],
-                     b11 = H[qI + EM_LD * qJ];
+        const double b00 = H[pI + LDH * pJ], b01 = H[pI + LDH * qJ], b10 = H[qI + LDH * pJ],
+                     b11 = H[qI + LDH * qJ];
         const double c00 = fma(cJ, b00, -(sJ * b01)), c01 = fma(sJ, b00, cJ * b01);
         const double c10 = fma(cJ, b10, -(sJ * b11)), c11 = fma(sJ, b10, cJ * b11);
         const double d00 = fma(cI, c00, -(sI * c10)), d01 = fma(cI, c01, -(sI * c11));
         const double d10 = fma(sI, c00, cI * c10), d11 = fma(sI, c01, cI * c11);
-        H[pI + EM_LD * pJ] = d00;
-        H[qI + EM_LD * qJ] = d11;
-        H[pI + EM_LD * qJ] = d01;
+        H[pI + LDH * pJ] = d00;
+        H[qI + LDH * qJ] = d11;
+        H[pI + LDH * qJ] = d01;
         if (I == J) {
-          H[qI + EM_LD * pI] = d01;
+          H[qI + LDH * pI] = d01;
         } else {
-          H[qI + EM_LD * pJ] = d10;
-          H[pJ + EM_LD * pI] = d00;
-          H[qJ + EM_LD * pI] = d01;
-          H[pJ + EM_LD * qI] = d10;
-          H[qJ + EM_LD * qI] = d11;
+          H[qI + LDH * pJ] = d10;
+          H[pJ + LDH * pI] = d00;
+          H[qJ + LDH * pI] = d01;
+          H[pJ + LDH * qI] = d10;
+          H[qJ + LDH * qI] = d11;
         }
       }
       __syncthreads();
@@ -374,16 +385,21 @@ __device__ bool em_jacobi(double* H, int m, double tol, double2* rot, unsigned* 
   }
 }
 
-// Shared memory (doubles): the factor's [G | I], G, X, H; the CTA's rows of Q and Z; the C Z
-// reduction.
-__host__ __device__ constexpr size_t em_fixed() { return (size_t)EM_LD * EM_M * 2 + 3 * (size_t)EM_LD * EM_M + 4 * 64; }
-__host__ __device__ inline size_t em_smem(int rows, int mp) {
-  return sizeof(double) * (em_fixed() + 2 * (size_t)rows * mp + (size_t)EM_W * EM_RC * mp);
+// Shared memory (doubles): the factor's [G | I], G, X, H (where C itself goes for a mode that is
+// solved whole); the CTA's rows of Q and Z; the C Z reduction (all three the rows of the whole
+// solve, if it comes to that).
+__host__ __device__ constexpr size_t em_fixed() { return 5 * (size_t)EM_LD * EM_M + 64 + 64 + EM_D + 64; }
+static_assert(5 * EM_LD * EM_M >= EM_DLD * EM_D, "C of a mode solved whole");
+__host__ __device__ inline size_t em_smem(int n, int mp, int rows) {
+  size_t v = 2 * (size_t)rows * mp + (size_t)EM_W * EM_RC * mp;
+  const size_t whole = n <= EM_D ? (size_t)rows * ((n + 7) & ~7) : 0;
+  if (v < whole) v = whole;
+  return sizeof(double) * (em_fixed() + v);
 }
 
 __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
   extern __shared__ __align__(16) double em_sm[];
-  __shared__ int abort_sh, ord[64], pq[128];
+  __shared__ int abort_sh, ord[EM_D], pq[128];
   __shared__ unsigned done_sh;
   int md = 0;
   while (md + 1 < a.p && (int)blockIdx.x >= a.mode[md + 1].cta0) ++md;
@@ -396,9 +412,9 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
   double* H = X + EM_LD * EM_M;              // Q^T Z
   double* dsc = H + EM_LD * EM_M;            // 64
   double* mult = dsc + 64;                   // 64
-  double* cs = mult + 64;                    // 64 (pairs' c, s) and 64 for sums
-  double* red = cs + 64;
-  double* Qr = cs + 128;                     // this CTA's rows of Q (nr x mp)
+  double* cs = mult + 64;                    // EM_D (pairs' c, s)
+  double* red = cs + EM_D;                   // 64 for sums
+  double* Qr = red + 64;                     // this CTA's rows of Q (nr x mp)
   // the group's first CTA runs the Jacobi and owns no rows (a group has at least two)
   const int nb = B - 1;
   const int r_lo = b == 0 ? 0 : (int)((int64_t)n * (b - 1) / nb), r_hi = b == 0 ? 0 : (int)((int64_t)n * b / nb);
@@ -427,12 +443,8 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
     return true;
   };
   double delta = 0.0;                        // the shift of the iterated matrix, below
-  if (m == n) {
-    // every vector is kept: Q = I, H = C
-    for (int e = t; e < nr * mp; e += EM_T) Qr[e] = (r_lo + e / mp == e % mp) ? 1.0 : 0.0;
-    for (int e = t; e < nful; e += EM_T) H[(e % m) + EM_LD * (e / m)] = M.C[e];
-    __syncthreads();
-  } else {
+  bool whole = m == n;                       // every vector is kept: Q = I, H = C
+  if (!whole) {
     const double u = 1.1102230246251565e-16;
     const double s0 = 11.0 * ((double)n * m + (double)m * (m + 1)) * u * m;
     // C + delta I is iterated, delta one rounding of C's largest diagonal entry (the Ritz values
@@ -501,7 +513,11 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
         } else {
           --extra;
         }
-        if (extra == 0 || it == EM_ITERS) break;
+        if (extra == 0) break;
+        if (it == EM_ITERS) {
+          whole = n <= EM_D;
+          break;
+        }
       }
       // Q = orth(Z)
       for (int pass = 0; pass < 6; ++pass) {
@@ -538,14 +554,33 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
       for (int e = t; e < nr * mp; e += EM_T) M.Q[(int64_t)(r_lo + e / mp) * mp + e % mp] = Qr[e];
       if (!em_sync(M.bar, ++nbar, B, a.flags, &abort_sh)) return;
     }
-    for (int e = t; e < nful; e += EM_T) {
-      const int i = e % m, j = e / m;
-      if (i < j) {
-        const double h = 0.5 * (H[i + EM_LD * j] + H[j + EM_LD * i]);
-        H[i + EM_LD * j] = h;
-        H[j + EM_LD * i] = h;
+    if (!whole) {
+      for (int e = t; e < nful; e += EM_T) {
+        const int i = e % m, j = e / m;
+        if (i < j) {
+          const double h = 0.5 * (H[i + EM_LD * j] + H[j + EM_LD * i]);
+          H[i + EM_LD * j] = h;
+          H[j + EM_LD * i] = h;
+        }
       }
+      __syncthreads();
     }
+  }
+  // the matrix to diagonalise: dm x dm at Hd (ld dld), the rows of its basis at Qr (ld dmp)
+  int dm = m, dmp = mp, dld = EM_LD;
+  double* Hd = H;
+  if (whole) {
+    dm = n;
+    dmp = (n + 7) & ~7;
+    if (n > EM_M) {
+      dld = EM_DLD;
+      Hd = em_sm;
+    }
+    delta = 0.0;
+    __syncthreads();
+    for (int e = t; e < nr * dmp; e += EM_T) Qr[e] = (r_lo + e / dmp == e % dmp) ? 1.0 : 0.0;
+    if (b == 0)
+      for (int e = t; e < n * n; e += EM_T) Hd[(e % n) + dld * (e / n)] = M.C[e];
     __syncthreads();
   }
   // Ritz values and vectors
@@ -553,35 +588,37 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
   int* order = (int*)(M.sums + kEigPart - 64);        // past the sums
   auto apply_from = [&](unsigned have, unsigned upto) {
     for (unsigned s = have; s < upto; ++s)
-      em_apply_sweep(Qr, nr, m, mp, rot + (int64_t)s * (EM_M - 1) * (EM_M / 2));
+      em_apply_sweep(Qr, nr, dm, dmp, rot + s * em_sweep_pairs(dm));
   };
   if (b == 0) {
     // scaled by a power of two so that the float angles neither overflow nor vanish
     int ex = 0;
     {
       double big = 0.0;
-      for (int j = 0; j < m; ++j) big = fmax(big, fabs(H[j + EM_LD * j]));
+      for (int j = 0; j < dm; ++j) big = fmax(big, fabs(Hd[j + dld * j]));
       if (big > 0.0 && isfinite(big)) frexp(big, &ex);
     }
     __syncthreads();
     const double sc = ldexp(1.0, -ex), un = ldexp(1.0, ex);
-    const int nn = (m + 1) & ~1;
+    const int nn = (dm + 1) & ~1;
     for (int e = t; e < nn * nn; e += EM_T) {
       const int i = e % nn, j = e / nn;
-      H[i + EM_LD * j] = (i < m && j < m) ? H[i + EM_LD * j] * sc : 0.0;
+      Hd[i + dld * j] = (i < dm && j < dm) ? Hd[i + dld * j] * sc : 0.0;
     }
     __syncthreads();
-    if (!em_jacobi(H, m, M.tol, rot, M.done, cs, pq, red) && t == 0) atomicOr(a.flags, kFlagEigNoConv);
+    const bool conv = dm > EM_M ? em_jacobi<5, EM_DLD>(Hd, dm, M.tol, rot, M.done, cs, pq, red)
+                                : em_jacobi<2, EM_LD>(Hd, dm, M.tol, rot, M.done, cs, pq, red);
+    if (!conv && t == 0) atomicOr(a.flags, kFlagEigNoConv);
     // descending order by integer keys, ties by index: a permutation whatever the values
-    for (int j = t; j < m; j += EM_T) {
-      const long long kj = em_key(H[j + EM_LD * j]);
+    for (int j = t; j < dm; j += EM_T) {
+      const long long kj = em_key(Hd[j + dld * j]);
       int rank = 0;
-      for (int l = 0; l < m; ++l) {
-        const long long kl = em_key(H[l + EM_LD * l]);
+      for (int l = 0; l < dm; ++l) {
+        const long long kl = em_key(Hd[l + dld * l]);
         rank += (kl > kj) || (kl == kj && l < j);
       }
       order[rank] = j;
-      if (rank < k) M.ev[rank] = H[j + EM_LD * j] * un - delta;
+      if (rank < k) M.ev[rank] = Hd[j + dld * j] * un - delta;
     }
   } else {
     unsigned have = 0;
@@ -604,7 +641,7 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
     if (lane == 0) *M.trace = s;
   }
   if (!em_sync(M.bar, ++nbar, B, a.flags, &abort_sh)) return;
-  for (int j = t; j < m; j += EM_T) ord[j] = __ldcg(&order[j]);
+  for (int j = t; j < dm; j += EM_T) ord[j] = __ldcg(&order[j]);
   __syncthreads();
   // per-CTA column sums of squares, largest |entry| and its row
   double* col = M.part + (int64_t)b * M.pstride;
@@ -612,14 +649,14 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
     double nrm = 0.0, best = -1.0;
     int ib = 0x7fffffff;
     for (int r = 0; r < nr; ++r) {
-      const double v = Qr[r * mp + ord[j]];
+      const double v = Qr[r * dmp + ord[j]];
       nrm = fma(v, v, nrm);
       if (fabs(v) > best) { best = fabs(v); ib = r_lo + r; }
     }
     col[j] = nrm;
     col[EM_M + j] = best;
     col[2 * EM_M + j] = ib < n ? (double)ib : (double)n;
-    col[3 * EM_M + j] = ib < n && Qr[(ib - r_lo) * mp + ord[j]] < 0.0 ? -1.0 : 1.0;
+    col[3 * EM_M + j] = ib < n && Qr[(ib - r_lo) * dmp + ord[j]] < 0.0 ? -1.0 : 1.0;
   }
   if (!em_sync(M.bar, ++nbar, B, a.flags, &abort_sh)) return;
   for (int j = w; j < k; j += EM_W) {
@@ -643,7 +680,7 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
   __syncthreads();
   for (int e = t; e < nr * k; e += EM_T) {
     const int r = e % nr, j = e / nr;
-    M.out[r_lo + r + (int64_t)n * j] = Qr[r * mp + ord[j]] * dsc[j];
+    M.out[r_lo + r + (int64_t)n * j] = Qr[r * dmp + ord[j]] * dsc[j];
   }
 }
 
@@ -667,9 +704,9 @@ bool em_split(const int* n, const int* k, int p, int nsm, size_t limit, EmSplit&
   int need[kMaxModes], sum = 0;
   for (int i = 0; i < p; ++i) {
     const int m = em_cols(n[i], k[i]), mp = (m + 7) & ~7;
-    if (em_smem(1, mp) > limit) return false;
     int rows = n[i];                         // the most rows of a CTA
-    if (em_smem(rows, mp) > limit) rows = (int)((limit - em_smem(0, mp)) / (em_smem(1, mp) - em_smem(0, mp)));
+    while (rows > 0 && em_smem(n[i], mp, rows) > limit) --rows;
+    if (rows == 0) return false;
     need[i] = (n[i] + rows - 1) / rows;
     const int want = avail > 0 ? (int)((double)avail * ((double)n[i] * n[i] / tot)) : 0;
     const int most = m == n[i] ? (n[i] + EM_W - 1) / EM_W : n[i];
@@ -686,7 +723,7 @@ bool em_split(const int* n, const int* k, int p, int nsm, size_t limit, EmSplit&
   out.smem = 0;
   for (int i = 0; i < p; ++i) {
     const int nb = out.nct[i] - 1, mp = (em_cols(n[i], k[i]) + 7) & ~7;
-    out.smem = std::max(out.smem, em_smem((n[i] + nb - 1) / nb, mp));
+    out.smem = std::max(out.smem, em_smem(n[i], mp, (n[i] + nb - 1) / nb));
   }
   return true;
 }
@@ -696,7 +733,7 @@ bool em_split(const int* n, const int* k, int p, int nsm, size_t limit, EmSplit&
 size_t eig_modes_scratch(int n, int k) {
   const size_t m = em_cols(n, k), mp = (m + 7) & ~(size_t)7;
   return (size_t)n * mp + (size_t)std::min(152, n + 1) * kEigPart + kEigPart +
-         (size_t)kEigSweeps * (EM_M - 1) * (EM_M / 2) * 2 + 8;
+         (size_t)kEigSweeps * 2 * em_sweep_pairs(n <= EM_D ? n : (int)m) + 8;
 }
 
 tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsigned* flags, cudaStream_t s) {
@@ -748,7 +785,7 @@ tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsig
     M.sums = w;
     w += kEigPart;
     M.rot = w;
-    w += (size_t)kEigSweeps * (EM_M - 1) * (EM_M / 2) * 2;
+    w += (size_t)kEigSweeps * 2 * em_sweep_pairs(M.n <= EM_D ? M.n : M.m);
     M.bar = (unsigned*)w;
     M.done = M.bar + 4;
     M.ev = pr[i].ev;
