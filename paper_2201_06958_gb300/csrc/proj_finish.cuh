@@ -55,7 +55,8 @@ struct FinArgs {
 };
 
 // Row stride of A_2 in the fused finish's shared memory: = 4 (mod 32), so that the lanes
-// of a warp (eight columns b x four i2 phases) read 32 different banks.
+// of a warp (eight columns b x four i2 phases) read 32 different banks.  Never above that of
+// N2 = FS_TE for the N2 up to FS_TE that it serves.
 __host__ __device__ constexpr int a2_stride(int N2) { return N2 + ((36 - N2 % 32) % 32); }
 
 // Four consecutive values in shared memory (16-byte aligned).
@@ -519,16 +520,23 @@ struct Finish {
     count_launch();
   }
 
+  // The limit is set once, to the most that any launch needs (FS_JMAX outputs, A_2 of 32 ranks):
+  // with each launch's own need another thread's smaller one could lower it just before this
+  // launch, and a need of 48 KB less the static part and more was left at the default.
+  static constexpr size_t smem_max = sizeof(T) * (FS_SC * FS_JMAX + FS_SC * FS_TE + (size_t)a2_stride(FS_TE) * kMaxRank);
+  template <int NQ, int JB>
+  void launch_sk_nq(int grid) {
+    static const cudaError_t once = cudaFuncSetAttribute(
+        k_finish_sk<T, NQ, JB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+    (void)once;
+    launch_pdl(k_finish_sk<T, NQ, JB>, grid, smem);
+  }
   template <int JB>
   void launch_sk(int grid) {
-    auto go = [&](auto kern) {
-      if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      launch_pdl(kern, grid, smem);
-    };
-    if (nqm <= 1) go(k_finish_sk<T, 1, JB>);
-    else if (nqm <= 2) go(k_finish_sk<T, 2, JB>);
-    else if (nqm <= 4) go(k_finish_sk<T, 4, JB>);
-    else go(k_finish_sk<T, 8, JB>);
+    if (nqm <= 1) launch_sk_nq<1, JB>(grid);
+    else if (nqm <= 2) launch_sk_nq<2, JB>(grid);
+    else if (nqm <= 4) launch_sk_nq<4, JB>(grid);
+    else launch_sk_nq<8, JB>(grid);
   }
 
   void launch(int nsplit) {
