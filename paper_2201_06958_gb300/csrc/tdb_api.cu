@@ -265,7 +265,12 @@ struct tdb_batch {
   cudaEvent_t fork = nullptr;
   std::vector<cudaEvent_t> join;
   cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-  std::vector<uint64_t> keys[2];
+  struct Key {                       // what a member's recorded step depends on
+    uint64_t step;
+    const void* slot[2];
+    bool operator==(const Key& o) const { return step == o.step && slot[0] == o.slot[0] && slot[1] == o.slot[1]; }
+  };
+  std::vector<Key> keys[2];
   long long gcount[2] = {0, 0};
   bool broken = false;
   int64_t replays = 0, records = 0;
@@ -2356,7 +2361,11 @@ tdb_status tdb_batch_push(tdb_batch* b, int parity, tdb_step_info* infos) {
   }
   for (size_t i = 0; i < n; ++i) prepare_step(b->m[i]);
   bool fresh = b->gexec[parity] != nullptr && b->keys[parity].size() == n;
-  for (size_t i = 0; i < n && fresh; ++i) fresh = b->keys[parity][i] == graph_key(b->m[i]);
+  auto key = [&](size_t i) {
+    const tdb_ctx* c = b->m[i];
+    return tdb_batch::Key{graph_key(c), {c->slot[0], c->slot[1]}};
+  };
+  for (size_t i = 0; i < n && fresh; ++i) fresh = b->keys[parity][i] == key(i);
   if (!fresh) {
     if (b->gexec[parity]) cudaGraphExecDestroy(b->gexec[parity]);
     b->gexec[parity] = nullptr;
@@ -2376,7 +2385,7 @@ tdb_status tdb_batch_push(tdb_batch* b, int parity, tdb_step_info* infos) {
       return worst;
     }
     b->keys[parity].resize(n);
-    for (size_t i = 0; i < n; ++i) b->keys[parity][i] = graph_key(b->m[i]);
+    for (size_t i = 0; i < n; ++i) b->keys[parity][i] = key(i);
     b->records++;
   }
   b->replays++;
