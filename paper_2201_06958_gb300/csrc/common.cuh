@@ -40,6 +40,24 @@ __device__ __forceinline__ T block_sum(T v, T* sh) {
   return r;
 }
 
+// A sum of floats carried in two (Knuth's TwoSum): what double holds of it, without the 64 cycles
+// a warp pays per double instruction.
+struct FloatPair {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x, float x_lo = 0.f) {
+    const float s = hi + x, b = s - hi;
+    lo += ((hi - (s - b)) + (x - b)) + x_lo;
+    hi = s;
+  }
+  // adds (wh + wl) x, the product's rounding included
+  __device__ __forceinline__ void add_product(float wh, float wl, float x) {
+    const float p = wh * x;
+    add(p, fmaf(wl, x, fmaf(wh, x, -p)));
+  }
+  // (an overflowed sum leaves its error term undefined)
+  __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
+};
+
 // ---------------------------------------------------------------------------
 // Per-mode descriptors passed by value to small-matrix kernels
 // ---------------------------------------------------------------------------

@@ -86,7 +86,8 @@ template void launch_cast<double, double>(const double*, double*, int64_t, cudaS
 // weighted squared norm (Eq. 2.2 with the quadrature of Eq. 2.17) in one pass, for the mode
 // products' route of the projection:
 //   sum_i w_1(i_1) ... w_p(i_p) out[i]^2
-// A warp per mode-1 column, the column weights prod_{m>1} w_m from `wcol`.  Deterministic:
+// A warp per mode-1 column; a lane's products of a column are added in double (float: in a pair of
+// floats) and weighted by the column's prod_{m>1} w_m in double (double: from `wcol`).  Deterministic:
 // warp and CTA partials in a fixed order, added by the last CTA to finish (`counter` is zero
 // before and after).  64^3 double from a cold cache: 12.7 us, as difference, norm and
 // sum apart 23.7 us.
@@ -94,7 +95,8 @@ template void launch_cast<double, double>(const double*, double*, int64_t, cudaS
 template <typename T>
 __global__ void __launch_bounds__(256) k_diff_norm(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out,
                                                    int N1, unsigned ncol, T scale, const T* __restrict__ w1,
-                                                   const T* __restrict__ wcol, double* __restrict__ partial,
+                                                   const T* __restrict__ wcol, WeightView wv,
+                                                   double* __restrict__ partial,
                                                    unsigned* __restrict__ counter, double* __restrict__ norm2,
                                                    unsigned* flags) {
   __shared__ double sh[32];
@@ -105,14 +107,26 @@ __global__ void __launch_bounds__(256) k_diff_norm(const T* __restrict__ a, cons
   bool bad = false;
   for (unsigned c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < ncol; c += nw) {
     const size_t o = (size_t)N1 * c;
-    T s = T(0);
+    typename std::conditional<sizeof(T) == 4, FloatPair, double>::type s{};
     for (int i = lane; i < N1; i += 32) {
       const T d = (a[o + i] - b[o + i]) * scale;
       out[o + i] = d;
       bad |= !isfinite(d);
-      s = fma(w1[i] * d, d, s);
+      if constexpr (sizeof(T) == 4) s.add((w1[i] * d) * d);
+      else s = fma(w1[i] * d, d, s);
     }
-    acc = fma((double)wcol[c], (double)s, acc);
+    if constexpr (sizeof(T) == 4) {
+      double wc = 1.0;
+      unsigned rem = c;
+      for (int m = 1; m < wv.p; ++m) {
+        const unsigned nm = (unsigned)wv.N[m];
+        wc *= wv.w[m][rem % nm];
+        rem /= nm;
+      }
+      acc = fma(wc, s.value(), acc);
+    } else {
+      acc = fma(wcol[c], s, acc);
+    }
   }
   acc = block_sum(acc, sh);
   if (bad && flags) atomicOr(flags, kFlagNonFinite);
@@ -135,15 +149,17 @@ __global__ void __launch_bounds__(256) k_diff_norm(const T* __restrict__ a, cons
 
 template <typename T>
 void launch_diff_norm(const T* a, const T* b, T* out, int N1, int64_t ncol, T scale, const T* w1, const T* wcol,
+                      const WeightView& wv,
                       double* partial, unsigned* counter, int nblocks, double* norm2, unsigned* flags, cudaStream_t s) {
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(nblocks, (ncol + 7) / 8));
-  k_diff_norm<T><<<blocks, 256, 0, s>>>(a, b, out, N1, (unsigned)ncol, scale, w1, wcol, partial, counter, norm2, flags);
+  k_diff_norm<T><<<blocks, 256, 0, s>>>(a, b, out, N1, (unsigned)ncol, scale, w1, wcol, wv, partial, counter, norm2,
+                                     flags);
   count_launch();
 }
 template void launch_diff_norm<float>(const float*, const float*, float*, int, int64_t, float, const float*,
-                                      const float*, double*, unsigned*, int, double*, unsigned*, cudaStream_t);
+                                      const float*, const WeightView&, double*, unsigned*, int, double*, unsigned*, cudaStream_t);
 template void launch_diff_norm<double>(const double*, const double*, double*, int, int64_t, double, const double*,
-                                       const double*, double*, unsigned*, int, double*, unsigned*, cudaStream_t);
+                                       const double*, const WeightView&, double*, unsigned*, int, double*, unsigned*, cudaStream_t);
 
 // Exact error of Eq. 2.20 without materialising V^TDB: with H = T x_2 U_2 ... x_p U_p
 // (r_1 x N_2 x ... x N_p), every mode-1 column of the reconstruction is U_1 H[:, c].

@@ -128,6 +128,7 @@ void launch_state_pack(const StateViews& v, double* out, cudaStream_t s);
 template <typename Ts, typename Td> void launch_cast(const Ts* a, Td* b, int64_t n, cudaStream_t s);
 template <typename T>
 void launch_diff_norm(const T* a, const T* b, T* out, int N1, int64_t ncol, T scale, const T* w1, const T* wcol,
+                      const WeightView& wv,
                       double* partial, unsigned* counter, int nblocks, double* norm2, unsigned* flags, cudaStream_t s);
 template <typename T>
 void launch_recon_err(const T* V, const T* U1, const T* H, int r1, int N1, int64_t ncol, const T* w1, const T* wcol,

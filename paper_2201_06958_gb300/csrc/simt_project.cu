@@ -13,6 +13,8 @@
 // products that contract S points took 428 us; 126^3 double at (5, 5, 5): 87 us against 251
 // us.  One CTA of eight warps per SM with the next rows prefetched into registers measured the
 // same as three of four without.
+#include <type_traits>
+
 #include "proj_finish.cuh"
 #include "simt_project.h"
 
@@ -69,7 +71,7 @@ constexpr int sp_warp_elems(int rb) {
 
 template <typename T, int RB>
 constexpr size_t sp_smem(int ti2) {
-  return sizeof(T) * ((size_t)RB * SP_T1 + (size_t)ti2 * RB * kSpDup<T> + ti2 + (size_t)RB * ti2 +
+  return sizeof(T) * ((size_t)RB * SP_T1 + (size_t)ti2 * RB * kSpDup<T> + (size_t)ti2 * kSpDup<T> + (size_t)RB * ti2 +
                       (size_t)SP_WARPS * sp_warp_elems<T>(RB));
 }
 
@@ -100,7 +102,7 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
   T* Z1s = A2s + ti2 * RB * kSpDup<T>;         // [RB][ti2]
   T* Z2s = Z1s + RB * ti2;                     // [4][RB][128]
   constexpr int ZW = sp_warp_elems<T>(RB);     // a warp's part of it
-  T* w2s = Z2s + SP_WARPS * ZW;                // [ti2]
+  T* w2s = Z2s + SP_WARPS * ZW;                // [ti2] (float: the weight in two floats)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) fin_dep_launch();
   const int nq12 = P.nq1 * P.nq2;
@@ -122,7 +124,15 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
 #pragma unroll
     for (int u = 0; u < kSpDup<T>; ++u) A2s[(x * RB + b) * kSpDup<T> + u] = a;
   }
-  for (int x = tid; x < ti2; x += SP_THREADS) w2s[x] = b2 + x < N2 ? (T)P.w2[b2 + x] : T(0);
+  for (int x = tid; x < ti2; x += SP_THREADS) {
+    const double w = b2 + x < N2 ? P.w2[b2 + x] : 0.0;
+    if constexpr (sizeof(T) == 4) {
+      w2s[2 * x] = (float)w;
+      w2s[2 * x + 1] = (float)(w - (double)(float)w);
+    } else {
+      w2s[x] = w;
+    }
+  }
   T w1r[4];
   bool in1[4];
 #pragma unroll
@@ -193,7 +203,9 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
     for (int b = 0; b < RB; ++b)
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc2[b][j] = T(0);
-    T nrm = T(0);
+    // ||dV||_W^2 of this lane's points of the slice: the four points of a row in T, everything
+    // after that in double (float: in a pair of floats)
+    typename std::conditional<sizeof(T) == 4, FloatPair, double>::type nrm{};
     for (int grp = 0; grp < ngrp; ++grp) {
       const int x0 = warp * wrows + grp * G;               // first row of the group within the tile
       T d[G][4];
@@ -212,7 +224,10 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
             q = fma(w1r[j] * d[g][j], d[g][j], q);
           }
           odd |= expo_bits(q) >= kExpInf<T>;
-          if (grp * G + g < wrows) nrm = fma(w2s[x0 + g], q, nrm);
+          if (grp * G + g < wrows) {
+            if constexpr (sizeof(T) == 4) nrm.add_product(w2s[2 * (x0 + g)], w2s[2 * (x0 + g) + 1], q);
+            else nrm = fma(w2s[x0 + g], q, nrm);
+          }
         }
         if (odd) {                                         // ... by a difference, or only by its square
 #pragma unroll
@@ -337,7 +352,10 @@ __global__ void __launch_bounds__(SP_THREADS, kSpPerSm<T>) k_sp_project(SpParams
         }
       }
     }
-    if (r0 == 0) acc_norm += P.wsl[sl] * (double)nrm;
+    if (r0 == 0) {
+      if constexpr (sizeof(T) == 4) acc_norm += P.wsl[sl] * nrm.value();
+      else acc_norm += P.wsl[sl] * nrm;
+    }
     // the slice's partials leave: Z1 as it is, Z2 summed over the warps in order
     __syncwarp();
 #pragma unroll

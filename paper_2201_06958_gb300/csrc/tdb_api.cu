@@ -1201,7 +1201,7 @@ tdb_status project_step(tdb_ctx* ctx, const Tc* Vn, const Tc* Vfrom, double scal
                        ctx->flags, s, evm, ctx->err, (Tc)scale));
   } else {
     launch_diff_norm<Tc>(Vn, Vfrom, (Tc*)ctx->dV, (int)ctx->N[0], ctx->S / ctx->N[0], (Tc)scale,
-                         (const Tc*)ctx->w1T, (const Tc*)ctx->wcolT, ctx->npart, ctx->redcnt + 1, ctx->nblk,
+                         (const Tc*)ctx->w1T, (const Tc*)ctx->wcolT, weight_view(ctx), ctx->npart, ctx->redcnt + 1, ctx->nblk,
                          &ctx->rb_dev->dv2, ctx->flags, s);
     CHECK_LAUNCH();
     TRY(project_tree<Tc>(ctx, (const Tc*)ctx->dV, evm));
