@@ -281,9 +281,9 @@ __device__ void em_apply_sweep(double* A, int nr, int m, int mp, const double2* 
 // Cyclic Jacobi on the symmetric H (m x m, full, ld LDH; row and column nn - 1 zero for odd
 // m; NB blocks of 2 x 2 a thread at most) by this CTA, the rotations of sweep s written to rot[s]
 // and announced through *done (s + 1; the last one with kEmLast set).  Every pair rotates: the block's columns are not
-// sorted, so a wanted Ritz value can sit in its tail.  The angle's tangent is float (a rotation by it
-// leaves 1e-7 of the pair's off-diagonal, which the next sweep takes), its cosine and sine
-// double.  The 2 x 2 blocks above the diagonal are updated and mirrored.  Ends when the
+// sorted, so a wanted Ritz value can sit in its tail.  The angle's tangent is a
+// float root of b t^2 + (a_qq - a_pp) t - b = 0 with one Newton step in double, its cosine and
+// sine are double.  The 2 x 2 blocks above the diagonal are updated and mirrored.  Ends when the
 // off-diagonal mass is below tol^2 of the diagonal's, or at the rounding
 // floor (a sweep after the third that does not quarter it).
 constexpr unsigned kEmLast = 0x80000000u;
@@ -340,7 +340,10 @@ __device__ bool em_jacobi(double* H, int m, double tol, double2* rot, unsigned* 
           const float theta = (float)(aqq - app) / (2.f * fpq);
           const float at = fabsf(theta);
           const float root = at < 1e18f ? sqrtf(fmaf(at, at, 1.f)) : at;
-          const double tt = (double)copysignf(1.f / (at + root), theta);
+          const float t0 = copysignf(1.f / (at + root), theta);
+          const double diff = aqq - app;
+          const float slope = fmaf(2.f * fpq, t0, (float)diff);          // (both terms of t0's sign)
+          const double tt = fma(-fma(fma(apq, (double)t0, diff), (double)t0, -apq), (double)(1.f / slope), (double)t0);
           c = drsqrt(fma(tt, tt, 1.0));
           s = tt * c;
         }
