@@ -733,9 +733,14 @@ bool em_split(const int* n, const int* k, int p, int nsm, size_t limit, EmSplit&
 
 }  // namespace
 
+// A CTA's partial sums: the block's m x m and its upper triangle, or four statistics a column.
+// (Even: the rotations that follow are read 16 bytes at a time.)
+static int em_pstride(int m) { return (std::max(m * (m + 1) / 2 + m * m, 4 * EM_M) + 1) & ~1; }
+static_assert(EM_M * (EM_M + 1) / 2 + EM_M * EM_M + 64 <= kEigPart && EM_D <= 128, "the sums, and the order after them");
+
 size_t eig_modes_scratch(int n, int k) {
   const size_t m = em_cols(n, k), mp = (m + 7) & ~(size_t)7;
-  return (size_t)n * mp + (size_t)std::min(152, n + 1) * kEigPart + kEigPart +
+  return (size_t)n * mp + (size_t)std::min(152, n + 1) * em_pstride((int)m) + kEigPart +
          (size_t)kEigSweeps * 2 * em_sweep_pairs(n <= EM_D ? n : (int)m) + 8;
 }
 
@@ -783,8 +788,8 @@ tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsig
     M.Q = w;
     w += (size_t)M.n * M.mp;
     M.part = w;
-    M.pstride = kEigPart;
-    w += (size_t)std::min(152, M.n + 1) * kEigPart;
+    M.pstride = em_pstride(M.m);
+    w += (size_t)std::min(152, M.n + 1) * M.pstride;
     M.sums = w;
     w += kEigPart;
     M.rot = w;

@@ -193,7 +193,7 @@ void launch_gram_weighted(const float* Vw, int64_t L, int64_t Nn, int64_t Q, dou
 constexpr int kEigBlock = 50;              // most columns of a block: 16 more than the wanted pairs (<= 34)
 constexpr int kEigSweeps = 16;             // Jacobi sweeps at most
 constexpr int kEigWhole = 96;              // most points of a mode that can be solved whole
-constexpr int kEigPart = 3840;             // a CTA's partial sums: block^2 and its upper triangle, and 64
+constexpr int kEigPart = 3840;             // a group's sums: block^2 and its upper triangle, and 64
 struct EigProblem {
   const double* C;                         // n x n, symmetric
   int n, k;                                // k wanted pairs, k <= min(n, 34)

@@ -417,14 +417,45 @@ __global__ void k_slice_weights(int p, const double* w3, int N3, const double* w
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-// Split partials a plan keeps: (FS_CTAS + tiles) x 256 x J values bound nsplit x tiles x 256 x J
-// for the split count the launch picks.
+// Split partials a tuned plan keeps: (FS_CTAS + tiles) x 256 x J values bound nsplit x tiles x 256 x J
+// for the split counts that the tuner tries first.
 inline size_t finish_part_elems(int p, const int64_t* N, const int* cap) {
   const int jmax = p == 2 ? 1 : (p == 3 ? cap[2] : cap[2] * cap[3]);
   const int64_t ntmax = ((int64_t)cap[0] * N[1] + FS_TE - 1) / FS_TE + ((int64_t)N[0] * cap[1] + FS_TE - 1) / FS_TE;
   return (size_t)(FS_CTAS + ntmax) * FS_TE * jmax;
 }
 inline int finish_outputs(int p, const int* r) { return p == 2 ? 1 : (p == 3 ? r[2] : r[2] * r[3]); }
+
+// The tiling of a finish: W inside it (its first-side CTAs hold whole i2 columns), the elements of
+// a first-side CTA, the tiles of both sides.
+struct FinTiles {
+  bool fuse_w;
+  int te1, nt1, nt2;
+};
+inline FinTiles finish_tiles(int p, const int64_t* N, const int* r) {
+  FinTiles t;
+  t.fuse_w = p >= 3 && N[1] <= FS_TE;
+  t.te1 = t.fuse_w ? (int)N[1] * (FS_TE / (int)N[1]) : FS_TE;
+  t.nt1 = (int)((r[0] * N[1] + t.te1 - 1) / t.te1);
+  t.nt2 = (int)((N[0] * r[1] + FS_TE - 1) / FS_TE);
+  return t;
+}
+// A split takes at least 16 slices in float and 4 in double, whose arithmetic (64 cycles per
+// warp instruction and sub-partition) is worth more SMs than the split's partials cost.
+template <typename T>
+constexpr int kFinMinSlices = sizeof(T) == 4 ? FS_SC : 4;
+// Split partials (values) of the launches that aim at FS_CTAS CTAs, at any ranks up to `cap`: none
+// where the slices do not split, else at most FS_CTAS tiles (or all the splits' tiles) of at most
+// FS_JMAX outputs.
+template <typename T>
+size_t finish_split_elems(int p, const int64_t* N, const int* cap) {
+  int64_t ns = 1;
+  for (int n = 2; n < p; ++n) ns *= N[n];
+  const int64_t most = std::min<int64_t>(FS_SPLIT_MAX, ns / kFinMinSlices<T>);
+  if (most < 2) return 0;
+  const FinTiles t = finish_tiles(p, N, cap);
+  return (size_t)std::min<int64_t>(FS_CTAS, most * (t.nt1 + t.nt2)) * FS_TE * std::min(finish_outputs(p, cap), FS_JMAX);
+}
 
 // The finish of one projection: Y_1, Y_2 (and Z1) from the tile partials, the slices
 // contracted with B = A_3 (x A_4); then Y_3 (three modes) or W = Z1 x_2 A_2^T (four modes).
@@ -451,11 +482,11 @@ struct Finish {
     nslice = 1;
     for (int n = 2; n < p; ++n) nslice *= (int)N[n];
     J = finish_outputs(p, r);
-    // W = Z1 x_2 A_2^T inside the finish when its first-side CTAs can hold whole i2 columns
-    fuse_w = p >= 3 && N2 <= FS_TE;
-    const int te1 = fuse_w ? N2 * (FS_TE / N2) : FS_TE;
-    nt1 = (int)(((int64_t)r[0] * N2 + te1 - 1) / te1);
-    nt2 = (int)(((int64_t)N1 * r[1] + FS_TE - 1) / FS_TE);
+    const FinTiles t = finish_tiles(p, N, r);
+    fuse_w = t.fuse_w;
+    const int te1 = t.te1;
+    nt1 = t.nt1;
+    nt2 = t.nt2;
     nqm = std::max(nq1, nq2);
     memset(&f, 0, sizeof(f));
     f.Z1p = z1p;
@@ -489,15 +520,11 @@ struct Finish {
     smem = sizeof(T) * (FS_SC * ((J + 3) & ~3) + (fuse_w ? FS_SC * FS_TE + (size_t)a2_stride(N2) * r[1] : 0));
   }
 
-  // A split takes at least 16 slices in float and 4 in double, whose arithmetic (64 cycles per
-  // warp instruction and sub-partition) is worth more SMs than the split's partials cost.
-  static constexpr int min_slices = sizeof(T) == 4 ? FS_SC : 4;
-
   // splits per tile: the grid stays within the target (whole waves of resident CTAs: two
   // per SM), at least one split
   int nsplit_for(int target) const {
     int ns = (int)std::max<int64_t>(1, target / (nt1 + nt2));
-    ns = std::min({ns, std::max(1, nslice / min_slices), FS_SPLIT_MAX});
+    ns = std::min({ns, std::max(1, nslice / kFinMinSlices<T>), FS_SPLIT_MAX});
     while (ns > 1 && (size_t)ns * (nt1 + nt2) * FS_TE * J > part_cap) --ns;
     return ns;
   }

@@ -420,11 +420,12 @@ int64_t slices(int p, const int64_t* N) {
   return v;
 }
 
-// Most tiles along mode 2 that sp_shape makes.
+// Most tiles along mode 2 that sp_shape makes: with one rank block (more blocks fill the SMs with
+// taller tiles).
 template <typename T>
-int64_t sp_tiles2_max(int64_t N2) {
-  const int low = SP_WARPS * SpCfg<T>::G;
-  return std::max<int64_t>((N2 + 127) / 128, std::min<int64_t>((N2 + low - 1) / low, FS_NQ_MAX));
+int64_t sp_tiles2_max(const int64_t* N, int64_t nslice) {
+  const int r[2] = {1, 1};
+  return sp_shape<T>(N, r, nslice).nq2;
 }
 
 template <typename T, int RB>
@@ -442,20 +443,23 @@ void sp_launch(const SpParams<T>& P, const SpShape& h, int vec, cudaStream_t s) 
 
 bool sp_supported(int p, const int* r) { return finish_outputs(p, r) <= FS_JMAX; }
 
+void sp_carve_weights(SpPlan& plan, Carver& cv, int p, const int64_t* N) {
+  plan.wsl = cv.take<double>((size_t)slices(p, N));
+}
+
 template <typename T>
-void sp_carve(SpPlan& plan, Carver& cv, int p, const int64_t* N, const int* cap) {
+void sp_carve_pass(SpPlan& plan, Carver& cv, int p, const int64_t* N, const int* cap) {
   const int64_t ns = slices(p, N);
-  const int64_t nq1 = (N[0] + SP_T1 - 1) / SP_T1, nq2 = sp_tiles2_max<T>(N[1]);
+  const int64_t nq1 = (N[0] + SP_T1 - 1) / SP_T1, nq2 = sp_tiles2_max<T>(N, ns);
   plan.z1p = cv.take<T>((size_t)(nq1 * ns * N[1] * cap[0]));
   plan.z2p = cv.take<T>((size_t)(nq2 * ns * N[0] * cap[1]));
-  plan.wsl = cv.take<double>((size_t)ns);
   plan.npart = cv.take<double>((size_t)std::max<int64_t>(kSpCtas<T>, nq1 * nq2) * SP_WARPS);
-  plan.fpart_cap = finish_part_elems(p, N, cap);
+  plan.fpart_cap = finish_split_elems<T>(p, N, cap);
   plan.fpart = cv.take<T>(plan.fpart_cap);
   plan.wrest = p == 4 ? cv.take<T>((size_t)cap[0] * cap[1] * ns) : nullptr;
 }
-template void sp_carve<float>(SpPlan&, Carver&, int, const int64_t*, const int*);
-template void sp_carve<double>(SpPlan&, Carver&, int, const int64_t*, const int*);
+template void sp_carve_pass<float>(SpPlan&, Carver&, int, const int64_t*, const int*);
+template void sp_carve_pass<double>(SpPlan&, Carver&, int, const int64_t*, const int*);
 
 void sp_prepare(SpPlan& plan, int p, const int64_t* N, const double* const* w, cudaStream_t s) {
   const int64_t ns = slices(p, N);

@@ -19,8 +19,10 @@ struct SpPlan {
 
 // Whether sp_project takes these ranks (r_3 r_4 of four modes at most 128).
 bool sp_supported(int p, const int* r);
+// The slice weights, kept for the context's life, and the buffers of a pass, free between passes.
+void sp_carve_weights(SpPlan& plan, Carver& cv, int p, const int64_t* N);
 template <typename T>
-void sp_carve(SpPlan& plan, Carver& cv, int p, const int64_t* N, const int* cap);
+void sp_carve_pass(SpPlan& plan, Carver& cv, int p, const int64_t* N, const int* cap);
 // The slice weights, once per context (before any capture).
 void sp_prepare(SpPlan& plan, int p, const int64_t* N, const double* const* w, cudaStream_t s);
 // Y_n of dV = dscale (Vn - Vp) (Eqs. 2.15, 2.16; dscale a power of two) and ||dV||_W^2 into

@@ -367,6 +367,16 @@ int rank_from_core(const double* s2, int r, double eps, double gamma_th) {
   return r;
 }
 
+// Whether a context without the tensor cores projects in one fused pass (simt_project.cu).
+// Measured per projection, fused against mode products: float 256 x 128 x 512 at ranks
+// (11, 8, 16) 60 against 430 us, double 126^3 at (5, 5, 5) 100 against 410 us.  Small double
+// tensors keep the mode products: at 64^3 the pass is latency-bound on both routes (12 us
+// apart), and an error 1e-8 of ||V||_W there rests on the last bits of the double state,
+// which the mode products' order of summation has always given.
+constexpr int64_t kSpDoubleMin = (int64_t)1 << 19;
+bool sp_context(const tdb_ctx* c) { return c->prec != TDB_BF16_TTM && (!c->f64 || c->S >= kSpDoubleMin); }
+bool sp_route(const tdb_ctx* c) { return sp_context(c) && sp_supported(c->p, c->r); }
+
 // ---------------------------------------------------------------------------
 // Workspace layout
 // ---------------------------------------------------------------------------
@@ -391,12 +401,6 @@ void carve(tdb_ctx* c, Carver& cv) {
     c->Y[n] = cv.take<char>(ysz * tsz);
   }
   c->T = cv.take<double>(Rprod);
-  {
-    int64_t tot = Rprod;
-    for (int n = 0; n < p; ++n) tot += c->N[n] * c->cap[n];
-    c->packed = cv.take<double>(tot);
-  }
-  c->T2 = cv.take<double>(Rprod);
   c->Tbak = cv.take<double>(Rprod);
   c->Tcore = c->f64 ? (void*)c->T : (void*)cv.take<char>(Rprod * tsz);
   c->dS = cv.take<char>(Rprod * tsz);
@@ -406,9 +410,6 @@ void carve(tdb_ctx* c, Carver& cv) {
   tree = std::max<int64_t>(tree, Rprod);
   c->tree_elems = tree;
   c->ping = cv.take<char>(tree * tsz);
-  c->pong = cv.take<char>(tree * tsz);
-  c->dV = cv.take<char>(c->S * tsz);
-  c->rec = cv.take<char>(c->S * tsz);
   c->G = cv.take<double>(p * kMaxRank * kMaxRank);
   c->Ginv = cv.take<double>(p * kMaxRank * kMaxRank);
   c->Ginvf = c->f64 ? nullptr : cv.take<float>(p * kMaxRank * kMaxRank);
@@ -436,7 +437,35 @@ void carve(tdb_ctx* c, Carver& cv) {
   c->rb_dev = cv.take<Readback>(1);
   c->est_dev = cv.take<EstState>(1);
   c->flags = &c->rb_dev->flags;
-  // HOSVD scratch (sized by the Gram dimension: N_n, or the short side of a long mode)
+  // What nothing reads after the call or the launch that wrote it: four sets of buffers in the same
+  // place, as no two of them are ever in use at once.  (Apart they made up to ten times the rest: double 20^4 at ranks up to 20.)
+  const size_t shared = cv.off;
+  size_t shared_end = shared;
+  auto close = [&] {
+    shared_end = std::max(shared_end, cv.off);
+    cv.off = shared;
+  };
+  // a packed state on its way from or to the host
+  int64_t packed = Rprod;
+  for (int n = 0; n < p; ++n) packed += c->N[n] * c->cap[n];
+  c->packed = cv.take<double>(packed);
+  close();
+  // the update's core between its phases
+  c->T2 = cv.take<double>(Rprod);
+  close();
+  // the fused projection pass
+  if (sp_context(c)) {
+    if (c->f64) sp_carve_pass<double>(c->sp, cv, c->p, c->N, c->cap);
+    else sp_carve_pass<float>(c->sp, cv, c->p, c->N, c->cap);
+  }
+  close();
+  // mode products (projection, column factors of the error and the reconstruction, HOSVD) and
+  // the HOSVD.  The difference is formed where ranks up to the caps can take the mode products;
+  // the tensor-core projection has its four-mode scratch there.  Float types weight the data.
+  c->pong = cv.take<char>(tree * tsz);
+  c->dV = sp_context(c) && sp_supported(p, c->cap) ? nullptr : (void*)cv.take<char>(c->S * tsz);
+  c->rec = c->f64 ? nullptr : (void*)cv.take<char>(c->S * tsz);
+  // (sized by the Gram dimension: N_n, or the short side of a long mode)
   if (c->f64) {
     const int ntile = (int)((Ng + 31) / 32);
     c->wpart_cap = std::max<size_t>((size_t)(ntile * (ntile + 1) / 2) * 8 * 1024, (size_t)152 * 64 * 64);
@@ -460,6 +489,9 @@ void carve(tdb_ctx* c, Carver& cv) {
   for (int n = 0; n < p; ++n) kmax = std::max(kmax, c->kcap[n]);
   c->Zs = cv.take<double>(Ng * kmax);
   c->wq = cv.take<double>(2 * Ng);
+  close();
+  cv.off = shared_end;
+  if (sp_context(c)) sp_carve_weights(c->sp, cv, c->p, c->N);
   c->mlpP = cv.take<float>(MLP_NPARAM);
   c->mlpNorm = cv.take<float>(2 * MLP_F + 2);
   c->mlpM = cv.take<float>(MLP_NPARAM);
@@ -471,8 +503,6 @@ void carve(tdb_ctx* c, Carver& cv) {
   c->trX = cv.take<float>((size_t)c->tr_cap * MLP_F);
   c->trT = cv.take<float>(c->tr_cap);
   if (c->prec == TDB_BF16_TTM) tc_carve(c->tc, cv, c->p, c->N, c->cap);
-  else if (c->f64) sp_carve<double>(c->sp, cv, c->p, c->N, c->cap);
-  else sp_carve<float>(c->sp, cv, c->p, c->N, c->cap);
 }
 
 tdb_status validate(const tdb_config* cfg, std::string& err) {
@@ -545,17 +575,6 @@ WeightView weight_view(const tdb_ctx* c) {
     wv.w[n] = n < c->p ? c->w[n] : nullptr;
   }
   return wv;
-}
-
-// Whether a context without the tensor cores projects in one fused pass (simt_project.cu).
-// Measured per projection, fused against mode products: float 256 x 128 x 512 at ranks
-// (11, 8, 16) 60 against 430 us, double 126^3 at (5, 5, 5) 100 against 410 us.  Small double
-// tensors keep the mode products: at 64^3 the pass is latency-bound on both routes (12 us
-// apart), and an error 1e-8 of ||V||_W there rests on the last bits of the double state,
-// which the mode products' order of summation has always given.
-constexpr int64_t kSpDoubleMin = (int64_t)1 << 19;
-bool sp_route(const tdb_ctx* c) {
-  return !c->use_tc && sp_supported(c->p, c->r) && (!c->f64 || c->S >= kSpDoubleMin);
 }
 
 // ---------------------------------------------------------------------------
@@ -1710,7 +1729,7 @@ tdb_status common_init(tdb_ctx** out, const tdb_config* cfg, void* ws, size_t ws
     launch_weights_T<double>(weight_view(ctx), (double*)ctx->w1T, (double*)ctx->wcolT, ctx->stream);
   else
     launch_weights_T<float>(weight_view(ctx), (float*)ctx->w1T, (float*)ctx->wcolT, ctx->stream);
-  if (!ctx->use_tc) sp_prepare(ctx->sp, ctx->p, ctx->N, (const double* const*)ctx->w, ctx->stream);
+  if (sp_context(ctx)) sp_prepare(ctx->sp, ctx->p, ctx->N, (const double* const*)ctx->w, ctx->stream);
   memset(&ctx->est, 0, sizeof(ctx->est));
   ctx->est.last_log_eps = -30.0;
   ctx->est.max_skip = std::max(1, ctx->cfg.error_every);
