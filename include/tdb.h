@@ -299,12 +299,13 @@ typedef struct tdb_profile {
   double ms_error;            /* exact error (Eq. 2.20) or its estimate */
   double ms_control;          /* rank control including HOSVD re-initialisations (host clock) */
   int64_t launches_main;      /* launches of the main projection kernel */
-  int64_t update_phases;      /* entries of us_update_phase in use (6 + number of modes) */
+  int64_t update_phases;      /* entries of us_update_phase in use: seven */
   double us_update_phase[12]; /* microseconds summed over the timed steps, per phase of the
                                  fused update kernel (device global timer at its grid barriers):
                                  rows M/X/P with dS, rows U'/C, Cholesky-QR factors with rows
                                  U'', core products of modes 1 and 2, of modes 3..p, Gram
-                                 partials, Gram finish; the entries after these are zero */
+                                 partials, Gram finish (next to zero where it is a launch of its
+                                 own, beside the error); the entries after these are zero */
   double us_project_span;     /* TDB_BF16_TTM: microseconds summed over the timed steps from the
                                  first CTA's start to the last CTA's end of the main projection
                                  kernel (device global timer); the CUDA-event time of

@@ -1115,7 +1115,7 @@ __global__ void __launch_bounds__(UPD_THREADS, 1) k_update(UpdArgs a) {
   if (threadIdx.x == 0) abort_sh = 0;
   __syncthreads();
   __shared__ unsigned long long st_sh[16];
-  int nst = 0;
+  int nst = 0;                             // kUpdPhases at the end, whatever p
   unsigned nbar = 0;
   stamp(st_sh, a.stamps, 0);
   const int p = a.d.p;

@@ -170,6 +170,9 @@ void launch_orthonormalize(RowArgs& a, double* R, double* Rinv, unsigned* flags,
 // CTAs that hold all of dS = Y_2 x_2 A_2^T at once (eight threads of 1024 per element)
 __host__ __device__ inline int64_t update_ds_ctas(int64_t rprod) { return (rprod + 127) / 128; }
 
+// Phases that a profiled update times: those of the kernel (k_update.cu), whatever the modes.
+constexpr int kUpdPhases = 7;
+
 // k_update.cu: a.bar must hold zero
 template <typename Tc>
 tdb_status launch_update(UpdArgs& a, int grid_hint, cudaStream_t s);

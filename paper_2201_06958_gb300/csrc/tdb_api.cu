@@ -2150,7 +2150,7 @@ tdb_status tdb_get_profile(tdb_ctx* ctx, tdb_profile* out) {
   CK(cudaStreamSynchronize(ctx->stream));
   ctx->pacc.us_project_span = 1e-3 * (double)sp[2];
   ctx->pacc.spans = (int64_t)sp[3];
-  ctx->pacc.update_phases = std::min(6 + ctx->p, 12);
+  ctx->pacc.update_phases = kUpdPhases;
   for (int k = 0; k < 12; ++k) ctx->pacc.us_update_phase[k] = k < ctx->pacc.update_phases ? 1e-3 * (double)st[16 + k] : 0.0;
   *out = ctx->pacc;
   return TDB_OK;
