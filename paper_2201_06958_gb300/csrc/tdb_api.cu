@@ -1906,7 +1906,9 @@ tdb_status tdb_reinit(tdb_ctx* ctx, const void* V_now) {
 tdb_status tdb_get_factors(tdb_ctx* ctx, double* core, double* const* U, int* ranks) {
   if (!ctx) return TDB_ERR_INVALID_ARG;
   if (!ctx->ready) { ctx->err = "not initialised"; return TDB_ERR_STATE; }
-  if (core || U) {
+  bool all = core && U;
+  for (int n = 0; n < ctx->p; ++n) all = all && U[n];
+  if (all) {
     // packed on the device, so that one copy leaves it
     const StateViews v = state_views(ctx, false, nullptr);
     launch_state_pack(v, ctx->packed, ctx->stream);
@@ -1921,13 +1923,20 @@ tdb_status tdb_get_factors(tdb_ctx* ctx, double* core, double* const* U, int* ra
     CK(cudaMemcpyAsync(h.data(), ctx->packed, sizeof(double) * v.total, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     const double* src = h.data();
-    if (core) memcpy(core, src, sizeof(double) * v.nT);
+    memcpy(core, src, sizeof(double) * v.nT);
     src += v.nT;
     for (int n = 0; n < ctx->p; ++n) {
-      if (U && U[n]) memcpy(U[n], src, sizeof(double) * ctx->N[n] * ctx->r[n]);
+      memcpy(U[n], src, sizeof(double) * ctx->N[n] * ctx->r[n]);
       src += ctx->N[n] * ctx->r[n];
     }
   } else {
+    // part of it: what is asked for and no more
+    int64_t Rprod = 1;
+    for (int n = 0; n < ctx->p; ++n) Rprod *= ctx->r[n];
+    if (core) CK(cudaMemcpyAsync(core, ctx->T, sizeof(double) * Rprod, cudaMemcpyDeviceToHost, ctx->stream));
+    for (int n = 0; U && n < ctx->p; ++n)
+      if (U[n])
+        CK(cudaMemcpyAsync(U[n], ctx->U[n], sizeof(double) * ctx->N[n] * ctx->r[n], cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
   }
   if (ranks)
