@@ -77,9 +77,7 @@ void launch_cast(const Ts* a, Td* b, int64_t n, cudaStream_t s) {
   if (blocks < 1) blocks = 1;
   k_cast<Ts, Td><<<blocks, 256, 0, s>>>(a, b, n); count_launch();
 }
-template void launch_cast<double, float>(const double*, float*, int64_t, cudaStream_t);
 template void launch_cast<float, double>(const float*, double*, int64_t, cudaStream_t);
-template void launch_cast<double, double>(const double*, double*, int64_t, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // The snapshot difference out = scale (a - b) (scale 1, or a central difference's) and its
@@ -1099,8 +1097,5 @@ void launch_modeprod(const Tin* in, Tacc* out, const Tm* M, int64_t L, int K, in
                                                int64_t, cudaStream_t, const int*);
 INST_MP(float, float, float)
 INST_MP(double, double, double)
-INST_MP(double, float, float)
-INST_MP(float, double, double)
-INST_MP(double, double, float)
 
 }  // namespace tdb

@@ -32,16 +32,11 @@ struct WeightView {
   const double* w[kMaxModes];
 };
 
+// The weighted Cholesky-QR of freshly computed bases (k_small.cu).
 struct RowArgs {
   ModeDesc d;
-  const void* Y[kMaxModes];      // projection tensors (Tc)
-  const void* Tc;                // core in the compute type
-  const double* U[kMaxModes];
   const double* w[kMaxModes];
-  const double* Ginv;            // p x LD x LD
-  const double* P;               // p x LD x LD
   const double* Rinv;            // p x LD x LD
-  double* X[kMaxModes];
   double* Up[kMaxModes];
   double* Uout[kMaxModes];
   void* A[kMaxModes];            // weighted bases (Ta)

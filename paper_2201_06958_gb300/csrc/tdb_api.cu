@@ -131,7 +131,6 @@ struct tdb_ctx {
   double* G;
   double* Ginv;
   float* Ginvf;                   // float copy of Ginv (float compute types)
-  double* P;
   double* R;
   double* Rinv;
   double* Gpart;
@@ -413,7 +412,6 @@ void carve(tdb_ctx* c, Carver& cv) {
   c->G = cv.take<double>(p * kMaxRank * kMaxRank);
   c->Ginv = cv.take<double>(p * kMaxRank * kMaxRank);
   c->Ginvf = c->f64 ? nullptr : cv.take<float>(p * kMaxRank * kMaxRank);
-  c->P = cv.take<double>(p * kMaxRank * kMaxRank);
   c->R = cv.take<double>(p * kMaxRank * kMaxRank);
   c->Rinv = cv.take<double>(p * kMaxRank * kMaxRank);
   c->gsplit = 64;
@@ -921,7 +919,6 @@ tdb_status hosvd_state(tdb_ctx* ctx, const Tc* V, const int* ranks) {
   memset(&a, 0, sizeof(a));
   a.d = mode_desc(ctx);
   for (int n = 0; n < ctx->p; ++n) {
-    a.U[n] = ctx->U[n];
     a.w[n] = ctx->w[n];
     a.Up[n] = ctx->Up[n];
     a.Uout[n] = ctx->U[n];
