@@ -189,7 +189,7 @@ void launch_gram_weighted(const float* Vw, int64_t L, int64_t Nn, int64_t Q, dou
 
 // k_eig_modes.cu: leading eigenpairs of several symmetric positive semi-definite matrices
 constexpr int kEigBlock = 50;              // most columns of a block: 16 more than the wanted pairs (<= 34)
-constexpr int kEigSweeps = 16;             // Jacobi sweeps at most
+constexpr int kEigSweeps = 32;             // Jacobi sweeps at most
 constexpr int kEigWhole = 96;              // most points of a mode that can be solved whole
 constexpr int kEigPart = 3840;             // a group's sums: block^2 and its upper triangle, and 64
 struct EigProblem {
