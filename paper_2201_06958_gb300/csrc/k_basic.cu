@@ -812,7 +812,8 @@ __global__ void __launch_bounds__(256) k_mp_cols(const float* __restrict__ in, f
 // r_1), the next 32 on their way by cp.async.  Bound: HBM, N_1 ncol values written once.
 // 256 x 128 x 512 float at r_1 = 11, 17.7 us from a cold cache (18.3 with H through registers);
 // a whole reconstruction of 192 x 129 x 192 x 3 at r_1 = 13 31.7 us (33.0), where the product
-// of the last mode with a thread per output took 91 us, and the mode before it as long.
+// of the last mode with a thread per output took 91 us, and the mode before it as long.  A warp
+// takes eight columns at least: 64^3 float at rank 4 in 11 us, with 32 at least 15 us.
 template <typename T, int R, int RM>
 __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, const T* __restrict__ H, int r1, int N1,
                                                       unsigned ncol, int vec, T* __restrict__ V) {
@@ -867,6 +868,23 @@ __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, 
   }
 }
 
+// Mode 1 last where its rows fill a warp's lanes and the last mode does not; the mode products in
+// order, with a thread per output of the last, elsewhere.  Float, us of a reconstruction, this
+// against the products: 7 x 100 000 (rank 4) 31 to 23, 24 x 200 x 200 (4) 15 to 12, 33 x 300 x 300
+// (14) 29 to 21, 48 x 150 x 150 13 to 13, 80 x 120 x 120 12 to 13, 260 x 300 x 300 33 to 39, 192 x
+// 129 x 192 x 3 37 to 74; two modes 10 to 8.  Double runs at its arithmetic, which the products
+// share out better: 64^3 (4) 17 to 17, 130 x 300 x 300 242 to 93, 256 x 128 x 64 (14) 72 to 80; with
+// a last mode of three points next to none of it is left to them (427 to 500 us).
+template <typename T>
+bool recon_mode1_last(int p, const int64_t* N, const int* r) {
+  if (p == 2) return false;
+  const bool short_last = 4 * (int64_t)r[p - 1] >= 3 * N[p - 1];
+  if (sizeof(T) == 8) return N[0] >= 128 && short_last;
+  return N[0] >= 64 || (N[0] >= 32 && short_last);
+}
+template bool recon_mode1_last<float>(int, const int64_t*, const int*);
+template bool recon_mode1_last<double>(int, const int64_t*, const int*);
+
 template <typename T>
 void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* V, cudaStream_t s) {
   const uintptr_t va = (uintptr_t)V;
@@ -874,8 +892,8 @@ void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* 
     constexpr int R = decltype(rows)::value, RM = decltype(rmax)::value;
     const size_t sm = sizeof(T) * 8 * 2 * kChunk<T, RM> * RM;
     if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    // a warp per 32 columns of a row block at least, two CTAs per SM at most
-    const int64_t units = ((N1 + 32 * R - 1) / (32 * R)) * ((ncol + 31) / 32);
+    // a warp per eight columns of a row block at least, two CTAs per SM at most
+    const int64_t units = ((N1 + 32 * R - 1) / (32 * R)) * ((ncol + 7) / 8);
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((units + 7) / 8, 2 * 152));
     const int vec = N1 % R == 0 && va % (R * sizeof(T)) == 0;
     kern<<<blocks, 256, sm, s>>>(U1, H, r1, N1, (unsigned)ncol, vec, V);
