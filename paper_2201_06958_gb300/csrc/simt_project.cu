@@ -428,6 +428,14 @@ int64_t sp_tiles2_max(const int64_t* N, int64_t nslice) {
   return sp_shape<T>(N, r, nslice).nq2;
 }
 
+// Points that the tiles of a pass cover, over the tensor's (with one rank block).
+template <typename T>
+double sp_padding(int p, const int64_t* N) {
+  const int r[2] = {1, 1};
+  const SpShape h = sp_shape<T>(N, r, slices(p, N));
+  return (double)h.nq1 * SP_T1 / N[0] * ((double)h.nq2 * h.ti2 / N[1]);
+}
+
 template <typename T, int RB>
 void sp_launch(const SpParams<T>& P, const SpShape& h, int vec, cudaStream_t s) {
   static bool attr = false;
@@ -440,6 +448,29 @@ void sp_launch(const SpParams<T>& P, const SpShape& h, int vec, cudaStream_t s) 
 }
 
 }  // namespace
+
+// The pass against the mode products, a step of 650 random sizes each way (us, pass to products):
+// Float: faster nearly everywhere (256 x 128 x 512 at ranks (11, 8, 16) 60 to 430, 32^3 (3) 65 to 69);
+//   a short mode 2 of four wastes its tiles (64 x 3 x 64 x 64 (3) 193 to 114, 3 x 3 x 3 x 20 000 (8)
+//   2263 to 652; 64 x 64 x 3 x 64 (3) 77 to 110): the line at 20 points.
+// Double, two modes: a warp's lanes lie along mode 1 (20 x 50 000 872 to 446, 7 x 100 000 1676 to 810;
+//   200 x 200 80 to 195, 50 000 x 20 233 to 1769): the line lay between 48 and 55 points.
+// Double, three modes: modes of up to 64 points have a cheaper product (64^3 at ranks 3 and 16 86 to
+//   89 and 220 to 182, 400 x 400 x 8 (8) 231 to 157; 96^3 (3, 16) 114 to 255 and 297 to 405, 126^3 (5)
+//   100 to 410); so has a product over a long mode 2 with few slices (4 x 1000 x 250 (3) 937 to 363), and
+//   tiles that are mostly padding cost their arithmetic (5 x 300 x 300 (8) 519 to 312 at 27 times the
+//   points, 300 x 5 x 300 (8) 205 to 600 at four times).
+// Double, four modes: the finish forms r_3 r_4 outputs a slice with double's arithmetic (40 x 40 x 40 x 8
+//   (8) 375 to 185); even at 1.5 times the points.
+template <typename T>
+bool sp_worth(int p, const int64_t* N) {
+  if (sizeof(T) == 4) return p < 4 || N[1] > 20;
+  if (p == 2) return N[0] >= 52;
+  if (p == 3) return N[2] > 64 && N[1] <= 256 && sp_padding<T>(p, N) <= 30;
+  return sp_padding<T>(p, N) <= 1.5;
+}
+template bool sp_worth<float>(int, const int64_t*);
+template bool sp_worth<double>(int, const int64_t*);
 
 bool sp_supported(int p, const int* r) { return finish_outputs(p, r) <= FS_JMAX; }
 

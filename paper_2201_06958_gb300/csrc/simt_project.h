@@ -17,6 +17,9 @@ struct SpPlan {
   void* wrest = nullptr;              // W = Z1 x_2 A_2^T of four modes (r1 x r2 x N3 x N4)
 };
 
+// Whether the pass is the faster way for tensors of these sizes.
+template <typename T>
+bool sp_worth(int p, const int64_t* N);
 // Whether sp_project takes these ranks (r_3 r_4 of four modes at most 128).
 bool sp_supported(int p, const int* r);
 // The slice weights, kept for the context's life, and the buffers of a pass, free between passes.

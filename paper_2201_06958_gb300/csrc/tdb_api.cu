@@ -367,13 +367,9 @@ int rank_from_core(const double* s2, int r, double eps, double gamma_th) {
 }
 
 // Whether a context without the tensor cores projects in one fused pass (simt_project.cu).
-// Measured per projection, fused against mode products: float 256 x 128 x 512 at ranks
-// (11, 8, 16) 60 against 430 us, double 126^3 at (5, 5, 5) 100 against 410 us.  Small double
-// tensors keep the mode products: at 64^3 the pass is latency-bound on both routes (12 us
-// apart), and an error 1e-8 of ||V||_W there rests on the last bits of the double state,
-// which the mode products' order of summation has always given.
-constexpr int64_t kSpDoubleMin = (int64_t)1 << 19;
-bool sp_context(const tdb_ctx* c) { return c->prec != TDB_BF16_TTM && (!c->f64 || c->S >= kSpDoubleMin); }
+bool sp_context(const tdb_ctx* c) {
+  return c->prec != TDB_BF16_TTM && (c->f64 ? sp_worth<double>(c->p, c->N) : sp_worth<float>(c->p, c->N));
+}
 bool sp_route(const tdb_ctx* c) { return sp_context(c) && sp_supported(c->p, c->r); }
 
 // ---------------------------------------------------------------------------
