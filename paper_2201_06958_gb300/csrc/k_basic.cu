@@ -690,6 +690,27 @@ __global__ void k_mp_expand1(const Tin* __restrict__ in, Tacc* __restrict__ out,
   }
 }
 
+// K small, many outputs: a thread per output element, l fastest, K products in order.  Where the
+// lanes of a thread per (l, q) would be empty (a last mode far longer than the product of the
+// others' ranks and sizes), and for double outputs that outnumber their inputs: double runs at its
+// arithmetic, which the finest grain shares out best (reconstructions of 7 x 100 000 at rank 7 17 us
+// against 62 with eight outputs a thread, 126^3 at rank 14 65 against 72; float 7 x 100 000 12 against 25).
+template <typename Tin, typename Tm, typename Tacc>
+__global__ void __launch_bounds__(256) k_mp_expand_out(const Tin* __restrict__ in, Tacc* __restrict__ out,
+                                                       const Tm* __restrict__ M, int64_t L, int K, int J, int64_t Q,
+                                                       int64_t sMj, int64_t sMk, const int* __restrict__ gate) {
+  if (gate && *gate == 0) return;
+  const unsigned total = (unsigned)(L * J * Q), uL = (unsigned)L, uJ = (unsigned)J;
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+    const unsigned l = e % uL, jq = e / uL, j = jq % uJ, q = jq / uJ;
+    const Tin* base = in + l + (size_t)uL * K * q;
+    const Tm* mrow = M + j * sMj;
+    Tacc acc = Tacc(0);
+    for (int k = 0; k < K; ++k) acc = fma((Tacc)__ldg(&mrow[k * sMk]), (Tacc)base[(size_t)k * uL], acc);
+    out[e] = acc;
+  }
+}
+
 // K small: a thread per (l, q), l fastest, and JT consecutive outputs j: every value of `in` is
 // read once for the JT of them, their M (blockIdx.y's rows) comes from shared memory.  Each
 // output sums its K products in order whatever JT is.  Bound: the stores of L J Q values;
@@ -869,18 +890,19 @@ __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, 
 }
 
 // Mode 1 last where its rows fill a warp's lanes and the last mode does not; the mode products in
-// order, with a thread per output of the last, elsewhere.  Float, us of a reconstruction, this
-// against the products: 7 x 100 000 (rank 4) 31 to 23, 24 x 200 x 200 (4) 15 to 12, 33 x 300 x 300
-// (14) 29 to 21, 48 x 150 x 150 13 to 13, 80 x 120 x 120 12 to 13, 260 x 300 x 300 33 to 39, 192 x
-// 129 x 192 x 3 37 to 74; two modes 10 to 8.  Double runs at its arithmetic, which the products
-// share out better: 64^3 (4) 17 to 17, 130 x 300 x 300 242 to 93, 256 x 128 x 64 (14) 72 to 80; with
-// a last mode of three points next to none of it is left to them (427 to 500 us).
+// order elsewhere.  Float, us of a reconstruction, this against the products: 7 x 100 000 (rank 4)
+// 31 to 11, 24 x 200 x 200 (4) 15 to 12, 33 x 300 x 300 (14) 29 to 21, 64 x 3 x 64 x 64 (4) 30 to 20,
+// 130 x 300 x 300 (4) 27 to 25; 80 x 120 x 120 (4) 12 to 13, 260 x 300 x 300 (4) 33 to 39, 192 x 129 x
+// 192 x 3 (14) 37 to 74; two modes 10 to 8.  The lines: three fifths of the rows that a warp's blocks
+// hold, or a quarter beside a last mode that is next to uncompressed.  Double runs at its arithmetic, which the products
+// share out better: 64^3 (4) 17 to 14, 130 x 300 x 300 (4) 242 to 93, 256 x 128 x 64 (14) 72 to 72;
+// beside a last mode of three points they have little of it to share (192 x 129 x 192 x 3 427 to 451).
 template <typename T>
 bool recon_mode1_last(int p, const int64_t* N, const int* r) {
   if (p == 2) return false;
   const bool short_last = 4 * (int64_t)r[p - 1] >= 3 * N[p - 1];
   if (sizeof(T) == 8) return N[0] >= 128 && short_last;
-  return N[0] >= 64 || (N[0] >= 32 && short_last);
+  return 5 * N[0] >= 3 * 128 * ((N[0] + 127) / 128) || (N[0] >= 32 && short_last);
 }
 template bool recon_mode1_last<float>(int, const int64_t*, const int*);
 template bool recon_mode1_last<double>(int, const int64_t*, const int*);
@@ -1034,7 +1056,10 @@ void launch_modeprod(const Tin* in, Tacc* out, const Tm* M, int64_t L, int K, in
   count_launch();
   if (K <= 64) {
     const int64_t lq = L * Q;
-    if (J >= 5 && ((lq + 255) / 256) * ((J + 7) / 8) >= 2 * 152) {
+    if ((lq < 128 || (sizeof(Tacc) == 8 && J > K)) && lq * J >= 2 * 152 * 256) {
+      k_mp_expand_out<Tin, Tm, Tacc><<<(unsigned)std::min<int64_t>((lq * J + 255) / 256, 152 * 32), 256, 0, s>>>(
+          in, out, M, L, K, J, Q, sMj, sMk, gate);
+    } else if (J >= 5 && ((lq + 255) / 256) * ((J + 7) / 8) >= 2 * 152) {
       const dim3 grid((unsigned)std::min<int64_t>((lq + 255) / 256, 152 * 32), (unsigned)std::min((J + 7) / 8, 16384));
       k_mp_expand<Tin, Tm, Tacc, 8><<<grid, 256, 0, s>>>(in, out, M, L, K, J, Q, sMj, sMk, gate);
     } else if (((lq + 255) / 256) * ((J + 3) / 4) >= 2 * 152) {

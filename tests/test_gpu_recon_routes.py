@@ -16,12 +16,14 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("shift", [0, 1])
 @pytest.mark.parametrize("dims,ranks", [
     ((64, 48), (6, 6)), ((200, 9), (5, 5)),                       # two modes
-    ((63, 20, 11), (5, 4, 3)), ((64, 20, 11), (5, 4, 3)),         # the rows of float
+    ((76, 20, 11), (5, 4, 3)), ((77, 20, 11), (5, 4, 3)),         # the rows of float, one block
+    ((153, 20, 11), (5, 4, 3)), ((154, 20, 11), (5, 4, 3)),       # ... two blocks
     ((31, 20, 4), (5, 4, 3)), ((32, 20, 4), (5, 4, 3)),           # ... beside a last mode kept whole
     ((127, 9, 4), (9, 5, 3)), ((128, 9, 4), (9, 5, 3)),           # the rows of double
     ((128, 9, 5), (9, 5, 3)),                                     # a last mode that is shortened
     ((130, 7, 3), (17, 6, 3)), ((129, 3, 5, 3), (20, 3, 5, 3)),   # a ragged block, ranks above sixteen
     ((5, 40, 300), (3, 4, 5)), ((6, 5, 4, 400), (3, 3, 3, 6)),    # a short first mode
+    ((7, 20000), (7, 7)), ((16, 8, 700), (4, 4, 9)), ((127, 640), (6, 6)), ((129, 640), (6, 6)),   # outputs a thread
     ((260, 1, 9), (3, 1, 3)), ((1, 30, 20), (1, 4, 4)),
 ])
 def test_reconstruction_within_rounding(precision, dims, ranks, shift):
