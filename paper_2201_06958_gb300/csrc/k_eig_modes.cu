@@ -14,9 +14,12 @@
 //            of Q meanwhile, so no vector matrix is formed.
 //   output   the k leading columns, unit length, entry of largest magnitude positive.
 // A mode of at most m points skips the iteration (Q = I, H = C).  A mode of up to 96 points whose
-// iteration has not settled after 27 rounds is solved whole in the same way: a spectrum that
+// iteration has not settled after 30 rounds is solved whole in the same way: a spectrum that
 // hardly decays (noise) would take hundreds, and its vectors were still off by up to 0.3 in angle.
-// (A longer mode keeps the block that it has by then.)
+// (A longer mode keeps the block that it has by then.)  In the float types pairs below 1e-5 of the
+// largest eigenvalue are waited for three rounds at most once the others have settled: under a cap
+// above the rank they are noise more often than not (float 1000 x 4 x 250 at rank 4, two pairs in
+// noise: a re-initialisation 2.1 ms, waiting for them to the end 6.7 ms).
 //
 // Bound: chains of dependent double operations on one CTA (GB300 issues one double warp
 // instruction per 64 cycles per SM sub-partition), so the design cuts the number of chains
@@ -41,8 +44,9 @@ constexpr int EM_M = kEigBlock;             // most columns of a block (50)
 constexpr int EM_LD = EM_M + 1;             // leading dimension of m x m matrices in shared memory
 constexpr int EM_RC = 8;                    // rows of C Z formed at a time
 constexpr int EM_MP = (EM_M + 7) & ~7;      // columns padded to whole groups of eight (56)
-constexpr int EM_ITERS = 27;                // iterations at most
+constexpr int EM_ITERS = 30;                // iterations at most
 constexpr int EM_SWEEPS = kEigSweeps;
+constexpr double EM_TOL = 1e-15;            // off-diagonal mass left by the Jacobi
 constexpr int EM_D = kEigWhole, EM_DLD = EM_D + 1;   // most points of a mode solved whole (96)
 
 __device__ __forceinline__ unsigned em_ld_acquire(const unsigned* p) {
@@ -471,6 +475,7 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
       M.Q[(int64_t)row * mp + c] = v;
     }
     int extra = -1;                          // iterations still to do once the block has settled
+    int waited = 0;                          // iterations since the columns above M.least have
     if (!em_sync(M.bar, ++nbar, B, a.flags, &abort_sh)) return;
     for (int it = 0;; ++it) {
       em_cz(M.C, n, M.Q, mp, r_lo, nr, Zr, czr);
@@ -485,7 +490,7 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
         // tau lambda_1 / lambda_j, the perturbation of that eigenvector by the Gram's rounding.
         if (extra < 0) {
           double need = 0.0;
-          bool settled = true;
+          bool settled = true, large = true;     // every wanted column, those above M.least
           double top = 0.0, low = H[0];
           for (int j = 0; j < m; ++j) {
             const double h = fmax(H[j + EM_LD * j], 0.0);
@@ -499,6 +504,7 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
               for (int i = 0; i < m; ++i) in = fma(H[i + EM_LD * t], H[i + EM_LD * t], in);
               const double g = G[t + EM_LD * t];
               settled = g - in <= 4e-14 * g;
+              large = settled || hj <= M.least * top;
               const float aim = (float)(M.tau * 5e6 * top / hj);      // relative to the 2e-7 reached
               if (aim < 1.f) {
                 const float rate = fminf((float)(low / hj), 0.999f);
@@ -507,7 +513,10 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
             }
           }
           settled = __syncthreads_and(settled);
-          if (settled) {
+          large = __syncthreads_and(large);
+          if (!settled && large && ++waited > 3) {
+            extra = 0;
+          } else if (settled) {
             // the largest count any column asks for
             if (t < 64) red[t] = t < k ? need : 0.0;
             __syncthreads();
@@ -612,8 +621,8 @@ __global__ void __launch_bounds__(EM_T, 1) k_eig_modes(EigModes a) {
       Hd[i + dld * j] = (i < dm && j < dm) ? Hd[i + dld * j] * sc : 0.0;
     }
     __syncthreads();
-    const bool conv = dm > EM_M ? em_jacobi<5, EM_DLD>(Hd, dm, M.tol, rot, M.done, cs, pq, red)
-                                : em_jacobi<2, EM_LD>(Hd, dm, M.tol, rot, M.done, cs, pq, red);
+    const bool conv = dm > EM_M ? em_jacobi<5, EM_DLD>(Hd, dm, EM_TOL, rot, M.done, cs, pq, red)
+                                : em_jacobi<2, EM_LD>(Hd, dm, EM_TOL, rot, M.done, cs, pq, red);
     if (!conv && t == 0) atomicOr(a.flags, kFlagEigNoConv);
     // descending order by integer keys, ties by index: a permutation whatever the values
     for (int j = t; j < dm; j += EM_T) {
@@ -747,7 +756,7 @@ size_t eig_modes_scratch(int n, int k) {
          (size_t)kEigSweeps * 2 * em_sweep_pairs(n <= EM_D ? n : (int)m) + 8;
 }
 
-tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsigned* flags, cudaStream_t s) {
+tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double least, unsigned* flags, cudaStream_t s) {
   // (read once; what the device gives less than 2 KB for the kernel's static shared memory)
   struct Device {
     int nsm = 0, coop = 0;
@@ -803,7 +812,7 @@ tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsig
     M.out = pr[i].Q;
     M.trace = pr[i].trace;
     M.tau = tau;
-    M.tol = tol;
+    M.least = least;
     cudaMemsetAsync(M.bar, 0, 8 * sizeof(unsigned), s);
   }
   // (the limit, not this launch's need: another thread's launch may need more)

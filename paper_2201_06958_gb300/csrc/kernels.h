@@ -217,7 +217,7 @@ struct EigMode {
   double* ev;
   double* out;
   double* trace;
-  double tau, tol;
+  double tau, least;
 };
 struct EigModes {
   int p;
@@ -226,8 +226,9 @@ struct EigModes {
 };
 size_t eig_modes_scratch(int n, int k);
 // All p problems in one cooperative launch.  tau: relative accuracy of the matrices' entries
-// (what the iteration converges to); tol: off-diagonal mass left by the Jacobi.
-tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double tol, unsigned* flags, cudaStream_t s);
+// (what the iteration converges to); least: pairs below it, relative to the largest, are waited
+// for three rounds at most.
+tdb_status launch_eig_modes(EigProblem* pr, int p, double tau, double least, unsigned* flags, cudaStream_t s);
 
 // k_hosvd.cu
 template <typename Tv>

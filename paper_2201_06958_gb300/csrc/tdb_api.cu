@@ -897,7 +897,7 @@ tdb_status hosvd_spectrum(tdb_ctx* ctx, const Tc* V) {
   // that.  (A float eigensolver resolves eigenvectors only where the eigenvalue gaps exceed
   // about 1e-6 of the largest eigenvalue; those the rank rule keeps at gamma_th = 99.999 %
   // sit below that.)
-  const tdb_status st = launch_eig_modes(pr, ctx->p, ctx->f64 ? 2e-16 : 1e-10, 1e-15, ctx->flags, s);
+  const tdb_status st = launch_eig_modes(pr, ctx->p, ctx->f64 ? 2e-16 : 1e-10, ctx->f64 ? 0.0 : 1e-5, ctx->flags, s);
   if (st != TDB_OK) { ctx->err = "eigensolver launch failed"; return st; }
   for (int n = 0; n < ctx->p; ++n) {
     if (!short_side(ctx, n)) continue;
