@@ -692,7 +692,7 @@ __global__ void k_mp_expand1(const Tin* __restrict__ in, Tacc* __restrict__ out,
 
 // K small, many outputs: a thread per output element, l fastest, K products in order.  Where the
 // lanes of a thread per (l, q) would be empty (a last mode far longer than the product of the
-// others' ranks and sizes), and for double outputs that outnumber their inputs: double runs at its
+// others' ranks and sizes), and for double outputs that are no fewer than their inputs: double runs at its
 // arithmetic, which the finest grain shares out best (reconstructions of 7 x 100 000 at rank 7 17 us
 // against 62 with eight outputs a thread, 126^3 at rank 14 65 against 72; float 7 x 100 000 12 against 25).
 template <typename Tin, typename Tm, typename Tacc>
@@ -827,7 +827,7 @@ __global__ void __launch_bounds__(256) k_mp_cols(const float* __restrict__ in, f
   }
 }
 
-// V^TDB = U_1 H with H = T x_2 U_2 ... x_p U_p (r_1 x ncol): the last and only large product of
+// V^TDB = U_1 H in float with H = T x_2 U_2 ... x_p U_p (r_1 x ncol): the last and only large product of
 // a reconstruction.  Lane l of a warp owns R rows of a block of 32 R with U_1's in registers
 // and walks a range of columns, 32 columns' H at a time in shared memory (padded to RM, zeros past
 // r_1), the next 32 on their way by cp.async.  Bound: HBM, N_1 ncol values written once.
@@ -835,9 +835,10 @@ __global__ void __launch_bounds__(256) k_mp_cols(const float* __restrict__ in, f
 // a whole reconstruction of 192 x 129 x 192 x 3 at r_1 = 13 31.7 us (33.0), where the product
 // of the last mode with a thread per output took 91 us, and the mode before it as long.  A warp
 // takes eight columns at least: 64^3 float at rank 4 in 11 us, with 32 at least 15 us.
-template <typename T, int R, int RM>
-__global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, const T* __restrict__ H, int r1, int N1,
-                                                      unsigned ncol, int vec, T* __restrict__ V) {
+template <int R, int RM>
+__global__ void __launch_bounds__(256, 2) k_recon_out(const float* __restrict__ U1, const float* __restrict__ H, int r1,
+                                                      int N1, unsigned ncol, int vec, float* __restrict__ V) {
+  using T = float;
   constexpr int CC = kChunk<T, RM>;
   extern __shared__ __align__(16) unsigned char ro_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -869,14 +870,10 @@ __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, 
         T* o = V + (size_t)N1 * (c0 + c) + i0;
         if (vec) {
           if (i0 < N1) {
-            if constexpr (R * sizeof(T) == 16 && sizeof(T) == 4)
-              __stcs((float4*)o, make_float4(rec[0], rec[1 % R], rec[2 % R], rec[3 % R]));
-            else if constexpr (R == 2 && sizeof(T) == 4)
-              __stcs((float2*)o, make_float2(rec[0], rec[1 % R]));
-            else if constexpr (R == 2)
-              __stcs((double2*)o, make_double2(rec[0], rec[1 % R]));
+            if constexpr (R == 4)
+              __stcs((float4*)o, make_float4(rec[0], rec[1], rec[2], rec[3]));
             else
-              __stcs(o, rec[0]);
+              __stcs((float2*)o, make_float2(rec[0], rec[1]));
           }
         } else {
 #pragma unroll
@@ -894,21 +891,17 @@ __global__ void __launch_bounds__(256, 2) k_recon_out(const T* __restrict__ U1, 
 // 31 to 11, 24 x 200 x 200 (4) 15 to 12, 33 x 300 x 300 (14) 29 to 21, 64 x 3 x 64 x 64 (4) 30 to 20,
 // 130 x 300 x 300 (4) 27 to 25; 80 x 120 x 120 (4) 12 to 13, 260 x 300 x 300 (4) 33 to 39, 192 x 129 x
 // 192 x 3 (14) 37 to 74; two modes 10 to 8.  The lines: three fifths of the rows that a warp's blocks
-// hold, or a quarter beside a last mode that is next to uncompressed.  Double runs at its arithmetic, which the products
-// share out better: 64^3 (4) 17 to 14, 130 x 300 x 300 (4) 242 to 93, 256 x 128 x 64 (14) 72 to 72;
-// beside a last mode of three points they have little of it to share (192 x 129 x 192 x 3 427 to 451).
-template <typename T>
+// hold, or a quarter beside a last mode that is next to uncompressed.  Double runs at its arithmetic,
+// which the products share out better: 64^3 (4) 17 to 14, 130 x 300 x 300 (4) 242 to 93, 300 x 200 x 3
+// (12) 30 to 17; at 256 x 128 x 64 (14) 72 us each, at 192 x 129 x 192 x 3 (14) 427 to 451.
 bool recon_mode1_last(int p, const int64_t* N, const int* r) {
   if (p == 2) return false;
   const bool short_last = 4 * (int64_t)r[p - 1] >= 3 * N[p - 1];
-  if (sizeof(T) == 8) return N[0] >= 128 && short_last;
   return 5 * N[0] >= 3 * 128 * ((N[0] + 127) / 128) || (N[0] >= 32 && short_last);
 }
-template bool recon_mode1_last<float>(int, const int64_t*, const int*);
-template bool recon_mode1_last<double>(int, const int64_t*, const int*);
 
-template <typename T>
-void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* V, cudaStream_t s) {
+void launch_recon_out(const float* U1, const float* H, int r1, int N1, int64_t ncol, float* V, cudaStream_t s) {
+  using T = float;
   const uintptr_t va = (uintptr_t)V;
   auto go = [&](auto kern, auto rows, auto rmax) {
     constexpr int R = decltype(rows)::value, RM = decltype(rmax)::value;
@@ -921,19 +914,11 @@ void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* 
     kern<<<blocks, 256, sm, s>>>(U1, H, r1, N1, (unsigned)ncol, vec, V);
     count_launch();
   };
-  if constexpr (sizeof(T) == 4) {
-    if (r1 <= 8) go(k_recon_out<float, 4, 8>, IntC<4>(), IntC<8>());
-    else if (r1 <= 12) go(k_recon_out<float, 4, 12>, IntC<4>(), IntC<12>());
-    else if (r1 <= 16) go(k_recon_out<float, 4, 16>, IntC<4>(), IntC<16>());
-    else go(k_recon_out<float, 2, 32>, IntC<2>(), IntC<32>());
-  } else {
-    if (r1 <= 8) go(k_recon_out<double, 2, 8>, IntC<2>(), IntC<8>());
-    else if (r1 <= 16) go(k_recon_out<double, 2, 16>, IntC<2>(), IntC<16>());
-    else go(k_recon_out<double, 1, 32>, IntC<1>(), IntC<32>());
-  }
+  if (r1 <= 8) go(k_recon_out<4, 8>, IntC<4>(), IntC<8>());
+  else if (r1 <= 12) go(k_recon_out<4, 12>, IntC<4>(), IntC<12>());
+  else if (r1 <= 16) go(k_recon_out<4, 16>, IntC<4>(), IntC<16>());
+  else go(k_recon_out<2, 32>, IntC<2>(), IntC<32>());
 }
-template void launch_recon_out<float>(const float*, const float*, int, int, int64_t, float*, cudaStream_t);
-template void launch_recon_out<double>(const double*, const double*, int, int, int64_t, double*, cudaStream_t);
 
 // H = T x_2 U_2 x_3 U_3 (x_4 U_4) in float, r_1 x N_2 x slices, in one launch: a CTA forms the
 // r_1 x r_2 slice G = sum_j T[:, :, j] c_j, c_j = U_3[i_3, c] U_4[i_4, d] over the J = r_3 r_4
@@ -1056,7 +1041,7 @@ void launch_modeprod(const Tin* in, Tacc* out, const Tm* M, int64_t L, int K, in
   count_launch();
   if (K <= 64) {
     const int64_t lq = L * Q;
-    if ((lq < 128 || (sizeof(Tacc) == 8 && J > K)) && lq * J >= 2 * 152 * 256) {
+    if ((lq < 128 || (sizeof(Tacc) == 8 && J >= K)) && lq * J >= 2 * 152 * 256) {
       k_mp_expand_out<Tin, Tm, Tacc><<<(unsigned)std::min<int64_t>((lq * J + 255) / 256, 152 * 32), 256, 0, s>>>(
           in, out, M, L, K, J, Q, sMj, sMk, gate);
     } else if (J >= 5 && ((lq + 255) / 256) * ((J + 7) / 8) >= 2 * 152) {

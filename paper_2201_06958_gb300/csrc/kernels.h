@@ -129,12 +129,10 @@ template <typename T>
 void launch_recon_err(const T* V, const T* U1, const T* H, int r1, int N1, int64_t ncol, const T* w1, const T* wcol,
                       double* partial, unsigned* counter, int nblocks, double* out, unsigned* flags, cudaStream_t s,
                       const int* gate = nullptr);
-// Whether a reconstruction takes mode 1 last, in launch_recon_out
-template <typename T>
+// Whether a float reconstruction takes mode 1 last, in launch_recon_out
 bool recon_mode1_last(int p, const int64_t* N, const int* r);
 // V = U1 H (N1 x ncol; H: r1 x ncol)
-template <typename T>
-void launch_recon_out(const T* U1, const T* H, int r1, int N1, int64_t ncol, T* V, cudaStream_t s);
+void launch_recon_out(const float* U1, const float* H, int r1, int N1, int64_t ncol, float* V, cudaStream_t s);
 // H = T x_2 U_2 ... x_p U_p in one launch (three and four modes of few enough products), or false
 bool launch_core_cols(const float* T, const float* const* U, int p, const int64_t* N, const int* r, float* H,
                       cudaStream_t s, const int* gate);

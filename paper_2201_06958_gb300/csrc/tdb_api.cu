@@ -692,27 +692,29 @@ const Tc* column_factors(tdb_ctx* ctx, const int* gate) {
 // of S values reads H and writes V^TDB once, or the modes in order.
 template <typename Tc>
 tdb_status reconstruct_into(tdb_ctx* ctx, Tc* out) {
-  if (!recon_mode1_last<Tc>(ctx->p, ctx->N, ctx->r)) {
-    const int p = ctx->p;
-    int64_t cur[kMaxModes];
-    for (int m = 0; m < p; ++m) cur[m] = ctx->r[m];
-    const Tc* src = (const Tc*)ctx->Tcore;
-    Tc* bufs[2] = {(Tc*)ctx->ping, (Tc*)ctx->pong};
-    for (int n = 0; n < p; ++n) {
-      Tc* dst = n == p - 1 ? out : bufs[n & 1];
-      int64_t L = 1, Q = 1;
-      for (int m = 0; m < n; ++m) L *= cur[m];
-      for (int m = n + 1; m < p; ++m) Q *= cur[m];
-      launch_modeprod<Tc, Tc, Tc>(src, dst, (const Tc*)ctx->Uc[n], L, ctx->r[n], (int)ctx->N[n], Q, 1, ctx->N[n],
-                                  ctx->stream);
-      cur[n] = ctx->N[n];
-      src = dst;
+  const int p = ctx->p;
+  cudaStream_t s = ctx->stream;
+  if constexpr (sizeof(Tc) == 4) {
+    if (recon_mode1_last(p, ctx->N, ctx->r)) {
+      const Tc* H = column_factors<Tc>(ctx, nullptr);
+      launch_recon_out((const Tc*)ctx->Uc[0], H, ctx->r[0], (int)ctx->N[0], ctx->S / ctx->N[0], out, s);
+      CHECK_LAUNCH();
+      return TDB_OK;
     }
-    CHECK_LAUNCH();
-    return TDB_OK;
   }
-  const Tc* H = column_factors<Tc>(ctx, nullptr);
-  launch_recon_out<Tc>((const Tc*)ctx->Uc[0], H, ctx->r[0], (int)ctx->N[0], ctx->S / ctx->N[0], out, ctx->stream);
+  int64_t cur[kMaxModes];
+  for (int m = 0; m < p; ++m) cur[m] = ctx->r[m];
+  const Tc* src = (const Tc*)ctx->Tcore;
+  Tc* bufs[2] = {(Tc*)ctx->ping, (Tc*)ctx->pong};
+  for (int n = 0; n < p; ++n) {
+    Tc* dst = n == p - 1 ? out : bufs[n & 1];
+    int64_t L = 1, Q = 1;
+    for (int m = 0; m < n; ++m) L *= cur[m];
+    for (int m = n + 1; m < p; ++m) Q *= cur[m];
+    launch_modeprod<Tc, Tc, Tc>(src, dst, (const Tc*)ctx->Uc[n], L, ctx->r[n], (int)ctx->N[n], Q, 1, ctx->N[n], s);
+    cur[n] = ctx->N[n];
+    src = dst;
+  }
   CHECK_LAUNCH();
   return TDB_OK;
 }
