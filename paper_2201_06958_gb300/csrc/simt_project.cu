@@ -449,24 +449,28 @@ void sp_launch(const SpParams<T>& P, const SpShape& h, int vec, cudaStream_t s) 
 
 }  // namespace
 
-// The pass against the mode products, a step of 650 random sizes each way (us, pass to products):
+// The pass against the mode products, a step of 800 sizes each way (us, pass to products):
 // Float: faster nearly everywhere (256 x 128 x 512 at ranks (11, 8, 16) 60 to 430, 32^3 (3) 65 to 69);
 //   a short mode 2 of four wastes its tiles (64 x 3 x 64 x 64 (3) 193 to 114, 3 x 3 x 3 x 20 000 (8)
-//   2263 to 652; 64 x 64 x 3 x 64 (3) 77 to 110): the line at 20 points.
+//   2263 to 652; 64 x 64 x 3 x 64 (3) 77 to 110), and so does one of three with many slices (5 x 5 x
+//   42 223 (5) 1004 to 726, 35 x 4 x 7332 (27) 459 to 294; 31 x 9 x 738 (9) 108 to 125): the line at
+//   20 points, and 4096 slices with three modes.
 // Double, two modes: a warp's lanes lie along mode 1 (20 x 50 000 872 to 446, 7 x 100 000 1676 to 810;
 //   200 x 200 80 to 195, 50 000 x 20 233 to 1769): the line lay between 48 and 55 points.
-// Double, three modes: modes of up to 64 points have a cheaper product (64^3 at ranks 3 and 16 86 to
-//   89 and 220 to 182, 400 x 400 x 8 (8) 231 to 157; 96^3 (3, 16) 114 to 255 and 297 to 405, 126^3 (5)
-//   100 to 410); so has a product over a long mode 2 with few slices (4 x 1000 x 250 (3) 937 to 363), and
-//   tiles that are mostly padding cost their arithmetic (5 x 300 x 300 (8) 519 to 312 at 27 times the
-//   points, 300 x 5 x 300 (8) 205 to 600 at four times).
+// Double, three modes: a last mode of up to 64 points has a cheaper product (64^3 at ranks 3 and 16 86
+//   to 89 and 220 to 182, 400 x 400 x 8 (8) 231 to 157; 96^3 (3, 16) 114 to 269 and 297 to 459, 126^3 (5)
+//   100 to 410).  Above that, tiles that are mostly padding cost their arithmetic (13 x 4 x 1928 (10)
+//   634 to 156 at 39 times the points, 19 x 9 x 10 281 (6) 1557 to 5554 at twelve); beside a mode 2 that
+//   fills its tiles a short mode 1 does already (41 x 582 x 116 (16) 1645 to 1063, 224 x 332 x 97 (4) 412
+//   to 660); and a mode 1 of seven tiles and more is cheap for the products (9633 x 4 x 85 (6) 987
+//   to 834).
 // Double, four modes: the finish forms r_3 r_4 outputs a slice with double's arithmetic (40 x 40 x 40 x 8
 //   (8) 375 to 185); even at 1.5 times the points.
 template <typename T>
 bool sp_worth(int p, const int64_t* N) {
-  if (sizeof(T) == 4) return p < 4 || N[1] > 20;
+  if (sizeof(T) == 4) return p == 2 || N[1] > 20 || (p == 3 && N[2] <= 4096);
   if (p == 2) return N[0] >= 52;
-  if (p == 3) return N[2] > 64 && N[1] <= 256 && sp_padding<T>(p, N) <= 30;
+  if (p == 3) return N[2] > 64 && (N[1] <= 256 ? N[0] <= 7 * SP_T1 && sp_padding<T>(p, N) <= 30 : N[0] >= 48);
   return sp_padding<T>(p, N) <= 1.5;
 }
 template bool sp_worth<float>(int, const int64_t*);

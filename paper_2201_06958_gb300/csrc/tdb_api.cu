@@ -588,10 +588,12 @@ tdb_status project_tree(tdb_ctx* ctx, const Tc* dV, cudaEvent_t* evm) {
   };
   Tc* ping = (Tc*)ctx->ping;
   Tc* pong = (Tc*)ctx->pong;
-  if (p == 3 && ctx->aux && ctx->ev_fork && ctx->ev_join) {
+  if (p == 3 && ctx->N[2] <= 64 && ctx->aux && ctx->ev_fork && ctx->ev_join) {
     // Three modes: six launches, each too small to fill the GPU, in two chains on the context's
     // streams: Z1 = dV x_1 A_1^T, Y_3, dS beside dV x_2 A_2^T, Y_1 and (once Z1 is there) Y_2.
-    // 64^3 double: 67 us, one after another 86 us.
+    // 64^3 double: 67 us, one after another 86 us.  (The contraction of a longer last mode is a
+    // long launch of few CTAs that shares the SMs badly: a step of 1000 x 4 x 250 at rank 14 533 us
+    // in two chains, 346 in one.)
     for (int m = 0; m < p; ++m) dims[m] = ctx->N[m];
     int64_t side[kMaxModes];
     for (int m = 0; m < p; ++m) side[m] = ctx->N[m];

@@ -11,13 +11,15 @@ pytestmark = pytest.mark.gpu
 DOUBLE = [
     ((51, 40), (6, 6), 0), ((52, 40), (6, 6), 0), ((53, 31), (17, 17), 1),         # two modes
     ((30, 20, 64), (5, 4, 6), 0), ((30, 20, 65), (5, 4, 6), 0),                    # the last of three
-    ((40, 256, 65), (9, 17, 5), 0), ((40, 257, 65), (9, 17, 5), 0),                # the middle
+    ((40, 256, 65), (9, 17, 5), 0), ((47, 257, 65), (9, 17, 5), 0), ((48, 257, 65), (9, 17, 5), 0),   # the middle
+    ((896, 4, 66), (7, 4, 5), 0), ((897, 4, 66), (7, 4, 5), 0),                    # a long first
     ((8, 33, 70), (3, 9, 5), 0), ((9, 9, 70), (3, 9, 5), 0), ((3, 9, 70), (3, 9, 5), 1),   # padding of 30 times
     ((131, 65, 66), (8, 3, 4), 0), ((128, 128, 65), (5, 5, 5), 0), ((128, 250, 66), (4, 4, 4), 1),
     ((130, 129, 65), (9, 17, 5), 0), ((19076, 28), (6, 6), 1),
     ((120, 64, 5, 3), (6, 5, 4, 3), 0), ((120, 60, 5, 3), (6, 5, 4, 3), 0), ((85, 64, 5, 3), (6, 5, 4, 3), 0),
 ]
 FLOAT = [
+    ((7, 20, 4096), (3, 4, 5), 0), ((7, 20, 4097), (3, 4, 5), 0), ((7, 21, 4097), (3, 4, 5), 1),
     ((40, 20, 9, 7), (6, 5, 4, 3), 0), ((40, 21, 9, 7), (6, 5, 4, 3), 0), ((5, 3, 4, 90), (3, 3, 3, 6), 1),
 ]
 
