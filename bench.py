@@ -457,13 +457,14 @@ def run_tdb(args, world, rank, local):
         lib.tdb_get_profile(c.ctx, C.byref(prof))
         lib.tdb_set_profiling(c.ctx, 0)
         counters = c.counters()
+        route = c.projection_route()
         try:
             tuning = c.tuning() if prec == "bf16" else None
         except tdb.TDBError:
             tuning = None
         c.close()
         return {"ms": ms, "host_s": t_host, "eps": eps, "prof": prof, "clocks": clocks, "launches": launches,
-                "counters": counters, "acts": acts, "tuning": tuning}
+                "counters": counters, "acts": acts, "tuning": tuning, "route": route}
 
     # timed run: recorded steps, no instrumentation; then a profiled run of the same stream
     # (CUDA events around each phase and the projection kernel, recorded into the step's graph
@@ -486,6 +487,8 @@ def run_tdb(args, world, rank, local):
     kernel_ms = prof.ms_project_main / max(prof.launches_main, 1)
     if precision == "bf16":
         kname, kfiles = "tc_project", ["tc_project.cu"]
+    elif resp["route"] == "fused pass":
+        kname, kfiles = "sp_project", ["simt_project.cu"]
     else:
         kname, kfiles = "mode-1 product", ["k_basic.cu"]
         alg_bytes = esz * S_el                      # the mode-1 product reads the materialised difference once

@@ -386,6 +386,13 @@ tdb_status tdb_selftest_timeout(int which, int64_t limit_cycles, unsigned* scrat
 tdb_status tdb_selftest_eig_split(int nmodes, const int* n, const int* k, int num_sms, int64_t smem_bytes, int* ctas,
                                   int64_t* smem);
 
+/* How a step of this context projects at its present ranks (no counterpart in the paper): 0 on the
+ * tensor cores (TDB_BF16_TTM), 1 in the fused float or double pass, 2 by mode products; -1 for a
+ * NULL context.  tdb_profile's ms_project_main times that route's main kernel: both first
+ * contractions of the snapshot difference (0, 1), or the mode-1 product of the difference as it
+ * lies in memory (2). */
+int tdb_projection_route(const tdb_ctx* ctx);
+
 /* The launch shape the tensor-core projection's tuner chose for this context (TDB_BF16_TTM
  * only; the paper has no counterpart).  The tile is fixed (128 x 128, eight strips); the
  * tuner times, on the context's first step outside stream capture, each candidate number

@@ -2461,6 +2461,11 @@ tdb_status tdb_get_graph_counters(const tdb_ctx* ctx, const tdb_batch* b, int64_
 
 void tdb_batch_destroy(tdb_batch* b) { delete b; }
 
+int tdb_projection_route(const tdb_ctx* ctx) {
+  if (!ctx) return -1;
+  return ctx->use_tc ? 0 : (sp_route(ctx) ? 1 : 2);
+}
+
 tdb_status tdb_tc_tuning(const tdb_ctx* ctx, int* ctas, int* fin_target, int* ncand, int* cand, float* cand_us,
                          int* fin_cand, float* fin_us) {
   if (!ctx) return TDB_ERR_INVALID_ARG;

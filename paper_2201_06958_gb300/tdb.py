@@ -110,7 +110,7 @@ EXPORTS = [
     "tdb_estimator_params", "tdb_estimator_trace", "tdb_set_input_slots", "tdb_push_slot",
     "tdb_batch_create", "tdb_batch_push", "tdb_batch_last_error", "tdb_batch_destroy", "tdb_get_graph_counters",
     "tdb_selftest_recip", "tdb_selftest_timeout", "tdb_tc_tuning", "tdb_estimator_load_trace",
-    "tdb_selftest_eig_split",
+    "tdb_selftest_eig_split", "tdb_projection_route",
 ]
 
 
@@ -185,6 +185,8 @@ def load(path: str = LIB_PATH):
     lib.tdb_tc_tuning.argtypes = [vp, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int),
                                   C.POINTER(C.c_int), C.POINTER(C.c_float), C.POINTER(C.c_int), C.POINTER(C.c_float)]
     lib.tdb_tc_tuning.restype = st
+    lib.tdb_projection_route.argtypes = [vp]
+    lib.tdb_projection_route.restype = C.c_int
     lib.tdb_selftest_recip.argtypes = [vp, vp, vp, C.c_int64, vp]
     lib.tdb_selftest_recip.restype = st
     lib.tdb_selftest_timeout.argtypes = [C.c_int, C.c_int64, vp, vp]
@@ -417,6 +419,10 @@ class TDB:
         self._check(self.lib.tdb_get_graph_counters(self.ctx, None, C.byref(g), C.byref(gr)))
         return {"steps": s.value, "reinits": r.value, "exact_evals": e.value, "graph_replays": g.value,
                 "graph_records": gr.value}
+
+    def projection_route(self) -> str:
+        """How a step projects at the present ranks (tdb_projection_route)."""
+        return ("tensor cores", "fused pass", "mode products")[self.lib.tdb_projection_route(self.ctx)]
 
     def tuning(self) -> dict:
         """The tensor-core projection's launch shape (tdb_tc_tuning): CTAs per tile position,

@@ -5,6 +5,7 @@ them, against the oracle."""
 import pytest
 
 import test_gpu_projection as base
+from paper_2201_06958_gb300 import tdb
 
 pytestmark = pytest.mark.gpu
 
@@ -27,3 +28,17 @@ FLOAT = [
 @pytest.mark.parametrize("precision,dims,ranks,shift", [("fp64", *c) for c in DOUBLE] + [("fp32", *c) for c in FLOAT])
 def test_both_routes_within_rounding(precision, dims, ranks, shift):
     base.test_projection_and_error_within_rounding(precision, dims, ranks, shift)
+
+
+@pytest.mark.parametrize("precision,dims,ranks,route", [
+    ("bf16", (40, 30, 20), (4, 4, 4), "tensor cores"), ("fp32", (40, 30, 20), (4, 4, 4), "fused pass"),
+    ("fp32", (16, 21, 16, 16), (6, 6, 11, 11), "fused pass"), ("fp32", (16, 21, 16, 16), (6, 6, 12, 12), "mode products"),
+    ("fp64", (52, 40), (6, 6), "fused pass"), ("fp64", (51, 40), (6, 6), "mode products"),
+    ("fp64", (30, 20, 65), (4, 4, 4), "fused pass"), ("fp64", (30, 20, 64), (4, 4, 4), "mode products"),
+])
+def test_route_by_shape(precision, dims, ranks, route):
+    w, U, T, V0, _ = base._case(dims, ranks, 3, precision != "fp64")
+    c = tdb.TDB(dims, ranks, weights=w, precision=precision)
+    c.init_from_factors(T, U, base._device(V0, c.dtype, 0))
+    assert c.projection_route() == route
+    c.close()
