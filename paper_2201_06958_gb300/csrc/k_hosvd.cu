@@ -259,7 +259,7 @@ __global__ void k_col_unit_sign(double* __restrict__ Q, int64_t n) {
     long long i0 = bi[0];
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
       if (bv[w] > b0 || (bv[w] == b0 && bi[w] < i0)) { b0 = bv[w]; i0 = bi[w]; }
-    imax = i0;
+    imax = i0 < n ? i0 : 0;      // (a column without a comparable entry has no largest one)
   }
   __syncthreads();
   const double sc = (q[imax] < 0.0 ? -1.0 : 1.0) / sqrt(nrm > 0.0 ? nrm : 1.0);
