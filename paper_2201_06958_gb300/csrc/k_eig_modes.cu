@@ -26,9 +26,9 @@
 // (iterations, factors, Jacobi sweeps) and runs the modes' chains side by side; the products
 // are spread over all CTAs.  The result is a function of C alone, summed in a fixed order.
 //
-// Measured, all modes of a re-initialisation: 256 x 128 x 512 float (k = 18, 13, 10) 1.07 ms,
+// Measured, all modes of a re-initialisation: 256 x 128 x 512 float (k = 18, 13, 10) 1.11 ms,
 // where a float subspace iteration refined by double iterations and a one-CTA Jacobi, mode
-// after mode in 130 launches, took 6.0 ms; 126^3 double (k = 7) 0.34 ms, where 24 iterations
+// after mode in 130 launches, took 6.0 ms; 126^3 double (k = 7) 0.35 ms, where 24 iterations
 // of single launches took 11.2 ms; 90^3 double against a one-CTA Jacobi of the whole Gram, a
 // re-initialisation 1.1 against 76 ms.
 #include "common.cuh"

@@ -8,8 +8,9 @@
 //
 // Bound: float by latency (12 warps an SM of one group after the other: loads, then products
 // through shared memory), double by its arithmetic (two lanes per clock and SM).  256 x 128 x
-// 512 float at ranks (11, 8, 16): 53 us (58 with the sums of Z1 over the lanes formed by a
-// butterfly of 31 shuffles and nothing fetched ahead), where difference, norm and the mode
+// 512 float at ranks (11, 8, 16): 56 us, 53 with ||dV||^2 summed in single floats, which cost the
+// norm its last bits (58 so with the sums of Z1 over the lanes formed by a butterfly of 31 shuffles
+// and nothing fetched ahead), where difference, norm and the mode
 // products that contract S points took 428 us; 126^3 double at (5, 5, 5): 87 us against 251
 // us.  One CTA of eight warps per SM with the next rows prefetched into registers measured the
 // same as three of four without.
